@@ -221,130 +221,72 @@ __device__ __forceinline__ int fx_chol_bad(const fx &p00, const fx &det) {
     return fx_pivot_bad(det);
 }
 
-// floor(A R / 2^64) for A < 2^127 and R < 2^64 (limbs of columns 2..5 of the 192-bit
-// product); the partial products of columns 0 and 1 are dropped (result low by <= 3)
-__device__ __forceinline__ fx fx_mul_r64(const fx &a, unsigned long long R) {
-    const uint32_t r0 = (uint32_t)R, r1 = (uint32_t)(R >> 32);
-    fx q;
-    asm("mul.lo.u32 %0, %6, %8;\n\t"
-        "mul.lo.u32 %1, %7, %8;\n\t"
-        "mad.hi.cc.u32 %0, %5, %8, %0;\n\t"
-        "madc.hi.cc.u32 %1, %6, %8, %1;\n\t"
-        "madc.hi.u32 %2, %7, %8, 0;\n\t"
-        "mad.lo.cc.u32 %0, %5, %9, %0;\n\t"
-        "madc.lo.cc.u32 %1, %6, %9, %1;\n\t"
-        "madc.lo.cc.u32 %2, %7, %9, %2;\n\t"
-        "addc.u32 %3, 0, 0;\n\t"
-        "mad.hi.cc.u32 %0, %4, %9, %0;\n\t"
-        "madc.hi.cc.u32 %1, %5, %9, %1;\n\t"
-        "madc.hi.cc.u32 %2, %6, %9, %2;\n\t"
-        "madc.hi.u32 %3, %7, %9, %3;"
-        : "=&r"(q.w[0]), "=&r"(q.w[1]), "=&r"(q.w[2]), "=&r"(q.w[3])
-        : "r"(a.w[0]), "r"(a.w[1]), "r"(a.w[2]), "r"(a.w[3]), "r"(r0), "r"(r1));
-    return q;
-}
-
-// x^{-1/2} for x in [2^-16, 2^16) (pivots lie in [2^-8, 4]), built for a short
-// dependency chain (Newton's iteration r <- r + r e / 2, e = 1 - x r^2):
-//  * x = x_m 4^h with x_m = W / 2^64 in [1/4, 1), W the 64 bits after the leading zeros;
-//  * an FP32 estimate of r = x_m^{-1/2} in (1, 2] (~22 bits);
-//  * two Newton steps on W in 64-bit integer arithmetic, R = r 2^61 (~56 bits);
-//  * one Newton step against the whole of x: e from the top 128 bits of X R^2 (X the
-//    normalised 128-bit x), then y += y e / 2 (error ~ (3/2) e^2 + truncation 2^-110).
-// Inputs outside the range (checked by the callers) give a finite, meaningless result.
-static __device__ __noinline__ fx fx_rsqrt(fx x) {
-    uint32_t lz = __clz(x.w[3]);
-    lz = lz < 1u ? 1u : (lz > 31u ? 31u : lz);
-    int k = 16 - (int)lz;  // x = (W / 2^64) 2^k
-    unsigned long long W = ((unsigned long long)__funnelshift_l(x.w[2], x.w[3], lz) << 32) |
-                           __funnelshift_l(x.w[1], x.w[2], lz);
-    const int odd = k & 1;
-    W >>= odd;
-    k += odd;
-    const int h = k / 2;
-    // FP32 estimate, turned into R = r 2^61 through its bits
-    const float rf = rsqrtf(__uint2float_rn((uint32_t)(W >> 32)) * 0x1p-32f);
-    const uint32_t fb = __float_as_uint(rf);
-    int s0 = (int)((fb >> 23) & 0xffu) - 127 + 38;
-    s0 = s0 < 0 ? 0 : (s0 > 39 ? 39 : s0);
-    unsigned long long R = (unsigned long long)((fb & 0x7fffffu) | 0x800000u) << s0;
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        const unsigned long long S = __umul64hi(R, R);         // r^2 2^58
-        const unsigned long long P = __umul64hi(W, S);         // x_m r^2 2^58
-        const long long E = (long long)((1ull << 58) - P);     // e 2^58
-        R += (unsigned long long)__mul64hi((long long)R, (long long)((unsigned long long)E << 5));
-    }
-    // y = r 2^-h in Q16.112: Y = R 2^(51 - h)
-    int s2 = 19 - h;
-    s2 = s2 < 11 ? 11 : (s2 > 26 ? 26 : s2);
-    const uint32_t q0 = (uint32_t)R, q1 = (uint32_t)(R >> 32);
-    const fx y{{0u, q0 << s2, __funnelshift_l(q0, q1, s2), q1 >> (32 - s2)}};
-    // e = 1 - x y^2 = 1 - T2 2^(-121 - odd), T2 = top 128 bits of X_n R^2, X_n = X 2^(lz - 1)
-    const int sx = (int)lz - 1;
-    const fx xn{{x.w[0] << sx, __funnelshift_l(x.w[0], x.w[1], sx), __funnelshift_l(x.w[1], x.w[2], sx),
-                 __funnelshift_l(x.w[2], x.w[3], sx)}};
-    const fx t2 = fx_mul_r64(fx_mul_r64(xn, R), R);
-    const int se = 9 + odd;  // e in units of 2^-112: its low 64 bits suffice (|e| < 2^-50)
-    const unsigned long long tl = ((unsigned long long)__funnelshift_r(t2.w[1], t2.w[2], se) << 32) |
-                                  __funnelshift_r(t2.w[0], t2.w[1], se);
-    const long long E = -(long long)tl;
-    // y e / 2 in units of 2^-112: R E 2^(-62 - h)
-    const unsigned long long plo = R * (unsigned long long)E;
-    const long long phi = __mul64hi((long long)R, E);
-    int sd = 62 + h;
-    sd = sd < 55 ? 55 : (sd > 70 ? 70 : sd);
-    const long long dlt = sd < 64 ? (long long)(((unsigned long long)phi << (64 - sd)) | (plo >> sd))
-                                  : (phi >> (sd - 64));
+// x^{-1/2} in Q16.112 for a packed x with ulp 2^-(127 - h0) (h0 = 15: Q16.112; h0 = 13: ulp
+// 2^-114) in [2^-11, 2^11); pivots lie in [2^-9, 25].
+//  * x = m 4^h', m in [1/2, 2): an odd shift s of X (m = 1 for the powers of four, which stay exact);
+//  * an FP32 estimate r0 of r = m^{-1/2} (relative error below 2^-22), 24 bits, scale 30;
+//  * one step of third order on the top 64 bits W of m: with e = 1 - m r0^2, r = r0 (1 + e/2 +
+//    3/8 e^2) leaves 5/16 e^3 < 2^-64, so one step stands for the two Newton steps a quadratic
+//    iteration needs: R = r 2^62 to 2^-61;
+//  * one Newton step against the whole of x: with |e| < 2^-59 known, only the bits of m R^2 below
+//    2^-59 are formed (columns 3, 4 and the low half of 5 of X R^2: nine products instead of two
+//    full 128 x 64 ones), E = e 2^121, and y += y e / 2.
+// The result is within 1.1 units of 2^-112 (a big-integer emulation over [2^-10, 2^5]); exact for
+// powers of four.  Inputs outside the range (checked by the callers) give a finite, meaningless
+// result.
+static __device__ __noinline__ fx fx_rsqrt_at(fx x, int h0) {
+    int lz = __clz((int)x.w[3]);
+    lz = lz < 3 ? 3 : (lz > 31 ? 31 : lz);
+    const int s = (lz - 1) | 1;
+    const int h = (h0 - s) >> 1;
+    const unsigned long long W = ((unsigned long long)__funnelshift_l(x.w[2], x.w[3], s) << 32) |
+                                 __funnelshift_l(x.w[1], x.w[2], s);
+    const int sx = s - 2;
+    const uint32_t x0 = x.w[0] << sx, x1 = __funnelshift_l(x.w[0], x.w[1], sx),
+                   x2 = __funnelshift_l(x.w[1], x.w[2], sx), x3 = __funnelshift_l(x.w[2], x.w[3], sx);
+    const uint32_t fb = __float_as_uint(rsqrtf(__uint2float_rn((uint32_t)(W >> 32)) * 0x1p-31f));
+    const uint32_t r0 = ((fb & 0x7fffffu) | 0x800000u) << (((fb >> 23) - 120u) & 7u);
+    const unsigned long long P = __umul64hi(W, ((unsigned long long)r0 * r0) << 2);  // m r0^2 2^61
+    const long long E0 = (long long)((1ull << 61) - P);
+    const int e32 = (int)(E0 >> 11);
+    const int t = (int)(((long long)e32 * e32) >> 32);  // e^2 2^68
+    const long long D = E0 + ((3 * t) >> 9);            // (e/2 + 3/8 e^2) 2^62
+    const unsigned long long R = ((unsigned long long)r0 << 32) +
+                                 (((unsigned long long)((long long)(int)r0 * (int)(D >> 32))) << 2) +
+                                 (((unsigned long long)r0 * (uint32_t)D) >> 30);
+    // Q = R^2, 128 bits
+    const uint32_t ra = (uint32_t)R, rb = (uint32_t)(R >> 32);
+    const unsigned long long aa = (unsigned long long)ra * ra, ab = (unsigned long long)ra * rb,
+                             bb = (unsigned long long)rb * rb;
+    const unsigned long long mid = (ab << 1) + (aa >> 32);  // ab < 2^63: no carry lost
+    const unsigned long long top = bb + (mid >> 32) + ((mid < (aa >> 32)) ? (1ull << 32) : 0ull);
+    const uint32_t q0 = (uint32_t)aa, q1 = (uint32_t)mid, q2 = (uint32_t)top, q3 = (uint32_t)(top >> 32);
+    const unsigned long long S = ((unsigned long long)__umulhi(x0, q3) + __umulhi(x1, q2)) +
+                                 ((unsigned long long)__umulhi(x2, q1) + __umulhi(x3, q0)) +
+                                 (unsigned long long)x1 * q3 + (unsigned long long)x2 * q2 +
+                                 (unsigned long long)x3 * q1 + ((unsigned long long)(x2 * q3 + x3 * q2) << 32);
+    const long long E = -(long long)S;  // e 2^121 modulo 2^64
+    // y = r 2^-h in Q16.112: R 2^(50 - h), plus R E 2^(-72 - h)
+    int s2 = 18 - h;
+    s2 = s2 > 26 ? 26 : s2;
+    const long long dlt = __mul64hi((long long)R, E) >> (8 + h);
     const uint32_t ext = (uint32_t)(dlt >> 63);
-    return y + fx{{(uint32_t)dlt, (uint32_t)((unsigned long long)dlt >> 32), ext, ext}};
+    return fx{{0u, ra << s2, __funnelshift_l(ra, rb, s2), rb >> (32 - s2)}} +
+           fx{{(uint32_t)dlt, (uint32_t)((unsigned long long)dlt >> 32), ext, ext}};
 }
+__device__ __forceinline__ fx fx_rsqrt(const fx &x) { return fx_rsqrt_at(x, 15); }
 // det of the SPD 2x2 block [[p00, p01], [p01, p11]]
 __device__ __forceinline__ fx fx_det2(const fx &p00, const fx &p01, const fx &p11) {
     const fx a = fx_abs(p01);
     return fx_mul_uu(p00, p11) - fx_mul_uu(a, a);
 }
 
-// Symmetric form of the 2x2 block elimination used by the fixed-point sweep.  With
+// Symmetric form of the 2x2 block elimination used by the fixed-point sweeps.  With
 // the pivot block P = R R^T (R lower triangular, 1/r00 = a, r10, 1/r11 = b), the
 // Schur update C - B P^{-1} B^T equals C - U U^T, U = B R^{-T}: row i of U is
 // u0 = b_i0 a, u1 = (b_i1 - r10 u0) b = b_i1 b - u0 c with c = r10 b = p01 det^{-1/2}
-// (two products side by side).  |u_ik| <= sqrt(c_ii) <= sqrt(2), so the rows
-// are stored offset, u' = u + 2 > 0, and each entry needs two unsigned products:
-//   c_ij - u_i . u_j = c_ij - (u'_i0 u'_j0 + u'_i1 u'_j1) + t_i + t_j,  t = 2 (u'0 + u'1) - 4.
-struct fx_piv {
-    fx a, c, b, rs, det;
-};
-// the Cholesky quantities from a = p00^{-1/2} and rs = det^{-1/2} (independent, so the
-// two rsqrts need not wait for each other): b = x^{-1/2} = rs sqrt(p00) = rs p00 a
-__device__ __forceinline__ fx_piv fx_pivot_from(const fx &p00, const fx &p01, const fx &det, const fx &a,
-                                               const fx &rs) {
-    fx_piv v;
-    v.a = a;
-    v.rs = rs;
-    v.det = det;
-    v.c = fx_mul_su(p01, rs);
-    v.b = fx_mul_uu(rs, fx_mul_uu(p00, a));
-    return v;
-}
-__device__ __forceinline__ fx_piv fx_pivot(const fx &p00, const fx &p01, const fx &p11) {
-    const fx det = fx_det2(p00, p01, p11);
-    return fx_pivot_from(p00, p01, det, fx_rsqrt(p00), fx_rsqrt(det));
-}
-// offset row (u'0, u'1, t) of U from the pivot-row entries b0 = P(0, .), b1 = P(1, .)
-__device__ __forceinline__ void fx_urow(const fx_piv &v, const fx &b0, const fx &b1, fx &u0, fx &u1, fx &t) {
-    const fx x0 = fx_mul_su(b0, v.a);
-    const fx x1 = fx_mul_su(b1, v.b) - x0 * v.c;
-    u0 = fx_add_top(x0, 2 << 16);
-    u1 = fx_add_top(x1, 2 << 16);
-    const fx s = u0 + u1;
-    t = fx_add_top(s + s, -(4 << 16));
-}
-// c - u_i . u_j from the offset rows
-__device__ __forceinline__ fx fx_sym_update(const fx &c, const fx &ui0, const fx &ui1, const fx &ti,
-                                            const fx &uj0, const fx &uj1, const fx &tj) {
-    return ((c + ti) + tj) - (fx_mul_uu(ui0, uj0) + fx_mul_uu(ui1, uj1));
-}
+// (two products side by side), and |u_ik| <= sqrt(c_ii).  a = p00^{-1/2} and rs = det^{-1/2}
+// are independent, so the two rsqrts need not wait for each other: b = rs sqrt(p00) = rs p00 a.
 
 // ---- prefactors as mantissa x 2^e, and exponent-aligned sums -------------------------
 // The breadth-first prefactors (products of up to seven det^{-1/2} in [1/2, 16]) leave

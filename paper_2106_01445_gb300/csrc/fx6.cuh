@@ -230,7 +230,10 @@ __device__ __forceinline__ fx6 fx_det2(const fx6 &p00, const fx6 &p01, const fx6
     return fx_mul_uu(p00, p11) - fx_mul_uu(a, a);
 }
 
-// the symmetric 2x2 block elimination of the fixed-point sweep (see fx_piv in fx.cuh)
+// the symmetric 2x2 block elimination of the fixed-point sweeps (see fx.cuh).  Rows are
+// stored offset, u' = u + 2 > 0 (|u| <= sqrt(2) for a physical state), so that each entry needs
+// two unsigned products:
+//   c_ij - u_i . u_j = c_ij - (u'_i0 u'_j0 + u'_i1 u'_j1) + t_i + t_j,  t = 2 (u'0 + u'1) - 4.
 struct fx6_piv {
     fx6 a, c, b, rs, det;
 };

@@ -4,7 +4,7 @@
 // in 128-bit fixed point, four independent chains per thread with loop-carried
 // operands.  Used as the denominators of the arithmetic roofline of the subset sweep.
 #include "dd.cuh"
-#include "fx.cuh"
+#include "fl.cuh"
 #include "gbs_internal.cuh"
 
 namespace {
@@ -38,20 +38,20 @@ __global__ void dd_update_loop(double *out, int iters) {
     if (s == -12345.678) out[0] = s;
 }
 
-// the sweep's own fixed-point update entry, the symmetric form c + t_i + t_j -
-// (u'_i0 u'_j0 + u'_i1 u'_j1) with two unsigned truncated products (fx_sym_update)
+// the sweep's own fixed-point update entry in limb form, c - (u_i0 u_j0 + u_i1 u_j1)
+// (fl_sym_update)
 __global__ void fx_update_loop(double *out, int iters) {
-    fx c0 = fx_from_double(0.5 + threadIdx.x * 1e-6), c1 = fx_from_double(0.25);
-    fx c2 = fx_from_double(1.125), c3 = fx_from_double(0.0625);
-    const fx w0 = fx_from_double(1.3), w1 = fx_from_double(2.1), t0 = fx_from_double(-0.5);
+    fl c0 = fl_from_fx(fx_from_double(0.5 + threadIdx.x * 1e-6)), c1 = fl_from_fx(fx_from_double(0.25));
+    fl c2 = fl_from_fx(fx_from_double(1.125)), c3 = fl_from_fx(fx_from_double(0.0625));
+    const fl w0 = fl_from_fx(fx_from_double(1.3)), w1 = fl_from_fx(fx_from_double(2.1));
     for (int it = 0; it < iters; ++it) {
-        const fx n0 = fx_sym_update(c0, c1, c2, t0, c3, w0, t0);
-        const fx n1 = fx_sym_update(c1, c2, c3, t0, c0, w1, t0);
-        const fx n2 = fx_sym_update(c2, c3, c0, t0, c1, w0, t0);
-        const fx n3 = fx_sym_update(c3, c0, c1, t0, c2, w1, t0);
+        const fl n0 = fl_sym_update(c0, c1, c2, c3, w0);
+        const fl n1 = fl_sym_update(c1, c2, c3, c0, w1);
+        const fl n2 = fl_sym_update(c2, c3, c0, c1, w0);
+        const fl n3 = fl_sym_update(c3, c0, c1, c2, w1);
         c0 = n0; c1 = n1; c2 = n2; c3 = n3;
     }
-    const uint32_t s = c0.w[0] ^ c1.w[1] ^ c2.w[2] ^ c3.w[3];
+    const uint32_t s = (uint32_t)(c0.w[0] ^ c1.w[1] ^ c2.w[2] ^ c3.w[3]);
     if (s == 0x9e3779b9u) out[0] = 1.0;
 }
 

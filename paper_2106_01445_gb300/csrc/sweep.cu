@@ -29,6 +29,7 @@
 #include <type_traits>
 
 #include "dd.cuh"
+#include "fl.cuh"
 #include "fx.cuh"
 #include "fx6.cuh"
 #include "gbs_internal.cuh"
@@ -82,17 +83,18 @@ template <> struct Prec<dd> {
     static constexpr int wrow = 2;
     static constexpr double u = 1.2325951644078309e-32, u_sum = 1.2325951644078309e-32;
 };
-// Q16.112 fixed point: truncated products (2^-112) and the pivot rsqrt (residual
-// 1 - x y^2 within 2^-108) give each factor a relative error far below 2^-100 while its
-// pivot determinant stays >= 2^-8; prefactors and sums in double-double.
+// 128-bit fixed point: the matrices of the breadth-first levels and of the register bottom
+// in limb form (fl.cuh), the prefix, the prefactors and the sums packed Q16.112 (fx.cuh).
+// Products truncated to 2^-112 or finer and the pivot rsqrt (within 1.1 units of 2^-112) give
+// each factor a relative error far below 2^-100 while its pivot determinant stays >= 2^-8;
+// unit sums in double-double.
 template <> struct Prec<fx> {
     static constexpr int B = 2, idx = GBS_FX;
     using Tau = dd;
     using Abs = float;
     using Node = fxe;  // prefactors m 2^e
     static constexpr bool fixed = true;
-    static constexpr int wrow = 3;  // offset rows (u'0, u'1, t) of U = B R^{-T}
-    using Piv = fx_piv;
+    static constexpr int wrow = 2;  // rows (u0, u1) of U = B R^{-T}, in limb form
     static constexpr double u = 7.888609052210118e-31, u_sum = 1.2325951644078309e-32;
 };
 // Q16.176 fixed point (fx6.cuh): the same sweep 64 bits wider, per-term relative error far
@@ -108,6 +110,12 @@ template <> struct Prec<fx6> {
     using Piv = fx6_piv;
     static constexpr double u = 4.2351647362715017e-50, u_sum = 6.617444900424222e-52;  // 2^-164, 2^-170
 };
+// the type of the level matrices' entries
+template <typename T> struct EntOf { using type = T; };
+template <> struct EntOf<fx> { using type = fl; };
+__device__ __forceinline__ void store_entry(fl &d, const fx &v) { d = fl_from_fx(v); }
+template <typename T> __device__ __forceinline__ void store_entry(T &d, const T &v) { d = v; }
+static_assert(sizeof(fl) == sizeof(fx), "a level buffer holds either form");
 // doubles per unit partial: (hi, lo, sum |terms|), or the 192-bit fxe6 sum (mantissa in three
 // words, exponent) and sum |terms| for fx6
 template <typename T> constexpr int partial_words() { return std::is_same<T, fx6>::value ? 5 : 3; }
@@ -171,7 +179,6 @@ template <> __device__ __forceinline__ fxe6 node_one<fxe6>() { return fxe6(1.0);
 template <> __device__ __forceinline__ fxe6 node_times<fxe6, fx6>(const fxe6 &p, const fx6 &rs) { return fxe_mul(p, rs); }
 // product of two non-negative factors
 template <typename T> __device__ __forceinline__ T mul_pos(T a, T b) { return a * b; }
-template <> __device__ __forceinline__ fx mul_pos<fx>(fx a, fx b) { return fx_mul_uu(a, b); }
 template <> __device__ __forceinline__ fx6 mul_pos<fx6>(fx6 a, fx6 b) { return fx_mul_uu(a, b); }
 // pivot check: 0 fine, 1 not positive (or NaN), 2 outside the fixed-point range
 template <typename T> __device__ __forceinline__ int pivot_bad(T det) { return det > T(0) ? 0 : 1; }
@@ -396,7 +403,7 @@ __device__ __forceinline__ double tau_hi(dd x) { return x.hi; }
 
 
 // ---- register-resident bottom levels ----------------------------------------------
-template <typename T, int MD> struct RegMat {
+template <typename T, int MD> struct RegMat {  // T: the entry type
     T v[sym(2 * MD)];
     __device__ __forceinline__ T operator()(int i, int j) const { return v[pidx(2 * MD, i, j)]; }
 };
@@ -431,11 +438,35 @@ __device__ __forceinline__ void leaf_pair(BinAcc<T, NB> &acc, T inc, T tau, bool
 // with it are skipped
 template <typename T, int MD, int O, bool NEG, bool ONE = true, typename Src, typename AccT>
 __device__ __forceinline__ void dfs(const Src &A, T tau, int depth, int nreal, AccT &acc, int cnt) {
+    using Ent = typename EntOf<T>::type;
     constexpr int m = MD - O;
     constexpr int o = 2 * O;
-    const T p00 = A(o, o), p01 = A(o, o + 1), p11 = A(o + 1, o + 1);
+    const Ent p00 = A(o, o), p01 = A(o, o + 1), p11 = A(o + 1, o + 1);
     const bool real = depth < nreal;
-    if constexpr (m == 1) {
+    if constexpr (std::is_same<T, fx>::value) {
+        const fx det = fl_det2(p00, p01, p11);
+        const fx rs = fl_rsqrt(det);
+        if constexpr (m == 1) {
+            acc.bad |= fl_pivot_bad(det);
+            leaf_pair<NEG>(acc, ONE ? rs : fx_mul_uu(tau, rs), tau, real, cnt);
+        } else {
+            // symmetric form C - U U^T, U = B R^{-T}, in limbs
+            constexpr int d = 2 * (m - 1);
+            acc.bad |= fl_chol_bad(p00, det);
+            const fl_piv v = fl_pivot_from(p00, p01, fl_rsqrt(fl_pack(p00)), rs);
+            fl u0[d], u1[d];
+#pragma unroll
+            for (int i = 0; i < d; ++i) fl_urow(v.a, v.b, v.c, A(o, o + 2 + i), A(o + 1, o + 2 + i), u0[i], u1[i]);
+            RegMat<fl, m - 1> C;
+#pragma unroll
+            for (int i = 0; i < d; ++i)
+#pragma unroll
+                for (int j = i; j < d; ++j)
+                    C.v[pidx(d, i, j)] = fl_sym_update(A(o + 2 + i, o + 2 + j), u0[i], u1[i], u0[j], u1[j]);
+            dfs<T, m - 1, 0, NEG, false>(C, ONE ? rs : fx_mul_uu(tau, rs), depth + 1, nreal, acc, cnt + 1);
+            if (real) dfs<T, MD, O + 1, !NEG, ONE>(A, tau, depth + 1, nreal, acc, cnt);
+        }
+    } else if constexpr (m == 1) {
         const T det = det2(p00, p01, p11);
         if constexpr (Prec<T>::fixed) acc.bad |= pivot_bad(det);
         const T rs = rsq<T>(det);
@@ -653,9 +684,11 @@ __device__ __forceinline__ typename Prec<T>::Tau elim_pivot(T *Mx, int D, int c0
 }
 // The same pivot with the source kept: Dst (packed, D - c0 - 2 rows) receives the
 // trailing block's Schur complement, Mx is only read (the same operations in the same
-// order as elim_pivot, so the values are those it would leave in place).
+// order as elim_pivot, so the values are those it would leave in place).  level: Dst is a
+// level-0 matrix, stored in the levels' entry form.
 template <typename T>
-__device__ __forceinline__ typename Prec<T>::Tau elim_into(const T *Mx, int D, int c0, T *Dst, T *Wb, int *flag) {
+__device__ __forceinline__ typename Prec<T>::Tau elim_into(const T *Mx, int D, int c0, T *Dst, bool level, T *Wb,
+                                                           int *flag) {
     const int t = threadIdx.x;
     const T p00 = Mx[pidx(D, c0, c0)], p01 = Mx[pidx(D, c0, c0 + 1)], p11 = Mx[pidx(D, c0 + 1, c0 + 1)];
     const T det = det2(p00, p01, p11);
@@ -678,8 +711,10 @@ __device__ __forceinline__ typename Prec<T>::Tau elim_into(const T *Mx, int D, i
     for (int f = t; f < E; f += kThreads) {
         int i, j;
         fold_ij(f, Dt, i, j);
-        Dst[pidx(Dt, i, j)] = fms2(Mx[pidx(D, c0 + 2 + i, c0 + 2 + j)], Wb[2 * i], Mx[pidx(D, c0, c0 + 2 + j)],
-                                   Wb[2 * i + 1], Mx[pidx(D, c0 + 1, c0 + 2 + j)]);
+        const T v = fms2(Mx[pidx(D, c0 + 2 + i, c0 + 2 + j)], Wb[2 * i], Mx[pidx(D, c0, c0 + 2 + j)], Wb[2 * i + 1],
+                         Mx[pidx(D, c0 + 1, c0 + 2 + j)]);
+        if (level) store_entry(((typename EntOf<T>::type *)Dst)[pidx(Dt, i, j)], v);
+        else Dst[pidx(Dt, i, j)] = v;
     }
     __syncthreads();
     return rt;
@@ -716,6 +751,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
     T *X = (T *)(smem + Lay::off_X);
     T *Y = (T *)(smem + Lay::off_Y);
     using Node = typename Prec<T>::Node;
+    using Ent = typename EntOf<T>::type;
     using NIO = NodeIO<Node>;
     unsigned char *tauX = smem + Lay::off_tauX;
     unsigned char *tauY = smem + Lay::off_tauY;
@@ -867,7 +903,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 const int j0 = jv[ds], D = 2 * (rp - j0);
                 const T *src = j0 ? Sl + Lay::slot_off(j0) : Ub;
                 T *dst = ds + 1 < ss ? Sl + Lay::slot_off(ds + 1) : X;
-                const Tau rs = elim_into<T>(src, D, 2 * (ds - j0), dst, Wpre, &s_flag);
+                const Tau rs = elim_into<T>(src, D, 2 * (ds - j0), dst, ds + 1 == ss, Wpre, &s_flag);
                 for (int e = ds + 1; e <= ss; ++e) {
                     jv[e] = ds + 1;
                     tv[e] = tv[ds] * rs;
@@ -887,7 +923,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 for (int f = t; f < (d >> 1) * (d + 1); f += kThreads) {
                     int i, j;
                     fold_ij(f, d, i, j);
-                    X[pidx(d, i, j)] = src[pidx(D, o + i, o + j)];
+                    store_entry(((Ent *)X)[pidx(d, i, j)], src[pidx(D, o + i, o + j)]);
                 }
             }
             if (t == 0) NIO::st(tauX, 0, node_one<Node>());
@@ -895,16 +931,43 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
             // breadth-first expansion of L_eff levels: node c at level l + 1 is child
             // c & 1 (0 exclude, 1 include) of parent c >> 1
             for (int l = 0; l < L_eff; ++l) {
-                const T *src = (l & 1) ? Y : X;
-                T *dst = (l & 1) ? X : Y;
+                const Ent *src = (const Ent *)((l & 1) ? Y : X);
+                Ent *dst = (Ent *)((l & 1) ? X : Y);
                 const unsigned char *tsrc = (l & 1) ? tauY : tauX;
                 unsigned char *tdst = (l & 1) ? tauX : tauY;
-                T *Qb = dst;  // the parents' pivot quantities, read before the children are written
+                T *Qb = (T *)dst;  // the parents' pivot quantities, read before the children are written
                 const int d = 2 * (r - l), dc = d - 2;
                 const int sstr = nstride(d), dstr = nstride(dc), Ec = sym(dc);
                 const int np = 1 << l;
                 // (a) the parents' pivot quantities and the children's prefactors
-                if constexpr (Prec<T>::fixed) {
+                if constexpr (std::is_same<T, fx>::value) {
+                    // two lanes per parent: the even lane's p00^{-1/2} and the odd lane's
+                    // det^{-1/2} run side by side (whole warps, for the shuffle)
+                    if (t < ((2 * np + 31) & ~31)) {
+                        const int cp = min(t >> 1, np - 1), odd = t & 1;
+                        const fl *P = src + cp * sstr;
+                        const fl p00 = P[pidx(d, 0, 0)], p01 = P[pidx(d, 0, 1)], p11 = P[pidx(d, 1, 1)];
+                        const fx det = fl_det2(p00, p01, p11), pk = fl_pack(p00);
+                        fx in;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) in.w[k] = odd ? det.w[k] : pk.w[k];
+                        const fx y = fl_rsqrt(in);
+                        const fx yo = fx_shfl_xor(y, 1);
+                        if (!odd && t < 2 * np) {
+                            const fl_piv v = fl_pivot_from(p00, p01, y, yo);
+                            int4 *Q = (int4 *)Qb + 4 * cp;
+                            Q[0] = make_int4(v.a.w[0], v.a.w[1], v.a.w[2], v.a.w[3]);
+                            Q[1] = make_int4(v.b.w[0], v.b.w[1], v.b.w[2], v.b.w[3]);
+                            Q[2] = make_int4(v.c.w[0], v.c.w[1], v.c.w[2], v.c.w[3]);
+                            Q[3] = make_int4(v.a.w[4], v.b.w[4], v.c.w[4], 0);
+                            const Node tp = NIO::ld(tsrc, cp);
+                            NIO::st(tdst, 2 * cp, tp);
+                            NIO::st(tdst, 2 * cp + 1, node_times(tp, v.rs));
+                            const int bad = fl_chol_bad(p00, det);
+                            if (bad) atomicOr(&s_flag, bad);
+                        }
+                    }
+                } else if constexpr (Prec<T>::fixed) {
                     // two lanes per parent: the even lane's p00^{-1/2} and the odd lane's
                     // det^{-1/2} run side by side (whole warps, for the shuffle)
                     if (t < ((2 * np + 31) & ~31)) {
@@ -945,9 +1008,17 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 // (b) the rows of W = B P^{-1} (fixed point: of U = B R^{-T}), dc per parent
                 for (int f = t; f < np * dc; f += kThreads) {
                     const int cp = f / dc, i = f - cp * dc;
-                    const T *P = src + cp * sstr;
-                    const T b0 = P[pidx(d, 0, i + 2)], b1 = P[pidx(d, 1, i + 2)];
-                    if constexpr (Prec<T>::fixed) {
+                    const Ent *P = src + cp * sstr;
+                    const Ent b0 = P[pidx(d, 0, i + 2)], b1 = P[pidx(d, 1, i + 2)];
+                    if constexpr (std::is_same<T, fx>::value) {
+                        const int4 *Q = (const int4 *)Qb + 4 * cp;
+                        const int4 qa = Q[0], qb = Q[1], qc = Q[2], qt = Q[3];
+                        const fl5 a{{qa.x, qa.y, qa.z, qa.w, qt.x}}, b{{qb.x, qb.y, qb.z, qb.w, qt.y}},
+                            c{{qc.x, qc.y, qc.z, qc.w, qt.z}};
+                        // u0 rows, then u1 rows (16-byte stride: no bank conflicts)
+                        fl *Wl = (fl *)Wb;
+                        fl_urow(a, b, c, b0, b1, Wl[f], Wl[np * dc + f]);
+                    } else if constexpr (Prec<T>::fixed) {
                         const typename Prec<T>::Piv v{Qb[3 * cp], Qb[3 * cp + 1], Qb[3 * cp + 2], konst<T>(0.0),
                                                       konst<T>(0.0)};
                         fx_urow(v, b0, b1, Wb[3 * f], Wb[3 * f + 1], Wb[3 * f + 2]);
@@ -966,10 +1037,13 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 for (int f = t; f < np * Ec; f += kThreads) {
                     const int ij = dtab[e];
                     const int i = ij & 0xff, j = ij >> 8;
-                    const T *P = src + cp * sstr;
-                    const T v = P[pidx(d, i + 2, j + 2)];
+                    const Ent *P = src + cp * sstr;
+                    const Ent v = P[pidx(d, i + 2, j + 2)];
                     dst[(2 * cp) * dstr + e] = v;
-                    if constexpr (Prec<T>::fixed) {
+                    if constexpr (std::is_same<T, fx>::value) {
+                        const fl *U0 = (const fl *)Wb + cp * dc, *U1 = U0 + np * dc;
+                        dst[(2 * cp + 1) * dstr + e] = fl_sym_update(v, U0[i], U1[i], U0[j], U1[j]);
+                    } else if constexpr (Prec<T>::fixed) {
                         const T *Ui = Wb + 3 * (cp * dc + i), *Uj = Wb + 3 * (cp * dc + j);
                         dst[(2 * cp + 1) * dstr + e] = fx_sym_update(v, Ui[0], Ui[1], Ui[2], Uj[0], Uj[1], Uj[2]);
                     } else {
@@ -999,10 +1073,10 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 BT sb[NB];
                 const bool has = t < (1 << L_eff);
                 if (has) {
-                    const T *node = ((L_eff & 1) ? Y : X) + t * nstride(2 * B);
+                    const Ent *node = (const Ent *)((L_eff & 1) ? Y : X) + t * nstride(2 * B);
                     const Node tn = NIO::ld((L_eff & 1) ? tauY : tauX, t);
                     const int nreal = n - (n_eff - B);
-                    SmemMat<T, B> A{node};
+                    SmemMat<Ent, B> A{node};
                     dfs<T, B, 0, false>(A, konst<T>(1.0), 0, nreal, acc, 0);
 #pragma unroll
                     for (int b = 0; b < NB; ++b) sb[b] = scale_bin(tn, tsub, acc.v[b]);
@@ -1032,11 +1106,11 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 int e = -(1 << 20);
                 float ab = 0.0f;
                 if (t < (1 << L_eff)) {
-                    const T *node = ((L_eff & 1) ? Y : X) + t * nstride(2 * B);
+                    const Ent *node = (const Ent *)((L_eff & 1) ? Y : X) + t * nstride(2 * B);
                     const Node tn = NIO::ld((L_eff & 1) ? tauY : tauX, t);
                     const int nreal = n - (n_eff - B);
                     Acc<T> acc{konst<T>(0.0), konst<T>(0.0), 0, 0};
-                    SmemMat<T, B> A{node};
+                    SmemMat<Ent, B> A{node};
                     dfs<T, B, 0, false>(A, konst<T>(1.0), 0, nreal, acc, 0);
                     const int excl = (qs - k) + (ss - kk) + (L_eff - __popc(t));
                     v = fx_neg_if(fx_mul_su(acc.hi, tn.m), excl & 1);   // |v| < 2^11
@@ -1083,11 +1157,11 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                     u_abs += tau_abs(tsub) * ldexp((double)AB, em);
                 }
             } else if (t < (1 << L_eff)) {
-                const T *node = ((L_eff & 1) ? Y : X) + t * nstride(2 * B);
+                const Ent *node = (const Ent *)((L_eff & 1) ? Y : X) + t * nstride(2 * B);
                 const Node tau_node = NIO::ld((L_eff & 1) ? tauY : tauX, t);
                 const int nreal = n - (n_eff - B);
                 Acc<T> acc{konst<T>(0.0), konst<T>(0.0), 0, 0};
-                SmemMat<T, B> A{node};
+                SmemMat<Ent, B> A{node};
                 dfs<T, B, 0, false>(A, konst<T>(1.0), 0, nreal, acc, 0);
                 const int excl = (qs - k) + (ss - kk) + (L_eff - __popc(t));
                 const Tau sc = Tau((excl & 1) ? -1.0 : 1.0) * Tau(tau_node) * tsub;
