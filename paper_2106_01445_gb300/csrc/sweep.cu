@@ -92,9 +92,7 @@ template <> struct Prec<fx> {
     static constexpr int B = 2, idx = GBS_FX;
     using Tau = dd;
     using Abs = float;
-    using Node = fxe;  // prefactors m 2^e
     static constexpr bool fixed = true;
-    static constexpr int wrow = 2;  // rows (u0, u1) of U = B R^{-T}, in limb form
     static constexpr double u = 7.888609052210118e-31, u_sum = 1.2325951644078309e-32;
 };
 // Q16.176 fixed point (fx6.cuh): the same sweep 64 bits wider, per-term relative error far
@@ -106,16 +104,13 @@ template <> struct Prec<fx6> {
     using Abs = float;
     using Node = fxe6;
     static constexpr bool fixed = true;
-    static constexpr int wrow = 3;
+    static constexpr int wrow = 3;  // offset rows (u'0, u'1, t) of U = B R^{-T}
     using Piv = fx6_piv;
     static constexpr double u = 4.2351647362715017e-50, u_sum = 6.617444900424222e-52;  // 2^-164, 2^-170
 };
 // the type of the level matrices' entries
 template <typename T> struct EntOf { using type = T; };
 template <> struct EntOf<fx> { using type = fl; };
-__device__ __forceinline__ void store_entry(fl &d, const fx &v) { d = fl_from_fx(v); }
-template <typename T> __device__ __forceinline__ void store_entry(T &d, const T &v) { d = v; }
-static_assert(sizeof(fl) == sizeof(fx), "a level buffer holds either form");
 // doubles per unit partial: (hi, lo, sum |terms|), or the 192-bit fxe6 sum (mantissa in three
 // words, exponent) and sum |terms| for fx6
 template <typename T> constexpr int partial_words() { return std::is_same<T, fx6>::value ? 5 : 3; }
@@ -148,7 +143,6 @@ template <> __device__ __forceinline__ zf rsq<zf>(zf x) { return zf_rsqrt(x); }
 template <> __device__ __forceinline__ float rsq<float>(float x) { return rsqrtf(x); }
 template <> __device__ __forceinline__ double rsq<double>(double x) { return rsqrt(x); }
 template <> __device__ __forceinline__ dd rsq<dd>(dd x) { return dd_rsqrt(x); }
-template <> __device__ __forceinline__ fx rsq<fx>(fx x) { return fx_rsqrt(x); }
 template <> __device__ __forceinline__ fx6 rsq<fx6>(fx6 x) { return fx6_rsqrt(x); }
 
 // 1/sqrt(det) as a prefix factor, in the Tau type of the precision, given rs = rsq(det)
@@ -156,14 +150,12 @@ template <> __device__ __forceinline__ fx6 rsq<fx6>(fx6 x) { return fx6_rsqrt(x)
 __device__ __forceinline__ double tau_of(float det, float) { return rsqrt((double)det); }
 __device__ __forceinline__ double tau_of(double, double rs) { return rs; }
 __device__ __forceinline__ dd tau_of(dd, dd rs) { return rs; }
-__device__ __forceinline__ dd tau_of(fx, fx rs) { return fx_to_dd(rs); }
 __device__ __forceinline__ fxe6 tau_of(fx6, fx6 rs) { return fxe6_from(rs); }
 __device__ __forceinline__ zc tau_of(zc, zc rs) { return rs; }
 __device__ __forceinline__ zf tau_of(zf, zf rs) { return rs; }
 
 // constants and conversions of the working type
 template <typename T> __device__ __forceinline__ T konst(double v) { return T(v); }
-template <> __device__ __forceinline__ fx konst<fx>(double v) { return fx_from_double(v); }
 template <> __device__ __forceinline__ fx6 konst<fx6>(double v) { return fx6_from_double(v); }
 __device__ __forceinline__ float to_node(float x) { return x; }
 __device__ __forceinline__ double to_node(double x) { return x; }
@@ -172,9 +164,7 @@ __device__ __forceinline__ zc to_node(zc x) { return x; }
 __device__ __forceinline__ zf to_node(zf x) { return x; }
 // a child's prefactor: the parent's times det^{-1/2} of the parent's pivot
 template <typename N, typename T> __device__ __forceinline__ N node_times(const N &p, const T &rs) { return p * to_node(rs); }
-template <> __device__ __forceinline__ fxe node_times<fxe, fx>(const fxe &p, const fx &rs) { return fxe_mul(p, rs); }
 template <typename N> __device__ __forceinline__ N node_one() { return N(1.0); }
-template <> __device__ __forceinline__ fxe node_one<fxe>() { return fxe_one(); }
 template <> __device__ __forceinline__ fxe6 node_one<fxe6>() { return fxe6(1.0); }
 template <> __device__ __forceinline__ fxe6 node_times<fxe6, fx6>(const fxe6 &p, const fx6 &rs) { return fxe_mul(p, rs); }
 // product of two non-negative factors
@@ -182,7 +172,6 @@ template <typename T> __device__ __forceinline__ T mul_pos(T a, T b) { return a 
 template <> __device__ __forceinline__ fx6 mul_pos<fx6>(fx6 a, fx6 b) { return fx_mul_uu(a, b); }
 // pivot check: 0 fine, 1 not positive (or NaN), 2 outside the fixed-point range
 template <typename T> __device__ __forceinline__ int pivot_bad(T det) { return det > T(0) ? 0 : 1; }
-template <> __device__ __forceinline__ int pivot_bad<fx>(fx det) { return fx_pivot_bad(det); }
 template <> __device__ __forceinline__ int pivot_bad<fx6>(fx6 det) { return fx_pivot_bad(det); }
 // complex pivots: their determinants may have any argument in (-pi, pi); only zero or NaN is bad
 template <> __device__ __forceinline__ int pivot_bad<zc>(zc det) {
@@ -198,15 +187,11 @@ template <> __device__ __forceinline__ dd dot2<dd>(dd a0, dd b0, dd a1, dd b1) {
 template <typename T> __device__ __forceinline__ T fms2(T c, T a0, T b0, T a1, T b1) { return c - a0 * b0 - a1 * b1; }
 template <> __device__ __forceinline__ dd fms2<dd>(dd c, dd a0, dd b0, dd a1, dd b1) { return dd_fms2(c, a0, b0, a1, b1); }
 template <typename T> __device__ __forceinline__ T det2(T p00, T p01, T p11) { return dot2(p00, p11, -p01, p01); }
-template <> __device__ __forceinline__ fx det2<fx>(fx p00, fx p01, fx p11) { return fx_det2(p00, p01, p11); }
 template <> __device__ __forceinline__ fx6 det2<fx6>(fx6 p00, fx6 p01, fx6 p11) { return fx_det2(p00, p01, p11); }
 
 // an entry of A = I - O from its FP64 data (exact in double-double)
 template <typename T> __device__ __forceinline__ T a_entry(double delta, double o) { return (T)(delta - o); }
 template <> __device__ __forceinline__ dd a_entry<dd>(double delta, double o) { return dd_two_sum(delta, -o); }
-template <> __device__ __forceinline__ fx a_entry<fx>(double delta, double o) {
-    return fx_from_double(delta) - fx_from_double(o);
-}
 template <> __device__ __forceinline__ fx6 a_entry<fx6>(double delta, double o) {
     return fx6_from_double(delta) - fx6_from_double(o);
 }
@@ -247,23 +232,6 @@ template <typename N> struct NodeIO {
     static constexpr int bytes = sizeof(N), align = alignof(N);
     static __device__ __forceinline__ N ld(const unsigned char *b, int i) { return ((const N *)b)[i]; }
     static __device__ __forceinline__ void st(unsigned char *b, int i, const N &v) { ((N *)b)[i] = v; }
-};
-template <> struct NodeIO<fxe> {
-    static constexpr int bytes = 20, align = 4;
-    static __device__ __forceinline__ fxe ld(const unsigned char *b, int i) {
-        const uint32_t *q = (const uint32_t *)(b + bytes * i);
-        fxe r;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) r.m.w[k] = q[k];
-        r.e = (int)q[4];
-        return r;
-    }
-    static __device__ __forceinline__ void st(unsigned char *b, int i, const fxe &v) {
-        uint32_t *q = (uint32_t *)(b + bytes * i);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) q[k] = v.m.w[k];
-        q[4] = (uint32_t)v.e;
-    }
 };
 template <> struct NodeIO<fxe6> {
     static constexpr int bytes = 28, align = 4;
@@ -684,11 +652,9 @@ __device__ __forceinline__ typename Prec<T>::Tau elim_pivot(T *Mx, int D, int c0
 }
 // The same pivot with the source kept: Dst (packed, D - c0 - 2 rows) receives the
 // trailing block's Schur complement, Mx is only read (the same operations in the same
-// order as elim_pivot, so the values are those it would leave in place).  level: Dst is a
-// level-0 matrix, stored in the levels' entry form.
+// order as elim_pivot, so the values are those it would leave in place).
 template <typename T>
-__device__ __forceinline__ typename Prec<T>::Tau elim_into(const T *Mx, int D, int c0, T *Dst, bool level, T *Wb,
-                                                           int *flag) {
+__device__ __forceinline__ typename Prec<T>::Tau elim_into(const T *Mx, int D, int c0, T *Dst, T *Wb, int *flag) {
     const int t = threadIdx.x;
     const T p00 = Mx[pidx(D, c0, c0)], p01 = Mx[pidx(D, c0, c0 + 1)], p11 = Mx[pidx(D, c0 + 1, c0 + 1)];
     const T det = det2(p00, p01, p11);
@@ -711,10 +677,8 @@ __device__ __forceinline__ typename Prec<T>::Tau elim_into(const T *Mx, int D, i
     for (int f = t; f < E; f += kThreads) {
         int i, j;
         fold_ij(f, Dt, i, j);
-        const T v = fms2(Mx[pidx(D, c0 + 2 + i, c0 + 2 + j)], Wb[2 * i], Mx[pidx(D, c0, c0 + 2 + j)], Wb[2 * i + 1],
-                         Mx[pidx(D, c0 + 1, c0 + 2 + j)]);
-        if (level) store_entry(((typename EntOf<T>::type *)Dst)[pidx(Dt, i, j)], v);
-        else Dst[pidx(Dt, i, j)] = v;
+        Dst[pidx(Dt, i, j)] = fms2(Mx[pidx(D, c0 + 2 + i, c0 + 2 + j)], Wb[2 * i], Mx[pidx(D, c0, c0 + 2 + j)],
+                                   Wb[2 * i + 1], Mx[pidx(D, c0 + 1, c0 + 2 + j)]);
     }
     __syncthreads();
     return rt;
@@ -731,10 +695,6 @@ template <typename T, typename N, typename Tau> __device__ __forceinline__ typen
 scale_bin(const N &tn, const Tau &tsub, T v) {
     return (Tau(tn) * tsub) * v;
 }
-template <> __device__ __forceinline__ dd scale_bin<fx, fxe, dd>(const fxe &tn, const dd &tsub, fx v) {
-    return (fxe_to_dd(tn) * tsub) * fx_to_dd(v);
-}
-__device__ __forceinline__ bool node_nan(const fxe &) { return false; }
 template <typename N> __device__ __forceinline__ bool node_nan(const N &x) { return is_nan(x); }
 __device__ __forceinline__ void store2(double *o, zc v) { o[0] = v.re; o[1] = v.im; }
 __device__ __forceinline__ void store2(double *o, zf v) { o[0] = ff_to_double(v.re); o[1] = ff_to_double(v.im); }
@@ -751,7 +711,6 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
     T *X = (T *)(smem + Lay::off_X);
     T *Y = (T *)(smem + Lay::off_Y);
     using Node = typename Prec<T>::Node;
-    using Ent = typename EntOf<T>::type;
     using NIO = NodeIO<Node>;
     unsigned char *tauX = smem + Lay::off_tauX;
     unsigned char *tauY = smem + Lay::off_tauY;
@@ -903,7 +862,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 const int j0 = jv[ds], D = 2 * (rp - j0);
                 const T *src = j0 ? Sl + Lay::slot_off(j0) : Ub;
                 T *dst = ds + 1 < ss ? Sl + Lay::slot_off(ds + 1) : X;
-                const Tau rs = elim_into<T>(src, D, 2 * (ds - j0), dst, ds + 1 == ss, Wpre, &s_flag);
+                const Tau rs = elim_into<T>(src, D, 2 * (ds - j0), dst, Wpre, &s_flag);
                 for (int e = ds + 1; e <= ss; ++e) {
                     jv[e] = ds + 1;
                     tv[e] = tv[ds] * rs;
@@ -923,7 +882,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 for (int f = t; f < (d >> 1) * (d + 1); f += kThreads) {
                     int i, j;
                     fold_ij(f, d, i, j);
-                    store_entry(((Ent *)X)[pidx(d, i, j)], src[pidx(D, o + i, o + j)]);
+                    X[pidx(d, i, j)] = src[pidx(D, o + i, o + j)];
                 }
             }
             if (t == 0) NIO::st(tauX, 0, node_one<Node>());
@@ -931,43 +890,16 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
             // breadth-first expansion of L_eff levels: node c at level l + 1 is child
             // c & 1 (0 exclude, 1 include) of parent c >> 1
             for (int l = 0; l < L_eff; ++l) {
-                const Ent *src = (const Ent *)((l & 1) ? Y : X);
-                Ent *dst = (Ent *)((l & 1) ? X : Y);
+                const T *src = (l & 1) ? Y : X;
+                T *dst = (l & 1) ? X : Y;
                 const unsigned char *tsrc = (l & 1) ? tauY : tauX;
                 unsigned char *tdst = (l & 1) ? tauX : tauY;
-                T *Qb = (T *)dst;  // the parents' pivot quantities, read before the children are written
+                T *Qb = dst;  // the parents' pivot quantities, read before the children are written
                 const int d = 2 * (r - l), dc = d - 2;
                 const int sstr = nstride(d), dstr = nstride(dc), Ec = sym(dc);
                 const int np = 1 << l;
                 // (a) the parents' pivot quantities and the children's prefactors
-                if constexpr (std::is_same<T, fx>::value) {
-                    // two lanes per parent: the even lane's p00^{-1/2} and the odd lane's
-                    // det^{-1/2} run side by side (whole warps, for the shuffle)
-                    if (t < ((2 * np + 31) & ~31)) {
-                        const int cp = min(t >> 1, np - 1), odd = t & 1;
-                        const fl *P = src + cp * sstr;
-                        const fl p00 = P[pidx(d, 0, 0)], p01 = P[pidx(d, 0, 1)], p11 = P[pidx(d, 1, 1)];
-                        const fx det = fl_det2(p00, p01, p11), pk = fl_pack(p00);
-                        fx in;
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) in.w[k] = odd ? det.w[k] : pk.w[k];
-                        const fx y = fl_rsqrt(in);
-                        const fx yo = fx_shfl_xor(y, 1);
-                        if (!odd && t < 2 * np) {
-                            const fl_piv v = fl_pivot_from(p00, p01, y, yo);
-                            int4 *Q = (int4 *)Qb + 4 * cp;
-                            Q[0] = make_int4(v.a.w[0], v.a.w[1], v.a.w[2], v.a.w[3]);
-                            Q[1] = make_int4(v.b.w[0], v.b.w[1], v.b.w[2], v.b.w[3]);
-                            Q[2] = make_int4(v.c.w[0], v.c.w[1], v.c.w[2], v.c.w[3]);
-                            Q[3] = make_int4(v.a.w[4], v.b.w[4], v.c.w[4], 0);
-                            const Node tp = NIO::ld(tsrc, cp);
-                            NIO::st(tdst, 2 * cp, tp);
-                            NIO::st(tdst, 2 * cp + 1, node_times(tp, v.rs));
-                            const int bad = fl_chol_bad(p00, det);
-                            if (bad) atomicOr(&s_flag, bad);
-                        }
-                    }
-                } else if constexpr (Prec<T>::fixed) {
+                if constexpr (Prec<T>::fixed) {
                     // two lanes per parent: the even lane's p00^{-1/2} and the odd lane's
                     // det^{-1/2} run side by side (whole warps, for the shuffle)
                     if (t < ((2 * np + 31) & ~31)) {
@@ -1008,17 +940,9 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 // (b) the rows of W = B P^{-1} (fixed point: of U = B R^{-T}), dc per parent
                 for (int f = t; f < np * dc; f += kThreads) {
                     const int cp = f / dc, i = f - cp * dc;
-                    const Ent *P = src + cp * sstr;
-                    const Ent b0 = P[pidx(d, 0, i + 2)], b1 = P[pidx(d, 1, i + 2)];
-                    if constexpr (std::is_same<T, fx>::value) {
-                        const int4 *Q = (const int4 *)Qb + 4 * cp;
-                        const int4 qa = Q[0], qb = Q[1], qc = Q[2], qt = Q[3];
-                        const fl5 a{{qa.x, qa.y, qa.z, qa.w, qt.x}}, b{{qb.x, qb.y, qb.z, qb.w, qt.y}},
-                            c{{qc.x, qc.y, qc.z, qc.w, qt.z}};
-                        // u0 rows, then u1 rows (16-byte stride: no bank conflicts)
-                        fl *Wl = (fl *)Wb;
-                        fl_urow(a, b, c, b0, b1, Wl[f], Wl[np * dc + f]);
-                    } else if constexpr (Prec<T>::fixed) {
+                    const T *P = src + cp * sstr;
+                    const T b0 = P[pidx(d, 0, i + 2)], b1 = P[pidx(d, 1, i + 2)];
+                    if constexpr (Prec<T>::fixed) {
                         const typename Prec<T>::Piv v{Qb[3 * cp], Qb[3 * cp + 1], Qb[3 * cp + 2], konst<T>(0.0),
                                                       konst<T>(0.0)};
                         fx_urow(v, b0, b1, Wb[3 * f], Wb[3 * f + 1], Wb[3 * f + 2]);
@@ -1037,13 +961,10 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 for (int f = t; f < np * Ec; f += kThreads) {
                     const int ij = dtab[e];
                     const int i = ij & 0xff, j = ij >> 8;
-                    const Ent *P = src + cp * sstr;
-                    const Ent v = P[pidx(d, i + 2, j + 2)];
+                    const T *P = src + cp * sstr;
+                    const T v = P[pidx(d, i + 2, j + 2)];
                     dst[(2 * cp) * dstr + e] = v;
-                    if constexpr (std::is_same<T, fx>::value) {
-                        const fl *U0 = (const fl *)Wb + cp * dc, *U1 = U0 + np * dc;
-                        dst[(2 * cp + 1) * dstr + e] = fl_sym_update(v, U0[i], U1[i], U0[j], U1[j]);
-                    } else if constexpr (Prec<T>::fixed) {
+                    if constexpr (Prec<T>::fixed) {
                         const T *Ui = Wb + 3 * (cp * dc + i), *Uj = Wb + 3 * (cp * dc + j);
                         dst[(2 * cp + 1) * dstr + e] = fx_sym_update(v, Ui[0], Ui[1], Ui[2], Uj[0], Uj[1], Uj[2]);
                     } else {
@@ -1073,10 +994,10 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 BT sb[NB];
                 const bool has = t < (1 << L_eff);
                 if (has) {
-                    const Ent *node = (const Ent *)((L_eff & 1) ? Y : X) + t * nstride(2 * B);
+                    const T *node = ((L_eff & 1) ? Y : X) + t * nstride(2 * B);
                     const Node tn = NIO::ld((L_eff & 1) ? tauY : tauX, t);
                     const int nreal = n - (n_eff - B);
-                    SmemMat<Ent, B> A{node};
+                    SmemMat<T, B> A{node};
                     dfs<T, B, 0, false>(A, konst<T>(1.0), 0, nreal, acc, 0);
 #pragma unroll
                     for (int b = 0; b < NB; ++b) sb[b] = scale_bin(tn, tsub, acc.v[b]);
@@ -1106,11 +1027,11 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 int e = -(1 << 20);
                 float ab = 0.0f;
                 if (t < (1 << L_eff)) {
-                    const Ent *node = (const Ent *)((L_eff & 1) ? Y : X) + t * nstride(2 * B);
+                    const T *node = ((L_eff & 1) ? Y : X) + t * nstride(2 * B);
                     const Node tn = NIO::ld((L_eff & 1) ? tauY : tauX, t);
                     const int nreal = n - (n_eff - B);
                     Acc<T> acc{konst<T>(0.0), konst<T>(0.0), 0, 0};
-                    SmemMat<Ent, B> A{node};
+                    SmemMat<T, B> A{node};
                     dfs<T, B, 0, false>(A, konst<T>(1.0), 0, nreal, acc, 0);
                     const int excl = (qs - k) + (ss - kk) + (L_eff - __popc(t));
                     v = fx_neg_if(fx_mul_su(acc.hi, tn.m), excl & 1);   // |v| < 2^11
@@ -1157,11 +1078,11 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                     u_abs += tau_abs(tsub) * ldexp((double)AB, em);
                 }
             } else if (t < (1 << L_eff)) {
-                const Ent *node = (const Ent *)((L_eff & 1) ? Y : X) + t * nstride(2 * B);
+                const T *node = ((L_eff & 1) ? Y : X) + t * nstride(2 * B);
                 const Node tau_node = NIO::ld((L_eff & 1) ? tauY : tauX, t);
                 const int nreal = n - (n_eff - B);
                 Acc<T> acc{konst<T>(0.0), konst<T>(0.0), 0, 0};
-                SmemMat<Ent, B> A{node};
+                SmemMat<T, B> A{node};
                 dfs<T, B, 0, false>(A, konst<T>(1.0), 0, nreal, acc, 0);
                 const int excl = (qs - k) + (ss - kk) + (L_eff - __popc(t));
                 const Tau sc = Tau((excl & 1) ? -1.0 : 1.0) * Tau(tau_node) * tsub;
@@ -1237,6 +1158,18 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
         }
     }
 }
+
+#include "sweep_fx.cuh"
+
+// the sweep kernel of a precision and its dynamic shared memory
+template <typename T, bool BIN = false> struct Sweep {
+    static constexpr size_t bytes = Layout<T>::bytes;
+    static constexpr auto kernel = sweep_kernel<T, BIN>;
+};
+template <bool BIN> struct Sweep<fx, BIN> {
+    static constexpr size_t bytes = fxk::Lay::bytes(BIN);
+    static constexpr auto kernel = fxk::sweep_fx_kernel<BIN>;
+};
 
 // ---- per-pattern result ---------------------------------------------------------------
 // log P, kappa, the a-posteriori bound and the status of one pattern from its signed sum
@@ -1487,16 +1420,16 @@ Plan plan_from(void *ws, int n_pat) {
 template <typename T>
 int run_sweep(gbs_ctx *ctx, int M, const double *O, const double *logdet, const uint64_t *pats,
               int n_pat, double *logP, double *kappa, double *err_bound, int32_t *status) {
-    using Lay = Layout<T>;
+    using Lay = Sweep<T>;
     const int pi = Prec<T>::idx;
     if (ctx->reserved && n_pat > ctx->cap_pat)
         return gbs_fail(ctx, GBS_E_INVALID, "gbs_prob: %d patterns exceed the reservation of %d",
                         n_pat, ctx->cap_pat);
     if (ctx->sweep_blocks_per_sm[pi] == 0) {
-        GBS_CUDA(ctx, cudaFuncSetAttribute(sweep_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        GBS_CUDA(ctx, cudaFuncSetAttribute(Sweep<T>::kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)Lay::bytes));
         int nb = 0;
-        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<T>, kThreads,
+        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Sweep<T>::kernel, kThreads,
                                                                     Lay::bytes));
         if (nb < 1) return gbs_fail(ctx, GBS_E_CUDA, "sweep kernel does not fit on an SM");
         ctx->sweep_blocks_per_sm[pi] = nb;
@@ -1532,7 +1465,7 @@ int run_sweep(gbs_ctx *ctx, int M, const double *O, const double *logdet, const 
     const int grid = ctx->num_sms * ctx->sweep_blocks_per_sm[pi];
     int st = gbs_timing_begin(ctx);
     if (st) return st;
-    sweep_kernel<T><<<grid, kThreads, Lay::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
+    Sweep<T>::kernel<<<grid, kThreads, Lay::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
     GBS_CUDA(ctx, cudaGetLastError());
     st = gbs_timing_end(ctx);
     if (st) return st;
@@ -1552,13 +1485,13 @@ template <typename T>
 int run_sweep_on(gbs_ctx *ctx, void *ws, size_t ws_bytes, int M, const double *O,
                  const double *logdet, const uint64_t *pats, int n_pat, double *logP,
                  double *kappa, double *err_bound, int32_t *status) {
-    using Lay = Layout<T>;
+    using Lay = Sweep<T>;
     const int pi = Prec<T>::idx;
     if (ctx->sweep_blocks_per_sm[pi] == 0) {
-        GBS_CUDA(ctx, cudaFuncSetAttribute(sweep_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        GBS_CUDA(ctx, cudaFuncSetAttribute(Sweep<T>::kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)Lay::bytes));
         int nb = 0;
-        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<T>, kThreads,
+        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Sweep<T>::kernel, kThreads,
                                                                     Lay::bytes));
         if (nb < 1) return gbs_fail(ctx, GBS_E_CUDA, "sweep kernel does not fit on an SM");
         ctx->sweep_blocks_per_sm[pi] = nb;
@@ -1572,7 +1505,7 @@ int run_sweep_on(gbs_ctx *ctx, void *ws, size_t ws_bytes, int M, const double *O
     plan_kernel<T><<<1, kPlanThreads, 0, ctx->stream>>>(M, pats, n_pat, cap, pl);
     GBS_CUDA(ctx, cudaGetLastError());
     const int grid = ctx->num_sms * ctx->sweep_blocks_per_sm[pi];
-    sweep_kernel<T><<<grid, kThreads, Lay::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
+    Sweep<T>::kernel<<<grid, kThreads, Lay::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
     GBS_CUDA(ctx, cudaGetLastError());
     const int fthreads = 256, fblocks = (n_pat * 32 + fthreads - 1) / fthreads;
     finalize_kernel<T><<<fblocks, fthreads, 0, ctx->stream>>>(n_pat, logdet, pl, logP, kappa,
@@ -1586,16 +1519,16 @@ int run_sweep_on(gbs_ctx *ctx, void *ws, size_t ws_bytes, int M, const double *O
 template <typename T>
 int run_sweep_slice(gbs_ctx *ctx, int M, const double *O, const uint64_t *pats, int n_pat, int part,
                     int nparts, double *partial, int32_t *pflag) {
-    using Lay = Layout<T>;
+    using Lay = Sweep<T>;
     const int pi = Prec<T>::idx;
     if (ctx->reserved && n_pat > ctx->cap_pat)
         return gbs_fail(ctx, GBS_E_INVALID, "gbs_prob_partial: %d patterns exceed the reservation of %d",
                         n_pat, ctx->cap_pat);
     if (ctx->sweep_blocks_per_sm[pi] == 0) {
-        GBS_CUDA(ctx, cudaFuncSetAttribute(sweep_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        GBS_CUDA(ctx, cudaFuncSetAttribute(Sweep<T>::kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)Lay::bytes));
         int nb = 0;
-        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<T>, kThreads,
+        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Sweep<T>::kernel, kThreads,
                                                                     Lay::bytes));
         if (nb < 1) return gbs_fail(ctx, GBS_E_CUDA, "sweep kernel does not fit on an SM");
         ctx->sweep_blocks_per_sm[pi] = nb;
@@ -1629,7 +1562,7 @@ int run_sweep_slice(gbs_ctx *ctx, int M, const double *O, const uint64_t *pats, 
     const int grid = ctx->num_sms * ctx->sweep_blocks_per_sm[pi];
     int st = gbs_timing_begin(ctx);
     if (st) return st;
-    sweep_kernel<T><<<grid, kThreads, Lay::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
+    Sweep<T>::kernel<<<grid, kThreads, Lay::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
     GBS_CUDA(ctx, cudaGetLastError());
     st = gbs_timing_end(ctx);
     if (st) return st;
@@ -1983,7 +1916,7 @@ constexpr int kRetryInDD = -1;
 template <typename T>
 int click_distribution_in(gbs_ctx *ctx, int M, const double *O, const double *logdet, double *logp,
                           double *kappa) {
-    using Lay = Layout<T>;
+    using Lay = Sweep<T, true>;
     const int pi = Prec<T>::idx;
     const int split = sweep_split_of(ctx, pi);
     const long long units = sweep_units_upper_bound(1, M, pi, split);
@@ -2001,14 +1934,14 @@ int click_distribution_in(gbs_ctx *ctx, int M, const double *O, const double *lo
     all_modes_kernel<<<1, 1, 0, ctx->stream>>>(M, pat);
     plan_kernel<T><<<1, kPlanThreads, 0, ctx->stream>>>(M, pat, 1, units, pl);
     GBS_CUDA(ctx, cudaGetLastError());
-    GBS_CUDA(ctx, cudaFuncSetAttribute(sweep_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    GBS_CUDA(ctx, cudaFuncSetAttribute(Sweep<T, true>::kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)Lay::bytes));
     int nbk = 0;
-    GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbk, sweep_kernel<T, true>, kThreads, Lay::bytes));
+    GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbk, Sweep<T, true>::kernel, kThreads, Lay::bytes));
     if (nbk < 1) return gbs_fail(ctx, GBS_E_CUDA, "binned sweep kernel does not fit on an SM");
     st = gbs_timing_begin(ctx);
     if (st) return st;
-    sweep_kernel<T, true><<<ctx->num_sms * nbk, kThreads, Lay::bytes, ctx->stream>>>(M, O, pat, 1, pl);
+    Sweep<T, true>::kernel<<<ctx->num_sms * nbk, kThreads, Lay::bytes, ctx->stream>>>(M, O, pat, 1, pl);
     GBS_CUDA(ctx, cudaGetLastError());
     st = gbs_timing_end(ctx);
     if (st) return st;
@@ -2036,7 +1969,7 @@ namespace {
 template <typename T>
 int sector_distribution_in(gbs_ctx *ctx, int M, const double *O, const double *logdet, int L, double rho, int K,
                            int even, double *pkn) {
-    using Lay = Layout<T>;
+    using Lay = Sweep<T, true>;
     if (M < 4 || M > kMaxDevice)
         return gbs_fail(ctx, GBS_E_INVALID, "gbs_sector_distribution: M = %d outside 4..%d", M, kMaxDevice);
     if (L < 4 || L > 4096 || (L & (L - 1)))
@@ -2063,10 +1996,10 @@ int sector_distribution_in(gbs_ctx *ctx, int M, const double *O, const double *l
     uint64_t *pat = (uint64_t *)((char *)ctx->ws + off_pat);
     double *G = (double *)((char *)ctx->ws + off_G);
     int *bad = (int *)((char *)ctx->ws + off_bad);
-    GBS_CUDA(ctx, cudaFuncSetAttribute(sweep_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    GBS_CUDA(ctx, cudaFuncSetAttribute(Sweep<T, true>::kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)Lay::bytes));
     int nbk = 0;
-    GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbk, sweep_kernel<T, true>, kThreads, Lay::bytes));
+    GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbk, Sweep<T, true>::kernel, kThreads, Lay::bytes));
     if (nbk < 1) return gbs_fail(ctx, GBS_E_CUDA, "complex binned sweep kernel does not fit on an SM");
     all_modes_kernel<<<1, 1, 0, ctx->stream>>>(M, pat);
     GBS_CUDA(ctx, cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream));
@@ -2081,7 +2014,7 @@ int sector_distribution_in(gbs_ctx *ctx, int M, const double *O, const double *l
         GBS_CUDA(ctx, cudaGetLastError());
         st = gbs_timing_begin(ctx);
         if (st) return st;
-        sweep_kernel<T, true><<<ctx->num_sms * nbk, kThreads, Lay::bytes, ctx->stream>>>(M, O, pat, 1, pl);
+        Sweep<T, true>::kernel<<<ctx->num_sms * nbk, kThreads, Lay::bytes, ctx->stream>>>(M, O, pat, 1, pl);
         GBS_CUDA(ctx, cudaGetLastError());
         st = gbs_timing_end(ctx);
         if (st) return st;
