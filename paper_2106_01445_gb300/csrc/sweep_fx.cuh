@@ -64,6 +64,11 @@ __device__ __forceinline__ node node_mul(const node &a, const fx &rs) {
 }
 // the mantissa packed, Q16.112
 __device__ __forceinline__ fx node_packed(const node &a) { return fx_shr_small(fl_pack(a.m), 5); }
+__device__ __forceinline__ node node_mul(const node &a, const node &b) {
+    node r = node_mul(a, node_packed(b));
+    r.e += b.e;
+    return r;
+}
 __device__ __forceinline__ dd node_dd(const node &a) {
     const dd v = fx_to_dd(node_packed(a));
     const double s = ldexp(1.0, a.e);
@@ -116,7 +121,7 @@ struct Lay {
     static_assert(sizeof(fl) * sym(2 * kMaxN) <= W, "prefix matrix must fit in X, Y, Ub and Sl");
 };
 // 228 KB an SM, 1 KB of it reserved a CTA
-static_assert(3 * (Lay::bytes(true) + 1024 + 1024) <= 228 * 1024, "three CTAs must fit on an SM");
+static_assert(3 * (Lay::bytes(true) + 1024 + 1600) <= 228 * 1024, "three CTAs must fit on an SM");
 
 // f / w for the folded-triangle indices (f < 2^12, w <= 2 kMaxN + 1), by a reciprocal
 __device__ __forceinline__ void fold_fast(int f, int D, uint32_t inv, int &i, int &j) {
@@ -128,12 +133,11 @@ __device__ __forceinline__ void fold_fast(int f, int D, uint32_t inv, int &i, in
 constexpr int kInv = sym(2 * (R - 1)) + 1;  // reciprocals 2^20 / w + 1 of w < kInv
 
 // One 2x2 block pivot eliminated by the whole CTA: rows c0, c0 + 1 of the packed D x D matrix Mx;
-// the trailing Schur complement is written to Dst (packed), or in place (Dst null).  Returns
-// det^{-1/2} on thread 0.  Two barriers; the caller's data must be visible on entry.
-__device__ __forceinline__ fx elim(const fl *Mx, fl *inplace, int D, int c0, fl *Dst, fl *U, int4 *Qs,
-                                   const uint32_t *inv20, int *flag) {
+// the trailing Schur complement is written to Dst (packed), or in place (Dst null), and
+// det^{-1/2} to *rs.  Two barriers; the caller's data must be visible on entry.
+__device__ __forceinline__ void elim(const fl *Mx, fl *inplace, int D, int c0, fl *Dst, fl *U, int4 *Qs, fx *rs,
+                                     const uint32_t *inv20, int *flag) {
     const int t = threadIdx.x, Dt = D - c0 - 2;
-    fx rs = fx_zero();
     if (t < ((Dt + 31) & ~31)) {
         const fl p00 = Mx[pidx(D, c0, c0)], p01 = Mx[pidx(D, c0, c0 + 1)], p11 = Mx[pidx(D, c0 + 1, c0 + 1)];
         const fx det = fl_det2(p00, p01, p11), pk = fl_pack(p00);
@@ -150,8 +154,8 @@ __device__ __forceinline__ fx elim(const fl *Mx, fl *inplace, int D, int c0, fl 
             Q[1] = make_int4(v.b.w[0], v.b.w[1], v.b.w[2], v.b.w[3]);
             Q[2] = make_int4(v.c.w[0], v.c.w[1], v.c.w[2], v.c.w[3]);
             Q[3] = make_int4(v.a.w[4], v.b.w[4], v.c.w[4], 0);
-            rs = yo;
             if (t == 0) {
+                *rs = yo;
                 // a positive determinant of a negative block is outside this form's range only
                 const int bad = fl_pivot_bad(det) | (fl_positive(p00) ? 0 : 2);
                 if (bad) atomicOr(flag, bad);
@@ -177,7 +181,6 @@ __device__ __forceinline__ fx elim(const fl *Mx, fl *inplace, int D, int c0, fl 
         else inplace[at] = v;
     }
     __syncthreads();
-    return rs;
 }
 
 template <bool BIN>
@@ -201,7 +204,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
     __shared__ int s_flag;
     __shared__ float s_abs[kSub * kW];
     __shared__ int s_exp[kSub * kW];
-    __shared__ int s_kk[kSub];
+    __shared__ fx s_rs[kSub + kMaxN];  // the tree's and the prefix's det^{-1/2}
     __shared__ uint32_t inv20[kInv];
 
     const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
@@ -271,11 +274,8 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
         }
         __syncthreads();
         // eliminate the included prefix modes (2x2 block pivots)
-        node tpre = node_unit();  // thread 0
-        for (int e = 0; e < k; ++e) {
-            const fx rs = elim(X, X, D0, 2 * e, nullptr, Wb, Qs, inv20, &s_flag);
-            if (t == 0) tpre = node_mul(tpre, rs);
-        }
+        for (int e = 0; e < k; ++e)
+            elim(X, X, D0, 2 * e, nullptr, Wb, Qs, s_rs + kSub + e, inv20, &s_flag);
         // the unit's trailing block -> Ub, through registers: the prefix matrix may extend over Ub
         {
             const int d = 2 * rp, o = 2 * k, E = (d >> 1) * (d + 1);
@@ -305,15 +305,11 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
         // stored (in slot e + 1, or in X at the last depth), an exclude is a view of the same
         // matrix one mode further on; leaf `leaf` takes the choices of its bits from the top, so
         // consecutive leaves share every choice above the one that turns include.  jv[e]: the
-        // slot of the matrix the node at depth e views (0: Ub); tv[e] (thread 0): the product of
-        // the includes' det^{-1/2} above depth e.
+        // slot of the matrix the node at depth e views (0: Ub).  The include that leaf `leaf`
+        // starts with leaves its det^{-1/2} in s_rs[leaf].
         int jv[kS + 1];
-        node tv[kS + 1];
 #pragma unroll
-        for (int e = 0; e <= kS; ++e) {
-            jv[e] = 0;
-            tv[e] = node_unit();
-        }
+        for (int e = 0; e <= kS; ++e) jv[e] = 0;
         for (int leaf = 0; leaf < nsub; ++leaf) {
             const int kk = __popc(leaf);
             // the depth whose choice turns include (none at the first leaf); deeper choices
@@ -329,17 +325,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
             if (leaf) {
                 in_x = ds + 1 == ss;
                 fl *dst = in_x ? X : Sl + (ds == 1 ? slot_off(2) : 0);
-                const fx rs = elim(src, nullptr, D, 2 * (ds - j0), dst, Wb, Qs, inv20, &s_flag);
-                if (t == 0) {
-                    node pr = node_unit();
-#pragma unroll
-                    for (int e = 0; e <= kS; ++e)
-                        if (e == ds) pr = tv[e];
-                    pr = node_mul(pr, rs);
-#pragma unroll
-                    for (int e = 0; e <= kS; ++e)
-                        if (e > ds) tv[e] = pr;
-                }
+                elim(src, nullptr, D, 2 * (ds - j0), dst, Wb, Qs, s_rs + leaf, inv20, &s_flag);
 #pragma unroll
                 for (int e = 0; e <= kS; ++e)
                     if (e > ds) jv[e] = ds + 1;
@@ -357,15 +343,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                     X[pidx(d, i, j)] = s1[pidx(D1, o + i, o + j)];
                 }
             }
-            if (t == 0) {
-                node_st(tauX, 0, node_unit());
-                node ts = tv[0];
-#pragma unroll
-                for (int e = 0; e <= kS; ++e)
-                    if (e == ss) ts = tv[e];
-                node_st(s_ts, leaf, ts);
-                s_kk[leaf] = kk;
-            }
+            if (t == 0) node_st(tauX, 0, node_unit());
             __syncthreads();
             // breadth-first expansion of L_eff levels: node c at level l + 1 is child
             // c & 1 (0 exclude, 1 include) of parent c >> 1
@@ -454,19 +432,39 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                 const uint32_t einv = inv20[Ec];
                 const int qstep = (int)((kThreads * einv) >> 20), rstep = kThreads - qstep * Ec;
                 int cp = (int)(((uint32_t)t * einv) >> 20), e = t - cp * Ec;
-                for (int f = t; f < np * Ec; f += kThreads) {
-                    const int ij = dtab[e];
-                    const int i = ij & 0xff, j = ij >> 8;
-                    const fl v = src[cp * sstr + pidx(d, i + 2, j + 2)];
-                    dst[(2 * cp) * dstr + e] = v;
-                    const fl *U0 = Wb + cp * dc, *U1 = U0 + nr;
-                    dst[(2 * cp + 1) * dstr + e] = fl_sym_update(v, U0[i], U1[i], U0[j], U1[j]);
+                auto step = [&]() {
                     e += rstep;
                     cp += qstep;
                     if (e >= Ec) {
                         e -= Ec;
                         ++cp;
                     }
+                };
+                int f = t;
+                for (; f + kThreads < np * Ec; f += 2 * kThreads) {
+                    const int ij = dtab[e], i = ij & 0xff, j = ij >> 8, at = 2 * cp * dstr + e;
+                    const fl v = src[cp * sstr + pidx(d, i + 2, j + 2)];
+                    const fl *U0 = Wb + cp * dc, *U1 = U0 + nr;
+                    const fl a0 = U0[i], a1 = U1[i], b0 = U0[j], b1 = U1[j];
+                    step();
+                    const int ij2 = dtab[e], i2 = ij2 & 0xff, j2 = ij2 >> 8, at2 = 2 * cp * dstr + e;
+                    const fl v2 = src[cp * sstr + pidx(d, i2 + 2, j2 + 2)];
+                    const fl *V0 = Wb + cp * dc, *V1 = V0 + nr;
+                    const fl c0 = V0[i2], c1 = V1[i2], d0 = V0[j2], d1 = V1[j2];
+                    step();
+                    const fl r1 = fl_sym_update(v, a0, a1, b0, b1);
+                    const fl r2 = fl_sym_update(v2, c0, c1, d0, d1);
+                    dst[at] = v;
+                    dst[at2] = v2;
+                    dst[at + dstr] = r1;
+                    dst[at2 + dstr] = r2;
+                }
+                if (f < np * Ec) {
+                    const int ij = dtab[e], i = ij & 0xff, j = ij >> 8, at = 2 * cp * dstr + e;
+                    const fl v = src[cp * sstr + pidx(d, i + 2, j + 2)];
+                    const fl *U0 = Wb + cp * dc, *U1 = U0 + nr;
+                    dst[at] = v;
+                    dst[at + dstr] = fl_sym_update(v, U0[i], U1[i], U0[j], U1[j]);
                 }
                 __syncthreads();
             }
@@ -543,8 +541,30 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                 // next sub-unit writes Y after a barrier only
             }
         }
-        if (t == 0) node_st(s_ts, kSub, tpre);
         __syncthreads();
+        if (t < 32) {
+            // the prefix factor (a tree of products over the lanes) and each sub-unit's (the
+            // includes on its path, from the top)
+            node tp = node_unit();
+            for (int e = t; e < k; e += 32) tp = node_mul(tp, s_rs[kSub + e]);
+            const int top = k < 32 ? k : 32;
+            for (int off = 1; off < top; off <<= 1) {
+                node o;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) o.m.w[c] = __shfl_down_sync(0xffffffffu, tp.m.w[c], off);
+                o.e = __shfl_down_sync(0xffffffffu, tp.e, off);
+                if ((t & (2 * off - 1)) == 0 && t + off < top) tp = node_mul(tp, o);
+            }
+            if (t == 0) node_st(s_ts, kSub, tp);
+            if (t < nsub) {
+                node ts = node_unit();
+                for (int b = ss - 1; b >= 0; --b)
+                    if (t >> b & 1) ts = node_mul(ts, s_rs[t & ~((1 << b) - 1)]);
+                node_st(s_ts, t, ts);
+            }
+        }
+        if constexpr (BIN) __syncthreads();
+        else __syncwarp();
         if constexpr (BIN) {
             // sub-unit `leaf`, size z (0..9 within it): the four warps' sums (warp w holds the
             // sizes popc(w) + 0..7) times the sub-unit's factor, then per size of the unit
@@ -570,7 +590,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
             for (int z = t; z <= n; z += kThreads) {
                 dd s = dd(0.0);
                 for (int leaf = 0; leaf < nsub; ++leaf) {
-                    const int b = z - k - s_kk[leaf];
+                    const int b = z - k - __popc(leaf);
                     if (b >= 0 && b < 10) s += part[10 * leaf + b];
                 }
                 store2(out + 2 * z, tp * s);
@@ -608,7 +628,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                 a += oa;
             }
             if (t == 0) {
-                const dd tp = node_dd(tpre);
+                const dd tp = node_dd(node_ld(s_ts, kSub));
                 s = s * tp;
                 double *out = pl.partials + 3 * u;
                 out[0] = s.hi;
