@@ -6,64 +6,133 @@
 //     sigma   = R diag(s) R^T,         s = eta sigma_in + (1 - eta)/2,
 //     sigma_Q = R diag(s + 1/2) R^T,   sigma_Q^{-1} = R diag(1/(s + 1/2)) R^T,
 //     log det sigma_Q = sum_j log1p(eta (2 - eta) sinh^2 r_j).
-// Every entry is an independent length-2M dot product: no factorisation, one
-// thread per entry, the whole GPU in one launch.
+// Every entry is an independent length-2M dot product: no factorisation, one launch.
+//
+// What bounds it: FP64 multiply-adds, which a quarter of an SM issues one warp instruction of every
+// 64 clocks, so the time is the longest chain on one warp as long as the grid does not fill the GPU
+// (91 tiles at 50 modes).  Hence
+//  * 8 x 8 tiles of the upper triangle, and each dot product split over four warps (sigma or A, x or p
+//    quadratures) of M multiply-adds each, on rows that are weighted once when they are staged;
+//  * the unitarity residual |U^dag U - 1| (Hermitian: the real part with the xx tiles, the imaginary
+//    part with the xp ones) on four more warps;
+//  * the 4M weights (an exp each) computed once per cluster of eight CTAs and read through
+//    distributed shared memory: computed per entry and per j, as before, the exp and the division
+//    were nearly all of the time, 241 us at 50 modes on a GB300 and 446 at 100.
+// Now 15 us at 50 modes and 37 at 100 (with the status' memset); one thread an entry on the same
+// tiles took 33 and 68.
+#include <cooperative_groups.h>
+
 #include "gbs_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
-__device__ __forceinline__ double R_entry(const double *U, int M, int i, int j) {
-    // R = [[Re U, -Im U], [Im U, Re U]] in xp order
-    int ui = i < M ? i : i - M, uj = j < M ? j : j - M;
-    double re = U[2 * (ui * M + uj)], im = U[2 * (ui * M + uj) + 1];
-    if (i < M) return j < M ? re : -im;
-    return j < M ? im : re;
-}
+constexpr int kTile = 8, kEnt = kTile * kTile, kCluster = 8, kMaxModes = 128;
+constexpr int kParts = 6, kStateThreads = kEnt * kParts;
 
-__global__ void state_kernel(int M, const double *__restrict__ U, const double *__restrict__ r,
-                             double eta, double *__restrict__ sigma, double *__restrict__ O,
-                             double *__restrict__ logdet, int32_t *__restrict__ status) {
-    const int N = 2 * M;
-    int i = blockIdx.y * blockDim.y + threadIdx.y;
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N && k < N) {
-        double acc_s = 0.0, acc_a = 0.0;
-        for (int j = 0; j < N; ++j) {
-            int jm = j < M ? j : j - M;
-            double rj = r[jm];
-            // x quadratures get e^{-2r}/2, p quadratures e^{2r}/2
-            double sin_ = 0.5 * exp(j < M ? -2.0 * rj : 2.0 * rj);
-            double s = eta * sin_ + 0.5 * (1.0 - eta);
-            double prod = R_entry(U, M, i, j) * R_entry(U, M, k, j);
-            acc_s = fma(prod, s, acc_s);
-            acc_a = fma(prod, 1.0 / (s + 0.5), acc_a);
-        }
-        if (sigma) sigma[i * N + k] = acc_s;
-        O[i * N + k] = (i == k ? 1.0 : 0.0) - acc_a;
-        // unitarity residual |U^dag U - 1| on the M x M block
-        if (i < M && k < M) {
-            double re = 0.0, im = 0.0;
-            for (int j = 0; j < M; ++j) {
-                double ar = U[2 * (j * M + i)], ai = -U[2 * (j * M + i) + 1];
-                double br = U[2 * (j * M + k)], bi = U[2 * (j * M + k) + 1];
-                re += ar * br - ai * bi;
-                im += ar * bi + ai * br;
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kStateThreads)
+    state_kernel(int M, int tiles, const double *__restrict__ U, const double *__restrict__ r, double eta,
+                 double *__restrict__ sigma, double *__restrict__ O, double *__restrict__ logdet,
+                 int32_t *__restrict__ status) {
+    __shared__ double2 w[2 * kMaxModes];  // (s_j, 1 / (s_j + 1/2)), j = x then p quadratures
+    // per quadrature half: the tile's rows i weighted for sigma and for A, and its rows k
+    __shared__ double ws[2][kTile][kMaxModes + 1], wa[2][kTile][kMaxModes + 1], rk[2][kTile][kMaxModes + 1];
+    __shared__ double part[kParts][kEnt];
+    const cg::cluster_group cl = cg::this_cluster();
+    const int t = threadIdx.x, N = 2 * M, rank = (int)cl.block_rank();
+    // this CTA's share of the weights: x quadratures get e^{-2r}/2, p quadratures e^{2r}/2
+    for (int j = rank + kCluster * t; j < N; j += kCluster * kStateThreads) {
+        const double rj = r[j < M ? j : j - M];
+        const double s = eta * (0.5 * exp(j < M ? -2.0 * rj : 2.0 * rj)) + 0.5 * (1.0 - eta);
+        w[j] = make_double2(s, 1.0 / (s + 0.5));
+    }
+    cl.sync();
+    for (int j = t; j < N; j += kStateThreads)
+        if ((j & (kCluster - 1)) != rank) w[j] = cl.map_shared_rank(w, j & (kCluster - 1))[j];
+    cl.sync();  // the weights are in, and no CTA still reads another's when that one exits
+
+    // tile (bi, bk), bi <= bk, of the upper triangle, in rows
+    int bi = 0, rest = blockIdx.x;
+    while (bi < tiles && rest >= tiles - bi) {
+        rest -= tiles - bi;
+        ++bi;
+    }
+    const int bk = bi + rest;
+    if (bi < tiles) {
+        // R = [[Re U, -Im U], [Im U, Re U]] in xp order
+        for (int f = t; f < 2 * kTile * M; f += kStateThreads) {
+            const int g = f / M, j = f - g * M, side = g >= kTile, l = g & (kTile - 1), row = (side ? bk : bi) * kTile + l;
+            if (row >= N) continue;
+            const bool ip = row >= M;
+            const double *u = U + 2 * ((size_t)(ip ? row - M : row) * M + j);  // 8-byte aligned
+            const double x = ip ? u[1] : u[0], q = ip ? u[0] : -u[1];
+            if (side) {
+                rk[0][l][j] = x;
+                rk[1][l][j] = q;
+            } else {
+                ws[0][l][j] = x * w[j].x;
+                ws[1][l][j] = q * w[M + j].x;
+                wa[0][l][j] = x * w[j].y;
+                wa[1][l][j] = q * w[M + j].y;
             }
-            re -= (i == k) ? 1.0 : 0.0;
-            if (!(fabs(re) <= 1e-10 && fabs(im) <= 1e-10)) atomicExch(status, (int32_t)GBS_E_INVALID);
+        }
+        __syncthreads();
+        const int e = t & (kEnt - 1), pt = t / kEnt, li = e / kTile, lk = e % kTile;
+        const int i = bi * kTile + li, k = bk * kTile + lk;
+        if (i < N && k < N) {
+            double acc = 0.0;
+            if (pt < 4) {
+                const double *a = pt < 2 ? ws[pt & 1][li] : wa[pt & 1][li], *b = rk[pt & 1][lk];
+#pragma unroll 4
+                for (int j = 0; j < M; ++j) acc = fma(a[j], b[j], acc);
+            } else if (i < M) {
+                // column i of U against column c: the real part (k < M), or the imaginary part
+                const bool kp = k >= M, im = pt == 5;
+                const int c = kp ? k - M : k;
+                const double *a = U + 2 * i + im, *b = U + 2 * c + (im != kp);
+                if (i <= c) {
+#pragma unroll 4
+                    for (int j = 0; j < M; ++j) acc = fma(a[(size_t)2 * j * M], b[(size_t)2 * j * M], acc);
+                    if (kp && im) acc = -acc;
+                }
+            }
+            part[pt][e] = acc;
+        }
+        __syncthreads();
+        if (i < N && k < N) {
+            if (pt == 0 && sigma && i <= k) {
+                const double v = part[0][e] + part[1][e];
+                sigma[i * N + k] = v;
+                sigma[k * N + i] = v;
+            } else if (pt == 2 && i <= k) {
+                const double v = (i == k ? 1.0 : 0.0) - (part[2][e] + part[3][e]);
+                O[i * N + k] = v;
+                O[k * N + i] = v;
+            } else if (pt == 4) {
+                const double v = part[4][e] + part[5][e] - (i == k && i < M ? 1.0 : 0.0);
+                if (!(fabs(v) <= 1e-10)) atomicExch(status, (int32_t)GBS_E_INVALID);
+            }
         }
     }
-    const int lin = threadIdx.y * blockDim.x + threadIdx.x;  // whole warp 0 of block (0, 0)
-    if (blockIdx.x == 0 && blockIdx.y == 0 && lin < 32) {
-        double acc = 0.0;
-        for (int j = lin; j < M; j += 32) {
-            double rj = r[j];
+    // log det by the last CTA of the grid: one term a thread (a sinh and a log1p are a long chain on
+    // this pipe), added in the order of a warp that strides the modes
+    if (blockIdx.x == gridDim.x - 1) {
+        __syncthreads();
+        double *term = &ws[0][0][0];
+        for (int j = t; j < M; j += kStateThreads) {
+            const double rj = r[j];
             if (!(rj >= 0.0) || !isfinite(rj)) atomicExch(status, (int32_t)GBS_E_INVALID);
-            double sh = sinh(rj);
-            acc += log1p(eta * (2.0 - eta) * sh * sh);
+            const double sh = sinh(rj);
+            term[j] = log1p(eta * (2.0 - eta) * sh * sh);
         }
-        for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lin == 0) *logdet = acc;
+        __syncthreads();
+        if (t < 32) {
+            double acc = 0.0;
+            for (int j = t; j < M; j += 32) acc += term[j];
+            for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (t == 0) *logdet = acc;
+        }
     }
 }
 
@@ -73,9 +142,9 @@ int launch_build_state(gbs_ctx *ctx, int M, const double *U, const double *r, do
                        double *sigma, double *O, double *logdet, int32_t *status_dev) {
     int32_t *st = status_dev ? status_dev : ctx->dscratch;
     GBS_CUDA(ctx, cudaMemsetAsync(st, 0, sizeof(int32_t), ctx->stream));
-    int N = 2 * M;
-    dim3 blk(16, 16), grd((N + 15) / 16, (N + 15) / 16);
-    state_kernel<<<grd, blk, 0, ctx->stream>>>(M, U, r, eta, sigma, O, logdet, st);
+    const int tiles = (2 * M + kTile - 1) / kTile, n = tiles * (tiles + 1) / 2;
+    const int grid = (n + kCluster - 1) / kCluster * kCluster;
+    state_kernel<<<grid, kStateThreads, 0, ctx->stream>>>(M, tiles, U, r, eta, sigma, O, logdet, st);
     GBS_CUDA(ctx, cudaGetLastError());
     if (status_dev) return GBS_OK;
     GBS_CUDA(ctx, cudaMemcpyAsync(ctx->pinned, st, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
