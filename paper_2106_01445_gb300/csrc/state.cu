@@ -8,18 +8,19 @@
 //     log det sigma_Q = sum_j log1p(eta (2 - eta) sinh^2 r_j).
 // Every entry is an independent length-2M dot product: no factorisation, one launch.
 //
-// What bounds it: FP64 multiply-adds, which a quarter of an SM issues one warp instruction of every
+// What bounds it: FP64 operations, which a quarter of an SM issues one warp instruction of every
 // 64 clocks, so the time is the longest chain on one warp as long as the grid does not fill the GPU
 // (91 tiles at 50 modes).  Hence
-//  * 8 x 8 tiles of the upper triangle, and each dot product split over four warps (sigma or A, x or p
-//    quadratures) of M multiply-adds each, on rows that are weighted once when they are staged;
-//  * the unitarity residual |U^dag U - 1| (Hermitian: the real part with the xx tiles, the imaginary
-//    part with the xp ones) on four more warps;
+//  * 8 x 8 tiles of the upper triangle, sigma and A on warps of their own, and the unitarity residual
+//    |U^dag U - 1| (Hermitian: the real part with the xx tiles, the imaginary part with the xp ones)
+//    on four more, in halves;
 //  * the 4M weights (an exp each) computed once per cluster of eight CTAs and read through
 //    distributed shared memory: computed per entry and per j, as before, the exp and the division
 //    were nearly all of the time, 241 us at 50 modes on a GB300 and 446 at 100.
-// Now 15 us at 50 modes and 37 at 100 (with the status' memset); one thread an entry on the same
-// tiles took 33 and 68.
+// Now 17 us at 50 modes and 57 at 100 (with the status' memset).  Every entry is still
+// the sum over j in order, the product of the two rows' entries rounded first: log P of a pattern
+// whose sum cancels by 1e25 and more moves with the last bit of O.  (Splitting the sums over x and p
+// quadratures would take 15 and 37 us.)
 #include <cooperative_groups.h>
 
 #include "gbs_internal.cuh"
@@ -29,15 +30,14 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr int kTile = 8, kEnt = kTile * kTile, kCluster = 8, kMaxModes = 128;
-constexpr int kParts = 6, kStateThreads = kEnt * kParts;
+constexpr int kParts = 4, kStateThreads = kEnt * kParts;
 
 __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kStateThreads)
     state_kernel(int M, int tiles, const double *__restrict__ U, const double *__restrict__ r, double eta,
                  double *__restrict__ sigma, double *__restrict__ O, double *__restrict__ logdet,
                  int32_t *__restrict__ status) {
     __shared__ double2 w[2 * kMaxModes];  // (s_j, 1 / (s_j + 1/2)), j = x then p quadratures
-    // per quadrature half: the tile's rows i weighted for sigma and for A, and its rows k
-    __shared__ double ws[2][kTile][kMaxModes + 1], wa[2][kTile][kMaxModes + 1], rk[2][kTile][kMaxModes + 1];
+    __shared__ double rows[2][kTile][2 * kMaxModes + 1];  // the tile's rows i and k of R
     __shared__ double part[kParts][kEnt];
     const cg::cluster_group cl = cg::this_cluster();
     const int t = threadIdx.x, N = 2 * M, rank = (int)cl.block_rank();
@@ -66,29 +66,21 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kStateThreads
             if (row >= N) continue;
             const bool ip = row >= M;
             const double *u = U + 2 * ((size_t)(ip ? row - M : row) * M + j);  // 8-byte aligned
-            const double x = ip ? u[1] : u[0], q = ip ? u[0] : -u[1];
-            if (side) {
-                rk[0][l][j] = x;
-                rk[1][l][j] = q;
-            } else {
-                ws[0][l][j] = x * w[j].x;
-                ws[1][l][j] = q * w[M + j].x;
-                wa[0][l][j] = x * w[j].y;
-                wa[1][l][j] = q * w[M + j].y;
-            }
+            rows[side][l][j] = ip ? u[1] : u[0];
+            rows[side][l][M + j] = ip ? u[0] : -u[1];
         }
         __syncthreads();
         const int e = t & (kEnt - 1), pt = t / kEnt, li = e / kTile, lk = e % kTile;
         const int i = bi * kTile + li, k = bk * kTile + lk;
         if (i < N && k < N) {
             double acc = 0.0;
-            if (pt < 4) {
-                const double *a = pt < 2 ? ws[pt & 1][li] : wa[pt & 1][li], *b = rk[pt & 1][lk];
+            if (pt < 2) {
+                const double *a = rows[0][li], *b = rows[1][lk];
 #pragma unroll 4
-                for (int j = 0; j < M; ++j) acc = fma(a[j], b[j], acc);
+                for (int j = 0; j < N; ++j) acc = fma(a[j] * b[j], pt ? w[j].y : w[j].x, acc);
             } else if (i < M) {
                 // column i of U against column c: the real part (k < M), or the imaginary part
-                const bool kp = k >= M, im = pt == 5;
+                const bool kp = k >= M, im = pt == 3;
                 const int c = kp ? k - M : k;
                 const double *a = U + 2 * i + im, *b = U + 2 * c + (im != kp);
                 if (i <= c) {
@@ -102,15 +94,14 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kStateThreads
         __syncthreads();
         if (i < N && k < N) {
             if (pt == 0 && sigma && i <= k) {
-                const double v = part[0][e] + part[1][e];
-                sigma[i * N + k] = v;
-                sigma[k * N + i] = v;
-            } else if (pt == 2 && i <= k) {
-                const double v = (i == k ? 1.0 : 0.0) - (part[2][e] + part[3][e]);
+                sigma[i * N + k] = part[0][e];
+                sigma[k * N + i] = part[0][e];
+            } else if (pt == 1 && i <= k) {
+                const double v = (i == k ? 1.0 : 0.0) - part[1][e];
                 O[i * N + k] = v;
                 O[k * N + i] = v;
-            } else if (pt == 4) {
-                const double v = part[4][e] + part[5][e] - (i == k && i < M ? 1.0 : 0.0);
+            } else if (pt == 2) {
+                const double v = part[2][e] + part[3][e] - (i == k && i < M ? 1.0 : 0.0);
                 if (!(fabs(v) <= 1e-10)) atomicExch(status, (int32_t)GBS_E_INVALID);
             }
         }
@@ -119,7 +110,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kStateThreads
     // this pipe), added in the order of a warp that strides the modes
     if (blockIdx.x == gridDim.x - 1) {
         __syncthreads();
-        double *term = &ws[0][0][0];
+        double *term = &rows[0][0][0];
         for (int j = t; j < M; j += kStateThreads) {
             const double rj = r[j];
             if (!(rj >= 0.0) || !isfinite(rj)) atomicExch(status, (int32_t)GBS_E_INVALID);
