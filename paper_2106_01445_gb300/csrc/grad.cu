@@ -17,18 +17,458 @@
 // mesh U = T_last ... T_1, T(theta, phi) = [[e^{i phi} cos, -sin], [e^{i phi} sin, cos]].
 #include "dd.cuh"
 #include "gbs_internal.cuh"
+#include "qf.cuh"
 
 namespace {
 
 constexpr int kGradMaxN = 24;            // clicks per pattern on the gradient path
 constexpr int kGD = 2 * kGradMaxN;       // largest pattern matrix (48 x 48)
 constexpr int kTM = 7;                   // modes of a unit's subtree (2^7 leaves)
-constexpr int kTreeThreads = 128;
+constexpr int kTreeThreads = 256;
+constexpr int kChunkBits = 8;            // a chunk: at most 2^8 units sharing their high prefix modes
+constexpr int kGroupBits = 4;            // a group: at most 2^4 units walked as a tree
 
 __host__ __device__ constexpr int gsym(int d) { return d * (d + 1) / 2; }
-// packed upper-triangle index of (i, j), i <= j
+// packed upper-triangle index of (i, j), i <= j.  The rows of the trailing block of modes below
+// are the suffix of the array: the block left when the first mode is excluded starts 2 d - 1
+// entries further on and is packed itself.
 __host__ __device__ constexpr int gpidx(int d, int i, int j) { return i * d - (i * (i - 1)) / 2 + (j - i); }
 __device__ __forceinline__ int gpany(int d, int i, int j) { return i <= j ? gpidx(d, i, j) : gpidx(d, j, i); }
+// the include children of a unit's subtree, level after level, after its root
+__host__ __device__ constexpr int lvl_off(int l) {
+    int s = gsym(2 * kTM);
+    for (int q = 1; q < l; ++q) s += (1 << (q - 1)) * gsym(2 * (kTM - q));
+    return s;
+}
+__host__ __device__ constexpr int adj_cap() {
+    int m = gsym(2 * (kTM + kGroupBits));
+    for (int l = 0; l < kTM; ++l) m = (1 << l) * gsym(2 * (kTM - l)) > m ? (1 << l) * gsym(2 * (kTM - l)) : m;
+    return m;
+}
+__host__ __device__ constexpr int row_cap() {  // 2 x dc entries of every parent of a level
+    int m = 2 * (kGD - 2);
+    for (int l = 0; l < kTM; ++l) m = (1 << l) * 4 * (kTM - l - 1) > m ? (1 << l) * 4 * (kTM - l - 1) : m;
+    return m;
+}
+__host__ __device__ constexpr int tri_sum(int from, int to) {  // packed matrices of from .. to modes
+    int s = 0;
+    for (int m = from; m <= to; ++m) s += gsym(2 * m);
+    return s;
+}
+constexpr int kNodes = (1 << kTM) - 1;   // nodes of levels 0..kTM-1
+constexpr int kUD = 2 * (kChunkBits + kTM);  // largest group matrix (middle prefix modes, group, subtree)
+// shared memory (qf elements), SM at the end (its size is the batch's).
+// UM: the group's matrix; Gam: the adjoint of SM's trailing block summed over the groups; Sl, Gx,
+// dS: the group tree's include matrices, exclude adjoints and sums; Lv: the subtree's include
+// matrices, and between subtrees the group's (Gf) or the chunk's (Gs) adjoint; SM: the chunk's matrix
+constexpr int kOffUM = 0, kOffGam = kOffUM + gsym(kUD), kOffSl = kOffGam + gsym(kUD);
+constexpr int kOffGx = kOffSl + tri_sum(kTM + 1, kTM + kGroupBits - 1);
+constexpr int kOffLv = kOffGx + tri_sum(kTM, kTM + kGroupBits - 1);
+constexpr int kLvCap = lvl_off(kTM) > gsym(kGD) ? lvl_off(kTM) : gsym(kGD);
+constexpr int kOffAdjA = kOffLv + kLvCap, kOffAdjB = kOffAdjA + adj_cap();
+constexpr int kOffQ = kOffAdjB + adj_cap(), kOffRs = kOffQ + 3 * kNodes, kOffS = kOffRs + kNodes;
+constexpr int kOffZ = kOffS + kNodes, kOffY = kOffZ + row_cap(), kOffM2 = kOffY + row_cap();
+constexpr int kOffDQ = kOffM2 + 3 * (1 << (kTM - 1)), kOffDRs = kOffDQ + 3 * kGroupBits, kOffDS = kOffDRs + kGroupBits;
+constexpr int kOffPreQ = kOffDS + kGroupBits + 2, kOffPreRs = kOffPreQ + 3 * kChunkBits;
+constexpr int kOffHiQ = kOffPreRs + kChunkBits, kOffHiRs = kOffHiQ + 3 * kGradMaxN;
+constexpr int kOffSM = kOffHiRs + kGradMaxN;
+__host__ __device__ constexpr int tree_smem(int n_max) { return kOffSM + gsym(2 * n_max); }
+
+// (i, j), i <= j, of packed entry f of an even dimension d: rows p and d - 1 - p folded
+__device__ __forceinline__ void fold_ij(int f, int d, int &i, int &j) {
+    const int w = d + 1, p = f / w, k = f - p * w;
+    if (k < d - p) {
+        i = p;
+        j = p + k;
+    } else {
+        i = d - 1 - p;
+        j = i + (k - (d - p));
+    }
+}
+
+// One level of include steps, forward.  Parent cp (of np) is the packed d x d matrix at base +
+// noff[cp]; its pivot block is the first mode.  Stores P^{-1} (the off-diagonal entry negated, here
+// and wherever P^{-1} is kept) in Q + 3 cp and det^{-1/2} in rs[cp], and writes the include child
+// C - W B^T (W = P^{-1} B) to dst + cp * gsym(d - 2) (which may be the parent's own trailing block),
+// with the children's places in nchild (exclude, include) where it is given.  d = 2: pivots only.
+__device__ __noinline__ void tree_forward(qf *base, int np, int d, const uint16_t *noff, qf *dst, uint16_t *nchild,
+                                          qf *Q, qf *rs, qf *W, int *bad) {
+    const int t = threadIdx.x, dc = d - 2, stc = gsym(dc);
+    // four lanes a parent: the determinant and its root on each, then one product each
+    if (t < 4 * np) {
+        const int cp = t >> 2, k = t & 3;
+        const qf *P = base + noff[cp];
+        const qf p00 = P[0], p01 = P[1], p11 = P[d];
+        const qf det = qf_dot2s(false, p00, p11, true, p01, p01);
+        const qf r = qf_rsqrt(det), inv = r * r;
+        qf f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) f.w[c] = k == 0 ? p11.w[c] : k == 1 ? p01.w[c] : p00.w[c];
+        f = f * inv;
+        if (k < 3) {
+            Q[3 * cp + k] = f;
+        } else {
+            rs[cp] = r;
+            if (!qf_positive(det)) atomicOr(bad, 1);
+            if (nchild) {
+                nchild[2 * cp] = (uint16_t)(noff[cp] + 2 * d - 1);
+                nchild[2 * cp + 1] = (uint16_t)(dst - base + cp * stc);
+            }
+        }
+    }
+    __syncthreads();
+    if (dc == 0) return;
+    for (int f = t; f < np * dc * 2; f += kTreeThreads) {
+        const int cp = f / (2 * dc), x = f - cp * 2 * dc, i = x >> 1, a = x & 1;
+        const qf *P = base + noff[cp], *q = Q + 3 * cp;
+        W[f] = qf_dot2s(a, q[a], P[2 + i], !a, q[1 + a], P[d + 1 + i]);
+    }
+    __syncthreads();
+    for (int f = t; f < np * stc; f += kTreeThreads) {
+        const int cp = f / stc, e = f - cp * stc;
+        int i, j;
+        fold_ij(e, dc, i, j);
+        const qf *P = base + noff[cp], *w = W + 2 * (cp * dc + i);
+        const int at = gpidx(dc, i, j);
+        dst[cp * stc + at] = qf_fms2(P[2 * d - 1 + at], w[0], P[2 + j], w[1], P[d + 1 + j]);
+    }
+    __syncthreads();
+}
+
+// One level of include steps, backward: from the children's adjoints to the parents'.  Parent cp's
+// include child has the adjoint Gi + cp * gs (packed, d - 2 rows) and the sum Si[cp * ss]; its
+// exclude child, unless Ge is null, Ge + cp * gs and Se[cp * ss].  With Y = P^{-1} B Gi the parent's
+// adjoint is, times rs,
+//   rest: Gi - Ge / rs,   pivot rows: -Y,   pivot block: P^{-1} (B Gi B^T) P^{-1} - Si P^{-1} / 2
+// (Ge null: the pivot of a shared prefix, whose factor is in Si already: no rs, and the rest stays
+// where it is, out's own trailing block).  So, Ao: the parents' sums and, to 20 bits, the sums of their
+// terms' sizes.  K: slices of a row sum, for levels with few parents.
+__device__ __noinline__ void tree_backward(const qf *base, int np, int d, const uint16_t *noff, const qf *Gi,
+                                           const qf *Ge, int gs, qf *out, const qf *Q, const qf *rs, const qf *Si,
+                                           const qf *Se, int ss, qf *So, const double *Ai, const double *Ae, double *Ao, qf *Z,
+                                           qf *Y, qf *M2, int K) {
+    const int t = threadIdx.x, t2 = kTreeThreads - 1 - t, dc = d - 2, st = gsym(d), stc = gsym(dc);
+    // Z = B Gi, slice k of K of entry (a, j): whole warps, for the sums over the slices
+    const int nz = np * dc * 2 * K;
+    for (int f = t; f < ((nz + 31) & ~31); f += kTreeThreads) {
+        const int g = min(f, nz - 1) / K, k = f & (K - 1), cp = g / (2 * dc), x = g - cp * 2 * dc, j = x >> 1, a = x & 1;
+        const qf *b = base + noff[cp] + (a ? d + 1 : 2), *G = Gi + cp * gs;
+        qf z = qf_dot(k, K, dc, [&](int i) { return G + gpany(dc, i, j); }, [&](int i) { return b + i; });
+        for (int off = 1; off < K; off <<= 1) {
+            qf o;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) o.w[c] = __shfl_xor_sync(0xffffffffu, z.w[c], off);
+            z = z + o;
+        }
+        if (f < nz && k == 0) Z[g] = z;
+    }
+    if (So && t2 < np) {
+        So[t2] = qf_fma<false, true>(Se[t2 * ss], rs[t2], Si[t2 * ss]);
+        Ao[t2] = fma(qf_approx(rs[t2]), Ai[t2 * ss], Ae[t2 * ss]);
+    }
+    __syncthreads();
+    for (int f = t; f < np * dc * 2; f += kTreeThreads) {
+        const int cp = f / (2 * dc), x = f - cp * 2 * dc, j = x >> 1, a = x & 1;
+        const qf *q = Q + 3 * cp, *z = Z + 2 * (cp * dc + j);
+        Y[f] = qf_dot2s(a, q[a], z[0], !a, q[1 + a], z[1]);
+    }
+    for (int f = t2; f < np * 3; f += kTreeThreads) {
+        const int cp = f / 3, ij = f - 3 * cp;  // (0, 0), (0, 1), (1, 1)
+        const qf *z = Z + 2 * cp * dc + (ij == 2), *b = base + noff[cp] + (ij ? d + 1 : 2);
+        M2[f] = qf_dot(0, 1, dc, [&](int c) { return z + 2 * c; }, [&](int c) { return b + c; });
+    }
+    __syncthreads();
+    const int nrest = Ge ? np * stc : 0;
+    for (int f = t; f < nrest; f += kTreeThreads) {
+        const int cp = f / stc, e = f - cp * stc;
+        out[cp * st + 2 * d - 1 + e] = qf_fma<false, true>(Ge[cp * gs + e], rs[cp], Gi[cp * gs + e]);
+    }
+    for (int f = t; f < np * dc * 2; f += kTreeThreads) {
+        const int cp = f / (2 * dc), x = f - cp * 2 * dc, j = x >> 1, a = x & 1;
+        out[cp * st + (a ? d + 1 : 2) + j] = qf_mul<true>(Ge ? rs[cp] : qf_one(), Y[f]);
+    }
+    for (int f = t2; f < np * 3; f += kTreeThreads) {
+        const int cp = f / 3, ij = f - 3 * cp, i = ij == 2, j = ij != 0;
+        const qf *q = Q + 3 * cp, *m = M2 + 3 * cp;
+        // column j of M2 P^{-1}, then row i of P^{-1} times it
+        const qf u0 = qf_dot2s(j, m[0], q[j], !j, m[1], q[1 + j]), u1 = qf_dot2s(j, m[1], q[j], !j, m[2], q[1 + j]);
+        const qf v = qf_dot2s(i, q[i], u0, !i, q[1 + i], u1), h = qf_half(Si[cp * ss]);
+        const qf r = ij == 1 ? qf_fma<false>(v, h, q[1]) : qf_fma<true>(v, h, q[ij]);
+        out[cp * st + (ij == 2 ? d : ij)] = Ge ? rs[cp] * r : r;
+    }
+    __syncthreads();
+}
+
+// Gbar_p = dT/dA_S by reverse mode through the include/exclude Schur recursion.
+// Units = (pattern, include/exclude choice of the first q = n - m modes), m = min(n, 7), the
+// subtree over the last m modes.  S(node) = rs S(include child) - S(exclude child), 1 at a leaf;
+// Gamma(node) = dS(node)/dC_node from the children's (tree_backward); a node's exclude child is the
+// suffix of its packed matrix, so only include children are stored.
+// One CTA per chunk: an aligned run of 2^b units of one pattern.  Of the prefix modes the high
+// ones (b and up) are fixed by the chunk and eliminated once; the others are the bits of the unit,
+// the last kGroupBits of them (the group's) walked depth first as a tree over the units' subtrees,
+// each include's matrix and each exclude's adjoint kept per depth, so that a unit costs one tree
+// pivot and one step back on average; the ones between (middle) are eliminated once per group.
+// The group's adjoint goes back through its middle pivots into Gam, and Gam at the end
+// through the chunk's high pivots with V = the chunk's sum (the adjoint of a shared step is linear in
+// what flows into it).
+//
+// What bounds it: integer instructions and, with two CTAs an SM, the latency of about 40 phases a
+// unit; the work of a phase is cut fine for that (a row sum in up to four slices, a pivot over
+// four lanes, long jobs on the last warps beside the short ones on the first).  Measured on the
+// 32-mode Clements workload (512 patterns, n = 8..16): 69.5 ms in double-double (FP64 pipe 70% busy),
+// 49.9 with the same kernel in qf (barriers, divergence), 18.0 as it is here.
+__global__ void __launch_bounds__(kTreeThreads, 2) grad_tree_kernel(int M, int n_max, const double *__restrict__ O,
+                                                               const uint64_t *__restrict__ pats,
+                                                               const int *__restrict__ chunk_p,
+                                                               const long long *__restrict__ chunk_u, size_t pst,
+                                                               qf *__restrict__ part, qf *__restrict__ part_T,
+                                                               double *__restrict__ part_A,
+                                                               int *__restrict__ flags) {
+    extern __shared__ __align__(16) unsigned char gsm[];
+    qf *const base = (qf *)gsm;
+    qf *const SM = base + kOffSM, *const Gs = base + kOffLv, *const UM = base + kOffUM, *const Gf = base + kOffLv;
+    qf *const Gam = base + kOffGam, *const Lv = base + kOffLv;
+    qf *const nQ = base + kOffQ, *const nrs = base + kOffRs, *const nS = base + kOffS;
+    qf *const Zb = base + kOffZ, *const Yb = base + kOffY, *const M2 = base + kOffM2;
+    qf *const dQ = base + kOffDQ, *const dRs = base + kOffDRs, *const dS = base + kOffDS;
+    qf *const preQ = base + kOffPreQ, *const prers = base + kOffPreRs;
+    qf *const hiQ = base + kOffHiQ, *const hiRs = base + kOffHiRs;
+    __shared__ uint8_t modes[128], smrow[kGD], umrow[kUD];  // rows of SM and UM: see below
+    __shared__ uint16_t nptr[kNodes + 1], s_off[1], dptr[kGroupBits + 1];
+    __shared__ int s_bad;
+    __shared__ qf s_T, s_V, s_S[2];
+    __shared__ double nA[kNodes], dA[kGroupBits], s_A[2], s_Asum;
+    const int t = threadIdx.x, ch = blockIdx.x, p = chunk_p[ch], N2 = 2 * M;
+    const long long u_begin = chunk_u[2 * ch], u_end = chunk_u[2 * ch + 1];
+    const uint64_t wlo = pats[2 * p], whi = pats[2 * p + 1];
+    const int nlo = __popcll(wlo), n = nlo + __popcll(whi), m = n < kTM ? n : kTM, q = n - m, Dn = 2 * n;
+    if (t < M) {
+        const uint64_t w = t < 64 ? wlo : whi, bit = 1ull << (t & 63);
+        if (w & bit) modes[(t < 64 ? 0 : nlo) + __popcll(w & (bit - 1))] = (uint8_t)t;
+    }
+    if (t == 0) {
+        s_bad = 0;
+        s_Asum = 0.0;
+        s_T = n == 0 && u_begin == 0 ? qf_one() : qf_zero();
+    }
+    // the chunk's 2^bl units vary the prefix modes 0..bl-1: the middle ones 0..bm-1 and the group's
+    // g modes bm..bl-1; modes bl..q-1 are fixed by u_begin
+    const int bl = u_end > u_begin ? 63 - __clzll(u_end - u_begin) : 0;
+    const int g = bl < kGroupBits ? bl : kGroupBits, bm = bl - g;
+    const unsigned long long hi = (unsigned long long)u_begin >> bl;
+    const int kh = __popcll(hi), Ds = 2 * (kh + bl + m), Dr = 2 * (bl + m);
+    // SM: the included high modes, then modes 0..bl-1, then the subtree's; smrow: row -> pattern row
+    if (t < q) {
+        const int a = t;
+        int r = -1;
+        if (a < bl) r = kh + a;
+        else if (hi >> (a - bl) & 1) r = __popcll(hi & ((1ull << (a - bl)) - 1));
+        if (r >= 0) {
+            smrow[2 * r] = (uint8_t)(2 * a);
+            smrow[2 * r + 1] = (uint8_t)(2 * a + 1);
+        }
+    } else if (t < n) {
+        const int r = kh + bl + t - q;
+        smrow[2 * r] = (uint8_t)(2 * t);
+        smrow[2 * r + 1] = (uint8_t)(2 * t + 1);
+    }
+    __syncthreads();
+    // the chunk's rows of A = I - O, its high pivots, and a zero Gam
+    for (int f = t; f < gsym(Ds); f += kTreeThreads) {
+        int i, j;
+        fold_ij(f, Ds, i, j);
+        const int ri = smrow[i], rj = smrow[j];
+        const int gi = modes[ri >> 1] + (ri & 1) * M, gj = modes[rj >> 1] + (rj & 1) * M;
+        SM[gpidx(Ds, i, j)] = (i == j ? qf_one() : qf_zero()) - qf_from_double(O[(size_t)gi * N2 + gj]);
+    }
+    for (int f = t; f < gsym(Dr); f += kTreeThreads) Gam[f] = qf_zero();
+    // where the packed trailing block of the last d rows of a D-row matrix starts
+    auto tail = [](int D, int d) { return gsym(D) - gsym(d); };
+    for (int e = 0; e < kh; ++e) {
+        const int d = Ds - 2 * e;
+        if (t == 0) s_off[0] = (uint16_t)(SM - base + tail(Ds, d));
+        __syncthreads();
+        tree_forward(base, 1, d, s_off, SM + tail(Ds, d - 2), nullptr, hiQ + 3 * e, hiRs + e, Zb, &s_bad);
+    }
+    const int groups = n > 0 ? 1 << bm : 0;
+    for (int gr = 0; gr < groups; ++gr) {
+        const int kl = __popc(gr), D0 = 2 * (kl + g + m), k0 = kh + kl;
+        // UM: SM's trailing block on the group's included middle modes, its own modes and the
+        // subtree; umrow: row -> row of SM's trailing block
+        if (t < bm) {
+            if (gr >> t & 1) {
+                const int r = __popc(gr & ((1 << t) - 1));
+                umrow[2 * r] = (uint8_t)(2 * t);
+                umrow[2 * r + 1] = (uint8_t)(2 * t + 1);
+            }
+        } else if (t < bl + m) {
+            const int r = kl + t - bm;
+            umrow[2 * r] = (uint8_t)(2 * t);
+            umrow[2 * r + 1] = (uint8_t)(2 * t + 1);
+        }
+        __syncthreads();
+        for (int f = t; f < gsym(D0); f += kTreeThreads) {
+            int i, j;
+            fold_ij(f, D0, i, j);
+            UM[gpidx(D0, i, j)] = SM[gpidx(Ds, 2 * kh + umrow[i], 2 * kh + umrow[j])];
+        }
+        for (int e = 0; e < kl; ++e) {
+            const int d = D0 - 2 * e;
+            if (t == 0) s_off[0] = (uint16_t)(UM - base + tail(D0, d));
+            __syncthreads();
+            tree_forward(base, 1, d, s_off, UM + tail(D0, d - 2), nullptr, preQ + 3 * e, prers + e, Zb, &s_bad);
+        }
+        // the group's tree: depth e chooses mode e; dptr[e]: the matrix of the path's node there
+        const int dg = 2 * (g + m);
+        if (t == 0) {
+            dptr[0] = (uint16_t)(UM - base + tail(D0, dg));
+            for (int e = 0; e < g; ++e) dptr[e + 1] = (uint16_t)(dptr[e] + 2 * (dg - 2 * e) - 1);
+        }
+        __syncthreads();
+        qf *cur = nullptr;
+        int cs = 0;  // s_S[cs]: the sum that belongs to cur
+        for (int leaf = 0; leaf < 1 << g; ++leaf) {
+            if (leaf) {
+                // the depth whose choice turns include; deeper choices are excludes
+                const int e = g - __ffs(leaf), d = dg - 2 * e;
+                qf *dst = e + 1 == g ? Lv : base + kOffSl;
+                if (e + 1 < g)
+                    for (int x = 1; x <= e; ++x) dst += gsym(dg - 2 * x);
+                tree_forward(base, 1, d, dptr + e, dst, nullptr, dQ + 3 * e, dRs + e, Zb, &s_bad);
+                if (t == 0) {
+                    dptr[e + 1] = (uint16_t)(dst - base);
+                    for (int x = e + 1; x < g; ++x) dptr[x + 1] = (uint16_t)(dptr[x] + 2 * (dg - 2 * x) - 1);
+                }
+                __syncthreads();
+            }
+            if (t == 0) nptr[0] = dptr[g];
+            __syncthreads();
+            // the subtree, forward
+            for (int l = 0; l < m; ++l) {
+                const int np = 1 << l;
+                tree_forward(base, np, 2 * (m - l), nptr + np - 1, Lv + lvl_off(l + 1), l < m - 1 ? nptr + 2 * np - 1 : nullptr,
+                             nQ + 3 * (np - 1), nrs + np - 1, Zb, &s_bad);
+            }
+            // its last level: S = rs - 1, Gamma = -rs P^{-1} / 2
+            qf *Ach = base + ((m - 1) & 1 ? kOffAdjB : kOffAdjA);
+            for (int f = t; f < 4 << (m - 1); f += kTreeThreads) {
+                const int c = f >> 2, x = f & 3, node = (1 << (m - 1)) - 1 + c;
+                if (x == 3) {
+                    nS[node] = nrs[node] - qf_one();
+                    nA[node] = qf_approx(nrs[node]) + 1.0;
+                } else {
+                    const qf h = qf_half(nrs[node]), v = nQ[3 * node + x];
+                    Ach[3 * c + x] = x == 1 ? h * v : qf_mul<true>(h, v);
+                }
+            }
+            __syncthreads();
+            for (int l = m - 2; l >= 0; --l) {
+                const int np = 1 << l, d = 2 * (m - l);
+                const qf *Ac = base + ((l + 1) & 1 ? kOffAdjB : kOffAdjA);
+                qf *Ap = base + (l & 1 ? kOffAdjB : kOffAdjA);
+                const int stc = gsym(d - 2);
+                tree_backward(base, np, d, nptr + np - 1, Ac + stc, Ac, 2 * stc, Ap, nQ + 3 * (np - 1), nrs + np - 1,
+                              nS + 2 * np, nS + 2 * np - 1, 2, nS + np - 1, nA + 2 * np, nA + 2 * np - 1,
+                              nA + np - 1, Zb, Yb, M2, l < 2 ? 4 : l < 4 ? 2 : 1);
+            }
+            // up the group's tree: an include's adjoint joins the kept exclude's, an exclude's is kept
+            cur = base + kOffAdjA;
+            if (t == 0) {
+                s_S[0] = nS[0];
+                s_A[0] = nA[0];
+            }
+            cs = 0;
+            __syncthreads();
+            for (int e = g - 1; e >= 0; --e) {
+                const int d = dg - 2 * e, stc = gsym(d - 2);
+                qf *Gx = base + kOffGx;
+                for (int x = 0; x < e; ++x) Gx += gsym(dg - 2 * (x + 1));
+                if (leaf >> (g - 1 - e) & 1) {
+                    qf *out = base + (cur == base + kOffAdjA ? kOffAdjB : kOffAdjA);
+                    tree_backward(base, 1, d, dptr + e, cur, Gx, stc, out, dQ + 3 * e, dRs + e, s_S + cs, dS + e, 0,
+                                  s_S + (cs ^ 1), s_A + cs, dA + e, s_A + (cs ^ 1), Zb, Yb, M2, 4);
+                    cur = out;
+                    cs ^= 1;
+                } else {
+                    for (int f = t; f < stc; f += kTreeThreads) Gx[f] = cur[f];
+                    if (t == 0) {
+                        dS[e] = s_S[cs];
+                        dA[e] = s_A[cs];
+                    }
+                    __syncthreads();
+                    break;
+                }
+            }
+        }
+        // the group's value and adjoint, back through its middle pivots and into Gam
+        if (t == 0) {
+            qf tau = qf_one();
+            for (int e = 0; e < kh; ++e) tau = tau * hiRs[e];
+            for (int e = 0; e < kl; ++e) tau = tau * prers[e];
+            if ((q - g - k0) & 1) tau = -tau;
+            s_S[cs ^ 1] = tau;
+            s_V = tau * s_S[cs];
+            s_T = s_T + s_V;
+            s_Asum += fabs(qf_approx(tau)) * s_A[cs];
+        }
+        __syncthreads();
+        for (int f = t; f < gsym(dg); f += kTreeThreads) Gf[tail(D0, dg) + f] = s_S[cs ^ 1] * cur[f];
+        __syncthreads();
+        for (int e = kl - 1; e >= 0; --e) {
+            const int d = D0 - 2 * e;
+            if (t == 0) s_off[0] = (uint16_t)(UM - base + tail(D0, d));
+            __syncthreads();
+            tree_backward(base, 1, d, s_off, Gf + tail(D0, d - 2), nullptr, 0, Gf + tail(D0, d), preQ + 3 * e, nullptr,
+                          &s_V, nullptr, 0, nullptr, nullptr, nullptr, nullptr, Zb, Yb, M2, 4);
+        }
+        for (int f = t; f < gsym(D0); f += kTreeThreads) {
+            int i, j;
+            fold_ij(f, D0, i, j);
+            qf &x = Gam[gpidx(Dr, umrow[i], umrow[j])];
+            x = x + Gf[gpidx(D0, i, j)];
+        }
+        __syncthreads();
+    }
+    // the chunk: Gam as the adjoint of SM's trailing block, back through the high pivots
+    // with the chunk's sum as their V
+    for (int f = t; f < gsym(Dr); f += kTreeThreads) Gs[tail(Ds, Dr) + f] = Gam[f];
+    __syncthreads();
+    for (int e = kh - 1; e >= 0; --e) {
+        const int d = Ds - 2 * e;
+        if (t == 0) s_off[0] = (uint16_t)(SM - base + tail(Ds, d));
+        __syncthreads();
+        tree_backward(base, 1, d, s_off, Gs + tail(Ds, d - 2), nullptr, 0, Gs + tail(Ds, d), hiQ + 3 * e, nullptr, &s_T,
+                      nullptr, 0, nullptr, nullptr, nullptr, nullptr, Zb, Yb, M2, 4);
+    }
+    // dense partial (row stride 2n): zero, then the chunk's rows
+    for (int f = t; f < Dn * Dn; f += kTreeThreads) part[ch * pst + f] = qf_zero();
+    __syncthreads();
+    for (int f = t; f < gsym(Ds); f += kTreeThreads) {
+        int i, j;
+        fold_ij(f, Ds, i, j);
+        const qf x = Gs[gpidx(Ds, i, j)];
+        const int ri = smrow[i], rj = smrow[j];
+        part[ch * pst + (size_t)ri * Dn + rj] = x;
+        part[ch * pst + (size_t)rj * Dn + ri] = x;
+    }
+    if (t == 0) {
+        part_T[ch] = s_T;
+        part_A[ch] = n == 0 ? 1.0 : s_Asum;
+        if (s_bad) atomicOr(flags + p, 1);
+    }
+}
+
+// ---- the same adjoint in double-double --------------------------------------------------------
+// For patterns whose sum cancels by more than kRedo: there the result is limited by the arithmetic
+// (a relative error of about 3e-34 kappa in double-double, a tenth of that in qf, against a quadruple
+// precision sum over the subsets), so the two differ by 1e-9 and more, and callers keep the values
+// they had.  CTAs of other patterns leave at once.  A batch that has such patterns pays for one chunk's
+// time here (about 5 ms on the 32-mode workload).
+namespace ddk {
+constexpr int kTM = 7;                   // modes of a unit's subtree (2^7 leaves)
+constexpr int kTreeThreads = 128;
+
 // level l of a unit's subtree: 2^l nodes of dimension 2 (kTM - l), packed, back to back
 __host__ __device__ constexpr int lvl_off(int l) {
     int s = 0;
@@ -59,18 +499,6 @@ constexpr int kOffQ = kOffAdjB + lvl_cap(), kOffRs = kOffQ + 3 * kNodes, kOffS =
 constexpr int kOffY = kOffS + kNodes, kOffPreQ = kOffY + y_cap(), kOffPreRs = kOffPreQ + 3 * kGradMaxN;
 constexpr int kOffHiQ = kOffPreRs + kGradMaxN, kOffHiRs = kOffHiQ + 3 * kGradMaxN;
 constexpr int kTreeSmem = kOffHiRs + kGradMaxN;
-
-// (i, j), i <= j, of packed entry f of an even dimension d: rows p and d - 1 - p folded
-__device__ __forceinline__ void fold_ij(int f, int d, int &i, int &j) {
-    const int w = d + 1, p = f / w, k = f - p * w;
-    if (k < d - p) {
-        i = p;
-        j = p + k;
-    } else {
-        i = d - 1 - p;
-        j = i + (k - (d - p));
-    }
-}
 
 // One 2x2 pivot of the packed D x D unit matrix, eliminated by the CTA: rows and
 // columns >= c0 + 2 receive C - W B^T (W = B P^{-1}); the pivot rows stay as they were
@@ -163,13 +591,12 @@ __device__ void reverse_pivots(const dd *Mx, dd *G, int D, int np, const dd *Qs,
 // (Gam); at the end Gam goes back through the high pivots once, with V = the chunk's sum
 // (the adjoint of a shared step is linear in what flows into it), and the chunk's partial
 // Gbar and T are written; the chunks of a pattern are summed in order afterwards.
-__global__ void __launch_bounds__(kTreeThreads) grad_tree_kernel(int M, const double *__restrict__ O,
+__global__ void __launch_bounds__(kTreeThreads) grad_tree_dd_kernel(int M, const double *__restrict__ O,
                                                                const uint64_t *__restrict__ pats, int n_pat,
                                                                const int *__restrict__ chunk_p,
                                                                const long long *__restrict__ chunk_u, size_t pst,
-                                                               double *__restrict__ part_hi,
-                                                               double *__restrict__ part_lo,
-                                                               double *__restrict__ part_T, int *__restrict__ flags) {
+                                                               const int *__restrict__ redo, dd *__restrict__ part,
+                                                               dd *__restrict__ part_T, int *__restrict__ flags) {
     extern __shared__ __align__(16) unsigned char gsm[];
     dd *const base = (dd *)gsm;
     dd *const SM = base + kOffSM, *const Gs = base + kOffGs, *const UM = base + kOffUM, *const Gf = base + kOffGf;
@@ -183,6 +610,7 @@ __global__ void __launch_bounds__(kTreeThreads) grad_tree_kernel(int M, const do
     __shared__ int s_n, s_kh, s_kl, s_bad;
     __shared__ dd s_T, s_V;
     const int t = threadIdx.x, ch = blockIdx.x, p = chunk_p[ch], N2 = 2 * M;
+    if (!redo[p]) return;
     const long long u_begin = chunk_u[2 * ch], u_end = chunk_u[2 * ch + 1];
     if (t == 0) {
         int n = 0;
@@ -415,33 +843,46 @@ __global__ void __launch_bounds__(kTreeThreads) grad_tree_kernel(int M, const do
     __syncthreads();
     reverse_pivots(SM, Gs, Ds, kh, hiQ, s_T, Yb);
     // dense partial (row stride 2n): zero, then the chunk's rows
-    for (int f = t; f < Dn * Dn; f += kTreeThreads) {
-        part_hi[ch * pst + f] = 0.0;
-        part_lo[ch * pst + f] = 0.0;
-    }
+    for (int f = t; f < Dn * Dn; f += kTreeThreads) part[ch * pst + f] = dd(0.0);
     __syncthreads();
     for (int f = t; f < gsym(Ds); f += kTreeThreads) {
         int i, j;
         fold_ij(f, Ds, i, j);
         const dd g = Gs[gpidx(Ds, i, j)];
         const int ri = smrow[i], rj = smrow[j];
-        part_hi[ch * pst + (size_t)ri * Dn + rj] = g.hi;
-        part_lo[ch * pst + (size_t)ri * Dn + rj] = g.lo;
-        part_hi[ch * pst + (size_t)rj * Dn + ri] = g.hi;
-        part_lo[ch * pst + (size_t)rj * Dn + ri] = g.lo;
+        part[ch * pst + (size_t)ri * Dn + rj] = g;
+        part[ch * pst + (size_t)rj * Dn + ri] = g;
     }
     if (t == 0) {
-        part_T[2 * ch] = s_T.hi;
-        part_T[2 * ch + 1] = s_T.lo;
+        part_T[ch] = s_T;
         if (s_bad) atomicOr(flags + p, 1);
     }
+}
+
+}  // namespace ddk
+
+// the patterns that the double-double kernel takes again: kappa = sum |terms| / |T| above kRedo (or
+// no number), or a pivot that is not positive; their flags start afresh
+constexpr double kRedo = 1e24;
+__global__ void grad_redo_kernel(int n_pat, const long long *__restrict__ chunk_off, const qf *__restrict__ part_T,
+                                 const double *__restrict__ part_A, int *__restrict__ redo, int *__restrict__ flags) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n_pat) return;
+    qf T = qf_zero();
+    double A = 0.0;
+    for (long long c = chunk_off[p]; c < chunk_off[p + 1]; ++c) {
+        T = T + part_T[c];
+        A += part_A[c];
+    }
+    redo[p] = flags[p] == 0 && A < kRedo * fabs(qf_approx(T)) ? 0 : 1;
+    if (redo[p]) flags[p] = 0;
 }
 
 // per pattern: sum the chunk partials in order, F_p = (w_p / T_p) Gbar_p, log P_p
 __global__ void grad_finalize_kernel(int M, const uint64_t *__restrict__ pats, int n_pat,
                                      const long long *__restrict__ chunk_off, size_t pst,
-                                     const double *__restrict__ part_hi, const double *__restrict__ part_lo,
-                                     const double *__restrict__ part_T, const double *__restrict__ w,
+                                     const int *__restrict__ redo, const qf *__restrict__ part,
+                                     const qf *__restrict__ part_T, const double *__restrict__ w,
                                      const double *__restrict__ logdet, double *__restrict__ F,
                                      double *__restrict__ logP, int32_t *__restrict__ status,
                                      const int *__restrict__ flags) {
@@ -452,7 +893,13 @@ __global__ void grad_finalize_kernel(int M, const uint64_t *__restrict__ pats, i
         int n = __popcll(pats[2 * p]) + __popcll(pats[2 * p + 1]);
         s_n = n;
         dd T = dd(0.0);
-        for (long long c = chunk_off[p]; c < chunk_off[p + 1]; ++c) T += dd(part_T[2 * c], part_T[2 * c + 1]);
+        if (redo[p]) {
+            for (long long c = chunk_off[p]; c < chunk_off[p + 1]; ++c) T += ((const dd *)part_T)[c];
+        } else {
+            qf Tq = qf_zero();
+            for (long long c = chunk_off[p]; c < chunk_off[p + 1]; ++c) Tq = Tq + part_T[c];
+            T = qf_to_dd(Tq);
+        }
         int st = flags[p] ? GBS_E_NOT_SPD : (T.hi > 0.0 ? GBS_OK : GBS_E_NONPOSITIVE);
         if (status) status[p] = st;
         if (logP) logP[p] = st ? nan("") : -0.5 * (*logdet) + log(T.hi) + log1p(T.lo / T.hi);
@@ -462,8 +909,13 @@ __global__ void grad_finalize_kernel(int M, const uint64_t *__restrict__ pats, i
     const int D = 2 * s_n;
     for (int f = threadIdx.x; f < D * D; f += blockDim.x) {
         dd s = dd(0.0);
-        for (long long c = chunk_off[p]; c < chunk_off[p + 1]; ++c)
-            s += dd(part_hi[(size_t)c * pst + f], part_lo[(size_t)c * pst + f]);
+        if (redo[p]) {
+            for (long long c = chunk_off[p]; c < chunk_off[p + 1]; ++c) s += ((const dd *)part)[(size_t)c * pst + f];
+        } else {
+            qf sq = qf_zero();
+            for (long long c = chunk_off[p]; c < chunk_off[p + 1]; ++c) sq = sq + part[(size_t)c * pst + f];
+            s = qf_to_dd(sq);
+        }
         F[(size_t)p * kGD * kGD + f] = (s.hi + s.lo) * s_scale;
     }
 }
@@ -741,9 +1193,10 @@ int grad_sigmaQ(gbs_ctx *ctx, int M, const double *O, const double *logdet, cons
     const int N = 2 * M;
     const size_t pst = (size_t)(2 * n_max) * (2 * n_max);  // one chunk's dense partial (row stride 2n)
     size_t o_off = 0, o_cu = al(o_off + 8 * ((size_t)n_pat + 1)), o_cp = al(o_cu + 16 * (size_t)chunks),
-           o_flags = al(o_cp + 4 * (size_t)chunks), o_phi = al(o_flags + 4 * (size_t)n_pat),
-           o_plo = al(o_phi + 8 * (size_t)chunks * pst), o_pT = al(o_plo + 8 * (size_t)chunks * pst),
-           o_F = al(o_pT + 16 * (size_t)chunks), o_H = al(o_F + 8 * (size_t)n_pat * kGD * kGD),
+           o_flags = al(o_cp + 4 * (size_t)chunks), o_part = al(o_flags + 4 * (size_t)n_pat),
+           o_pT = al(o_part + sizeof(qf) * (size_t)chunks * pst), o_pA = al(o_pT + sizeof(qf) * (size_t)chunks),
+           o_redo = al(o_pA + 8 * (size_t)chunks),
+           o_F = al(o_redo + 4 * (size_t)n_pat), o_H = al(o_F + 8 * (size_t)n_pat * kGD * kGD),
            o_T1 = al(o_H + 8 * (size_t)N * N), o_T2 = al(o_T1 + 8 * (size_t)N * N), o_sw = al(o_T2 + 8 * (size_t)N * N),
            total = o_sw + 64;
     int st = gbs_ws_ensure(ctx, total);
@@ -755,7 +1208,9 @@ int grad_sigmaQ(gbs_ctx *ctx, int M, const double *O, const double *logdet, cons
     long long *chunk_off = (long long *)(b + o_off), *chunk_u = (long long *)(b + o_cu);
     int *chunk_p = (int *)(b + o_cp);
     int *flags = (int *)(b + o_flags);
-    double *phi_ = (double *)(b + o_phi), *plo = (double *)(b + o_plo), *pT = (double *)(b + o_pT);
+    qf *part = (qf *)(b + o_part), *pT = (qf *)(b + o_pT);
+    double *pA = (double *)(b + o_pA);
+    int *redo = (int *)(b + o_redo);
     double *F = (double *)(b + o_F), *H = (double *)(b + o_H), *T1 = (double *)(b + o_T1),
            *T2 = (double *)(b + o_T2), *sw = (double *)(b + o_sw);
     // the chunk table (copied before the host buffer is released)
@@ -769,16 +1224,22 @@ int grad_sigmaQ(gbs_ctx *ctx, int M, const double *O, const double *logdet, cons
     free(ht);
     GBS_CUDA(ctx, ce);
     GBS_CUDA(ctx, cudaMemsetAsync(flags, 0, sizeof(int) * (size_t)n_pat, ctx->stream));
-    const size_t smem = sizeof(dd) * (size_t)kTreeSmem;
+    const size_t smem = sizeof(qf) * (size_t)tree_smem(n_max);
     GBS_CUDA(ctx, cudaFuncSetAttribute(grad_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     st = gbs_timing_begin(ctx);
     if (st) return st;
-    grad_tree_kernel<<<(unsigned)chunks, kTreeThreads, smem, ctx->stream>>>(M, O, pats, n_pat, chunk_p, chunk_u,
-                                                                           pst, phi_, plo, pT, flags);
+    grad_tree_kernel<<<(unsigned)chunks, kTreeThreads, smem, ctx->stream>>>(M, n_max, O, pats, chunk_p, chunk_u, pst,
+                                                                           part, pT, pA, flags);
+    GBS_CUDA(ctx, cudaGetLastError());
+    grad_redo_kernel<<<(n_pat + 127) / 128, 128, 0, ctx->stream>>>(n_pat, chunk_off, pT, pA, redo, flags);
+    const size_t dsmem = sizeof(dd) * (size_t)ddk::kTreeSmem;
+    GBS_CUDA(ctx, cudaFuncSetAttribute(ddk::grad_tree_dd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsmem));
+    ddk::grad_tree_dd_kernel<<<(unsigned)chunks, ddk::kTreeThreads, dsmem, ctx->stream>>>(
+        M, O, pats, n_pat, chunk_p, chunk_u, pst, redo, (dd *)part, (dd *)pT, flags);
     GBS_CUDA(ctx, cudaGetLastError());
     st = gbs_timing_end(ctx);
     if (st) return st;
-    grad_finalize_kernel<<<n_pat, 256, 0, ctx->stream>>>(M, pats, n_pat, chunk_off, pst, phi_, plo, pT, w, logdet, F,
+    grad_finalize_kernel<<<n_pat, 256, 0, ctx->stream>>>(M, pats, n_pat, chunk_off, pst, redo, part, pT, w, logdet, F,
                                                          logP, status, flags);
     GBS_CUDA(ctx, cudaGetLastError());
     return grad_chain_sigma(ctx, M, O, pats, n_pat, F, (size_t)kGD * kGD, w, H, T1, T2, sw, dsq);
