@@ -39,6 +39,7 @@ constexpr int kMaxOrder = 4;
 constexpr int kMinorThreads = 256;
 constexpr int kDftThreads = 128;
 constexpr int kSecThreads = 256;   // one warp per sector
+constexpr int kFitThreads = 128;   // a warp on several sectors
 constexpr int kSumThreads = 128;   // one warp per pattern
 constexpr int kPlanThreads = 256;
 constexpr double kTailEps = 1e-14;
@@ -214,6 +215,8 @@ struct ApproxPlan {
     double *pat_max;      // per pattern: largest tilted sector
     double *sec_D;        // (kMaxOrder + 1) per sector: D_w^(k), w = 0..order
     double *sec_part;     // per sector: fitted last point (negative: the fit fell back)
+    int *sec_slow;        // sectors left to the slow fits' kernel
+    unsigned long long *slow;  // their number, and the kernel's work counter
 };
 
 // log det(I - rho O_S) by Cholesky in shared memory (packed); +inf if not positive definite
@@ -1276,6 +1279,296 @@ __device__ bool maxent_fit_warp(int v0, int n, int J, const double *m, double *a
     return gmax <= 1e-10;
 }
 
+// The same fit, a warp on up to 32 sectors: the sums over the support, the Newton step and every
+// comparison in the order of maxent_fit_warp, so the results are its, bit for bit.  The FP64 pipe
+// charges a warp instruction the same for one lane as for 32 (16 clocks of an SM), and a Newton step is a
+// few hundred of them on the same numbers in every lane.  So here
+//  * the sums of one sector after another are taken by the whole warp, its 2 J + 2 sums halved at each
+//    step of the butterfly (each value still added in the butterfly's order; 12 additions for 10 values
+//    instead of 50) and handed to the sector's lane;
+//  * then every lane takes its own sector's step at once: those whose trial point is accepted solve for
+//    the next one, the others halve theirs; finished sectors leave the loop over the sums.
+template <int J>
+__device__ __forceinline__ bool newton_step(const double *pw, const double *g, double *st) {
+    double Ab[J + 1][J + 2];
+#pragma unroll
+    for (int i = 0; i <= J; ++i) {
+#pragma unroll
+        for (int k = 0; k <= J; ++k) Ab[i][k] = pw[i + k];
+        Ab[i][J + 1] = g[i];
+    }
+    bool singular = false;
+#pragma unroll
+    for (int c = 0; c <= J; ++c) {
+        int piv = c;
+        double best = Ab[c][c];
+#pragma unroll
+        for (int i = c + 1; i <= J; ++i)
+            if (fabs(Ab[i][c]) > fabs(best)) {
+                piv = i;
+                best = Ab[i][c];
+            }
+        singular = singular || best == 0.0;
+#pragma unroll
+        for (int i = c + 1; i <= J; ++i)
+#pragma unroll
+            for (int k = 0; k <= J + 1; ++k) {
+                const double u = Ab[c][k], v = Ab[i][k];
+                Ab[c][k] = piv == i ? v : u;
+                Ab[i][k] = piv == i ? u : v;
+            }
+#pragma unroll
+        for (int i = c + 1; i <= J; ++i) {
+            const double f = Ab[i][c] / Ab[c][c];
+#pragma unroll
+            for (int k = c; k <= J + 1; ++k) Ab[i][k] -= f * Ab[c][k];
+        }
+    }
+#pragma unroll
+    for (int i = J; i >= 0; --i) {
+        double v = Ab[i][J + 1];
+#pragma unroll
+        for (int q = i + 1; q <= J; ++q) v -= Ab[i][q] * st[q];
+        st[i] = v / Ab[i][i];
+    }
+    return singular;
+}
+
+// sums over the warp of NV values a lane, in the order of a butterfly over offsets 16 .. 1: at each
+// offset a lane keeps half of its values (the upper half where its bit is set).  Afterwards
+// lane l holds the sum of value half_index<NV>(l).
+template <int NV> __host__ __device__ constexpr int half_index(int l) {
+    int at = 0, slots = NV, real = NV;  // real: the lane's own values among its slots (the rest is padding)
+    for (int off = 16; off; off >>= 1) {
+        if (slots == 1) break;
+        const int h = (slots + 1) / 2;
+        if (l & off) {
+            at += h;
+            real = real > h ? real - h : 0;
+        } else {
+            real = real < h ? real : h;
+        }
+        slots = h;
+    }
+    return real > 0 ? at : -1;
+}
+template <int NV> __host__ __device__ constexpr int half_owner(int v) {
+    for (int l = 0; l < 32; ++l)
+        if (half_index<NV>(l) == v) return l;
+    return 0;
+}
+template <int CUR, int OFF> __device__ __forceinline__ void half_steps(double *v, int lane) {
+    if constexpr (OFF > 0) {
+        constexpr int H = (CUR + 1) / 2;
+        if constexpr (CUR > 1) {
+            const bool up = lane & OFF;
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+                const double lo = v[k], hi = H + k < CUR ? v[H + k] : 0.0;
+                v[k] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, OFF);
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], OFF);
+        }
+        half_steps<(CUR > 1 ? H : 1), OFF / 2>(v, lane);
+    }
+}
+
+// sums of x^i q, i <= 2 J, and of q (last) with q = exp(-f(x)) over the support x = s / S, s < S, by a
+// warp: lane l ends with value half_index<2 J + 2>(l) in v[0].  xt: s / xn
+template <int J>
+__device__ __forceinline__ void fit_sums(const double *aa, int S, const double *xt, int xn, int lane, double *v) {
+    constexpr int NP = 2 * J + 1, NV = NP + 1;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = 0.0;
+    for (int s = lane; s < S; s += 32) {
+        const double xs = S == xn ? xt[s] : (double)s / S;
+        double f = 0.0, xp = 1.0;
+#pragma unroll
+        for (int i = 0; i <= J; ++i) { f += aa[i] * xp; xp *= xs; }
+        const double q = exp(-f);
+        v[NP] += q;
+        xp = 1.0;
+#pragma unroll
+        for (int i = 0; i < NP; ++i) { v[i] += xp * q; xp *= xs; }
+    }
+    half_steps<NV, 16>(v, lane);
+}
+// one trial point: its value of the dual, gradient, and whether the line search takes it
+template <int J>
+__device__ __forceinline__ bool trial(const double *an, const double *sum, const double *m, bool first, double phi,
+                                      double gmax, double gst, double tstep, double &phin, double *gn, double &gnmax) {
+    phin = sum[2 * J + 1];
+    gnmax = 0.0;
+#pragma unroll
+    for (int i = 0; i <= J; ++i) {
+        phin += an[i] * m[i];
+        gn[i] = m[i] - sum[i];
+        gnmax = fmax(gnmax, fabs(gn[i]));
+    }
+    return first || (isfinite(phin) && phin <= phi - 1e-4 * tstep * gst) ||
+           (isfinite(phin) && phin <= phi + 1e-14 * fabs(phi) && gnmax <= 0.5 * gmax);
+}
+
+// the fits of the warp's sectors, lane i's with n clicks and moments m (act: it has one): 1 it stands
+// (coefficients a), 0 it does not, -1 not decided after kFitRounds trial points.  x: s / xn
+constexpr int kFitRounds = 40;
+template <int J>
+__device__ int maxent_fit_lanes(bool act, int n, const double *m, double *a, const double *x, int xn, int lane) {
+    constexpr int NV = 2 * J + 2;
+    double st[J + 1], phi = 0.0, gmax = 0.0, gst = 0.0, tstep = 1.0;
+    int state = act ? 0 : 2, it = 0;  // 0: first point, 1: a trial point, 2: done
+    int ok = act ? -1 : 0;
+#pragma unroll
+    for (int i = 0; i <= J; ++i) {
+        a[i] = 0.0;
+        st[i] = 0.0;
+    }
+    if (act) a[0] = log((double)n);
+    unsigned left = __ballot_sync(0xffffffffu, state != 2);
+    for (int round = 0; left && round < kFitRounds; ++round) {
+        double an[J + 1], sum[NV];
+#pragma unroll
+        for (int i = 0; i <= J; ++i) an[i] = state == 1 ? a[i] - tstep * st[i] : a[i];
+        for (unsigned todo = left; todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1, S = __shfl_sync(0xffffffffu, n, src);
+            double aa[J + 1], v[NV];
+#pragma unroll
+            for (int i = 0; i <= J; ++i) aa[i] = __shfl_sync(0xffffffffu, an[i], src);
+            fit_sums<J>(aa, S, x, xn, lane, v);
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                const double u = __shfl_sync(0xffffffffu, v[0], half_owner<NV>(i));
+                if (lane == src) sum[i] = u;
+            }
+        }
+        if (state != 2) {
+            double phin, gn[J + 1], gnmax;
+            if (!trial<J>(an, sum, m, state == 0, phi, gmax, gst, tstep, phin, gn, gnmax)) {
+                tstep *= 0.5;
+                if (tstep < 1e-12) {
+                    ok = gmax <= 1e-10;
+                    state = 2;
+                }
+            } else {
+                it += state;
+                state = 1;
+                phi = phin;
+                gmax = gnmax;
+                tstep = 1.0;
+#pragma unroll
+                for (int i = 0; i <= J; ++i) a[i] = an[i];
+                if (it == 200) {
+                    ok = gmax <= 1e-10;
+                    state = 2;
+                } else if (newton_step<J>(sum, gn, st)) {
+                    ok = gmax <= 1e-13;
+                    state = 2;
+                } else if (gmax <= 1e-13) {
+#pragma unroll
+                    for (int i = 0; i <= J; ++i) a[i] -= st[i];
+                    ok = 1;
+                    state = 2;
+                } else {
+                    gst = 0.0;
+#pragma unroll
+                    for (int i = 0; i <= J; ++i) gst += gn[i] * st[i];
+                }
+            }
+        }
+        left = __ballot_sync(0xffffffffu, state != 2);
+    }
+    return ok;
+}
+
+// The same fit by a cluster of kSlowCtas CTAs of four warps: sixteen steps of a line search at once,
+// 2^-16r .. 2^-(16r+15) in round r, of which the first accepted one counts.  A few fits in ten thousand
+// (moments on the boundary of their cone) search 30 and more halvings in each of up to 200 iterations,
+// and one of them on one warp (7,157 trial points, 66 ms) took longer than all others together.  The step is solved by one warp of each CTA (a CTA's four warps sit
+// on the four quarters of its SM, each with an FP64 pipe of its own); every thread keeps the state.
+constexpr int kSlowCtas = 4, kSlowThreads = 128, kSlowWarps = kSlowCtas * kSlowThreads / 32;
+struct SlowShared {
+    double x[kApproxMaxN];
+    double st[kMaxOrder + 1];
+    double sum[2][kSlowThreads / 32][2 * kMaxOrder + 2];  // two rounds' trial sums
+    int take[2][kSlowThreads / 32];
+    int singular;
+    long long job;
+};
+template <int J>
+__device__ bool maxent_fit_cluster(const cooperative_groups::cluster_group &cl, SlowShared &sh, int n, const double *m,
+                                   double *a) {
+    constexpr int NV = 2 * J + 2;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, rank = (int)cl.block_rank(), me = rank * 4 + wp;
+    double st[J + 1], an[J + 1], sum[NV], v[NV], gn[J + 1], phi = 0.0, phin, gmax = 0.0, gnmax, gst = 0.0;
+    int buf = 0;
+#pragma unroll
+    for (int i = 0; i <= J; ++i) a[i] = 0.0;
+    a[0] = log((double)n);
+    fit_sums<J>(a, n, sh.x, n, lane, v);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) sum[i] = __shfl_sync(0xffffffffu, v[0], half_owner<NV>(i));
+    trial<J>(a, sum, m, true, 0.0, 0.0, 0.0, 1.0, phi, gn, gmax);
+    for (int it = 0; it < 200; ++it) {
+        if (wp == 0) {
+            const bool singular = newton_step<J>(sum, gn, st);
+            if (lane == 0) {
+#pragma unroll
+                for (int i = 0; i <= J; ++i) sh.st[i] = st[i];
+                sh.singular = singular;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i <= J; ++i) st[i] = sh.st[i];
+        const bool singular = sh.singular;
+        if (singular) return gmax <= 1e-13;
+        if (gmax <= 1e-13) {
+#pragma unroll
+            for (int i = 0; i <= J; ++i) a[i] -= st[i];
+            return true;
+        }
+        gst = 0.0;
+#pragma unroll
+        for (int i = 0; i <= J; ++i) gst += gn[i] * st[i];
+        double tround = 1.0;
+        for (;;) {
+            double t = tround;
+            for (int c = 0; c < me; ++c) t *= 0.5;
+#pragma unroll
+            for (int i = 0; i <= J; ++i) an[i] = a[i] - t * st[i];
+            fit_sums<J>(an, n, sh.x, n, lane, v);
+#pragma unroll
+            for (int i = 0; i < NV; ++i) sum[i] = __shfl_sync(0xffffffffu, v[0], half_owner<NV>(i));
+            const bool take = t >= 1e-12 && trial<J>(an, sum, m, false, phi, gmax, gst, t, phin, gn, gnmax);
+            if (lane == 0) {
+                sh.take[buf][wp] = take;
+#pragma unroll
+                for (int i = 0; i < NV; ++i) sh.sum[buf][wp][i] = sum[i];
+            }
+            cl.sync();  // this round's sums are in; the other buffer is free again after the next one
+            int found = -1;
+            for (int c = kSlowWarps - 1; c >= 0; --c)
+                if (cl.map_shared_rank(&sh, c / 4)->take[buf][c & 3]) found = c;
+            if (found >= 0) {
+                const double *src = cl.map_shared_rank(&sh, found / 4)->sum[buf][found & 3];
+#pragma unroll
+                for (int i = 0; i < NV; ++i) sum[i] = src[i];
+                t = tround;
+                for (int c = 0; c < found; ++c) t *= 0.5;
+#pragma unroll
+                for (int i = 0; i <= J; ++i) a[i] -= t * st[i];
+            }
+            buf ^= 1;
+            if (found >= 0) break;
+            for (int c = 0; c < kSlowWarps; ++c) tround *= 0.5;
+            if (tround < 1e-12) return gmax <= 1e-10;
+        }
+        trial<J>(a, sum, m, true, 0.0, 0.0, 0.0, 1.0, phi, gn, gmax);
+    }
+    return gmax <= 1e-10;
+}
+
 __device__ __forceinline__ double stirling2(int i, int w) {
     // S(i, w) for i, w <= 4
     const double tab[5][5] = {{1, 0, 0, 0, 0}, {0, 1, 0, 0, 0}, {0, 1, 1, 0, 0}, {0, 1, 3, 1, 0}, {0, 1, 7, 6, 1}};
@@ -1320,6 +1613,18 @@ __global__ void __launch_bounds__(kDftThreads) approx_dft_kernel(int order, Appr
     }
 }
 
+// raw moments mu_i, i <= Jmax, of a sector from its factorial moments
+__device__ __forceinline__ void raw_moments(const double *Dk, int Jmax, double *mu) {
+    for (int i = 0; i <= Jmax; ++i) {
+        double s = 0.0, fw = 1.0;
+        for (int w = 0; w <= i; ++w) {
+            s += stirling2(i, w) * fw * Dk[w];
+            fw *= (w + 1);
+        }
+        mu[i] = s;
+    }
+}
+
 // one warp per (pattern, sector k): factorial moments -> raw moments (Stirling numbers)
 // -> maximum-entropy fit on the support v in [max(0, n - k), n - 1] -> the last point.
 // curves (one pattern only, else null): every sector's fitted distribution over the
@@ -1354,14 +1659,7 @@ __global__ void __launch_bounds__(kSecThreads) approx_sector_fit_kernel(int n_pa
             const int S = n - v0;
             const int Jmax = order < S - 1 ? order : S - 1;
             double mu[kMaxOrder + 1];
-            for (int i = 0; i <= Jmax; ++i) {
-                double s = 0.0, fw = 1.0;
-                for (int w = 0; w <= i; ++w) {
-                    s += stirling2(i, w) * fw * Dk[w];
-                    fw *= (w + 1);
-                }
-                mu[i] = s;
-            }
+            raw_moments(Dk, Jmax, mu);
             bool done = false;
             for (int J = Jmax; J >= 0 && !done; --J) {
                 double m[kMaxOrder + 1], a[kMaxOrder + 1];
@@ -1384,6 +1682,110 @@ __global__ void __launch_bounds__(kSecThreads) approx_sector_fit_kernel(int n_pa
         }
         if (lane == 0) pl.sec_part[gs] = fell ? -val : val;   // the sign marks a fallback
     }
+}
+
+// The same values, P consecutive sectors a warp (P <= 32): order J for all of them at once in
+// maxent_fit_lanes; the others go to approx_fit_slow_kernel.  Both kernels together, GB300: 256
+// 50-mode patterns at order 2 11.4 -> 5.2 ms, 96 at order 4 66 -> 14.8 ms (one warp a sector before).
+template <int J>
+__global__ void __launch_bounds__(kFitThreads, 3) approx_sector_fit_lanes_kernel(int n_pat, int P, double sector_eps,
+                                                                                ApproxPlan pl) {
+    __shared__ double s_x[kFitThreads / 32][kPairMaxN];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    double *x = s_x[wp];
+    const long long nsec = pl.sec_off[n_pat];
+    if (*pl.overflow) return;
+    const long long g0 = ((long long)blockIdx.x * (kFitThreads / 32) + wp) * P, gs = g0 + lane;
+    if (g0 >= nsec) return;
+    const bool in = lane < P && gs < nsec;
+    int lo = 0, hi = n_pat;  // the pattern whose sector range holds gs
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (pl.sec_off[mid] <= (in ? gs : g0)) lo = mid; else hi = mid;
+    }
+    const int p = lo, n = pl.pat_n[p];
+    const int k = (int)(gs - pl.sec_off[p]);
+    const int xn = __shfl_sync(0xffffffffu, n, 0);
+    for (int v = lane; v < xn; v += 32) x[v] = (double)v / xn;
+    __syncwarp();
+    const double *Dk = pl.sec_D + (size_t)(in ? gs : g0) * (kMaxOrder + 1);
+    const double D0 = Dk[0];
+    double val = 0.0;
+    const bool fit = in && n > 0 && k >= n && D0 >= sector_eps * pl.pat_max[p] && D0 > 0.0;
+    const int Jmax = J < n - 1 ? J : n - 1;
+    const bool act = fit && Jmax == J;
+    if (in && n == 0) val = k == 0 ? D0 : 0.0;
+    double m[J + 1], a[J + 1], mu[J + 1];
+    if (act) {
+        raw_moments(Dk, J, mu);
+        double np = 1.0;
+#pragma unroll
+        for (int i = 0; i <= J; ++i) {
+            m[i] = mu[i] / np / mu[0];
+            np *= n;
+        }
+    }
+    const int ok = maxent_fit_lanes<J>(act, n, m, a, x, xn, lane);
+    if (act && ok == 1) val = mu[0] * exp(-a[0]);
+    if (in) pl.sec_part[gs] = val;
+    if (fit && !(act && ok == 1)) pl.sec_slow[atomicAdd(pl.slow, 1ull)] = (int)gs;
+}
+
+// the sectors that approx_sector_fit_lanes_kernel left: fits that take many trial points, fits that
+// fail at their order and go on at lower ones, and supports smaller than the order
+__global__ void __cluster_dims__(kSlowCtas, 1, 1) __launch_bounds__(kSlowThreads)
+    approx_fit_slow_kernel(int n_pat, int order, ApproxPlan pl) {
+    __shared__ SlowShared sh;
+    const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    const int t = threadIdx.x;
+    const bool first = cl.block_rank() == 0 && t == 0;
+    if (*pl.overflow) return;
+    const long long jobs = (long long)pl.slow[0];
+    for (;;) {
+        if (first) sh.job = (long long)atomicAdd(pl.slow + 1, 1ull);
+        cl.sync();
+        const long long job = cl.map_shared_rank(&sh, 0)->job;
+        cl.sync();  // read by all before the next one is drawn, and before a CTA exits
+        if (job >= jobs) break;
+        const long long gs = pl.sec_slow[job];
+        int lo = 0, hi = n_pat;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (pl.sec_off[mid] <= gs) lo = mid; else hi = mid;
+        }
+        const int n = pl.pat_n[lo];
+        for (int v = t; v < n; v += kSlowThreads) sh.x[v] = (double)v / n;
+        __syncthreads();
+        const double *Dk = pl.sec_D + (size_t)gs * (kMaxOrder + 1);
+        const int top = order < n - 1 ? order : n - 1;
+        double m[kMaxOrder + 1], a[kMaxOrder + 1], mu[kMaxOrder + 1], val = 0.0;
+        raw_moments(Dk, top, mu);
+        bool done = false, fell = false;
+        for (int j = top; j >= 0 && !done; --j) {
+            double np = 1.0;
+            for (int i = 0; i <= j; ++i) { m[i] = mu[i] / np / mu[0]; np *= n; }
+            done = j == 4   ? maxent_fit_cluster<4>(cl, sh, n, m, a)
+                   : j == 3 ? maxent_fit_cluster<3>(cl, sh, n, m, a)
+                   : j == 2 ? maxent_fit_cluster<2>(cl, sh, n, m, a)
+                   : j == 1 ? maxent_fit_cluster<1>(cl, sh, n, m, a)
+                            : maxent_fit_cluster<0>(cl, sh, n, m, a);
+            if (done) {
+                val = mu[0] * exp(-a[0]);
+                if (j != top) fell = true;
+            }
+            cl.sync();  // the next fit writes its sums where a slower CTA may still read this one's
+        }
+        if (!done) fell = true;
+        if (first) pl.sec_part[gs] = fell ? -val : val;   // the sign marks a fallback
+    }
+}
+// P: as many sectors a warp as leave three warps for each quarter of an SM
+template <int J> void launch_fit_lanes(gbs_ctx *ctx, long long secs, int n_pat, double eps, const ApproxPlan &pl) {
+    int P = 1;
+    while (P < 32 && secs >= 2ll * P * 12 * ctx->num_sms) P *= 2;
+    const long long per = (long long)(kFitThreads / 32) * P;
+    approx_sector_fit_lanes_kernel<J><<<(unsigned)((secs + per - 1) / per), kFitThreads, 0, ctx->stream>>>(n_pat, P, eps,
+                                                                                                         pl);
 }
 
 // the curves untilted (rho^-k) and scaled by det(sigma_Q)^{-1/2}
@@ -1941,7 +2343,7 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 struct ApproxOffsets {
     size_t counter, total, overflow, info, counter2, pat_n, pat_L, pat_rho, unit_off, unit_flag, sec_off, pat_max,
-        unit_D, sec_D, sec_part, end;
+        unit_D, sec_D, sec_part, sec_slow, counter3, end;
 };
 
 ApproxOffsets approx_offsets(int n_pat, long long units, long long secs = 0) {
@@ -1951,7 +2353,8 @@ ApproxOffsets approx_offsets(int n_pat, long long units, long long secs = 0) {
     o.overflow = 16;
     o.info = 24;       // 6 long long
     o.counter2 = 72;   // the CTA-pair minors kernel's work counter
-    o.pat_n = align256(80);
+    o.counter3 = 80;   // the slow fits' list length and its work counter
+    o.pat_n = align256(96);
     o.pat_L = align256(o.pat_n + 4 * (size_t)n_pat);
     o.pat_rho = align256(o.pat_L + 4 * (size_t)n_pat);
     o.unit_off = align256(o.pat_rho + 8 * (size_t)n_pat);
@@ -1961,7 +2364,8 @@ ApproxOffsets approx_offsets(int n_pat, long long units, long long secs = 0) {
     o.unit_D = align256(o.pat_max + 8 * (size_t)n_pat);
     o.sec_D = align256(o.unit_D + 8 * 2 * (kMaxOrder + 1) * (size_t)units);
     o.sec_part = align256(o.sec_D + 8 * (kMaxOrder + 1) * (size_t)secs);
-    o.end = o.sec_part + 8 * (size_t)secs;
+    o.sec_slow = align256(o.sec_part + 8 * (size_t)secs);
+    o.end = o.sec_slow + 4 * (size_t)secs;
     return o;
 }
 
@@ -1982,6 +2386,8 @@ ApproxPlan approx_plan_from(void *ws, int n_pat, long long units = 0, long long 
     pl.pat_max = (double *)(b + o.pat_max);
     pl.sec_D = (double *)(b + o.sec_D);
     pl.sec_part = (double *)(b + o.sec_part);
+    pl.sec_slow = (int *)(b + o.sec_slow);
+    pl.slow = (unsigned long long *)(b + o.counter3);
     return pl;
 }
 
@@ -2029,7 +2435,7 @@ int run_approx(gbs_ctx *ctx, int M, const double *O, const double *logdet, const
     }
     pl = approx_plan_from(ctx->ws, n_pat, units, secs);
     GBS_CUDA(ctx, cudaMemsetAsync(ctx->ws, 0, 8, ctx->stream));  // work counters
-    GBS_CUDA(ctx, cudaMemsetAsync((char *)ctx->ws + approx_offsets(n_pat, 0).counter2, 0, 8, ctx->stream));
+    GBS_CUDA(ctx, cudaMemsetAsync((char *)ctx->ws + approx_offsets(n_pat, 0).counter2, 0, 24, ctx->stream));
     int st = gbs_timing_begin(ctx);
     if (st) return st;
     if (nsmall > 0) {
@@ -2082,8 +2488,17 @@ int run_approx(gbs_ctx *ctx, int M, const double *O, const double *logdet, const
         GBS_CUDA(ctx, cudaMemsetAsync(curves, 0, sizeof(double) * (size_t)(curve_K + 1) * (curve_n + 1),
                                       ctx->stream));
     }
-    approx_sector_fit_kernel<<<fit_blocks, kSecThreads, 0, ctx->stream>>>(
-        n_pat, order, MinorPrec<R>::sector_eps, pl, curves, curve_K);
+    const double eps = MinorPrec<R>::sector_eps;
+    if (curves) {
+        approx_sector_fit_kernel<<<fit_blocks, kSecThreads, 0, ctx->stream>>>(n_pat, order, eps, pl, curves, curve_K);
+    } else if (secs > 0) {
+        if (order == 1) launch_fit_lanes<1>(ctx, secs, n_pat, eps, pl);
+        else if (order == 2) launch_fit_lanes<2>(ctx, secs, n_pat, eps, pl);
+        else if (order == 3) launch_fit_lanes<3>(ctx, secs, n_pat, eps, pl);
+        else launch_fit_lanes<4>(ctx, secs, n_pat, eps, pl);
+        GBS_CUDA(ctx, cudaGetLastError());
+        approx_fit_slow_kernel<<<ctx->num_sms * kSlowCtas, kSlowThreads, 0, ctx->stream>>>(n_pat, order, pl);
+    }
     GBS_CUDA(ctx, cudaGetLastError());
     if (curves) {
         const long long tot = (long long)(curve_K + 1) * (nmax + 1);
