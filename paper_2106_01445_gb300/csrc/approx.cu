@@ -480,76 +480,113 @@ template <> struct GroupAcc<float> {
 // G <- -(I - t O_S)^{-1} in shared memory (packed upper triangle of 2n x 2n, then four
 // staged pivot columns of 2n entries), t = cs + i sn, by the symmetric sweep operator on
 // every pivot; Z_S(t) = prod of principal pivot^{-1/2} (the LDL^T pivots, one root per
-// pair) to s_zs on thread 0.  A pivot with Re <= 0 sets *s_bad.  All kMinorThreads threads
-// take part; ends with a barrier.
+// pair) to s_zs.  A pivot with Re <= 0 sets *s_bad.  All kMinorThreads threads take part; ends
+// with a barrier.
+//
+// One phase and one barrier a pivot.  Pivot k's column b and u = b / pivot are staged; in its phase
+//  * the first warps (a thread a row) form column k + 1 as pivot k leaves it, and stage it and its
+//    quotients by the next pivot in the other buffers;
+//  * the others begin with the entries outside rows and columns k and k + 1, e - b_i u_j; the first
+//    ones join after kHeadStart rounds, about what the column, two reciprocals' worth, costs them.
+// Every warp computing both pivots' reciprocals, with a barrier between the entries and the next
+// column, cost as much as the entries at 50 rows: 16 of a hundred instructions each on eight warps
+// against 40 rounds of 70.  Every entry's operations and their order are those of the plain form.
+// Float-float takes two entries at a time (8 warps on an SM at 100 modes: the wait for one update is
+// covered by the other); FP64, bound by its pipe, takes one.  Measured on a GB300, whole calls: order 2
+// at 50 modes 35.1 -> 31.9 ms, at 100 modes 165.3 -> 163.8, the FP64 gradient at 32 modes 74.2 -> 61.6.
+constexpr int kHeadStart = 4;
 template <typename R>
 __device__ __forceinline__ void sweep_inverse(int M, const double *__restrict__ O, const int *modes, int n,
                                               double cs, double sn, cx<R> *G, int *s_bad, double *s_zs) {
-    const int t = threadIdx.x;
+    constexpr int W = kMinorThreads / 32;
+    __shared__ cx<R> s_inv[2];
+    const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
     const int N = 2 * n, N2 = 2 * M;
-    for (int f = t; f < N * N; f += kMinorThreads) {
-        int i = f / N, j = f - i * N;
-        if (j < i) continue;
-        int si = modes[i >> 1] + (i & 1) * M, sj = modes[j >> 1] + (j & 1) * M;
-        double o = O[(size_t)si * N2 + sj];
-        G[pidx(N, i, j)] = init_entry<R>(i == j, cs, sn, o);
+    const int fw = N + 1, fE = n * fw;  // rows p and N - 1 - p folded: N + 1 entries
+    const uint32_t inv22 = (1u << 22) / (uint32_t)fw + 1u;  // f / fw = f inv22 >> 22 for f < fE <= 224 x 225 / 2
+    auto fold = [&](int f, int &i, int &j) {
+        const int fp = (int)(((uint32_t)f * inv22) >> 22), fq = f - fp * fw;
+        const bool low = fq < N - fp;
+        i = low ? fp : N - 1 - fp;
+        j = low ? fp + fq : i + (fq - (N - fp));
+    };
+    for (int f = t; f < fE; f += kMinorThreads) {
+        int i, j;
+        fold(f, i, j);
+        const int si = modes[i >> 1] + (i & 1) * M, sj = modes[j >> 1] + (j & 1) * M;
+        G[pidx(N, i, j)] = init_entry<R>(i == j, cs, sn, O[(size_t)si * N2 + sj]);
     }
     __syncthreads();
-    // symmetric sweep operator on every pivot: G <- -(I - t O_S)^{-1};
-    // Z_S(t) = prod of principal pivot^{-1/2} (pivots are the LDL^T pivots).
-    // Pivot k's column is staged in cb (and cb / pivot in cu) by the previous pivot's
-    // second phase, so an entry update is one complex product of staged values.
     cx<R> *const cb0 = G + sym(N), *const cb1 = cb0 + N, *const cu0 = cb0 + 2 * N, *const cu1 = cb0 + 3 * N;
-    {
+    const int NS = (N + 31) >> 5;  // warps that stage columns
+    if (wp < NS) {
         const cx<R> inv0 = cinv(G[0]);
-        for (int i = t; i < N; i += kMinorThreads) {
-            const cx<R> v = G[pidx(N, 0, i)];
-            cb0[i] = v;
-            cu0[i] = v * inv0;
+        if (t < N) {
+            const cx<R> v = G[t];
+            cb0[t] = v;
+            cu0[t] = v * inv0;
         }
+        if (t == 0) s_inv[0] = inv0;
     }
     __syncthreads();
-    cx<double> zs = mk<double>(1.0, 0.0);
+    cx<double> zs = mk<double>(1.0, 0.0);  // on the last warp's first thread
     cx<R> dprev = mk<R>(R(1), R(0));
-    const int fw = N + 1, fE = (N >> 1) * fw;  // rows p and N - 1 - p folded: N + 1 entries
+    const int rounds = (fE + 31) >> 5;
     for (int k = 0; k < N; ++k) {
         const cx<R> *cb = (k & 1) ? cb1 : cb0, *cu = (k & 1) ? cu1 : cu0;
-        const cx<R> d = cb[k];
-        if (!(d.re > R(0)) && t == 0) *s_bad = 1;
-        if ((k & 1) && t == 0) zs = zs * widen(crsqrt(dprev * d));
-        dprev = d;
-        const cx<R> inv = cinv(d);
-        int fp = t / fw, fq = t - fp * fw;
-        const int sp = kMinorThreads / fw, sq = kMinorThreads - sp * fw;
-        for (int f = t; f < fE; f += kMinorThreads) {
-            int i, j;
-            if (fq < N - fp) { i = fp; j = fp + fq; } else { i = N - 1 - fp; j = i + (fq - (N - fp)); }
-            if (i != k && j != k) {
-                cx<R> &e = G[i * N - (i * (i - 1)) / 2 + (j - i)];
-                e = cfms_inl(e, cb[i], cu[j]);
-            }
-            fq += sq;
-            fp += sp;
-            if (fq >= fw) { fq -= fw; ++fp; }
+        if (t == kMinorThreads - 32) {
+            const cx<R> d = cb[k];
+            if (!(d.re > R(0))) *s_bad = 1;
+            if (k & 1) zs = zs * widen(crsqrt(dprev * d));
+            dprev = d;
         }
-        __syncthreads();
-        // scale pivot k's row and column; stage pivot k + 1's column
-        cx<R> *cbn = (k & 1) ? cb0 : cb1, *cun = (k & 1) ? cu0 : cu1;
-        const bool more = k + 1 < N;
-        const cx<R> invn = more ? cinv(G[pidx(N, k + 1, k + 1)]) : mk<R>(R(0), R(0));
-        for (int i = t; i < N; i += kMinorThreads) {
-            if (i != k) G[pidx_any(N, i, k)] = cu[i];
-            if (more) {
-                // entry (k, k + 1) is the one just scaled: cu[k + 1]
-                const cx<R> v = i == k ? cu[k + 1] : G[pidx_any(N, i, k + 1)];
-                cbn[i] = v;
-                cun[i] = v * invn;
+        if (wp < NS) {
+            // scale pivot k's row and column (entry (k, k + 1) is the next column's)
+            if (t < N && t != k && t != k + 1) G[pidx_any(N, t, k)] = cu[t];
+            if (t == k) G[pidx(N, k, k)] = mk<R>(R(0), R(0)) - s_inv[k & 1];
+            if (k + 1 < N) {
+                cx<R> *cbn = (k & 1) ? cb0 : cb1, *cun = (k & 1) ? cu0 : cu1;
+                // the next pivot (its place in G stays as it is until its own phase)
+                const cx<R> dn = cfms_inl(G[pidx(N, k + 1, k + 1)], cb[k + 1], cu[k + 1]);
+                const cx<R> invn = cinv(dn);
+                if (t < N) {
+                    const int lo = t < k + 1 ? t : k + 1, hi = t < k + 1 ? k + 1 : t;
+                    cx<R> &e = G[pidx(N, lo, hi)];
+                    cx<R> v;
+                    if (t == k) v = cu[k + 1];
+                    else if (t == k + 1) v = dn;
+                    else v = cfms_inl(e, cb[lo], cu[hi]);
+                    if (t != k + 1) e = v;
+                    cbn[t] = v;
+                    cun[t] = v * invn;
+                    if (t == k + 1) s_inv[(k + 1) & 1] = invn;
+                }
             }
         }
-        if (t == 0) G[pidx(N, k, k)] = mk<R>(R(0), R(0)) - inv;
+        // the entries, 32 a round and warp
+        const int first = wp < NS || ((k & 1) && wp == W - 1) ? kHeadStart : 0;  // busy warps join later
+        const int m = NS < W ? W - NS - (k & 1) : 0;
+        auto entry = [&](int r, int &i, int &j) {  // this lane's entry of round r: its place, -1 none, -2 the end
+            const int c = r < kHeadStart ? r * m + (wp - NS) : kHeadStart * m + (r - kHeadStart) * W + wp;
+            const int f = c * 32 + lane;
+            fold(f < fE ? f : 0, i, j);
+            return c >= rounds ? -2 : f < fE && i != k && j != k && i != k + 1 && j != k + 1 ? pidx(N, i, j) : -1;
+        };
+        constexpr int U = std::is_same_v<R, ff> ? 2 : 1;  // independent updates at a time
+        const int dead = sym(N) + (k & 1) * N;  // cb[0], read and dropped in the place of a skipped entry
+        for (int r = first;; r += U) {
+            int a[U], i[U], j[U];
+            for (int q = 0; q < U; ++q) a[q] = entry(r + q, i[q], j[q]);
+            if (a[0] == -2) break;
+            cx<R> v[U];
+            for (int q = 0; q < U; ++q)
+                if (U > 1 || a[q] >= 0) v[q] = cfms_inl(G[a[q] < 0 ? dead : a[q]], cb[i[q]], cu[j[q]]);
+            for (int q = 0; q < U; ++q)
+                if (a[q] >= 0) G[a[q]] = v[q];
+        }
         __syncthreads();
     }
-    if (t == 0) { s_zs[0] = zs.re; s_zs[1] = zs.im; }
+    if (t == kMinorThreads - 32) { s_zs[0] = zs.re; s_zs[1] = zs.im; }
     __syncthreads();
 }
 
