@@ -33,6 +33,7 @@
 #include "fx.cuh"
 #include "fx6.cuh"
 #include "gbs_internal.cuh"
+#include "qf.cuh"
 #include "zc.cuh"
 
 namespace {
@@ -82,6 +83,27 @@ template <> struct Prec<dd> {
     static constexpr bool fixed = false;
     static constexpr int wrow = 2;
     static constexpr double u = 1.2325951644078309e-32, u_sum = 1.2325951644078309e-32;
+};
+// The double-double sweep on the integer pipes (qf.cuh): the same plan, units and trees in 110-bit
+// software floating point; the results whose last digits show the arithmetic are taken again in
+// double-double (kRedoKappa).  In double-double the sweep runs at the FP64 pipe's rate (a fused
+// update is 216 clocks of an SM a warp); here an update is about 35, and latency bounds it (12 warps
+// an SM, a third of the issue slots).  181 patterns of 10 to 18 clicks at 24 modes on a GB300: 7.9 ms
+// -> 3.9 (4.8 with dd's three register levels and two CTAs an SM).
+struct sq : qf {
+    sq() = default;
+    __device__ __forceinline__ sq(const qf &o) : qf(o) {}
+    __device__ __forceinline__ explicit sq(double d) : qf(d == 1.0 ? qf_one() : qf_from_double(d)) {}
+};
+template <> struct Prec<sq> {
+    // one register level less than dd (160 registers and 74 KB instead of 244 and 114: three CTAs an
+    // SM), and one prefix level more in the CTA's loop, so that the units are dd's (kSubMore)
+    static constexpr int B = 2, idx = GBS_DD;
+    using Tau = sq;
+    using Abs = double;
+    using Node = sq;
+    static constexpr bool fixed = false;
+    static constexpr int wrow = 2;
 };
 // 128-bit fixed point: the matrices of the breadth-first levels and of the register bottom
 // in limb form (fl.cuh), the prefix, the prefactors and the sums packed Q16.112 (fx.cuh).
@@ -143,6 +165,7 @@ template <> __device__ __forceinline__ zf rsq<zf>(zf x) { return zf_rsqrt(x); }
 template <> __device__ __forceinline__ float rsq<float>(float x) { return rsqrtf(x); }
 template <> __device__ __forceinline__ double rsq<double>(double x) { return rsqrt(x); }
 template <> __device__ __forceinline__ dd rsq<dd>(dd x) { return dd_rsqrt(x); }
+template <> __device__ __forceinline__ sq rsq<sq>(sq x) { return qf_rsqrt(x); }
 template <> __device__ __forceinline__ fx6 rsq<fx6>(fx6 x) { return fx6_rsqrt(x); }
 
 // 1/sqrt(det) as a prefix factor, in the Tau type of the precision, given rs = rsq(det)
@@ -150,6 +173,7 @@ template <> __device__ __forceinline__ fx6 rsq<fx6>(fx6 x) { return fx6_rsqrt(x)
 __device__ __forceinline__ double tau_of(float det, float) { return rsqrt((double)det); }
 __device__ __forceinline__ double tau_of(double, double rs) { return rs; }
 __device__ __forceinline__ dd tau_of(dd, dd rs) { return rs; }
+__device__ __forceinline__ sq tau_of(sq, sq rs) { return rs; }
 __device__ __forceinline__ fxe6 tau_of(fx6, fx6 rs) { return fxe6_from(rs); }
 __device__ __forceinline__ zc tau_of(zc, zc rs) { return rs; }
 __device__ __forceinline__ zf tau_of(zf, zf rs) { return rs; }
@@ -160,6 +184,7 @@ template <> __device__ __forceinline__ fx6 konst<fx6>(double v) { return fx6_fro
 __device__ __forceinline__ float to_node(float x) { return x; }
 __device__ __forceinline__ double to_node(double x) { return x; }
 __device__ __forceinline__ dd to_node(dd x) { return x; }
+__device__ __forceinline__ sq to_node(sq x) { return x; }
 __device__ __forceinline__ zc to_node(zc x) { return x; }
 __device__ __forceinline__ zf to_node(zf x) { return x; }
 // a child's prefactor: the parent's times det^{-1/2} of the parent's pivot
@@ -173,6 +198,8 @@ template <> __device__ __forceinline__ fx6 mul_pos<fx6>(fx6 a, fx6 b) { return f
 // pivot check: 0 fine, 1 not positive (or NaN), 2 outside the fixed-point range
 template <typename T> __device__ __forceinline__ int pivot_bad(T det) { return det > T(0) ? 0 : 1; }
 template <> __device__ __forceinline__ int pivot_bad<fx6>(fx6 det) { return fx_pivot_bad(det); }
+__device__ __forceinline__ bool saturated(const qf &x) { return (x.w[3] & 0x3ffu) == 1023u; }
+template <> __device__ __forceinline__ int pivot_bad<sq>(sq det) { return qf_positive(det) && !saturated(det) ? 0 : 1; }
 // complex pivots: their determinants may have any argument in (-pi, pi); only zero or NaN is bad
 template <> __device__ __forceinline__ int pivot_bad<zc>(zc det) {
     return fabs(det.re) + fabs(det.im) > 0.0 ? 0 : 1;
@@ -183,14 +210,22 @@ template <> __device__ __forceinline__ int pivot_bad<zf>(zf det) {
 
 // the Schur-update kernels: a0 b0 + a1 b1, c - a0 b0 - a1 b1, det of a 2x2 block
 template <typename T> __device__ __forceinline__ T dot2(T a0, T b0, T a1, T b1) { return a0 * b0 + a1 * b1; }
+template <> __device__ __forceinline__ sq dot2<sq>(sq a0, sq b0, sq a1, sq b1) { return qf_dot2<false, false>(a0, b0, a1, b1); }
 template <> __device__ __forceinline__ dd dot2<dd>(dd a0, dd b0, dd a1, dd b1) { return dd_dot2(a0, b0, a1, b1); }
 template <typename T> __device__ __forceinline__ T fms2(T c, T a0, T b0, T a1, T b1) { return c - a0 * b0 - a1 * b1; }
+template <> __device__ __forceinline__ sq fms2<sq>(sq c, sq a0, sq b0, sq a1, sq b1) { return qf_fms2(c, a0, b0, a1, b1); }
+template <typename T> __device__ __forceinline__ T mul_neg(T a, T b) { return -a * b; }
+template <> __device__ __forceinline__ sq mul_neg<sq>(sq a, sq b) { return qf_mul<true>(a, b); }
 template <> __device__ __forceinline__ dd fms2<dd>(dd c, dd a0, dd b0, dd a1, dd b1) { return dd_fms2(c, a0, b0, a1, b1); }
 template <typename T> __device__ __forceinline__ T det2(T p00, T p01, T p11) { return dot2(p00, p11, -p01, p01); }
+template <> __device__ __forceinline__ sq det2<sq>(sq p00, sq p01, sq p11) { return qf_dot2<false, true>(p00, p11, p01, p01); }
 template <> __device__ __forceinline__ fx6 det2<fx6>(fx6 p00, fx6 p01, fx6 p11) { return fx_det2(p00, p01, p11); }
 
 // an entry of A = I - O from its FP64 data (exact in double-double)
 template <typename T> __device__ __forceinline__ T a_entry(double delta, double o) { return (T)(delta - o); }
+template <> __device__ __forceinline__ sq a_entry<sq>(double delta, double o) {
+    return qf_from_double(delta) - qf_from_double(o);
+}
 template <> __device__ __forceinline__ dd a_entry<dd>(double delta, double o) { return dd_two_sum(delta, -o); }
 template <> __device__ __forceinline__ fx6 a_entry<fx6>(double delta, double o) {
     return fx6_from_double(delta) - fx6_from_double(o);
@@ -213,11 +248,20 @@ __device__ __forceinline__ double to_hi(double x) { return x; }
 __device__ __forceinline__ float abs_part(float x) { return x; }
 __device__ __forceinline__ double abs_part(double x) { return x; }
 __device__ __forceinline__ double abs_part(dd x) { return x.hi; }
+// of a positive number, truncated to a double's digits, put together on the integer pipe
+__device__ __forceinline__ double abs_part(const sq &x) {
+    const unsigned long long m = ((unsigned long long)(x.w[3] >> 10) << 34) | ((unsigned long long)x.w[2] << 4) | (x.w[1] >> 26);
+    const int e = (int)(x.w[3] & 0x3ffu) - 512, z = __clzll((long long)m);  // x = m 2^-54 4^e
+    const unsigned long long f = (m << z) << 1;                             // the digits after the first
+    return m == 0ull || e < -500 ? 0.0
+                                 : __longlong_as_double((long long)((f >> 12) | ((unsigned long long)(1023 + 9 - z + 2 * e) << 52)));
+}
 __device__ __forceinline__ float abs_part(fx x) { return (float)(int32_t)x.w[3] * (1.0f / 65536.0f); }
 __device__ __forceinline__ float abs_part(fx6 x) { return (float)(int32_t)x.w[5] * (1.0f / 65536.0f); }
 __device__ __forceinline__ bool is_nan(float x) { return x != x; }
 __device__ __forceinline__ bool is_nan(double x) { return x != x; }
 __device__ __forceinline__ bool is_nan(dd x) { return x.hi != x.hi; }
+__device__ __forceinline__ bool is_nan(const sq &x) { return saturated(x); }
 __device__ __forceinline__ bool is_nan(zc x) { return zc_nan(x); }
 __device__ __forceinline__ bool is_nan(zf x) { return zf_nan(x); }
 // a thread's subtree sum as (hi, lo) doubles
@@ -258,8 +302,10 @@ template <> struct NodeIO<fxe6> {
 // matrices, W the rows W = B P^{-1} of the level being eliminated; a level's pivot
 // quantities sit at the start of its destination buffer (read before the children are
 // written).  The prefactor arrays hold the W rows of a prefix pivot.
+template <typename T> constexpr int kSubMore = std::is_same_v<T, sq> ? Prec<dd>::B - Prec<sq>::B : 0;
 template <typename T> struct Layout {
     static constexpr int B = Prec<T>::B;
+    static constexpr int S = kS + kSubMore<T>;  // prefix levels looped over, at most
     static constexpr int R = kL + B;  // modes of a unit's level-0 matrix
     static constexpr int level_size(int l) { return (1 << l) * nstride(2 * (R - l)); }
     static constexpr int max_even() {
@@ -289,17 +335,17 @@ template <typename T> struct Layout {
     using Node = typename Prec<T>::Node;
     static constexpr size_t off_X = 0;
     static constexpr size_t off_Y = off_X + sizeof(T) * max_even();
-    static constexpr int ublk() { return sym(2 * (kS + R)); }
+    static constexpr int ublk() { return sym(2 * (S + R)); }
     static constexpr size_t off_U = off_Y + sizeof(T) * max_odd();
-    // the sub-unit tree's stored matrices: after an include at depth d < kS - 1, the
-    // 2 (kS + R - d - 1) rows of the modes below it
+    // the sub-unit tree's stored matrices: after an include at depth d < S - 1, the
+    // 2 (S + R - d - 1) rows of the modes below it
     static constexpr int slot_off(int d) {
         int o = 0;
-        for (int e = 1; e < d; ++e) o += sym(2 * (kS + R - e));
+        for (int e = 1; e < d; ++e) o += sym(2 * (S + R - e));
         return o;
     }
     static constexpr size_t off_Sl = off_U + sizeof(T) * ublk();
-    static constexpr size_t off_W = off_Sl + sizeof(T) * slot_off(kS);
+    static constexpr size_t off_W = off_Sl + sizeof(T) * slot_off(S);
     // prefactors: even levels hold at most kThreads / 2 nodes, odd levels kThreads
     static constexpr size_t off_tauX = off_W + sizeof(T) * w_entries();
     static constexpr size_t off_tauY = off_tauX + NodeIO<Node>::bytes * (kThreads / 2);
@@ -366,6 +412,8 @@ __device__ __forceinline__ void unit_scale(double &h, double &l, dd tp) {
     h = u.hi;
     l = u.lo;
 }
+template <typename Tau> __device__ __forceinline__ Tau tau_out(const Tau &x) { return x; }
+__device__ __forceinline__ dd tau_out(const sq &x) { return qf_to_dd(x); }
 __device__ __forceinline__ double tau_hi(double x) { return x; }
 __device__ __forceinline__ double tau_hi(dd x) { return x.hi; }
 
@@ -391,6 +439,16 @@ __device__ __forceinline__ void leaf_pair(Acc<T> &acc, T inc, T tau, bool real, 
     T comb = real ? inc - tau : inc;
     acc_add(acc, NEG ? -comb : comb);
     acc.abs += real ? abs_part(inc) + abs_part(tau) : abs_part(inc);
+}
+// ... with the include leaf still a product: inc = tau rs (tau 1 where ONE), one fused operation
+template <bool NEG, bool ONE>
+__device__ __forceinline__ void leaf_pair_sq(Acc<sq> &acc, const sq &rs, const sq &tau, bool real) {
+    sq c;
+    if (!real) c = ONE ? rs : sq(qf_mul<false>(tau, rs));
+    else c = ONE ? sq(rs - qf_one()) : sq(qf_fma<false, true>(tau, tau, rs));
+    acc.hi = NEG ? sq(acc.hi - c) : sq(acc.hi + c);
+    const double r = abs_part(rs) + (real ? 1.0 : 0.0);
+    acc.abs = ONE ? acc.abs + r : fma(abs_part(tau), r, acc.abs);
 }
 template <typename T, int NB> struct BinAcc {
     T v[NB];
@@ -436,9 +494,10 @@ __device__ __forceinline__ void dfs(const Src &A, T tau, int depth, int nreal, A
         }
     } else if constexpr (m == 1) {
         const T det = det2(p00, p01, p11);
-        if constexpr (Prec<T>::fixed) acc.bad |= pivot_bad(det);
+        if constexpr (Prec<T>::fixed || std::is_same_v<T, sq>) acc.bad |= pivot_bad(det);
         const T rs = rsq<T>(det);
-        leaf_pair<NEG>(acc, ONE ? rs : mul_pos(tau, rs), tau, real, cnt);
+        if constexpr (std::is_same_v<T, sq>) leaf_pair_sq<NEG, ONE>(acc, rs, tau, real);
+        else leaf_pair<NEG>(acc, ONE ? rs : mul_pos(tau, rs), tau, real, cnt);
     } else if constexpr (Prec<T>::fixed) {
         // symmetric form C - U U^T, U = B R^{-T} (offset rows)
         constexpr int d = 2 * (m - 1);
@@ -458,9 +517,10 @@ __device__ __forceinline__ void dfs(const Src &A, T tau, int depth, int nreal, A
     } else {
         constexpr int d = 2 * (m - 1);
         const T det = det2(p00, p01, p11);
+        if constexpr (std::is_same_v<T, sq>) acc.bad |= pivot_bad(det);
         const T rs = rsq<T>(det);
         const T inv = rs * rs;
-        const T q00 = p11 * inv, q01 = -p01 * inv, q11 = p00 * inv;
+        const T q00 = p11 * inv, q01 = mul_neg(p01, inv), q11 = p00 * inv;
         T b0[d], b1[d], w0[d], w1[d];
 #pragma unroll
         for (int i = 0; i < d; ++i) {
@@ -475,7 +535,7 @@ __device__ __forceinline__ void dfs(const Src &A, T tau, int depth, int nreal, A
 #pragma unroll
             for (int j = i; j < d; ++j)
                 C.v[pidx(d, i, j)] = fms2(A(o + 2 + i, o + 2 + j), w0[i], b0[j], w1[i], b1[j]);
-        dfs<T, m - 1, 0, NEG, false>(C, ONE ? rs : tau * rs, depth + 1, nreal, acc, cnt + 1);
+        dfs<T, m - 1, 0, NEG, false>(C, ONE ? rs : T(tau * rs), depth + 1, nreal, acc, cnt + 1);
         if (real) dfs<T, MD, O + 1, !NEG, ONE>(A, tau, depth + 1, nreal, acc, cnt);
     }
 }
@@ -505,7 +565,14 @@ struct Plan {
     double *partials;   // 3 per unit
     int split;          // prefix levels looped inside a unit (0..kS)
     double t_re, t_im;  // complex binned sweep: the generating variable t of A = I - t O
+    int *n_redo;        // patterns the first pass of GBS_DD leaves to the second
+    bool redo;          // a second pass: only the patterns with kRedoFlag in their status bits
 };
+constexpr int kRedoFlag = 256;
+// GBS_DD: patterns with kappa above this, and those without a result, are taken again in
+// double-double.  There the two arithmetics' last digits differ by more than 1e-9 of the result
+// (kappa 2^-106 times a few), and the sign of a sum that is all cancellation is the arithmetic's.
+constexpr double kRedoKappa = 1e22;
 
 template <typename T>
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(int M, const uint64_t *__restrict__ pats,
@@ -599,6 +666,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(int M, const uint64_
         *pl.total_units = over ? 0 : total;
         *pl.overflow = over ? 1 : 0;
         *pl.counter = 0;
+        *pl.n_redo = 0;
     }
 }
 
@@ -632,7 +700,7 @@ __device__ __forceinline__ typename Prec<T>::Tau elim_pivot(T *Mx, int D, int c0
     const T rs = rsq<T>(det);
     if (t < Dt) {
         const T inv = rs * rs;
-        const T q00 = p11 * inv, q01 = -p01 * inv, q11 = p00 * inv;
+        const T q00 = p11 * inv, q01 = mul_neg(p01, inv), q11 = p00 * inv;
         const T b0 = Mx[pidx(D, c0, c0 + 2 + t)], b1 = Mx[pidx(D, c0 + 1, c0 + 2 + t)];
         Wb[2 * t] = dot2(q00, b0, q01, b1);
         Wb[2 * t + 1] = dot2(q01, b0, q11, b1);
@@ -666,7 +734,7 @@ __device__ __forceinline__ typename Prec<T>::Tau elim_into(const T *Mx, int D, i
     const T rs = rsq<T>(det);
     if (t < Dt) {
         const T inv = rs * rs;
-        const T q00 = p11 * inv, q01 = -p01 * inv, q11 = p00 * inv;
+        const T q00 = p11 * inv, q01 = mul_neg(p01, inv), q11 = p00 * inv;
         const T b0 = Mx[pidx(D, c0, c0 + 2 + t)], b1 = Mx[pidx(D, c0 + 1, c0 + 2 + t)];
         Wb[2 * t] = dot2(q00, b0, q01, b1);
         Wb[2 * t + 1] = dot2(q01, b0, q11, b1);
@@ -703,7 +771,7 @@ __device__ __forceinline__ void store2(double *o, zf v) { o[0] = ff_to_double(v.
 // BIN: the click-number distribution mode (one pattern = all M modes): the subset
 // terms are summed unsigned into bins by subset size instead of into the signed sum
 template <typename T, bool BIN = false>
-__global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__restrict__ O,
+__global__ void __launch_bounds__(kThreads, std::is_same_v<T, sq> ? 3 : 0) sweep_kernel(int M, const double *__restrict__ O,
                                                         const uint64_t *__restrict__ pats, int n_pat, Plan pl) {
     using Lay = Layout<T>;
     constexpr int B = Prec<T>::B;
@@ -736,6 +804,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
 
     const int t = threadIdx.x;
     const int N2 = 2 * M;
+    if (pl.redo && *pl.n_redo == 0) return;
     // decode tables (i, j) of packed indices for every even dimension 2m <= 2R
     if (t == 0) {
         int off = 0;
@@ -764,6 +833,10 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
             if (pl.unit_off[mid] <= u) lo = mid; else hi = mid;
         }
         const int sp = lo;
+        if (pl.redo && !(pl.pflags[sp] & kRedoFlag)) {
+            __syncthreads();  // every thread has read s_unit
+            continue;
+        }
         const int p = pl.perm[sp];
         const long long prefix = u - pl.unit_off[sp];
         const uint64_t wlo = pats[2 * p], whi = pats[2 * p + 1];
@@ -779,7 +852,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
         __syncthreads();
         const int n = s_n;
         int n_eff, L_eff, q, ss;
-        unit_shape<T>(n, n_eff, L_eff, q, ss, pl.split);
+        unit_shape<T>(n, n_eff, L_eff, q, ss, pl.split + kSubMore<T>);
         const int r = L_eff + B;           // modes of a sub-unit's level-0 matrix
         const int qs = q - ss;             // prefix levels fixed by the unit index
         const int rp = ss + r;             // modes after the unit's prefix elimination
@@ -807,6 +880,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 const int si = modes[a] + (i & 1) * M, sj = modes[b] + (j & 1) * M;
                 const double o = O[(size_t)si * N2 + sj];
                 if (Prec<T>::fixed && !(fabs(o) <= 4.0)) atomicOr(&s_flag, 2);
+                if (std::is_same_v<T, sq> && !(fabs(o) <= 0x1p100)) atomicOr(&s_flag, 1);
                 v = a_entry_t<T>(i == j ? 1.0 : 0.0, o, pl.t_re, pl.t_im);
             }
             X[pidx(D0, i, j)] = v;
@@ -819,7 +893,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
         // matrix may extend over Ublk
         {
             const int d = 2 * rp, o = 2 * k;
-            constexpr int kDm = 2 * (kS + Lay::R), kPer = (kDm * kDm + kThreads - 1) / kThreads;
+            constexpr int kDm = 2 * (Lay::S + Lay::R), kPer = (kDm * kDm + kThreads - 1) / kThreads;
             T tmp[kPer];
 #pragma unroll
             for (int q = 0; q < kPer; ++q) {
@@ -837,6 +911,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
         const int nsub = 1 << ss;
         double u_hi = 0.0, u_lo = 0.0, u_abs = 0.0;
         fxe6 uacc6(fx6_zero(), -(1 << 20));  // fx6: the unit's sum (thread 0)
+        sq u_sq = qf_zero();                 // sq: the thread's sum
         if constexpr (BIN) {
             for (int z = t; z <= n; z += kThreads) s_ubin[z] = typename BinOf<T>::type(0.0);
         }
@@ -848,8 +923,8 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
         // every choice above the one that turns include.  jv[e]: the slot of the matrix the
         // node at depth e views (0: Ublk); tv[e]: the product of the includes' det^{-1/2}
         // above depth e.
-        int jv[kS + 1];
-        Tau tv[kS + 1];
+        int jv[Lay::S + 1];
+        Tau tv[Lay::S + 1];
         jv[0] = 0;
         tv[0] = Tau(1.0);
         for (int leaf = 0; leaf < nsub; ++leaf) {
@@ -928,7 +1003,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                     const T rs = rsq<T>(det);
                     const T inv = rs * rs;
                     Qb[3 * t] = p11 * inv;
-                    Qb[3 * t + 1] = -p01 * inv;
+                    Qb[3 * t + 1] = mul_neg(p01, inv);
                     Qb[3 * t + 2] = p00 * inv;
                     const int bad = pivot_bad(det);
                     const Node tp = NIO::ld(tsrc, t);
@@ -1085,12 +1160,19 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 SmemMat<T, B> A{node};
                 dfs<T, B, 0, false>(A, konst<T>(1.0), 0, nreal, acc, 0);
                 const int excl = (qs - k) + (ss - kk) + (L_eff - __popc(t));
+                if constexpr (std::is_same_v<T, sq>) {
+                    const sq sc = sq(tau_node * tsub), c = sq(sc * acc.hi);
+                    u_sq = (excl & 1) ? sq(u_sq - c) : sq(u_sq + c);
+                    u_abs += abs_part(sc) * acc.abs;
+                    if (acc.bad || is_nan(tau_node) || is_nan(tsub)) atomicOr(&s_flag, 1);
+                } else {
                 const Tau sc = Tau((excl & 1) ? -1.0 : 1.0) * Tau(tau_node) * tsub;
                 double sh, sl;
                 sum_parts(acc.hi, acc.lo, sh, sl);
                 unit_add(u_hi, u_lo, sc, sh, sl);
                 u_abs += tau_abs(sc) * to_hi(acc.abs);
                 if (is_nan(acc.abs) || is_nan(tau_node)) atomicOr(&s_flag, 1);
+                }
             }
             __syncthreads();   // X / Y are rewritten by the next sub-unit
         }
@@ -1117,6 +1199,11 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
             }
             __syncthreads();
         } else {
+        if constexpr (std::is_same_v<T, sq>) {
+            const dd v = qf_to_dd(u_sq);
+            u_hi = v.hi;
+            u_lo = v.lo;
+        }
         double c_hi = u_hi, c_lo = u_lo, c_abs = u_abs;
         // deterministic CTA reduction (TwoSum tree)
         for (int off = 16; off; off >>= 1) {
@@ -1145,7 +1232,7 @@ __global__ void __launch_bounds__(kThreads) sweep_kernel(int M, const double *__
                 l += red[3 * w + 1] + e;
                 a += red[3 * w + 2];
             }
-            const Tau tp = s_tpre;
+            const auto tp = tau_out(s_tpre);
             unit_scale(h, l, tp);
             double *out = pl.partials + 3 * u;
             out[0] = h;
@@ -1244,12 +1331,19 @@ __global__ void finalize_kernel(int n_pat, const double *__restrict__ logdet, Pl
     const int p = pl.perm[sp];
     const int n = pl.pat_n[p];
     const bool batch_over = *pl.overflow != 0;
+    if (std::is_same_v<T, sq> && sp == 0 && lane == 0) *pl.counter = 0;  // for the second pass
+    if (pl.redo && !(pl.pflags[sp] & kRedoFlag)) return;
     double h, l, a;
     warp_unit_sum(pl.partials, pl.unit_off[sp], batch_over ? pl.unit_off[sp] : pl.unit_off[sp + 1], lane, h, l, a);
     if (lane) return;
     double lp, kap, eb;
     int st;
-    finish_pattern<T>(n, batch_over, pl.pflags[sp], h, l, a, *logdet, lp, kap, eb, st);
+    finish_pattern<std::conditional_t<std::is_same_v<T, sq>, dd, T>>(n, batch_over, pl.pflags[sp] & ~kRedoFlag, h, l, a,
+                                                                    *logdet, lp, kap, eb, st);
+    if (std::is_same_v<T, sq> && (st == GBS_OK ? !(kap <= kRedoKappa) : st == GBS_E_NOT_SPD || st == GBS_E_NONPOSITIVE)) {
+        pl.pflags[sp] = kRedoFlag;
+        atomicAdd(pl.n_redo, 1);
+    }
     logP[p] = lp;
     if (kappa) kappa[p] = kap;
     if (err_bound) err_bound[p] = eb;
@@ -1414,31 +1508,74 @@ Plan plan_from(void *ws, int n_pat) {
     pl.split = kS;
     pl.t_re = 0.0;
     pl.t_im = 0.0;
+    pl.n_redo = (int *)(b + o.overflow) + 1;
+    pl.redo = false;
     return pl;
+}
+
+// the blocks of a sweep kernel an SM holds (a context's first call of it asks the runtime)
+template <typename T> int sweep_setup(gbs_ctx *ctx, int &blocks_per_sm) {
+    using Lay = Sweep<T>;
+    int &nb = ctx->sweep_blocks_per_sm[std::is_same_v<T, sq> ? 7 : Prec<T>::idx];
+    if (nb == 0) {
+        GBS_CUDA(ctx, cudaFuncSetAttribute(Sweep<T>::kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)Lay::bytes));
+        int b = 0;
+        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, Sweep<T>::kernel, kThreads, Lay::bytes));
+        if (b < 1) return gbs_fail(ctx, GBS_E_CUDA, "sweep kernel does not fit on an SM");
+        nb = b;
+    }
+    blocks_per_sm = nb;
+    return GBS_OK;
+}
+
+// a planned batch: the sweep of every unit (timed, if the context times its sweeps), then the
+// patterns' results
+template <typename T>
+int launch_sweep(gbs_ctx *ctx, bool timed, int M, const double *O, const double *logdet, const uint64_t *pats, int n_pat,
+                 const Plan &pl, double *logP, double *kappa, double *err_bound, int32_t *status) {
+    int nb;
+    int st = sweep_setup<T>(ctx, nb);
+    if (st) return st;
+    if (timed && (st = gbs_timing_begin(ctx))) return st;
+    Sweep<T>::kernel<<<ctx->num_sms * nb, kThreads, Sweep<T>::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
+    GBS_CUDA(ctx, cudaGetLastError());
+    if (timed && (st = gbs_timing_end(ctx))) return st;
+    const int fthreads = 256, fblocks = (n_pat * 32 + fthreads - 1) / fthreads;
+    if constexpr (std::is_same<T, fx6>::value)
+        finalize6_kernel<<<fblocks, fthreads, 0, ctx->stream>>>(n_pat, logdet, pl, logP, kappa, err_bound, status);
+    else
+        finalize_kernel<T><<<fblocks, fthreads, 0, ctx->stream>>>(n_pat, logdet, pl, logP, kappa, err_bound, status);
+    GBS_CUDA(ctx, cudaGetLastError());
+    return GBS_OK;
+}
+// GBS_DD: every pattern in software floating point, then those that kRedoKappa names in double-double
+int launch_sweep_dd(gbs_ctx *ctx, bool timed, int M, const double *O, const double *logdet, const uint64_t *pats,
+                    int n_pat, const Plan &pl, double *logP, double *kappa, double *err_bound, int32_t *status) {
+    int st = timed ? gbs_timing_begin(ctx) : GBS_OK;
+    if (st) return st;
+    st = launch_sweep<sq>(ctx, false, M, O, logdet, pats, n_pat, pl, logP, kappa, err_bound, status);
+    if (st) return st;
+    Plan again = pl;
+    again.redo = true;
+    st = launch_sweep<dd>(ctx, false, M, O, logdet, pats, n_pat, again, logP, kappa, err_bound, status);
+    if (st) return st;
+    return timed ? gbs_timing_end(ctx) : GBS_OK;
 }
 
 template <typename T>
 int run_sweep(gbs_ctx *ctx, int M, const double *O, const double *logdet, const uint64_t *pats,
-              int n_pat, double *logP, double *kappa, double *err_bound, int32_t *status) {
-    using Lay = Sweep<T>;
+              int n_pat, double *logP, double *kappa, double *err_bound, int32_t *status,
+              bool two_pass = true) {
     const int pi = Prec<T>::idx;
     if (ctx->reserved && n_pat > ctx->cap_pat)
         return gbs_fail(ctx, GBS_E_INVALID, "gbs_prob: %d patterns exceed the reservation of %d",
                         n_pat, ctx->cap_pat);
-    if (ctx->sweep_blocks_per_sm[pi] == 0) {
-        GBS_CUDA(ctx, cudaFuncSetAttribute(Sweep<T>::kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)Lay::bytes));
-        int nb = 0;
-        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Sweep<T>::kernel, kThreads,
-                                                                    Lay::bytes));
-        if (nb < 1) return gbs_fail(ctx, GBS_E_CUDA, "sweep kernel does not fit on an SM");
-        ctx->sweep_blocks_per_sm[pi] = nb;
-    }
     long long cap;
     if (ctx->reserved) {
         cap = (long long)((ctx->ws_bytes - ws_offsets(n_pat, 0).partials) / (8 * partial_words<T>()));
     } else {
-        int st = gbs_ws_ensure(ctx, ws_offsets(n_pat, 0).end);
+        const int st = gbs_ws_ensure(ctx, ws_offsets(n_pat, 0).end);
         if (st) return st;
         cap = (long long)((ctx->ws_bytes - ws_offsets(n_pat, 0).partials) / (8 * partial_words<T>()));
     }
@@ -1462,21 +1599,9 @@ int run_sweep(gbs_ctx *ctx, int M, const double *O, const double *logdet, const 
             GBS_CUDA(ctx, cudaGetLastError());
         }
     }
-    const int grid = ctx->num_sms * ctx->sweep_blocks_per_sm[pi];
-    int st = gbs_timing_begin(ctx);
-    if (st) return st;
-    Sweep<T>::kernel<<<grid, kThreads, Lay::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
-    GBS_CUDA(ctx, cudaGetLastError());
-    st = gbs_timing_end(ctx);
-    if (st) return st;
-    const int fthreads = 256, fblocks = (n_pat * 32 + fthreads - 1) / fthreads;
-    if constexpr (std::is_same<T, fx6>::value)
-        finalize6_kernel<<<fblocks, fthreads, 0, ctx->stream>>>(n_pat, logdet, pl, logP, kappa, err_bound, status);
-    else
-        finalize_kernel<T><<<fblocks, fthreads, 0, ctx->stream>>>(n_pat, logdet, pl, logP, kappa,
-                                                                 err_bound, status);
-    GBS_CUDA(ctx, cudaGetLastError());
-    return GBS_OK;
+    if constexpr (std::is_same_v<T, dd>)
+        if (two_pass) return launch_sweep_dd(ctx, true, M, O, logdet, pats, n_pat, pl, logP, kappa, err_bound, status);
+    return launch_sweep<T>(ctx, true, M, O, logdet, pats, n_pat, pl, logP, kappa, err_bound, status);
 }
 
 // The same launch sequence on a workspace the caller provides: no allocation,
@@ -1485,17 +1610,7 @@ template <typename T>
 int run_sweep_on(gbs_ctx *ctx, void *ws, size_t ws_bytes, int M, const double *O,
                  const double *logdet, const uint64_t *pats, int n_pat, double *logP,
                  double *kappa, double *err_bound, int32_t *status) {
-    using Lay = Sweep<T>;
     const int pi = Prec<T>::idx;
-    if (ctx->sweep_blocks_per_sm[pi] == 0) {
-        GBS_CUDA(ctx, cudaFuncSetAttribute(Sweep<T>::kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)Lay::bytes));
-        int nb = 0;
-        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Sweep<T>::kernel, kThreads,
-                                                                    Lay::bytes));
-        if (nb < 1) return gbs_fail(ctx, GBS_E_CUDA, "sweep kernel does not fit on an SM");
-        ctx->sweep_blocks_per_sm[pi] = nb;
-    }
     const size_t base = ws_offsets(n_pat, 0).partials;
     if (ws_bytes < base)
         return gbs_fail(ctx, GBS_E_INVALID, "workspace of %zu bytes cannot hold %d patterns", ws_bytes, n_pat);
@@ -1504,14 +1619,9 @@ int run_sweep_on(gbs_ctx *ctx, void *ws, size_t ws_bytes, int M, const double *O
     pl.split = sweep_split_of(ctx, pi);
     plan_kernel<T><<<1, kPlanThreads, 0, ctx->stream>>>(M, pats, n_pat, cap, pl);
     GBS_CUDA(ctx, cudaGetLastError());
-    const int grid = ctx->num_sms * ctx->sweep_blocks_per_sm[pi];
-    Sweep<T>::kernel<<<grid, kThreads, Lay::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
-    GBS_CUDA(ctx, cudaGetLastError());
-    const int fthreads = 256, fblocks = (n_pat * 32 + fthreads - 1) / fthreads;
-    finalize_kernel<T><<<fblocks, fthreads, 0, ctx->stream>>>(n_pat, logdet, pl, logP, kappa,
-                                                             err_bound, status);
-    GBS_CUDA(ctx, cudaGetLastError());
-    return GBS_OK;
+    if constexpr (std::is_same_v<T, dd>)
+        return launch_sweep_dd(ctx, false, M, O, logdet, pats, n_pat, pl, logP, kappa, err_bound, status);
+    return launch_sweep<T>(ctx, false, M, O, logdet, pats, n_pat, pl, logP, kappa, err_bound, status);
 }
 
 // One slice of the batch's work units (gbs_prob_partial): the plan of the whole batch,
@@ -1519,20 +1629,13 @@ int run_sweep_on(gbs_ctx *ctx, void *ws, size_t ws_bytes, int M, const double *O
 template <typename T>
 int run_sweep_slice(gbs_ctx *ctx, int M, const double *O, const uint64_t *pats, int n_pat, int part,
                     int nparts, double *partial, int32_t *pflag) {
-    using Lay = Sweep<T>;
     const int pi = Prec<T>::idx;
     if (ctx->reserved && n_pat > ctx->cap_pat)
         return gbs_fail(ctx, GBS_E_INVALID, "gbs_prob_partial: %d patterns exceed the reservation of %d",
                         n_pat, ctx->cap_pat);
-    if (ctx->sweep_blocks_per_sm[pi] == 0) {
-        GBS_CUDA(ctx, cudaFuncSetAttribute(Sweep<T>::kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)Lay::bytes));
-        int nb = 0;
-        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Sweep<T>::kernel, kThreads,
-                                                                    Lay::bytes));
-        if (nb < 1) return gbs_fail(ctx, GBS_E_CUDA, "sweep kernel does not fit on an SM");
-        ctx->sweep_blocks_per_sm[pi] = nb;
-    }
+    int nb;
+    const int st0 = sweep_setup<T>(ctx, nb);
+    if (st0) return st0;
     if (!ctx->reserved) {
         int st = gbs_ws_ensure(ctx, ws_offsets(n_pat, 0).end);
         if (st) return st;
@@ -1559,10 +1662,9 @@ int run_sweep_slice(gbs_ctx *ctx, int M, const double *O, const uint64_t *pats, 
     long long *range = (long long *)((char *)ctx->ws + ws_offsets(n_pat, 0).range);
     slice_kernel<<<1, 1, 0, ctx->stream>>>(pl, part, nparts, range);
     GBS_CUDA(ctx, cudaGetLastError());
-    const int grid = ctx->num_sms * ctx->sweep_blocks_per_sm[pi];
     int st = gbs_timing_begin(ctx);
     if (st) return st;
-    Sweep<T>::kernel<<<grid, kThreads, Lay::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
+    Sweep<T>::kernel<<<ctx->num_sms * nb, kThreads, Sweep<T>::bytes, ctx->stream>>>(M, O, pats, n_pat, pl);
     GBS_CUDA(ctx, cudaGetLastError());
     st = gbs_timing_end(ctx);
     if (st) return st;
@@ -1815,7 +1917,8 @@ int sweep_auto(gbs_ctx *ctx, int M, const double *O, const double *logdet, const
     const unsigned g = (unsigned)((n_pat + 255) / 256);
     auto_mark_kernel<<<g, 256, 0, ctx->stream>>>(n_pat, st1, patterns, redo);
     GBS_CUDA(ctx, cudaGetLastError());
-    r = sweep_exact(ctx, M, O, logdet, redo, n_pat, GBS_DD, lp2, ka2, er2, st2);
+    // (in one pass: mostly there is nothing to do, and a launch without work costs 2 us)
+    r = run_sweep<dd>(ctx, M, O, logdet, redo, n_pat, lp2, ka2, er2, st2, false);
     if (r) return r;
     auto_merge_kernel<<<g, 256, 0, ctx->stream>>>(n_pat, st1, lp2, ka2, er2, st2, logP, ka1, eb1, st1);
     GBS_CUDA(ctx, cudaGetLastError());
