@@ -96,6 +96,18 @@ __device__ __forceinline__ cx<ff> cfms_ff(cx<ff> e, cx<ff> a, cx<ff> b) {
 static __device__ GBS_FF_FMS_INLINE cx<ff> cfms(cx<ff> e, cx<ff> a, cx<ff> b) { return cfms_ff(e, a, b); }
 template <typename R> __device__ __forceinline__ cx<R> cfms_inl(cx<R> e, cx<R> a, cx<R> b) { return e - a * b; }
 __device__ __forceinline__ cx<ff> cfms_inl(cx<ff> e, cx<ff> a, cx<ff> b) { return cfms_ff(e, a, b); }
+// FP64 in fused multiply-adds, four an update instead of six: the gradient's (the forward keeps the
+// form above, whose last digits its fits go by)
+__device__ __forceinline__ cx<double> cfma_d(cx<double> c, cx<double> a, cx<double> b) {
+    return {fma(a.re, b.re, fma(-a.im, b.im, c.re)), fma(a.re, b.im, fma(a.im, b.re, c.im))};
+}
+__device__ __forceinline__ cx<double> cfms_d(cx<double> e, cx<double> a, cx<double> b) {
+    return {fma(-a.re, b.re, fma(a.im, b.im, e.re)), fma(-a.re, b.im, fma(-a.im, b.re, e.im))};
+}
+template <bool FUSED, typename R> __device__ __forceinline__ cx<R> cfms_inv(cx<R> e, cx<R> a, cx<R> b) {
+    if constexpr (FUSED) return cfms_d(e, a, b);
+    else return cfms_inl(e, a, b);
+}
 static __device__ __noinline__ cx<ff> cinv(cx<ff> a) { return cinv<ff>(a); }
 static __device__ __noinline__ cx<ff> crsqrt(cx<ff> p) { return crsqrt<ff>(p); }
 __device__ __forceinline__ cx<double> widen(cx<float> a) { return {(double)a.re, (double)a.im}; }
@@ -495,7 +507,7 @@ template <> struct GroupAcc<float> {
 // covered by the other); FP64, bound by its pipe, takes one.  Measured on a GB300, whole calls: order 2
 // at 50 modes 35.1 -> 31.9 ms, at 100 modes 165.3 -> 163.8, the FP64 gradient at 32 modes 74.2 -> 61.6.
 constexpr int kHeadStart = 4;
-template <typename R>
+template <typename R, bool FUSED = false>
 __device__ __forceinline__ void sweep_inverse(int M, const double *__restrict__ O, const int *modes, int n,
                                               double cs, double sn, cx<R> *G, int *s_bad, double *s_zs) {
     constexpr int W = kMinorThreads / 32;
@@ -547,7 +559,7 @@ __device__ __forceinline__ void sweep_inverse(int M, const double *__restrict__ 
             if (k + 1 < N) {
                 cx<R> *cbn = (k & 1) ? cb0 : cb1, *cun = (k & 1) ? cu0 : cu1;
                 // the next pivot (its place in G stays as it is until its own phase)
-                const cx<R> dn = cfms_inl(G[pidx(N, k + 1, k + 1)], cb[k + 1], cu[k + 1]);
+                const cx<R> dn = cfms_inv<FUSED>(G[pidx(N, k + 1, k + 1)], cb[k + 1], cu[k + 1]);
                 const cx<R> invn = cinv(dn);
                 if (t < N) {
                     const int lo = t < k + 1 ? t : k + 1, hi = t < k + 1 ? k + 1 : t;
@@ -555,7 +567,7 @@ __device__ __forceinline__ void sweep_inverse(int M, const double *__restrict__ 
                     cx<R> v;
                     if (t == k) v = cu[k + 1];
                     else if (t == k + 1) v = dn;
-                    else v = cfms_inl(e, cb[lo], cu[hi]);
+                    else v = cfms_inv<FUSED>(e, cb[lo], cu[hi]);
                     if (t != k + 1) e = v;
                     cbn[t] = v;
                     cun[t] = v * invn;
@@ -580,7 +592,7 @@ __device__ __forceinline__ void sweep_inverse(int M, const double *__restrict__ 
             if (a[0] == -2) break;
             cx<R> v[U];
             for (int q = 0; q < U; ++q)
-                if (U > 1 || a[q] >= 0) v[q] = cfms_inl(G[a[q] < 0 ? dead : a[q]], cb[i[q]], cu[j[q]]);
+                if (U > 1 || a[q] >= 0) v[q] = cfms_inv<FUSED>(G[a[q] < 0 ? dead : a[q]], cb[i[q]], cu[j[q]]);
             for (int q = 0; q < U; ++q)
                 if (a[q] >= 0) G[a[q]] = v[q];
         }
@@ -2165,7 +2177,7 @@ __device__ __forceinline__ cx<double> schur_tail(const cx<double> *__restrict__ 
         for (int i = k + 1; i < K; ++i) {
             const cx<double> li = a[pidx(K, k, i)] * inv;
 #pragma unroll
-            for (int j = i; j < K; ++j) a[pidx(K, i, j)] = a[pidx(K, i, j)] - li * a[pidx(K, k, j)];
+            for (int j = i; j < K; ++j) a[pidx(K, i, j)] = cfms_d(a[pidx(K, i, j)], li, a[pidx(K, k, j)]);
         }
     }
 #pragma unroll
@@ -2204,12 +2216,12 @@ __device__ __forceinline__ void diag_leaf(const cx<double> *__restrict__ Gs, int
                                           bool &bad) {
     cx<double> s[3];
     const cx<double> f = schur_tail<NV, 1>(Gs, N, m, s, bad);
-    const cx<double> det = s[0] * s[2] - s[1] * s[1];
+    const cx<double> det = cfms_d(s[0] * s[2], s[1], s[1]);
     if (!(s[0].re > 0.0) || !(det.re * s[0].re + det.im * s[0].im > 0.0)) bad = true;
     const cx<double> wgt = wz * f * crsqrt(det) * cinv(det);
-    k00 = k00 + wgt * s[2];
-    k01 = k01 - wgt * s[1];
-    k11 = k11 + wgt * s[0];
+    k00 = cfma_d(k00, wgt, s[2]);
+    k01 = cfms_d(k01, wgt, s[1]);
+    k11 = cfma_d(k11, wgt, s[0]);
 }
 
 // W = V + {a, b}, a < b: adds wz det(G_WW)^-1/2 [G_WW^-1]_ab to the off-diagonal block
@@ -2223,31 +2235,40 @@ __device__ __forceinline__ void off_leaf(const cx<double> *__restrict__ Gs, int 
     const cx<double> p00 = s[pidx(4, 0, 0)], p01 = s[pidx(4, 0, 1)], p11 = s[pidx(4, 1, 1)];
     const cx<double> q00 = s[pidx(4, 0, 2)], q01 = s[pidx(4, 0, 3)], q10 = s[pidx(4, 1, 2)], q11 = s[pidx(4, 1, 3)];
     const cx<double> r00 = s[pidx(4, 2, 2)], r01 = s[pidx(4, 2, 3)], r11 = s[pidx(4, 3, 3)];
-    const cx<double> detP = p00 * p11 - p01 * p01;
+    const cx<double> detP = cfms_d(p00 * p11, p01, p01);
     const cx<double> iP = cinv(detP);
     // X = P^-1 Q
-    const cx<double> x00 = (p11 * q00 - p01 * q10) * iP, x01 = (p11 * q01 - p01 * q11) * iP;
-    const cx<double> x10 = (p00 * q10 - p01 * q00) * iP, x11 = (p00 * q11 - p01 * q01) * iP;
-    const cx<double> c00 = r00 - (q00 * x00 + q10 * x10), c01 = r01 - (q00 * x01 + q10 * x11),
-                     c11 = r11 - (q01 * x01 + q11 * x11);
-    const cx<double> detC = c00 * c11 - c01 * c01;
+    const cx<double> x00 = cfms_d(p11 * q00, p01, q10) * iP, x01 = cfms_d(p11 * q01, p01, q11) * iP;
+    const cx<double> x10 = cfms_d(p00 * q10, p01, q00) * iP, x11 = cfms_d(p00 * q11, p01, q01) * iP;
+    const cx<double> c00 = cfms_d(cfms_d(r00, q00, x00), q10, x10), c01 = cfms_d(cfms_d(r01, q00, x01), q10, x11),
+                     c11 = cfms_d(cfms_d(r11, q01, x01), q11, x11);
+    const cx<double> detC = cfms_d(c00 * c11, c01, c01);
     const cx<double> iC = cinv(detC);
     if (!(p00.re > 0.0) || !(detP.re * p00.re + detP.im * p00.im > 0.0) || !(c00.re > 0.0) ||
         !(detC.re * c00.re + detC.im * c00.im > 0.0))
         bad = true;
     const cx<double> ci00 = c11 * iC, ci01 = mk<double>(0.0, 0.0) - c01 * iC, ci11 = c00 * iC;
     const cx<double> wgt = wz * f * crsqrt(detP) * crsqrt(detC);
-    ko[0] = ko[0] - wgt * (x00 * ci00 + x01 * ci01);
-    ko[1] = ko[1] - wgt * (x00 * ci01 + x01 * ci11);
-    ko[2] = ko[2] - wgt * (x10 * ci00 + x11 * ci01);
-    ko[3] = ko[3] - wgt * (x10 * ci01 + x11 * ci11);
+    ko[0] = cfms_d(ko[0], wgt, cfma_d(x00 * ci00, x01, ci01));
+    ko[1] = cfms_d(ko[1], wgt, cfma_d(x00 * ci01, x01, ci11));
+    ko[2] = cfms_d(ko[2], wgt, cfma_d(x10 * ci00, x11, ci01));
+    ko[3] = cfms_d(ko[3], wgt, cfma_d(x10 * ci01, x11, ci11));
 }
 
 // one CTA per (pattern, chunk of its contour points): per point t_l the inverse G (the
-// forward's sweep), K block by block (a thread or a warp per block), then Re(-1/2 t (s G - G K G)) added to
-// the chunk's own slot (packed upper triangle of 2n x 2n; every entry has one owner thread, so the
-// sums over l are in a fixed order)
-__global__ void __launch_bounds__(kMinorThreads, 1) approx_minors_adjoint_kernel(
+// forward's sweep), K block by block, then Re(-1/2 t (s G - G K G)) added to the chunk's own slot
+// (packed upper triangle of 2n x 2n; every entry has one owner thread, so the sums over l are in a
+// fixed order).
+//
+// Bound by the FP64 pipe (two lanes a clock and SM, whatever the number of active lanes): what counts
+// is the number of FP64 instructions a warp issues.  LOW (orders 1 and 2): a diagonal block's groups
+// over 16 lanes and the off-diagonal blocks, a single group each, in warps of their own; with a thread
+// a block every warp held a diagonal block and went through its n groups nearly alone.  Products are
+// fused, and of the second one, Re(h G T) with h multiplied into T first, only the real part is formed.
+// Measured on a GB300, 128 patterns of 8 to 16 clicks at order 2: 37.6 -> 10.4 ms (with 16 instead of two
+// CTAs an SM to choose from, so that the largest patterns do not finish alone).
+template <bool LOW>
+__global__ void __launch_bounds__(kMinorThreads, LOW ? 2 : 1) approx_minors_adjoint_kernel(
     int M, const double *__restrict__ O, const uint64_t *__restrict__ pats, int order, int chunks_per,
     ApproxPlan pl, const double *__restrict__ unit_B, double *__restrict__ slots, size_t sst,
     int *__restrict__ flags) {
@@ -2280,13 +2301,12 @@ __global__ void __launch_bounds__(kMinorThreads, 1) approx_minors_adjoint_kernel
     const double rho = pl.pat_rho[p];
     const int nb = n * (n + 1) / 2;
     bool bad = false;
-    auto gt = [&](int i, int j) -> cx<double> { const cx<double> v = Gs[pidx_any(N, i, j)]; return mk<double>(-v.re, -v.im); };
     for (int l = l0; l < l1; ++l) {
         double sn, cs;
         sincospi(2.0 * (double)l / (double)L, &sn, &cs);
         sn *= rho;
         cs *= rho;
-        sweep_inverse<double>(M, O, modes, n, cs, sn, Gs, &s_bad, s_zs);
+        sweep_inverse<double, true>(M, O, modes, n, cs, sn, Gs, &s_bad, s_zs);
         const size_t uo = ((size_t)pl.unit_off[p] + l) * 2 * (kMaxOrder + 1);
         cx<double> cb[kMaxOrder + 1];
         cx<double> sl = mk<double>(0.0, 0.0);
@@ -2295,13 +2315,59 @@ __global__ void __launch_bounds__(kMinorThreads, 1) approx_minors_adjoint_kernel
             sl = sl + cb[w] * mk<double>(pl.unit_D[uo + 2 * w], pl.unit_D[uo + 2 * w + 1]);
         }
         const cx<double> zs = mk<double>(s_zs[0], s_zs[1]);
-        // one 2 x 2 block (a, b) per segment of gw lanes at a time: a thread at orders <= 2,
-        // where a block holds few groups (an off-diagonal one a single group at order 2), a
-        // warp above.  The segment's lanes split the block's groups W = V + {a, b}: V over the
+        if constexpr (LOW) {
+            const cx<double> z0 = mk<double>(0.0, 0.0);
+            const cx<double> w1 = cb[1] * zs, w2 = cb[2] * zs;
+            const int lane = t & 31, nd = (n + 1) >> 1, no = (n * (n - 1) / 2 + 31) >> 5;
+            for (int task = t >> 5; task < nd + no; task += kMinorThreads / 32) {
+                if (task < nd) {
+                    // two diagonal blocks a warp: group q of block a is {a}, then {x, a} for the other modes
+                    const int a = 2 * task + (lane >> 4), total = order > 1 ? n : 1;
+                    cx<double> k00 = z0, k01 = z0, k11 = z0;
+                    if (a < n)
+                        for (int q = lane & 15; q < total; q += 16) {
+                            if (q == 0) {
+                                const int m[1] = {a};
+                                diag_leaf<0>(Gs, N, m, w1, k00, k01, k11, bad);
+                            } else {
+                                const int m[2] = {q - 1 < a ? q - 1 : q, a};
+                                diag_leaf<1>(Gs, N, m, w2, k00, k01, k11, bad);
+                            }
+                        }
+#pragma unroll
+                    for (int off = 8; off; off >>= 1) {
+                        k00.re += __shfl_xor_sync(0xffffffffu, k00.re, off);
+                        k00.im += __shfl_xor_sync(0xffffffffu, k00.im, off);
+                        k01.re += __shfl_xor_sync(0xffffffffu, k01.re, off);
+                        k01.im += __shfl_xor_sync(0xffffffffu, k01.im, off);
+                        k11.re += __shfl_xor_sync(0xffffffffu, k11.re, off);
+                        k11.im += __shfl_xor_sync(0xffffffffu, k11.im, off);
+                    }
+                    if (a < n && (lane & 15) == 0) {
+                        Kp[pidx(N, 2 * a, 2 * a)] = k00;
+                        Kp[pidx(N, 2 * a, 2 * a + 1)] = k01;
+                        Kp[pidx(N, 2 * a + 1, 2 * a + 1)] = k11;
+                    }
+                } else {
+                    const int r = (task - nd) * 32 + lane;  // the r-th pair a < b
+                    if (r < n * (n - 1) / 2) {
+                        int m[2];
+                        unrank_pair(r, m[0], m[1]);
+                        cx<double> ko[4] = {z0, z0, z0, z0};
+                        if (order > 1) off_leaf<0>(Gs, N, m, w2, ko, bad);
+                        Kp[pidx(N, 2 * m[0], 2 * m[1])] = ko[0];
+                        Kp[pidx(N, 2 * m[0], 2 * m[1] + 1)] = ko[1];
+                        Kp[pidx(N, 2 * m[0] + 1, 2 * m[1])] = ko[2];
+                        Kp[pidx(N, 2 * m[0] + 1, 2 * m[1] + 1)] = ko[3];
+                    }
+                }
+            }
+        } else {
+        // one 2 x 2 block (a, b) a warp at a time: its lanes split the block's groups W = V + {a, b}: V over the
         // other modes, sizes ascending and each size in colex order (neighbouring lanes mostly
         // share the size, so the leaf code rarely diverges); partial sums meet in a fixed
         // shuffle tree.  Every thread runs every round (the shuffles take the whole warp).
-        const int gw = order <= 2 ? 1 : 32;
+        constexpr int gw = 32;
         const int seg = t / gw, sg = t - seg * gw, nseg = kMinorThreads / gw;
         const int rounds = (nb + nseg - 1) / nseg;
         for (int rd = 0; rd < rounds; ++rd) {
@@ -2380,25 +2446,29 @@ __global__ void __launch_bounds__(kMinorThreads, 1) approx_minors_adjoint_kernel
                 }
             }
         }
+        }
         __syncthreads();
-        // Re(-1/2 t (s G - G K G)) on the upper triangle, kPanel columns at a time
-        const cx<double> ht = mk<double>(-0.5 * cs, -0.5 * sn);
+        // Re(-1/2 t (s G - G K G)) on the upper triangle, kPanel columns at a time (Gs = -G)
+        const cx<double> ht = mk<double>(-0.5 * cs, -0.5 * sn), hs = ht * sl;
         for (int j0 = 0; j0 < N; j0 += kPanel) {
             for (int f = t; f < N * kPanel; f += kMinorThreads) {
                 const int r = f / kPanel, j = j0 + (f - r * kPanel);
                 cx<double> acc = mk<double>(0.0, 0.0);
                 if (j < N)
-                    for (int q = 0; q < N; ++q) acc = acc + Kp[pidx_any(N, r, q)] * gt(q, j);
-                Tp[f] = acc;
+                    for (int q = 0; q < N; ++q) acc = cfma_d(acc, Kp[pidx_any(N, r, q)], Gs[pidx_any(N, q, j)]);
+                Tp[f] = ht * acc;
             }
             __syncthreads();
             for (int f = t; f < N * kPanel; f += kMinorThreads) {
                 const int i = f / kPanel, jj = f - i * kPanel, j = j0 + jj;
                 if (j >= N || i > j) continue;
-                cx<double> y = mk<double>(0.0, 0.0);
-                for (int q = 0; q < N; ++q) y = y + gt(i, q) * Tp[q * kPanel + jj];
-                const cx<double> v = ht * (sl * gt(i, j) - y);
-                slot[pidx(N, i, j)] += v.re;
+                double y = 0.0;
+                for (int q = 0; q < N; ++q) {
+                    const cx<double> g = Gs[pidx_any(N, i, q)], x = Tp[q * kPanel + jj];
+                    y = fma(g.re, x.re, fma(-g.im, x.im, y));
+                }
+                const cx<double> g = Gs[pidx(N, i, j)];
+                slot[pidx(N, i, j)] -= fma(hs.re, g.re, fma(-hs.im, g.im, y));
             }
             __syncthreads();
         }
@@ -2707,8 +2777,9 @@ int approx_grad(gbs_ctx *ctx, int M, const double *O, const double *logdet, cons
     const long long units = ((long long *)ctx->pinned)[0], secs = ((long long *)ctx->pinned)[3];
     const int Lmax = (int)((long long *)ctx->pinned)[2];
     pl = approx_plan_from(ctx->ws, n_pat, units, secs);
-    // contour points of a pattern split over chunks_per CTAs: about two CTAs per SM in all
-    const int want = (2 * ctx->num_sms + n_pat - 1) / n_pat;
+    // contour points of a pattern split over chunks_per CTAs: about 16 CTAs per SM in all (a pattern's
+    // work goes with the fourth power of its clicks, so a wave or two would wait for the largest)
+    const int want = (16 * ctx->num_sms + n_pat - 1) / n_pat;
     const int chunks_per = want < 1 ? 1 : (want > 64 ? 64 : want);
     const int Nm = 2 * (n_max > 0 ? n_max : 1);
     const size_t sst = (size_t)sym(Nm), fst = (size_t)Nm * Nm, N2 = (size_t)(2 * M) * (2 * M);
@@ -2741,9 +2812,9 @@ int approx_grad(gbs_ctx *ctx, int M, const double *O, const double *logdet, cons
     if (n_max > 0) {
         // swept matrix + four staged columns, K, one panel of K G
         const size_t smem = sizeof(cx<double>) * (2 * sst + 4 * (size_t)Nm + (size_t)Nm * kPanel);
-        GBS_CUDA(ctx, cudaFuncSetAttribute(approx_minors_adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem));
-        approx_minors_adjoint_kernel<<<(unsigned)(n_pat * chunks_per), kMinorThreads, smem, ctx->stream>>>(
+        const auto adjoint = order <= 2 ? approx_minors_adjoint_kernel<true> : approx_minors_adjoint_kernel<false>;
+        GBS_CUDA(ctx, cudaFuncSetAttribute(adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        adjoint<<<(unsigned)(n_pat * chunks_per), kMinorThreads, smem, ctx->stream>>>(
             M, O, pats, order, chunks_per, pl, unit_B, slots, sst, flags);
         GBS_CUDA(ctx, cudaGetLastError());
         approx_grad_finalize_kernel<<<n_pat, 256, 0, ctx->stream>>>(chunks_per, pl, slots, sst, w, lp_i, st_i, flags,
