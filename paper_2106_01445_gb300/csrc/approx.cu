@@ -37,6 +37,7 @@ namespace {
 
 constexpr int kMaxOrder = 4;
 constexpr int kMinorThreads = 256;
+constexpr int kWideThreads = 512;   // of a minors CTA that has its SM to itself, orders 1 and 2
 constexpr int kDftThreads = 128;
 constexpr int kSecThreads = 256;   // one warp per sector
 constexpr int kFitThreads = 128;   // a warp on several sectors
@@ -507,10 +508,10 @@ template <> struct GroupAcc<float> {
 // covered by the other); FP64, bound by its pipe, takes one.  Measured on a GB300, whole calls: order 2
 // at 50 modes 35.1 -> 31.9 ms, at 100 modes 165.3 -> 163.8, the FP64 gradient at 32 modes 74.2 -> 61.6.
 constexpr int kHeadStart = 4;
-template <typename R, bool FUSED = false>
+template <typename R, bool FUSED = false, int TH = kMinorThreads>
 __device__ __forceinline__ void sweep_inverse(int M, const double *__restrict__ O, const int *modes, int n,
                                               double cs, double sn, cx<R> *G, int *s_bad, double *s_zs) {
-    constexpr int W = kMinorThreads / 32;
+    constexpr int W = TH / 32;
     __shared__ cx<R> s_inv[2];
     const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
     const int N = 2 * n, N2 = 2 * M;
@@ -522,7 +523,7 @@ __device__ __forceinline__ void sweep_inverse(int M, const double *__restrict__ 
         i = low ? fp : N - 1 - fp;
         j = low ? fp + fq : i + (fq - (N - fp));
     };
-    for (int f = t; f < fE; f += kMinorThreads) {
+    for (int f = t; f < fE; f += TH) {
         int i, j;
         fold(f, i, j);
         const int si = modes[i >> 1] + (i & 1) * M, sj = modes[j >> 1] + (j & 1) * M;
@@ -546,7 +547,7 @@ __device__ __forceinline__ void sweep_inverse(int M, const double *__restrict__ 
     const int rounds = (fE + 31) >> 5;
     for (int k = 0; k < N; ++k) {
         const cx<R> *cb = (k & 1) ? cb1 : cb0, *cu = (k & 1) ? cu1 : cu0;
-        if (t == kMinorThreads - 32) {
+        if (t == TH - 32) {
             const cx<R> d = cb[k];
             if (!(d.re > R(0))) *s_bad = 1;
             if (k & 1) zs = zs * widen(crsqrt(dprev * d));
@@ -598,7 +599,7 @@ __device__ __forceinline__ void sweep_inverse(int M, const double *__restrict__ 
         }
         __syncthreads();
     }
-    if (t == kMinorThreads - 32) { s_zs[0] = zs.re; s_zs[1] = zs.im; }
+    if (t == TH - 32) { s_zs[0] = zs.re; s_zs[1] = zs.im; }
     __syncthreads();
 }
 
@@ -615,6 +616,11 @@ __host__ __device__ inline int minor_smem_entries(int n, int esz, int min_blocks
     if (items < n - 1) items = n - 1;
     const long long ent = inv + (15 * items > 8LL * n ? 15 * items : 8LL * n);
     return (int)ent;
+}
+
+// two CTAs of float-float patterns of n clicks share an SM
+__host__ __device__ inline bool minor_shares_sm(int n, int esz) {
+    return ((long long)n * (2 * n + 1) + 8LL * n) * esz <= 228 * 1024 / 2 - 4 * 1024;
 }
 
 // Read-only view of the swept matrix -G, G = (I - t O_S)^{-1}, packed upper triangle of
@@ -790,8 +796,8 @@ static __device__ __noinline__ PairItem<ff> pair_item_tab(const GView<ff> V, int
 // CTA); s_off holds 2 (n + 1) ints of shared memory; add3: this CTA adds the three-detector
 // terms (of a CTA pair, one computes them for its phase 2 only).  table: the group's pair
 // factorisations G_PP = L D L^T are computed once per b into `scratch` ahead of the items
-// (cap >= n - 1 then), instead of once per item.
-template <typename R>
+// (cap >= n - 1 then), instead of once per item.  LOW: order <= 2, whose terms need no barrier.
+template <typename R, bool LOW = false>
 __device__ __forceinline__ void group_terms(const GView<R> &V, int n, int order, int tid, int nthr, int t2,
                                             int n2, cx<R> *scratch, int cap, int *s_off, bool add3, bool table,
                                             GroupAcc<R> &acc, bool &bad) {
@@ -815,6 +821,7 @@ __device__ __forceinline__ void group_terms(const GView<R> &V, int n, int order,
                 for (int j = i; j < 4; ++j) m[pidx(4, i, j)] = V.g(rr[i], rr[j]);
             acc.add(2, ldl_rsqrt_prod<R, 4>(m, bad));
         }
+    if constexpr (LOW) return;
     // order 4 in FP64 and float-float: the pair phases below; order 3, and every order in
     // FP32 (whose arithmetic is cheap next to the phases' barriers): a 6 x 6 factorisation
     // per triple, each serving its fourth detectors through a 2 x 2 Schur block
@@ -1041,12 +1048,15 @@ __device__ __forceinline__ int unit_pattern(const ApproxPlan &pl, int n_pat, lon
     return p;
 }
 
-// One CTA per (pattern, nu_l) unit, for patterns of up to n_single clicks (the packed
+// One CTA per (pattern, nu_l) unit, for patterns of n_from to n_single clicks (the packed
 // inverse in this CTA's shared memory); larger patterns are left to the cluster kernel.
-template <typename R>
-__global__ void __launch_bounds__(kMinorThreads, MinorPrec<R>::min_blocks) approx_minors_kernel(int M, const double *__restrict__ O,
+// TH = 512: order <= 2 on an SM that holds one CTA only.  The inverse, nearly all of the work there,
+// takes all 16 warps; the group terms stay with the first 256 threads, whose split of the sums is
+// that of every other size.
+template <typename R, int TH>
+__global__ void __launch_bounds__(TH, TH > kMinorThreads ? 1 : MinorPrec<R>::min_blocks) approx_minors_kernel(int M, const double *__restrict__ O,
                                                                     const uint64_t *__restrict__ pats,
-                                                                    int n_pat, int order, int n_single,
+                                                                    int n_pat, int order, int n_from, int n_single,
                                                                     int smem_entries,
                                                                     unsigned long long *counter,
                                                                     ApproxPlan pl) {
@@ -1068,7 +1078,7 @@ __global__ void __launch_bounds__(kMinorThreads, MinorPrec<R>::min_blocks) appro
         const int p = unit_pattern(pl, n_pat, u);
         const int l = (int)(u - pl.unit_off[p]);
         const int n = pl.pat_n[p], L = pl.pat_L[p];
-        if (n > n_single) {   // a pattern for the CTA pairs
+        if (n < n_from || n > n_single) {   // a pattern for another launch
             __syncthreads();
             continue;
         }
@@ -1089,7 +1099,7 @@ __global__ void __launch_bounds__(kMinorThreads, MinorPrec<R>::min_blocks) appro
         const double rho = pl.pat_rho[p];
         sn *= rho;
         cs *= rho;
-        sweep_inverse<R>(M, O, modes, n, cs, sn, G, &s_bad, s_zs);
+        sweep_inverse<R, false, TH>(M, O, modes, n, cs, sn, G, &s_bad, s_zs);
         GroupAcc<R> acc;
         acc.zero();
         bool bad = false;
@@ -1098,9 +1108,11 @@ __global__ void __launch_bounds__(kMinorThreads, MinorPrec<R>::min_blocks) appro
         // items per group from this pattern's own n (not the batch's allocation): the work
         // split, and with it every rounding, is the same in any batch
         const int cap = (minor_smem_entries(n, (int)sizeof(cx<R>), MinorPrec<R>::min_blocks) - sym(N)) / 15;
-        group_terms<R>(V, n, order, t, kMinorThreads, t, kMinorThreads, G + sym(N), cap, s_off, true, true, acc, bad);
+        constexpr bool kLow = TH > kMinorThreads;
+        if (!kLow || t < kMinorThreads)
+            group_terms<R, kLow>(V, n, order, t, kMinorThreads, t, kMinorThreads, G + sym(N), cap, s_off, true, true, acc, bad);
         if (bad) s_bad = 1;
-        warp_group_sums<R>(acc, red[t >> 5]);
+        if (!kLow || t < kMinorThreads) warp_group_sums<R>(acc, red[t >> 5]);
         __syncthreads();
         if (t == 0) {
             write_unit(pl, u, order, s_zs, red, kMinorThreads / 32);
@@ -1131,93 +1143,131 @@ __host__ __device__ inline int pair_part_entries(int N) {  // the larger half
     return lo > tot - lo ? lo : tot - lo;
 }
 
-template <typename R>
+// The inverse of sweep_inverse on both halves, one phase and one cluster barrier a pivot (in the place
+// of three barriers, with every warp forming the pivot's reciprocal).  A CTA forms its own entries of
+// the next column and stages them, and their quotients, in both CTAs.  The pivot after the next one may
+// be the other CTA's: its diagonal entry is passed on a pivot ahead (dg), so that both know the next
+// pivot as soon as a phase begins.  Measured on a GB300, order 2, 64 patterns of 40 to 90
+// clicks at 100 modes: the pair kernel 83.6 -> 75.5 ms (with 512 threads), the one-CTA kernel 74.1 -> 61.5
+// (sizes that share an SM in a launch of their own, the others with 512 threads).
+template <typename R> struct PairPivots {
+    cx<R> inv[2];  // reciprocal of this pivot and of the next
+    cx<R> dg[2];   // the next pivot's diagonal entry as the pivot before this one left it
+};
+template <typename R, int TH>
 __device__ void sweep_inverse_pair(cg::cluster_group &cl, int rank, int M, const double *__restrict__ O,
                                    const uint8_t *modes, int n, double cs, double sn, cx<R> *Gl, cx<R> *stage,
-                                   cx<R> *stage_peer, int rsplit, int off1, int *s_bad, double *s_zs) {
-    const int t = threadIdx.x;
+                                   cx<R> *stage_peer, PairPivots<R> *pv, PairPivots<R> *pv_peer, int rsplit, int off1,
+                                   int *s_bad, double *s_zs) {
+    constexpr int W = TH / 32;
+    const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
     const int N = 2 * n, N2 = 2 * M;
     const int r_lo = rank ? rsplit : 0, r_hi = rank ? N : rsplit;
     const int base = rank ? off1 : 0;
     auto lidx = [&](int i, int j) { return i * N - (i * (i - 1)) / 2 + (j - i) - base; };  // own row i <= j
-    for (int f = t; f < (r_hi - r_lo) * N; f += kMinorThreads) {
-        const int i = r_lo + f / N, j = f - (f / N) * N;
-        if (j < i) continue;
+    auto own = [&](int i) { return i >= r_lo && i < r_hi; };
+    // own rows folded in pairs (r_lo + q, r_hi - 1 - q), fw entries a pair; then the unpaired middle row
+    const int nrows = r_hi - r_lo, npair = nrows >> 1, fw = 2 * N - r_lo - r_hi + 1;
+    const int rmid = r_lo + npair, fP = npair * fw, fE = fP + ((nrows & 1) ? N - rmid : 0);
+    const uint32_t inv24 = (1u << 24) / (uint32_t)fw + 1u;  // f / fw = f inv24 >> 24 for f fw < 2^24, f inv24 < 2^32
+    auto fold = [&](int f, int &i, int &j) {
+        const int fp = (int)(((uint32_t)f * inv24) >> 24), fq = f - fp * fw, a = r_lo + fp;
+        const bool low = fq < N - a;
+        i = f >= fP ? rmid : low ? a : r_hi - 1 - fp;
+        j = f >= fP ? rmid + (f - fP) : low ? a + fq : i + (fq - (N - a));
+    };
+    for (int f = t; f < fE; f += TH) {
+        int i, j;
+        fold(f, i, j);
         const int si = modes[i >> 1] + (i & 1) * M, sj = modes[j >> 1] + (j & 1) * M;
         Gl[lidx(i, j)] = init_entry<R>(i == j, cs, sn, O[(size_t)si * N2 + sj]);
     }
-    cx<R> *const cb0 = stage, *const cb1 = stage + N, *const cu = stage + 2 * N;
-    cx<R> *const pb0 = stage_peer, *const pb1 = stage_peer + N;
     __syncthreads();
-    // pivot 0's column is row 0: rank 0's
-    if (rank == 0)
-        for (int i = t; i < N; i += kMinorThreads) {
-            const cx<R> v = Gl[lidx(0, i)];
-            cb0[i] = v;
-            pb0[i] = v;
+    const int NS = (N + 31) >> 5;  // warps that stage columns
+    if (wp < NS && t < N) {
+        if (rank == 0) {  // pivot 0's column is row 0
+            const cx<R> inv0 = cinv(Gl[0]), v = Gl[t], u = v * inv0;
+            stage[t] = v;
+            stage_peer[t] = v;
+            stage[2 * N + t] = u;
+            stage_peer[2 * N + t] = u;
+            if (t == 0) pv->inv[0] = pv_peer->inv[0] = inv0;
         }
+        if (t == 1 && own(1)) pv->dg[1] = pv_peer->dg[1] = Gl[lidx(1, 1)];
+    }
     cl.sync();
-    cx<double> zs = mk<double>(1.0, 0.0);
+    cx<double> zs = mk<double>(1.0, 0.0);  // on the last warp's first thread
     cx<R> dprev = mk<R>(R(1), R(0));
-    // own rows folded in pairs (r_lo + q, r_hi - 1 - q): fw entries per pair
-    const int nrows = r_hi - r_lo, npair = nrows >> 1, fw = 2 * N - r_lo - r_hi + 1, fE = npair * fw;
-    const int sp = kMinorThreads / fw, sq = kMinorThreads - sp * fw;
-    const int rmid = r_lo + npair;  // the unpaired middle row when nrows is odd
+    const int rounds = (fE + 31) >> 5;
     for (int k = 0; k < N; ++k) {
-        const cx<R> *cb = (k & 1) ? cb1 : cb0;
-        cx<R> *cbn = (k & 1) ? cb0 : cb1, *pbn = (k & 1) ? pb0 : pb1;
-        const cx<R> d = cb[k];
-        if (!(d.re > R(0)) && t == 0) *s_bad = 1;
-        if ((k & 1) && t == 0) zs = zs * widen(crsqrt(dprev * d));
-        dprev = d;
-        const cx<R> inv = cinv(d);
-        for (int i = t; i < N; i += kMinorThreads) cu[i] = cb[i] * inv;
-        __syncthreads();
-        // entries (i, j), i, j != k, of the own rows: e -= cb_i cu_j
-        int fp = t / fw, fq = t - fp * fw;
-        for (int f = t; f < fE; f += kMinorThreads) {
-            int i, j;
-            const int a = r_lo + fp;
-            if (fq < N - a) { i = a; j = a + fq; } else { i = r_hi - 1 - fp; j = i + (fq - (N - a)); }
-            if (i != k && j != k) {
-                cx<R> &e = Gl[lidx(i, j)];
-                e = cfms_inl(e, cb[i], cu[j]);
-            }
-            fq += sq;
-            fp += sp;
-            if (fq >= fw) { fq -= fw; ++fp; }
+        const int oc = (k & 1) * N, on = N - oc;  // staged: b, b', u, u'
+        const cx<R> *cb = stage + oc, *cu = stage + 2 * N + oc;
+        if (t == TH - 32) {
+            const cx<R> d = cb[k];
+            if (!(d.re > R(0))) *s_bad = 1;
+            if (k & 1) zs = zs * widen(crsqrt(dprev * d));
+            dprev = d;
         }
-        if (nrows & 1)
-            for (int j = rmid + t; j < N; j += kMinorThreads)
-                if (rmid != k && j != k) {
-                    cx<R> &e = Gl[lidx(rmid, j)];
-                    e = cfms_inl(e, cb[rmid], cu[j]);
-                }
-        __syncthreads();
-        // scale pivot k's row and column (own entries), stage pivot k + 1's column into
-        // both CTAs (the owner of each entry writes it)
-        const bool more = k + 1 < N;
-        for (int i = t; i < N; i += kMinorThreads) {
-            const int lo = i < k ? i : k, hi = i < k ? k : i;
-            if (i != k && lo >= r_lo && lo < r_hi) Gl[lidx(lo, hi)] = cu[i];
-            if (more) {
-                const int l2 = i < k + 1 ? i : k + 1, h2 = i < k + 1 ? k + 1 : i;
-                if (l2 >= r_lo && l2 < r_hi) {
-                    // entry (k, k + 1) is the one just scaled: cu[k + 1]
-                    const cx<R> v = i == k ? cu[k + 1] : Gl[lidx(l2, h2)];
-                    cbn[i] = v;
-                    pbn[i] = v;
+        if (wp < NS) {
+            if (t < N && t != k + 1) {  // scale pivot k's row and column (entry (k, k + 1) is the next column's)
+                const int lo = t < k ? t : k, hi = t < k ? k : t;
+                if (own(lo)) Gl[lidx(lo, hi)] = t == k ? mk<R>(R(0), R(0)) - pv->inv[k & 1] : cu[t];
+            }
+            if (k + 1 < N) {
+                const cx<R> dn = cfms_inl(pv->dg[(k + 1) & 1], cb[k + 1], cu[k + 1]);
+                const cx<R> invn = cinv(dn);
+                if (t < N) {
+                    const int lo = t < k + 1 ? t : k + 1, hi = t < k + 1 ? k + 1 : t;
+                    if (own(lo)) {
+                        cx<R> &e = Gl[lidx(lo, hi)];
+                        cx<R> v;
+                        if (t == k) v = cu[k + 1];
+                        else if (t == k + 1) v = dn;
+                        else v = cfms_inl(e, cb[lo], cu[hi]);
+                        if (t != k + 1) e = v;
+                        const cx<R> u = v * invn;
+                        stage[on + t] = v;
+                        stage_peer[on + t] = v;
+                        stage[2 * N + on + t] = u;
+                        stage_peer[2 * N + on + t] = u;
+                    }
+                    if (t == k + 1) pv->inv[(k + 1) & 1] = invn;
+                    if (t == k + 2 && own(t)) {
+                        cx<R> &e = Gl[lidx(t, t)];
+                        e = cfms_inl(e, cb[t], cu[t]);
+                        pv->dg[k & 1] = pv_peer->dg[k & 1] = e;
+                    }
                 }
             }
         }
-        if (t == 0 && k >= r_lo && k < r_hi) Gl[lidx(k, k)] = mk<R>(R(0), R(0)) - inv;
+        // the entries, 32 a round and warp, as in sweep_inverse
+        const int first = wp < NS || ((k & 1) && wp == W - 1) ? kHeadStart : 0;
+        const int m = NS < W ? W - NS - (k & 1) : 0;
+        auto entry = [&](int r, int &i, int &j) {
+            const int c = r < kHeadStart ? r * m + (wp - NS) : kHeadStart * m + (r - kHeadStart) * W + wp;
+            const int f = c * 32 + lane;
+            fold(f < fE ? f : 0, i, j);
+            const bool skip = i == k || j == k || i == k + 1 || j == k + 1 || (i == k + 2 && j == k + 2);
+            return c >= rounds ? -2 : f < fE && !skip ? lidx(i, j) : -1;
+        };
+        constexpr int U = std::is_same_v<R, ff> ? 2 : 1;
+        for (int r = first;; r += U) {
+            int a[U], i[U], j[U];
+            for (int q = 0; q < U; ++q) a[q] = entry(r + q, i[q], j[q]);
+            if (a[0] == -2) break;
+            cx<R> v[U];
+            for (int q = 0; q < U; ++q)
+                if (U > 1 || a[q] >= 0) v[q] = cfms_inl(a[q] < 0 ? cb[0] : Gl[a[q]], cb[i[q]], cu[j[q]]);
+            for (int q = 0; q < U; ++q)
+                if (a[q] >= 0) Gl[a[q]] = v[q];
+        }
         cl.sync();
     }
-    if (t == 0) { s_zs[0] = zs.re; s_zs[1] = zs.im; }
+    if (t == TH - 32) { s_zs[0] = zs.re; s_zs[1] = zs.im; }
 }
 
-template <typename R>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMinorThreads, 1)
+template <typename R, int TH>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TH, 1)
 approx_minors_pair_kernel(int M, const double *__restrict__ O, const uint64_t *__restrict__ pats, int n_pat,
                           int order, int n_single, int smem_entries, unsigned long long *counter, ApproxPlan pl) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1227,6 +1277,8 @@ approx_minors_pair_kernel(int M, const double *__restrict__ O, const uint64_t *_
     __shared__ int s_bad;
     __shared__ double red[2 * (kMinorThreads / 32)][2 * (kMaxOrder + 1)];
     __shared__ double s_zs[2];
+    __shared__ PairPivots<R> s_pv;
+    constexpr bool kLow = TH > kMinorThreads;  // order <= 2: group terms on 256 threads, as in the one-CTA kernel
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank(), t = threadIdx.x;
     const long long total = *pl.total;
@@ -1265,7 +1317,8 @@ approx_minors_pair_kernel(int M, const double *__restrict__ O, const uint64_t *_
         const double rho = pl.pat_rho[p];
         sn *= rho;
         cs *= rho;
-        sweep_inverse_pair<R>(cl, rank, M, O, modes, n, cs, sn, Gl, stage, stage_peer, rsplit, off1, &s_bad, s_zs);
+        sweep_inverse_pair<R, TH>(cl, rank, M, O, modes, n, cs, sn, Gl, stage, stage_peer, &s_pv,
+                                  cl.map_shared_rank(&s_pv, rank ^ 1), rsplit, off1, &s_bad, s_zs);
         cx<R> *G0 = rank == 0 ? Gl : cl.map_shared_rank(Gl, 0);
         cx<R> *G1 = rank == 1 ? Gl : cl.map_shared_rank(Gl, 1);
         const GView<R> V{G0, G1, N, rsplit, off1};
@@ -1274,12 +1327,14 @@ approx_minors_pair_kernel(int M, const double *__restrict__ O, const uint64_t *_
         bool bad = false;
         // each CTA computes every pair item in its own scratch (the staging area and beyond),
         // rank 0 adds the three-detector terms, the four-detector ones are split over both
-        group_terms<R>(V, n, order, rank * kMinorThreads + t, 2 * kMinorThreads, rank * kMinorThreads + t,
+        if (!kLow || t < kMinorThreads)
+            group_terms<R, kLow>(V, n, order, rank * kMinorThreads + t, 2 * kMinorThreads, rank * kMinorThreads + t,
                        2 * kMinorThreads, stage, n - 2, s_off, rank == 0, false, acc, bad);
         if (bad) s_bad = 1;
         // warp sums: rank 1's into rank 0's table (rows 8..15), then rank 0 writes the unit
         double (*red0)[2 * (kMaxOrder + 1)] = rank == 0 ? red : cl.map_shared_rank(red, 0);
-        warp_group_sums<R>(acc, red0[rank * (kMinorThreads / 32) + (t >> 5)]);
+        if (!kLow || t < kMinorThreads)
+            warp_group_sums<R>(acc, red0[rank * (kMinorThreads / 32) + (t >> 5)]);
         __syncthreads();
         if (rank == 1 && t == 0 && s_bad) atomicOr(cl.map_shared_rank(&s_bad, 0), 1);
         cl.sync();
@@ -2513,7 +2568,7 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 struct ApproxOffsets {
     size_t counter, total, overflow, info, counter2, pat_n, pat_L, pat_rho, unit_off, unit_flag, sec_off, pat_max,
-        pat_ld, unit_D, sec_D, sec_part, sec_slow, counter3, end;
+        pat_ld, unit_D, sec_D, sec_part, sec_slow, counter3, counter4, end;
 };
 
 ApproxOffsets approx_offsets(int n_pat, long long units, long long secs = 0) {
@@ -2524,7 +2579,8 @@ ApproxOffsets approx_offsets(int n_pat, long long units, long long secs = 0) {
     o.info = 24;       // 6 long long
     o.counter2 = 72;   // the CTA-pair minors kernel's work counter
     o.counter3 = 80;   // the slow fits' list length and its work counter
-    o.pat_n = align256(96);
+    o.counter4 = 96;   // the work counter of the patterns with an SM to themselves
+    o.pat_n = align256(104);
     o.pat_L = align256(o.pat_n + 4 * (size_t)n_pat);
     o.pat_rho = align256(o.pat_L + 4 * (size_t)n_pat);
     o.unit_off = align256(o.pat_rho + 8 * (size_t)n_pat);
@@ -2587,6 +2643,32 @@ int launch_plan(gbs_ctx *ctx, int M, const double *O, const uint64_t *pats, int 
     return GBS_OK;
 }
 
+// one launch of the one-CTA minors kernel, for the patterns of n_from to n_to clicks
+template <typename R, int TH>
+int launch_minors(gbs_ctx *ctx, int M, const double *O, const uint64_t *pats, int n_pat, int order, int n_from, int n_to,
+                  size_t counter, const ApproxPlan &pl) {
+    // the packed inverse and four staged pivot columns, or the pair phases' items
+    // (15 entries each, at least n - 1 of them, up to 8 n while the CTAs per SM stay)
+    // (the largest over the range: the kernel sizes each pattern's items from its own n,
+    // and the floor to whole items makes the entries fall by up to 14 between some n)
+    int ent = sym(2 * n_to) + 8 * n_to;  // FP32: no pair phases
+    if constexpr (!std::is_same<R, float>::value)
+        for (int m = n_from > 1 ? n_from : 1; m <= n_to; ++m) {
+            const int e = minor_smem_entries(m, (int)sizeof(cx<R>), MinorPrec<R>::min_blocks);
+            if (e > ent) ent = e;
+        }
+    const size_t minor_smem = sizeof(cx<R>) * (size_t)ent;
+    const auto kernel = approx_minors_kernel<R, TH>;
+    GBS_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)minor_smem));
+    int nb = 0;
+    GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, TH, minor_smem));
+    if (nb < 1) nb = 1;
+    kernel<<<ctx->num_sms * nb, TH, minor_smem, ctx->stream>>>(M, O, pats, n_pat, order, n_from, n_to, ent,
+                                                               (unsigned long long *)((char *)ctx->ws + counter), pl);
+    GBS_CUDA(ctx, cudaGetLastError());
+    return GBS_OK;
+}
+
 template <typename R>
 int run_approx(gbs_ctx *ctx, int M, const double *O, const double *logdet, const uint64_t *pats,
                int n_pat, int order, double *logP, double *kappa, double *err_bound, int32_t *status,
@@ -2623,38 +2705,36 @@ int run_approx(gbs_ctx *ctx, int M, const double *O, const double *logdet, const
     }
     pl = approx_plan_from(ctx->ws, n_pat, units, secs);
     GBS_CUDA(ctx, cudaMemsetAsync(ctx->ws, 0, 8, ctx->stream));  // work counters
-    GBS_CUDA(ctx, cudaMemsetAsync((char *)ctx->ws + approx_offsets(n_pat, 0).counter2, 0, 24, ctx->stream));
+    GBS_CUDA(ctx, cudaMemsetAsync((char *)ctx->ws + approx_offsets(n_pat, 0).counter2, 0, 32, ctx->stream));
     int st = gbs_timing_begin(ctx);
     if (st) return st;
-    if (nsmall > 0) {
-        // the packed inverse and four staged pivot columns, or the pair phases' items
-        // (15 entries each, at least n - 1 of them, up to 8 n while the CTAs per SM stay)
-        // (the largest over n <= nsmall: the kernel sizes each pattern's items from its own n,
-        // and the floor to whole items makes the entries fall by up to 14 between some n)
-        int ent = sym(2 * nsmall) + 8 * nsmall;  // FP32: no pair phases
-        if constexpr (!std::is_same<R, float>::value)
-            for (int m = 1; m <= nsmall; ++m) {
-                const int e = minor_smem_entries(m, (int)sizeof(cx<R>), MinorPrec<R>::min_blocks);
-                if (e > ent) ent = e;
-            }
-        const size_t minor_smem = sizeof(cx<R>) * (size_t)ent;
-        GBS_CUDA(ctx, cudaFuncSetAttribute(approx_minors_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)minor_smem));
-        int nb = 0;
-        GBS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, approx_minors_kernel<R>, kMinorThreads,
-                                                                    minor_smem));
-        if (nb < 1) nb = 1;
-        approx_minors_kernel<R><<<ctx->num_sms * nb, kMinorThreads, minor_smem, ctx->stream>>>(
-            M, O, pats, n_pat, order, n_single, ent, (unsigned long long *)ctx->ws, pl);
-        GBS_CUDA(ctx, cudaGetLastError());
+    // one CTA a unit: up to n_two clicks two of them (of 256 threads) share an SM; above, the SM
+    // holds one, of 512 threads where the inverse is all that counts
+    int n_two = nsmall;
+    if (std::is_same<R, ff>::value)
+        while (n_two > 0 && !minor_shares_sm(n_two, (int)sizeof(cx<R>))) --n_two;
+    if (nsmall > n_two) {
+        const size_t c4 = approx_offsets(n_pat, 0).counter4;
+        if constexpr (std::is_same<R, ff>::value) {
+            if (order <= 2) st = launch_minors<R, kWideThreads>(ctx, M, O, pats, n_pat, order, n_two + 1, nsmall, c4, pl);
+            else st = launch_minors<R, kMinorThreads>(ctx, M, O, pats, n_pat, order, n_two + 1, nsmall, c4, pl);
+        }
+        if (st) return st;
+    }
+    if (n_two > 0) {
+        st = launch_minors<R, kMinorThreads>(ctx, M, O, pats, n_pat, order, 0, n_two, 0, pl);
+        if (st) return st;
     }
     if constexpr (MinorPrec<R>::pair) if (nmax > n_single) {
-        // half of the packed inverse, and three staged columns or the pair phases' items
-        const int pent = pair_part_entries(2 * nmax) + (6 * nmax > 15 * (nmax - 2) ? 6 * nmax : 15 * (nmax - 2));
+        // half of the packed inverse, and four staged columns or the pair phases' items
+        const int pent = pair_part_entries(2 * nmax) + (8 * nmax > 15 * (nmax - 2) ? 8 * nmax : 15 * (nmax - 2));
         const size_t pair_smem = sizeof(cx<R>) * (size_t)pent;
-        GBS_CUDA(ctx, cudaFuncSetAttribute(approx_minors_pair_kernel<R>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem));
-        approx_minors_pair_kernel<R><<<(ctx->num_sms / 2) * 2, kMinorThreads, pair_smem, ctx->stream>>>(
+        const bool wide = std::is_same<R, ff>::value && order <= 2;
+        auto kernel = approx_minors_pair_kernel<R, kMinorThreads>;
+        if constexpr (std::is_same<R, ff>::value)
+            if (wide) kernel = approx_minors_pair_kernel<R, kWideThreads>;
+        GBS_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem));
+        kernel<<<(ctx->num_sms / 2) * 2, wide ? kWideThreads : kMinorThreads, pair_smem, ctx->stream>>>(
             M, O, pats, n_pat, order, n_single, pent,
             (unsigned long long *)((char *)ctx->ws + approx_offsets(n_pat, 0).counter2), pl);
         GBS_CUDA(ctx, cudaGetLastError());
