@@ -490,8 +490,142 @@ template <> struct GroupAcc<float> {
     __device__ __forceinline__ double get(int q) const { return (double)hi[q] + (double)lo[q]; }
 };
 
-// G <- -(I - t O_S)^{-1} in shared memory (packed upper triangle of 2n x 2n, then four
-// staged pivot columns of 2n entries), t = cs + i sn, by the symmetric sweep operator on
+// ---- the inverse's working layout -----------------------------------------------------
+// The matrix entry (E) and the staged column b and quotients u = b / pivot of two pivots (parity
+// `par`), in `rows` entries a row behind the matrix.
+template <typename R, bool FUSED = false> struct InvOps {
+    using E = cx<R>;
+    static constexpr int rows = 4;
+    static constexpr bool eager = false;  // an update of a skipped entry costs the FP64 pipe
+    E *G;
+    cx<R> *st;
+    int N;
+    __device__ __forceinline__ InvOps(cx<R> *g, cx<R> *stage, int n) : G(g), st(stage), N(n) {}
+    static __device__ __forceinline__ E pack(cx<R> v) { return v; }
+    __device__ __forceinline__ cx<R> get(int a) const { return G[a]; }
+    __device__ __forceinline__ cx<R> b(int par, int i) const { return st[par * N + i]; }
+    __device__ __forceinline__ cx<R> u(int par, int i) const { return st[(2 + par) * N + i]; }
+    __device__ __forceinline__ void put(int par, int i, cx<R> bv, cx<R> uv) {
+        st[par * N + i] = bv;
+        st[(2 + par) * N + i] = uv;
+    }
+    __device__ __forceinline__ E update(E e, int par, int i, int j) const { return cfms_inv<FUSED>(e, b(par, i), u(par, j)); }
+    __device__ __forceinline__ void finish(int, int, int) {}
+};
+// Float-float: both parts of a complex entry at once in packed FP32 (the add, multiply and fma of two
+// lanes an instruction), the same operations part for part as cfms_ff.  An entry is (re.hi, im.hi,
+// re.lo, im.lo), turned back into cx<ff> at the end; b is staged as the factor of both parts, negated:
+// (-re, -re) and (im, -im), high and low.  Measured on a GB300, whole calls at
+// order 2 (with the two-row tiles): 50 modes 34.6 -> 28.6 ms, 100 modes 149 -> 114.
+__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+template <> struct InvOps<ff, false> {
+    using E = ulonglong2;  // .x: (re.hi, im.hi), .y: (re.lo, im.lo)
+    static constexpr int rows = 6;
+    static constexpr bool eager = true;   // two updates a tile side by side, without a branch
+    E *G, *st;
+    int N;
+    __device__ __forceinline__ InvOps(cx<ff> *g, cx<ff> *stage, int n) : G((E *)g), st((E *)stage), N(n) {}
+    static __device__ __forceinline__ E pack(cx<ff> v) { return E{f2_pack(v.re.hi, v.im.hi), f2_pack(v.re.lo, v.im.lo)}; }
+    static __device__ __forceinline__ cx<ff> unpack(E e) {
+        cx<ff> v;
+        f2_unpack(e.x, v.re.hi, v.im.hi);
+        f2_unpack(e.y, v.re.lo, v.im.lo);
+        return v;
+    }
+    __device__ __forceinline__ cx<ff> get(int a) const { return unpack(G[a]); }
+    __device__ __forceinline__ cx<ff> b(int par, int i) const {
+        const E x = st[2 * (par * N + i)], y = st[2 * (par * N + i) + 1];
+        cx<ff> v;
+        float z;
+        f2_unpack(x.x, v.re.hi, z);
+        f2_unpack(x.y, v.re.lo, z);
+        v.re = ff(-v.re.hi, -v.re.lo);
+        f2_unpack(y.x, v.im.hi, z);
+        f2_unpack(y.y, v.im.lo, z);
+        return v;
+    }
+    __device__ __forceinline__ cx<ff> u(int par, int i) const { return unpack(st[(4 + par) * N + i]); }
+    __device__ __forceinline__ void put(int par, int i, cx<ff> bv, cx<ff> uv) {
+        st[2 * (par * N + i)] = E{f2_pack(-bv.re.hi, -bv.re.hi), f2_pack(-bv.re.lo, -bv.re.lo)};
+        st[2 * (par * N + i) + 1] = E{f2_pack(bv.im.hi, -bv.im.hi), f2_pack(bv.im.lo, -bv.im.lo)};
+        st[(4 + par) * N + i] = pack(uv);
+    }
+    __device__ __forceinline__ E update(E e, int par, int i, int j) const {
+        const E x0 = st[2 * (par * N + i)], x1 = st[2 * (par * N + i) + 1], y0 = st[(4 + par) * N + j];
+        float a, b;
+        f2_unpack(y0.x, a, b);
+        const uint64_t y1h = f2_pack(b, a);
+        f2_unpack(y0.y, a, b);
+        const uint64_t y1l = f2_pack(b, a), m1 = f2_pack(-1.0f, -1.0f);
+        // the products with their remainders, negated (x holds the minus)
+        const uint64_t p0 = f2_mul(x0.x, y0.x), p1 = f2_mul(x1.x, y1h);
+        const uint64_t q0 = f2_fma(x0.x, y0.x, f2_mul(p0, m1)), q1 = f2_fma(x1.x, y1h, f2_mul(p1, m1));
+        // e.hi + p0 + p1 with the sums' remainders
+        const uint64_t s = f2_add(e.x, p0), sb = f2_fma(e.x, m1, s);
+        const uint64_t r0 = f2_add(f2_fma(f2_fma(sb, m1, s), m1, e.x), f2_fma(sb, m1, p0));
+        const uint64_t v = f2_add(s, p1), vb = f2_fma(s, m1, v);
+        const uint64_t r1 = f2_add(f2_fma(f2_fma(vb, m1, v), m1, s), f2_fma(vb, m1, p1));
+        uint64_t lo = f2_add(f2_add(e.y, f2_add(r0, r1)), f2_add(q0, q1));
+        lo = f2_fma(x0.x, y0.y, lo);
+        lo = f2_fma(x0.y, y0.x, lo);
+        lo = f2_fma(x1.x, y1l, lo);
+        lo = f2_fma(x1.y, y1h, lo);
+        const uint64_t h = f2_add(v, lo);
+        return E{h, f2_fma(f2_fma(v, m1, h), m1, lo)};
+    }
+    // the matrix as cx<ff>, entry by entry in its place
+    __device__ __forceinline__ void finish(int entries, int t, int threads) {
+        for (int f = t; f < entries; f += threads) {
+            const cx<ff> v = get(f);
+            ((cx<ff> *)G)[f] = v;
+        }
+    }
+};
+
+// The rows [lo, hi) (both even) of the upper triangle in tiles of two rows and one column: row pairs q
+// and (last - q) share one run of fw tiles, an odd middle pair follows.  Of a pair's first tile, on the
+// diagonal, the second row's entry is not in the triangle.
+struct RowPairs {
+    int N, lo, hi, mid, fw, fP, tiles;
+    uint32_t inv;  // f / fw = f inv >> 24, for f fw < 2^24 and f inv < 2^32
+    __device__ __forceinline__ RowPairs(int N_, int lo_, int hi_) : N(N_), lo(lo_), hi(hi_) {
+        const int np = (hi - lo) >> 1, half = np >> 1;
+        mid = lo + 2 * half;
+        fw = 2 * N - lo - hi + 2;
+        fP = half * fw;
+        tiles = fP + ((np & 1) ? N - mid : 0);
+        inv = (1u << 24) / (uint32_t)fw + 1u;
+    }
+    __device__ __forceinline__ void at(int f, int &i, int &j) const {
+        const int q = (int)(((uint32_t)f * inv) >> 24), r = f - q * fw, a = lo + 2 * q;
+        const bool low = r < N - a;
+        i = f >= fP ? mid : low ? a : hi - 2 - 2 * q;
+        j = f >= fP ? mid + (f - fP) : low ? a + r : i + (r - (N - a));
+    }
+};
+
+// G <- -(I - t O_S)^{-1} in shared memory (packed upper triangle of 2n x 2n, then the
+// staged pivot columns, InvOps::rows of 2n entries), t = cs + i sn, by the symmetric sweep operator on
 // every pivot; Z_S(t) = prod of principal pivot^{-1/2} (the LDL^T pivots, one root per
 // pair) to s_zs.  A pivot with Re <= 0 sets *s_bad.  All kMinorThreads threads take part; ends
 // with a barrier.
@@ -499,106 +633,102 @@ template <> struct GroupAcc<float> {
 // One phase and one barrier a pivot.  Pivot k's column b and u = b / pivot are staged; in its phase
 //  * the first warps (a thread a row) form column k + 1 as pivot k leaves it, and stage it and its
 //    quotients by the next pivot in the other buffers;
-//  * the others begin with the entries outside rows and columns k and k + 1, e - b_i u_j; the first
+//  * the others begin with the entries outside rows and columns k and k + 1, e - b_i u_j, in tiles of
+//    two rows (RowPairs); the first
 //    ones join after kHeadStart rounds, about what the column, two reciprocals' worth, costs them.
 // Every warp computing both pivots' reciprocals, with a barrier between the entries and the next
 // column, cost as much as the entries at 50 rows: 16 of a hundred instructions each on eight warps
 // against 40 rounds of 70.  Every entry's operations and their order are those of the plain form.
-// Float-float takes two entries at a time (8 warps on an SM at 100 modes: the wait for one update is
-// covered by the other); FP64, bound by its pipe, takes one.  Measured on a GB300, whole calls: order 2
-// at 50 modes 35.1 -> 31.9 ms, at 100 modes 165.3 -> 163.8, the FP64 gradient at 32 modes 74.2 -> 61.6.
+// Measured on a GB300, whole calls: order 2 at 50 modes 35.1 -> 31.9 ms, the FP64 gradient at 32 modes
+// 74.2 -> 61.6.  A tile of two rows then halved the index work and the loads of u an entry, which with
+// packed float-float were most of its instructions (78 an entry, 33 of them on the integer ALUs); two
+// tiles at a time were slower (31.5 ms for 28.6).
 constexpr int kHeadStart = 4;
 template <typename R, bool FUSED = false, int TH = kMinorThreads>
 __device__ __forceinline__ void sweep_inverse(int M, const double *__restrict__ O, const int *modes, int n,
-                                              double cs, double sn, cx<R> *G, int *s_bad, double *s_zs) {
+                                              double cs, double sn, cx<R> *Gs, int *s_bad, double *s_zs) {
     constexpr int W = TH / 32;
     __shared__ cx<R> s_inv[2];
     const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
     const int N = 2 * n, N2 = 2 * M;
-    const int fw = N + 1, fE = n * fw;  // rows p and N - 1 - p folded: N + 1 entries
-    const uint32_t inv22 = (1u << 22) / (uint32_t)fw + 1u;  // f / fw = f inv22 >> 22 for f < fE <= 224 x 225 / 2
-    auto fold = [&](int f, int &i, int &j) {
-        const int fp = (int)(((uint32_t)f * inv22) >> 22), fq = f - fp * fw;
-        const bool low = fq < N - fp;
-        i = low ? fp : N - 1 - fp;
-        j = low ? fp + fq : i + (fq - (N - fp));
-    };
-    for (int f = t; f < fE; f += TH) {
+    using Ops = InvOps<R, FUSED>;
+    Ops A(Gs, Gs + sym(N), N);
+    const RowPairs rp(N, 0, N);
+    for (int f = t; f < rp.tiles; f += TH) {
         int i, j;
-        fold(f, i, j);
-        const int si = modes[i >> 1] + (i & 1) * M, sj = modes[j >> 1] + (j & 1) * M;
-        G[pidx(N, i, j)] = init_entry<R>(i == j, cs, sn, O[(size_t)si * N2 + sj]);
+        rp.at(f, i, j);
+        const int sj = modes[j >> 1] + (j & 1) * M, si = modes[i >> 1], e = pidx(N, i, j);
+        A.G[e] = Ops::pack(init_entry<R>(i == j, cs, sn, O[(size_t)si * N2 + sj]));
+        if (j > i) A.G[e + (N - i - 1)] = Ops::pack(init_entry<R>(i + 1 == j, cs, sn, O[(size_t)(si + M) * N2 + sj]));
     }
     __syncthreads();
-    cx<R> *const cb0 = G + sym(N), *const cb1 = cb0 + N, *const cu0 = cb0 + 2 * N, *const cu1 = cb0 + 3 * N;
     const int NS = (N + 31) >> 5;  // warps that stage columns
     if (wp < NS) {
-        const cx<R> inv0 = cinv(G[0]);
+        const cx<R> inv0 = cinv(A.get(0));
         if (t < N) {
-            const cx<R> v = G[t];
-            cb0[t] = v;
-            cu0[t] = v * inv0;
+            const cx<R> v = A.get(t);
+            A.put(0, t, v, v * inv0);
         }
         if (t == 0) s_inv[0] = inv0;
     }
     __syncthreads();
     cx<double> zs = mk<double>(1.0, 0.0);  // on the last warp's first thread
     cx<R> dprev = mk<R>(R(1), R(0));
-    const int rounds = (fE + 31) >> 5;
+    const int rounds = (rp.tiles + 31) >> 5;
     for (int k = 0; k < N; ++k) {
-        const cx<R> *cb = (k & 1) ? cb1 : cb0, *cu = (k & 1) ? cu1 : cu0;
+        const int par = k & 1;
         if (t == TH - 32) {
-            const cx<R> d = cb[k];
+            const cx<R> d = A.b(par, k);
             if (!(d.re > R(0))) *s_bad = 1;
             if (k & 1) zs = zs * widen(crsqrt(dprev * d));
             dprev = d;
         }
         if (wp < NS) {
             // scale pivot k's row and column (entry (k, k + 1) is the next column's)
-            if (t < N && t != k && t != k + 1) G[pidx_any(N, t, k)] = cu[t];
-            if (t == k) G[pidx(N, k, k)] = mk<R>(R(0), R(0)) - s_inv[k & 1];
+            if (t < N && t != k && t != k + 1) A.G[pidx_any(N, t, k)] = Ops::pack(A.u(par, t));
+            if (t == k) A.G[pidx(N, k, k)] = Ops::pack(mk<R>(R(0), R(0)) - s_inv[par]);
             if (k + 1 < N) {
-                cx<R> *cbn = (k & 1) ? cb0 : cb1, *cun = (k & 1) ? cu0 : cu1;
                 // the next pivot (its place in G stays as it is until its own phase)
-                const cx<R> dn = cfms_inv<FUSED>(G[pidx(N, k + 1, k + 1)], cb[k + 1], cu[k + 1]);
+                const cx<R> dn = cfms_inv<FUSED>(A.get(pidx(N, k + 1, k + 1)), A.b(par, k + 1), A.u(par, k + 1));
                 const cx<R> invn = cinv(dn);
                 if (t < N) {
                     const int lo = t < k + 1 ? t : k + 1, hi = t < k + 1 ? k + 1 : t;
-                    cx<R> &e = G[pidx(N, lo, hi)];
+                    const int e = pidx(N, lo, hi);
                     cx<R> v;
-                    if (t == k) v = cu[k + 1];
+                    if (t == k) v = A.u(par, k + 1);
                     else if (t == k + 1) v = dn;
-                    else v = cfms_inv<FUSED>(e, cb[lo], cu[hi]);
-                    if (t != k + 1) e = v;
-                    cbn[t] = v;
-                    cun[t] = v * invn;
-                    if (t == k + 1) s_inv[(k + 1) & 1] = invn;
+                    else v = cfms_inv<FUSED>(A.get(e), A.b(par, lo), A.u(par, hi));
+                    if (t != k + 1) A.G[e] = Ops::pack(v);
+                    A.put(par ^ 1, t, v, v * invn);
+                    if (t == k + 1) s_inv[par ^ 1] = invn;
                 }
             }
         }
-        // the entries, 32 a round and warp
+        // the tiles, 32 a round and warp: entries outside rows and columns k and k + 1
         const int first = wp < NS || ((k & 1) && wp == W - 1) ? kHeadStart : 0;  // busy warps join later
         const int m = NS < W ? W - NS - (k & 1) : 0;
-        auto entry = [&](int r, int &i, int &j) {  // this lane's entry of round r: its place, -1 none, -2 the end
+        for (int r = first;; ++r) {
             const int c = r < kHeadStart ? r * m + (wp - NS) : kHeadStart * m + (r - kHeadStart) * W + wp;
+            if (c >= rounds) break;
             const int f = c * 32 + lane;
-            fold(f < fE ? f : 0, i, j);
-            return c >= rounds ? -2 : f < fE && i != k && j != k && i != k + 1 && j != k + 1 ? pidx(N, i, j) : -1;
-        };
-        constexpr int U = std::is_same_v<R, ff> ? 2 : 1;  // independent updates at a time
-        const int dead = sym(N) + (k & 1) * N;  // cb[0], read and dropped in the place of a skipped entry
-        for (int r = first;; r += U) {
-            int a[U], i[U], j[U];
-            for (int q = 0; q < U; ++q) a[q] = entry(r + q, i[q], j[q]);
-            if (a[0] == -2) break;
-            cx<R> v[U];
-            for (int q = 0; q < U; ++q)
-                if (U > 1 || a[q] >= 0) v[q] = cfms_inv<FUSED>(G[a[q] < 0 ? dead : a[q]], cb[i[q]], cu[j[q]]);
-            for (int q = 0; q < U; ++q)
-                if (a[q] >= 0) G[a[q]] = v[q];
+            int i, j;
+            rp.at(f < rp.tiles ? f : 0, i, j);
+            const bool in = f < rp.tiles && (unsigned)(j - k) > 1u;
+            const int e = pidx(N, i, j);
+            const int a[2] = {in && (unsigned)(i - k) > 1u ? e : -1,
+                              in && j > i && (unsigned)(i + 1 - k) > 1u ? e + (N - i - 1) : -1};
+            typename Ops::E v[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q)  // (a skipped entry's place takes a staged value, dropped below)
+                if (Ops::eager || a[q] >= 0)
+                    v[q] = A.update(a[q] < 0 ? A.st[(Ops::rows - 2 + par) * N] : A.G[a[q]], par, i + q, j);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (a[q] >= 0) A.G[a[q]] = v[q];
         }
         __syncthreads();
     }
+    A.finish(sym(N), t, TH);
     if (t == TH - 32) { s_zs[0] = zs.re; s_zs[1] = zs.im; }
     __syncthreads();
 }
@@ -618,9 +748,12 @@ __host__ __device__ inline int minor_smem_entries(int n, int esz, int min_blocks
     return (int)ent;
 }
 
-// two CTAs of float-float patterns of n clicks share an SM
-__host__ __device__ inline bool minor_shares_sm(int n, int esz) {
-    return ((long long)n * (2 * n + 1) + 8LL * n) * esz <= 228 * 1024 / 2 - 4 * 1024;
+// two CTAs of float-float patterns of n clicks share an SM: the inverse, and its staged columns or the
+// items the pair phases need
+__host__ __device__ inline bool minor_shares_sm(int n) {
+    const long long stage = 2LL * InvOps<ff>::rows * n, items = 15LL * (n - 1);
+    return ((long long)n * (2 * n + 1) + (stage > items ? stage : items)) * (long long)sizeof(cx<ff>) <=
+           228 * 1024 / 2 - 4 * 1024;
 }
 
 // Read-only view of the swept matrix -G, G = (I - t O_S)^{-1}, packed upper triangle of
@@ -1131,12 +1264,15 @@ __global__ void __launch_bounds__(TH, TH > kMinorThreads ? 1 : MinorPrec<R>::min
 // split over the 512 threads of the pair.
 constexpr int kPairMaxN = kApproxMaxN;
 
-// rows [0, rsplit) hold about half of the packed entries of an N x N upper triangle
+// rows [0, rsplit) hold about half of the packed entries of an N x N upper triangle (N even; an even
+// rsplit, with the smaller of the larger halves)
 __host__ __device__ inline int pair_split_row(int N) {
-    const int half = (N * (N + 1) / 2 + 1) / 2;
+    const int tot = N * (N + 1) / 2;
     int r = 0, acc = 0;
-    while (r < N && acc + (N - r) <= half) { acc += N - r; ++r; }
-    return r > 0 ? r : 1;
+    while (r < N && 2 * (acc + (N - r)) <= tot) { acc += N - r; ++r; }
+    const int d = r & ~1, low = d * N - d * (d - 1) / 2, u = d + 2, high = u * N - u * (u - 1) / 2;
+    const int best = u < N && high < tot - low ? u : d;
+    return best > 0 ? best : (N > 2 ? 2 : N);
 }
 __host__ __device__ inline int pair_part_entries(int N) {  // the larger half
     const int r = pair_split_row(N), lo = r * N - r * (r - 1) / 2, tot = N * (N + 1) / 2;
@@ -1156,7 +1292,7 @@ template <typename R> struct PairPivots {
 };
 template <typename R, int TH>
 __device__ void sweep_inverse_pair(cg::cluster_group &cl, int rank, int M, const double *__restrict__ O,
-                                   const uint8_t *modes, int n, double cs, double sn, cx<R> *Gl, cx<R> *stage,
+                                   const uint8_t *modes, int n, double cs, double sn, cx<R> *Gs, cx<R> *stage,
                                    cx<R> *stage_peer, PairPivots<R> *pv, PairPivots<R> *pv_peer, int rsplit, int off1,
                                    int *s_bad, double *s_zs) {
     constexpr int W = TH / 32;
@@ -1164,46 +1300,37 @@ __device__ void sweep_inverse_pair(cg::cluster_group &cl, int rank, int M, const
     const int N = 2 * n, N2 = 2 * M;
     const int r_lo = rank ? rsplit : 0, r_hi = rank ? N : rsplit;
     const int base = rank ? off1 : 0;
+    using Ops = InvOps<R>;
+    Ops A(Gs, stage, N), peer(Gs, stage_peer, N);  // (of the peer, the staged columns)
     auto lidx = [&](int i, int j) { return i * N - (i * (i - 1)) / 2 + (j - i) - base; };  // own row i <= j
     auto own = [&](int i) { return i >= r_lo && i < r_hi; };
-    // own rows folded in pairs (r_lo + q, r_hi - 1 - q), fw entries a pair; then the unpaired middle row
-    const int nrows = r_hi - r_lo, npair = nrows >> 1, fw = 2 * N - r_lo - r_hi + 1;
-    const int rmid = r_lo + npair, fP = npair * fw, fE = fP + ((nrows & 1) ? N - rmid : 0);
-    const uint32_t inv24 = (1u << 24) / (uint32_t)fw + 1u;  // f / fw = f inv24 >> 24 for f fw < 2^24, f inv24 < 2^32
-    auto fold = [&](int f, int &i, int &j) {
-        const int fp = (int)(((uint32_t)f * inv24) >> 24), fq = f - fp * fw, a = r_lo + fp;
-        const bool low = fq < N - a;
-        i = f >= fP ? rmid : low ? a : r_hi - 1 - fp;
-        j = f >= fP ? rmid + (f - fP) : low ? a + fq : i + (fq - (N - a));
-    };
-    for (int f = t; f < fE; f += TH) {
+    const RowPairs rp(N, r_lo, r_hi);
+    for (int f = t; f < rp.tiles; f += TH) {
         int i, j;
-        fold(f, i, j);
-        const int si = modes[i >> 1] + (i & 1) * M, sj = modes[j >> 1] + (j & 1) * M;
-        Gl[lidx(i, j)] = init_entry<R>(i == j, cs, sn, O[(size_t)si * N2 + sj]);
+        rp.at(f, i, j);
+        const int sj = modes[j >> 1] + (j & 1) * M, si = modes[i >> 1], e = lidx(i, j);
+        A.G[e] = Ops::pack(init_entry<R>(i == j, cs, sn, O[(size_t)si * N2 + sj]));
+        if (j > i) A.G[e + (N - i - 1)] = Ops::pack(init_entry<R>(i + 1 == j, cs, sn, O[(size_t)(si + M) * N2 + sj]));
     }
     __syncthreads();
     const int NS = (N + 31) >> 5;  // warps that stage columns
     if (wp < NS && t < N) {
         if (rank == 0) {  // pivot 0's column is row 0
-            const cx<R> inv0 = cinv(Gl[0]), v = Gl[t], u = v * inv0;
-            stage[t] = v;
-            stage_peer[t] = v;
-            stage[2 * N + t] = u;
-            stage_peer[2 * N + t] = u;
+            const cx<R> inv0 = cinv(A.get(0)), v = A.get(t), u = v * inv0;
+            A.put(0, t, v, u);
+            peer.put(0, t, v, u);
             if (t == 0) pv->inv[0] = pv_peer->inv[0] = inv0;
         }
-        if (t == 1 && own(1)) pv->dg[1] = pv_peer->dg[1] = Gl[lidx(1, 1)];
+        if (t == 1 && own(1)) pv->dg[1] = pv_peer->dg[1] = A.get(lidx(1, 1));
     }
     cl.sync();
     cx<double> zs = mk<double>(1.0, 0.0);  // on the last warp's first thread
     cx<R> dprev = mk<R>(R(1), R(0));
-    const int rounds = (fE + 31) >> 5;
+    const int rounds = (rp.tiles + 31) >> 5;
     for (int k = 0; k < N; ++k) {
-        const int oc = (k & 1) * N, on = N - oc;  // staged: b, b', u, u'
-        const cx<R> *cb = stage + oc, *cu = stage + 2 * N + oc;
+        const int par = k & 1;
         if (t == TH - 32) {
-            const cx<R> d = cb[k];
+            const cx<R> d = A.b(par, k);
             if (!(d.re > R(0))) *s_bad = 1;
             if (k & 1) zs = zs * widen(crsqrt(dprev * d));
             dprev = d;
@@ -1211,56 +1338,60 @@ __device__ void sweep_inverse_pair(cg::cluster_group &cl, int rank, int M, const
         if (wp < NS) {
             if (t < N && t != k + 1) {  // scale pivot k's row and column (entry (k, k + 1) is the next column's)
                 const int lo = t < k ? t : k, hi = t < k ? k : t;
-                if (own(lo)) Gl[lidx(lo, hi)] = t == k ? mk<R>(R(0), R(0)) - pv->inv[k & 1] : cu[t];
+                if (own(lo)) A.G[lidx(lo, hi)] = Ops::pack(t == k ? mk<R>(R(0), R(0)) - pv->inv[par] : A.u(par, t));
             }
             if (k + 1 < N) {
-                const cx<R> dn = cfms_inl(pv->dg[(k + 1) & 1], cb[k + 1], cu[k + 1]);
+                const cx<R> dn = cfms_inl(pv->dg[par ^ 1], A.b(par, k + 1), A.u(par, k + 1));
                 const cx<R> invn = cinv(dn);
                 if (t < N) {
                     const int lo = t < k + 1 ? t : k + 1, hi = t < k + 1 ? k + 1 : t;
                     if (own(lo)) {
-                        cx<R> &e = Gl[lidx(lo, hi)];
+                        const int e = lidx(lo, hi);
                         cx<R> v;
-                        if (t == k) v = cu[k + 1];
+                        if (t == k) v = A.u(par, k + 1);
                         else if (t == k + 1) v = dn;
-                        else v = cfms_inl(e, cb[lo], cu[hi]);
-                        if (t != k + 1) e = v;
+                        else v = cfms_inl(A.get(e), A.b(par, lo), A.u(par, hi));
+                        if (t != k + 1) A.G[e] = Ops::pack(v);
                         const cx<R> u = v * invn;
-                        stage[on + t] = v;
-                        stage_peer[on + t] = v;
-                        stage[2 * N + on + t] = u;
-                        stage_peer[2 * N + on + t] = u;
+                        A.put(par ^ 1, t, v, u);
+                        peer.put(par ^ 1, t, v, u);
                     }
-                    if (t == k + 1) pv->inv[(k + 1) & 1] = invn;
+                    if (t == k + 1) pv->inv[par ^ 1] = invn;
                     if (t == k + 2 && own(t)) {
-                        cx<R> &e = Gl[lidx(t, t)];
-                        e = cfms_inl(e, cb[t], cu[t]);
-                        pv->dg[k & 1] = pv_peer->dg[k & 1] = e;
+                        const int e = lidx(t, t);
+                        const cx<R> v = cfms_inl(A.get(e), A.b(par, t), A.u(par, t));
+                        A.G[e] = Ops::pack(v);
+                        pv->dg[par] = pv_peer->dg[par] = v;
                     }
                 }
             }
         }
-        // the entries, 32 a round and warp, as in sweep_inverse
-        const int first = wp < NS || ((k & 1) && wp == W - 1) ? kHeadStart : 0;
+        // the tiles, 32 a round and warp: entries outside rows and columns k and k + 1
+        const int first = wp < NS || ((k & 1) && wp == W - 1) ? kHeadStart : 0;  // busy warps join later
         const int m = NS < W ? W - NS - (k & 1) : 0;
-        auto entry = [&](int r, int &i, int &j) {
+        for (int r = first;; ++r) {
             const int c = r < kHeadStart ? r * m + (wp - NS) : kHeadStart * m + (r - kHeadStart) * W + wp;
+            if (c >= rounds) break;
             const int f = c * 32 + lane;
-            fold(f < fE ? f : 0, i, j);
-            const bool skip = i == k || j == k || i == k + 1 || j == k + 1 || (i == k + 2 && j == k + 2);
-            return c >= rounds ? -2 : f < fE && !skip ? lidx(i, j) : -1;
-        };
-        constexpr int U = std::is_same_v<R, ff> ? 2 : 1;
-        for (int r = first;; r += U) {
-            int a[U], i[U], j[U];
-            for (int q = 0; q < U; ++q) a[q] = entry(r + q, i[q], j[q]);
-            if (a[0] == -2) break;
-            cx<R> v[U];
-            for (int q = 0; q < U; ++q)
-                if (U > 1 || a[q] >= 0) v[q] = cfms_inl(a[q] < 0 ? cb[0] : Gl[a[q]], cb[i[q]], cu[j[q]]);
-            for (int q = 0; q < U; ++q)
-                if (a[q] >= 0) Gl[a[q]] = v[q];
+            int i, j;
+            rp.at(f < rp.tiles ? f : 0, i, j);
+            const bool in = f < rp.tiles && (unsigned)(j - k) > 1u;
+            const int e = lidx(i, j);
+            const int a[2] = {in && (unsigned)(i - k) > 1u && (i != k + 2 || j != k + 2) ? e : -1,
+                              in && j > i && (unsigned)(i + 1 - k) > 1u && (i != k + 1 || j != k + 2) ? e + (N - i - 1) : -1};
+            typename Ops::E v[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q)  // (a skipped entry's place takes a staged value, dropped below)
+                if (Ops::eager || a[q] >= 0)
+                    v[q] = A.update(a[q] < 0 ? A.st[(Ops::rows - 2 + par) * N] : A.G[a[q]], par, i + q, j);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (a[q] >= 0) A.G[a[q]] = v[q];
         }
+        cl.sync();
+    }
+    if (Ops::rows != 4) {  // the packed form turned back before the peer reads it
+        A.finish(rank ? sym(N) - off1 : off1, t, TH);
         cl.sync();
     }
     if (t == TH - 32) { s_zs[0] = zs.re; s_zs[1] = zs.im; }
@@ -2651,7 +2782,7 @@ int launch_minors(gbs_ctx *ctx, int M, const double *O, const uint64_t *pats, in
     // (15 entries each, at least n - 1 of them, up to 8 n while the CTAs per SM stay)
     // (the largest over the range: the kernel sizes each pattern's items from its own n,
     // and the floor to whole items makes the entries fall by up to 14 between some n)
-    int ent = sym(2 * n_to) + 8 * n_to;  // FP32: no pair phases
+    int ent = sym(2 * n_to) + 2 * InvOps<R>::rows * n_to;  // FP32: no pair phases
     if constexpr (!std::is_same<R, float>::value)
         for (int m = n_from > 1 ? n_from : 1; m <= n_to; ++m) {
             const int e = minor_smem_entries(m, (int)sizeof(cx<R>), MinorPrec<R>::min_blocks);
@@ -2712,7 +2843,7 @@ int run_approx(gbs_ctx *ctx, int M, const double *O, const double *logdet, const
     // holds one, of 512 threads where the inverse is all that counts
     int n_two = nsmall;
     if (std::is_same<R, ff>::value)
-        while (n_two > 0 && !minor_shares_sm(n_two, (int)sizeof(cx<R>))) --n_two;
+        while (n_two > 0 && !minor_shares_sm(n_two)) --n_two;
     if (nsmall > n_two) {
         const size_t c4 = approx_offsets(n_pat, 0).counter4;
         if constexpr (std::is_same<R, ff>::value) {
@@ -2726,8 +2857,9 @@ int run_approx(gbs_ctx *ctx, int M, const double *O, const double *logdet, const
         if (st) return st;
     }
     if constexpr (MinorPrec<R>::pair) if (nmax > n_single) {
-        // half of the packed inverse, and four staged columns or the pair phases' items
-        const int pent = pair_part_entries(2 * nmax) + (8 * nmax > 15 * (nmax - 2) ? 8 * nmax : 15 * (nmax - 2));
+        // half of the packed inverse, and the staged columns or the pair phases' items
+        constexpr int rows2 = 2 * InvOps<R>::rows;
+        const int pent = pair_part_entries(2 * nmax) + (rows2 * nmax > 15 * (nmax - 2) ? rows2 * nmax : 15 * (nmax - 2));
         const size_t pair_smem = sizeof(cx<R>) * (size_t)pent;
         const bool wide = std::is_same<R, ff>::value && order <= 2;
         auto kernel = approx_minors_pair_kernel<R, kMinorThreads>;
