@@ -56,8 +56,10 @@ typedef enum {
 typedef enum {
     GBS_FP64 = 0,        /* every factorisation and sum in FP64 */
     GBS_FP32_SPLIT = 1,  /* subset factorisations in FP32; signed sum compensated, FP64 result */
-    GBS_DD = 2,          /* double-double (~106-bit) factorisations and sum, on the FP64 pipes:
-                            for patterns whose signed sum cancels beyond FP64 (kappa u64 >~ 1e-10) */
+    GBS_DD = 2,          /* double-double (~106-bit) class factorisations and sum: for patterns whose
+                            signed sum cancels beyond FP64 (kappa u64 >~ 1e-10).  110-bit software
+                            floating point on the integer pipes, double-double itself on the FP64
+                            pipes where kappa exceeds 1e22 */
     GBS_FX = 3,          /* exact sum only: 128-bit fixed-point (Q16.112) factorisations on the
                             integer pipes, double-double prefactors and sum; accuracy as GBS_DD
                             (~2^-100 per term) at a fraction of its cost.  Needs every pivot

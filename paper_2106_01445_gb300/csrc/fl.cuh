@@ -36,7 +36,6 @@ constexpr int32_t kLimbMask = 0x3fffffff;
 
 __device__ __forceinline__ int64_t fl_mw(int32_t a, int32_t b) { return (int64_t)a * (int64_t)b; }
 
-__device__ __forceinline__ fl fl_zero() { return fl{{0, 0, 0, 0}}; }
 
 // Q16.112 -> scale 114 (|x| < 128)
 __device__ __forceinline__ fl fl_from_fx(const fx &a) {

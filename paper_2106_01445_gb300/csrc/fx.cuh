@@ -3,7 +3,7 @@
 //
 // Used for the Schur updates of the exact sweep, whose entries are bounded: A = I - O
 // = sigma_Q^{-1} <= 2 I, so every Schur complement of A has entries in [-2, 2]; with
-// pivot determinants >= 2^-8 (checked, see fx_pivot_bad) the inverse pivots, the rows
+// pivot determinants >= 2^-8 (checked, see fl_pivot_bad) the inverse pivots, the rows
 // W = B P^{-1} and every intermediate of c - w0 b0 - w1 b1 stay below 2^15.  Products
 // are truncated to 2^-112 (partial products below bit 96 are dropped, error < 2^-13
 // of the last place); sums are exact.
@@ -135,36 +135,7 @@ __device__ __forceinline__ fx fx_mul_su(const fx &a, const fx &b) {
     fx_sub_masked(p4, p5, p6, p7, b, fx_sign_mask(a));
     return fx_shift_out(p3, p4, p5, p6, p7);
 }
-__device__ __forceinline__ fx fx_abs(const fx &a) {
-    const uint32_t m = fx_sign_mask(a);
-    fx x;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) x.w[k] = a.w[k] ^ m;
-    fx r;
-    asm("sub.cc.u32 %0, %4, %8;\n\t"
-        "subc.cc.u32 %1, %5, %8;\n\t"
-        "subc.cc.u32 %2, %6, %8;\n\t"
-        "subc.u32 %3, %7, %8;"
-        : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3])
-        : "r"(x.w[0]), "r"(x.w[1]), "r"(x.w[2]), "r"(x.w[3]), "r"(m));
-    return r;
-}
-// a + k 2^-16 for a small integer k (top limb only: no carry below)
-__device__ __forceinline__ fx fx_add_top(const fx &a, int k) {
-    fx r = a;
-    r.w[3] = (uint32_t)((int32_t)a.w[3] + k);
-    return r;
-}
 __device__ __forceinline__ fx &operator*=(fx &a, const fx &b) { return a = a * b; }
-// a / 2 (arithmetic shift)
-__device__ __forceinline__ fx fx_half(const fx &a) {
-    fx r;
-    r.w[0] = __funnelshift_r(a.w[0], a.w[1], 1);
-    r.w[1] = __funnelshift_r(a.w[1], a.w[2], 1);
-    r.w[2] = __funnelshift_r(a.w[2], a.w[3], 1);
-    r.w[3] = (uint32_t)((int32_t)a.w[3] >> 1);
-    return r;
-}
 
 __device__ __forceinline__ fx fx_from_i128(__int128 v) {
     fx r;
@@ -173,11 +144,6 @@ __device__ __forceinline__ fx fx_from_i128(__int128 v) {
     r.w[2] = (uint32_t)(v >> 64);
     r.w[3] = (uint32_t)(v >> 96);
     return r;
-}
-__device__ __forceinline__ __int128 fx_to_i128(const fx &a) {
-    const unsigned __int128 u = (unsigned __int128)a.w[0] | ((unsigned __int128)a.w[1] << 32) |
-                                ((unsigned __int128)a.w[2] << 64) | ((unsigned __int128)a.w[3] << 96);
-    return (__int128)u;
 }
 // exact for |d| < 2^15 down to 2^-112 (lower bits truncated toward zero); zero outside
 __device__ __forceinline__ fx fx_from_double(double d) {
@@ -210,16 +176,6 @@ __device__ __forceinline__ dd fx_to_dd(const fx &a) {
     return dd(s.hi * 0x1p-48, s.lo * 0x1p-48);
 }
 
-// pivot check: 0 fine, 1 not positive, 2 below the fixed-point range (det < 2^-8)
-__device__ __forceinline__ int fx_pivot_bad(const fx &det) {
-    if (!fx_positive(det)) return 1;
-    return (int32_t)det.w[3] < 256 ? 2 : 0;
-}
-// the same for a pivot block given by p00 and det: both positive, det >= 2^-8
-__device__ __forceinline__ int fx_chol_bad(const fx &p00, const fx &det) {
-    if (!fx_positive(p00)) return 1;
-    return fx_pivot_bad(det);
-}
 
 // x^{-1/2} in Q16.112 for a packed x with ulp 2^-(127 - h0) (h0 = 15: Q16.112; h0 = 13: ulp
 // 2^-114) in [2^-11, 2^11); pivots lie in [2^-9, 25].
@@ -275,11 +231,6 @@ static __device__ __noinline__ fx fx_rsqrt_at(fx x, int h0) {
            fx{{(uint32_t)dlt, (uint32_t)((unsigned long long)dlt >> 32), ext, ext}};
 }
 __device__ __forceinline__ fx fx_rsqrt(const fx &x) { return fx_rsqrt_at(x, 15); }
-// det of the SPD 2x2 block [[p00, p01], [p01, p11]]
-__device__ __forceinline__ fx fx_det2(const fx &p00, const fx &p01, const fx &p11) {
-    const fx a = fx_abs(p01);
-    return fx_mul_uu(p00, p11) - fx_mul_uu(a, a);
-}
 
 // Symmetric form of the 2x2 block elimination used by the fixed-point sweeps.  With
 // the pivot block P = R R^T (R lower triangular, 1/r00 = a, r10, 1/r11 = b), the
@@ -288,14 +239,6 @@ __device__ __forceinline__ fx fx_det2(const fx &p00, const fx &p01, const fx &p1
 // (two products side by side), and |u_ik| <= sqrt(c_ii).  a = p00^{-1/2} and rs = det^{-1/2}
 // are independent, so the two rsqrts need not wait for each other: b = rs sqrt(p00) = rs p00 a.
 
-// ---- prefactors as mantissa x 2^e, and exponent-aligned sums -------------------------
-// The breadth-first prefactors (products of up to seven det^{-1/2} in [1/2, 16]) leave
-// the fixed-point range, so they are kept as m 2^e with m in [1, 2).
-struct __align__(16) fxe {
-    fx m;
-    int e;
-};
-__device__ __forceinline__ fxe fxe_one() { return fxe{fx_one(), 0}; }
 // a >> k for 0 <= k <= 31 (arithmetic)
 __device__ __forceinline__ fx fx_shr_small(const fx &a, int k) {
     fx r;
@@ -303,15 +246,6 @@ __device__ __forceinline__ fx fx_shr_small(const fx &a, int k) {
     r.w[1] = __funnelshift_r(a.w[1], a.w[2], k);
     r.w[2] = __funnelshift_r(a.w[2], a.w[3], k);
     r.w[3] = (uint32_t)((int32_t)a.w[3] >> k);
-    return r;
-}
-// a << k for 0 <= k <= 31
-__device__ __forceinline__ fx fx_shl_small(const fx &a, int k) {
-    fx r;
-    r.w[3] = __funnelshift_l(a.w[2], a.w[3], k);
-    r.w[2] = __funnelshift_l(a.w[1], a.w[2], k);
-    r.w[1] = __funnelshift_l(a.w[0], a.w[1], k);
-    r.w[0] = a.w[0] << k;
     return r;
 }
 // a >> s for any s >= 0 (arithmetic; s >= 127 leaves the sign)
@@ -325,21 +259,6 @@ __device__ __forceinline__ fx fx_shr(const fx &a, int s) {
     const uint32_t w2 = q == 0 ? a.w[2] : q == 1 ? a.w[3] : sg;
     const uint32_t w3 = q == 0 ? a.w[3] : sg;
     return fx_shr_small(fx{{w0, w1, w2, w3}}, b);
-}
-// m r 2^e renormalised, for r in (0, 32)
-__device__ __forceinline__ fxe fxe_mul(const fxe &a, const fx &r) {
-    const fx p = fx_mul_uu(a.m, r);  // (0, 64)
-    const int k = (31 - __clz((int)p.w[3])) - 16;  // floor(log2 p), in [-2, 5] for p >= 1/4
-    fxe o;
-    o.m = k >= 0 ? fx_shr_small(p, k) : fx_shl_small(p, -k);
-    o.e = a.e + k;
-    return o;
-}
-// m 2^e as a double-double
-__device__ __forceinline__ dd fxe_to_dd(const fxe &a) {
-    const dd v = fx_to_dd(a.m);
-    const double s = ldexp(1.0, a.e);
-    return dd(v.hi * s, v.lo * s);
 }
 __device__ __forceinline__ fx fx_shfl_xor(const fx &a, int mask) {
     fx r;

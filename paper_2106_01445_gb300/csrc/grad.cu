@@ -6,7 +6,8 @@
 //     dT = tr(Gbar dA_S),  Gbar = sum_Z (-1)^{n-|Z|} (-1/2) tau_Z A_Z^{-1},
 //     dL/dsigma_Q = -1/2 (sum_p w_p) A - A H A,   H = sum_p (w_p / T_p) embed(Gbar_p).
 // Gbar and T cancel together by the condition number kappa of the signed sum
-// (1e14..1e19 on improbable patterns), so the whole computation is double-double;
+// (1e14..1e19 on improbable patterns), so the whole computation is in 110-bit software floating
+// point (double-double for the patterns that cancel by more than 1e24);
 // after the division by T the result is an ordinary FP64 number.  Gbar = dT/dA_S is
 // computed in reverse mode through the same include/exclude Schur recursion that
 // evaluates T (O(2^n) work instead of a factorisation and inverse per subset); one
