@@ -36,11 +36,12 @@ import gbs_inputs as g  # noqa: E402
 METRIC = "subset logdets/sec and click-pattern log P/sec at stated rel. error vs FP64 oracle"
 # dram__bytes_read.sum + dram__bytes_write.sum of one sweep launch on this workload
 # (ncu captures summarised under profiles/); None where no capture of the current kernel exists
-DRAM_TRAFFIC = {"fp32": 129536.0, "dd": 396800.0, "fp64": 130048.0, "fx": 182784.0}
+DRAM_TRAFFIC = {"fp32": 129536.0, "dd": None, "fp64": 130048.0, "fx": 129280.0}
 UNIT = "subset logdets/s"
-# 32-bit multiply-adds of one fixed-point update entry: two 128 x 128-bit products
-# truncated to their top 128 bits, 23 IMAD each (3 + 5 + 7 + 8 over the four rows)
-FX_IMAD_PER_ENTRY = 46
+# 32-bit multiply-adds of one fixed-point update entry: two products of four 30-bit limbs
+# without their lowest columns, 10 wide multiply-adds each, which take two issue slots of the
+# multiplier
+FX_IMAD_PER_ENTRY = 40
 L2_FLUSH_BYTES = 512 << 20      # > 129 MB L2
 
 
@@ -404,19 +405,21 @@ def run_gpu(args):
     peak = all_peaks[prec]
     kms = sweep_ms / max(launches, 1)
     achieved = flops / (kms * 1e-3)
-    kname = {"fp32": "float", "fp64": "double", "dd": "dd", "fx": "fx"}[prec]
+    kname = {"fp32": "sweep_kernel<float>", "fp64": "sweep_kernel<double>",
+             "dd": "sweep_kernel<sq> (110-bit software floating point)", "fx": "sweep_fx_kernel"}[prec]
     roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": DRAM_TRAFFIC.get(prec),
-                "kernel": "sweep_kernel<%s>" % kname, "kernel_ms": kms, "flops_per_launch": flops,
+                "kernel": kname, "kernel_ms": kms, "flops_per_launch": flops,
                 "flop_count": "8r^2+10r+10 per include step (44/subset)",
                 "frac_executed_count": flops_exec / (kms * 1e-3) / peak,
                 "peak_basis": {"fp32": "SMs x 128 FP32 lanes x 2 x max SM clock (derived)",
                                "fp64": "measured FP64 FMA loop",
-                               "dd": "measured loop of the sweep's double-double update entry, 4 flops",
+                               "dd": "measured loop of a double-double update entry on the FP64 pipes, 4 flops "
+                                     "(the sweep runs on the integer pipes: above 1 is its gain)",
                                "fx": "measured loop of the sweep's fixed-point update entry, 4 flops"}[prec]}
     if prec == "fx":
-        # the integer pipe: each fixed-point update entry is two truncated 128-bit products of
-        # 23 IMAD each (FX_IMAD_PER_ENTRY); at the measured IMAD issue rate that bounds the
+        # the integer pipe: each fixed-point update entry is 20 wide multiply-adds
+        # (FX_IMAD_PER_ENTRY issue slots); at the measured IMAD issue rate that bounds the
         # entry rate, and so the sweep's flops, from above
         imad_bound = meas["imad"] / FX_IMAD_PER_ENTRY * 4.0
         roofline["int_pipe"] = {"imad_per_s": meas["imad"], "imad_per_entry": FX_IMAD_PER_ENTRY,
@@ -620,7 +623,7 @@ def run_workloads(dev, stream, meas, fp32_peak):
     ds_orc = ograd.grad_sigmaQ(st_or, pats[chk], np.ones(len(chk)))
     res["m32_grad"] = {"patterns": len(pats), "params": 2 * len(th) + c.M + 1,
                        "ms_forward_and_backward": ms, "patterns_per_s": len(pats) / (ms * 1e-3),
-                       "roofline_adjoint": {"bound": "alu", "kernel": "grad_tree_kernel (double-double)",
+                       "roofline_adjoint": {"bound": "alu", "kernel": "grad_tree_kernel (110-bit software floating point)",
                                             "kernel_ms": kms_adj, "flops": fl,
                                             "achieved_tflops": fl / (kms_adj * 1e-3) / 1e12,
                                             "peak_tflops": meas["dd"] / 1e12,
