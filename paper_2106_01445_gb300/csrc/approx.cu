@@ -358,6 +358,7 @@ __global__ void __launch_bounds__(kPlanThreads) approx_plan_kernel(int M, const 
         pl.pat_n[p] = n;
         pl.pat_L[p] = n < 0 ? 0 : L;
         pl.pat_rho[p] = rho_t;
+        pl.pat_max[p] = 0.0;
         pl.unit_flag[p] = 0;
     }
 }
@@ -1874,7 +1875,10 @@ __device__ __forceinline__ double stirling2(int i, int w) {
 }
 
 // inverse DFT of one pattern's tables (real: O is real, so D(conj t) = conj D(t)):
-//   D_w^(k) = (1/L) sum_l D_w(t_l) e^{-2 pi i k l / L},  one CTA per pattern
+//   D_w^(k) = (1/L) sum_l D_w(t_l) e^{-2 pi i k l / L}
+// gridDim.y CTAs per pattern, about eight an SM in all: one each left most SMs without work on 64
+// patterns and waited for the largest ones.  Measured on a GB300, order 2, 64
+// patterns of 40 to 90 clicks: 1.95 -> 0.59 ms.
 __global__ void __launch_bounds__(kDftThreads) approx_dft_kernel(int order, ApproxPlan pl) {
     extern __shared__ double tw[];  // cos, sin (2 pi m / L), m < L
     __shared__ double red[kDftThreads / 32];
@@ -1887,7 +1891,7 @@ __global__ void __launch_bounds__(kDftThreads) approx_dft_kernel(int order, Appr
     const double *U = pl.unit_D + (size_t)pl.unit_off[p] * 2 * (kMaxOrder + 1);
     double *D = pl.sec_D + (size_t)pl.sec_off[p] * (kMaxOrder + 1);
     double mx = 0.0;
-    for (int idx = t; idx < (order + 1) * L; idx += kDftThreads) {
+    for (int idx = blockIdx.y * kDftThreads + t; idx < (order + 1) * L; idx += gridDim.y * kDftThreads) {
         const int k = idx / (order + 1), w = idx - k * (order + 1);
         double s = U[2 * w];  // l = 0
         int m = 0;            // k l mod L
@@ -1907,7 +1911,8 @@ __global__ void __launch_bounds__(kDftThreads) approx_dft_kernel(int order, Appr
     __syncthreads();
     if (t == 0) {
         for (int w = 1; w < kDftThreads / 32; ++w) mx = fmax(mx, red[w]);
-        pl.pat_max[p] = mx;
+        if (mx > 0.0)  // (of the CTAs' maxima, none negative: as integers; the plan sets it to 0)
+            atomicMax((unsigned long long *)pl.pat_max + p, (unsigned long long)__double_as_longlong(mx));
     }
 }
 
@@ -2876,7 +2881,9 @@ int run_approx(gbs_ctx *ctx, int M, const double *O, const double *logdet, const
     const size_t dft_smem = sizeof(double) * 2 * (size_t)Lmax;
     GBS_CUDA(ctx, cudaFuncSetAttribute(approx_dft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)dft_smem));
-    approx_dft_kernel<<<n_pat, kDftThreads, dft_smem, ctx->stream>>>(order, pl);
+    const int dft_most = ((order + 1) * Lmax + kDftThreads - 1) / kDftThreads, dft_want = (8 * ctx->num_sms + n_pat - 1) / n_pat;
+    const unsigned dft_y = (unsigned)(dft_want < dft_most ? dft_want : dft_most > 0 ? dft_most : 1);
+    approx_dft_kernel<<<dim3((unsigned)n_pat, dft_y), kDftThreads, dft_smem, ctx->stream>>>(order, pl);
     GBS_CUDA(ctx, cudaGetLastError());
     const long long want = (secs + kSecThreads / 32 - 1) / (kSecThreads / 32);
     const int fit_blocks = (int)(want < (long long)ctx->num_sms * 16 ? (want > 0 ? want : 1) : ctx->num_sms * 16);
