@@ -13,8 +13,13 @@
 //   rows U = B R^-T            s = 117  (|u| <= sqrt(c_ii) < 4)
 //   1/r00 and 1/r11 (a, b)     s = 123, five limbs     r10/(r00 r11) (c)     s = 120, five limbs
 // with u u at 234 = 114 + 4 limbs and entry x a, u x c at 237 = 117 + 4 limbs.  Columns below
-// the one that feeds the carry are dropped: an entry update is low by at most 7 units of 2^-114
-// (the packed form: 2 units of 2^-112, i.e. 8 of these).
+// the one that feeds the carry are dropped from u u: an entry update is high by at most 7 units of
+// 2^-114 (the packed form: 2 units of 2^-112, i.e. 8 of these).
+//
+// Top limbs are cut to 32 bits, so the bounds above have to hold: the entries' do while every row
+// |u| < 4 (a diagonal entry loses at most 32 a pivot), and a row of a positive definite matrix always
+// is (u_i u_i <= c_ii <= 5, the gather admits |O| <= 4).  A row beyond tells that c_ii has become
+// negative; fl_urow reports it before the cut, the sweep refuses the pattern.
 //
 // Measured on a GB300 at 128 threads x 4 CTAs per SM, independent updates: 0.77 SM clocks an
 // entry against 1.18 for the packed form; IMAD.WIDE runs at 27 lanes per SM clock (plain IMAD at
@@ -73,8 +78,8 @@ __device__ __forceinline__ void fl_mac45(int64_t p[5], const fl &a, const fl5 &b
     p[3] += fl_mw(a.w[2], b.w[4]) + fl_mw(a.w[3], b.w[3]);
     p[4] += fl_mw(a.w[3], b.w[4]);
 }
-// limbs of columns 4..7 with the carry of column 3: x2^-120
-__device__ __forceinline__ fl fl_carry(const int64_t p[5]) {
+// limbs of columns 4..7 with the carry of column 3: x2^-120; top: the last one before it is cut to 32 bits
+__device__ __forceinline__ fl fl_carry(const int64_t p[5], int64_t &top) {
     fl r;
     int64_t x = p[1] + (p[0] >> 30);
     r.w[0] = (int32_t)x & kLimbMask;
@@ -82,8 +87,13 @@ __device__ __forceinline__ fl fl_carry(const int64_t p[5]) {
     r.w[1] = (int32_t)x & kLimbMask;
     x = p[3] + (x >> 30);
     r.w[2] = (int32_t)x & kLimbMask;
-    r.w[3] = (int32_t)(p[4] + (x >> 30));
+    top = p[4] + (x >> 30);
+    r.w[3] = (int32_t)top;
     return r;
+}
+__device__ __forceinline__ fl fl_carry(const int64_t p[5]) {
+    int64_t top;
+    return fl_carry(p, top);
 }
 __device__ __forceinline__ fl5 fl5_carry(const int64_t p[5]) {
     fl5 r;
@@ -119,10 +129,14 @@ __device__ __forceinline__ fx fl_det2(const fl &a, const fl &c, const fl &b) {
     return fx{{(l3 >> 24) | (l4 << 6), (l4 >> 26) | (l5 << 4), (l5 >> 28) | (l6 << 2), (uint32_t)(p6 >> 30)}};
 }
 
-// pivot check of a determinant with ulp 2^-114: 0 fine, 1 not positive, 2 below 2^-8
+// flags of a unit: 1 a pivot was not positive; kFlLost the arithmetic left its range (an entry of O beyond 4, a
+// determinant below 2^-8): what the unit finds besides, 1 included, may be noise, and it reports 2 alone
+constexpr int kFlLost = 4;
+__device__ __forceinline__ int fl_unit_flags(int f) { return f & kFlLost ? 2 : f; }
+// pivot check of a determinant with ulp 2^-114: 0 fine, 1 not positive, kFlLost below 2^-8
 __device__ __forceinline__ int fl_pivot_bad(const fx &det) {
     if (!fx_positive(det)) return 1;
-    return (int32_t)det.w[3] < 1024 ? 2 : 0;
+    return (int32_t)det.w[3] < 1024 ? kFlLost : 0;
 }
 __device__ __forceinline__ bool fl_positive(const fl &a) {
     return a.w[3] > 0 || (a.w[3] == 0 && (a.w[2] | a.w[1] | a.w[0]) != 0);
@@ -130,6 +144,12 @@ __device__ __forceinline__ bool fl_positive(const fl &a) {
 __device__ __forceinline__ int fl_chol_bad(const fl &p00, const fx &det) {
     if (!fl_positive(p00)) return 1;
     return fl_pivot_bad(det);
+}
+// the last pivot of a subset, of which only the determinant counts (a negative definite block passes):
+// no Cholesky check follows its rows, so a diagonal entry below -32 is where the range ends
+__device__ __forceinline__ int fl_last_bad(const fl &p00, const fl &p11, const fx &det) {
+    constexpr int32_t lo = -(32 << 24);
+    return p00.w[3] < lo || p11.w[3] < lo ? kFlLost : fl_pivot_bad(det);
 }
 __device__ __forceinline__ fx fl_rsqrt(const fx &x) { return fx_rsqrt_at(x, 13); }  // ulp 2^-114
 
@@ -152,16 +172,18 @@ __device__ __forceinline__ fl_piv fl_pivot_from(const fl &p00, const fl &p01, co
     v.b = fl5_carry(pb);
     return v;
 }
-// row (u0, u1) of U = B R^{-T}: u0 = b0 a, u1 = b1 b - u0 c
-__device__ __forceinline__ void fl_urow(const fl5 &a, const fl5 &b, const fl5 &c, const fl &b0, const fl &b1, fl &u0,
+// row (u0, u1) of U = B R^{-T}: u0 = b0 a, u1 = b1 b - u0 c; true if it is outside (-4, 4)
+__device__ __forceinline__ bool fl_urow(const fl5 &a, const fl5 &b, const fl5 &c, const fl &b0, const fl &b1, fl &u0,
                                         fl &u1) {
-    int64_t p[5] = {0, 0, 0, 0, 0}, q[5] = {0, 0, 0, 0, 0};
+    int64_t p[5] = {0, 0, 0, 0, 0}, q[5] = {0, 0, 0, 0, 0}, top0, top1;
     fl_mac45(p, b0, a);
     fl_mac45(q, b1, b);
-    u0 = fl_carry(p);
+    u0 = fl_carry(p, top0);
     const fl n{{-u0.w[0], -u0.w[1], -u0.w[2], -u0.w[3]}};
     fl_mac45(q, n, c);
-    u1 = fl_carry(q);
+    u1 = fl_carry(q, top1);
+    constexpr int64_t four = 1ll << 29;
+    return (uint64_t)((top0 + four) | (top1 + four)) >= 1ull << 30;
 }
 // c - u_i . u_j
 __device__ __forceinline__ fl fl_sym_update(const fl &c, const fl &a0, const fl &a1, const fl &b0, const fl &b1) {

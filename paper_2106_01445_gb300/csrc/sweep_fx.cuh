@@ -134,9 +134,10 @@ constexpr int kInv = sym(2 * (R - 1)) + 1;  // reciprocals 2^20 / w + 1 of w < k
 
 // One 2x2 block pivot eliminated by the whole CTA: rows c0, c0 + 1 of the packed D x D matrix Mx;
 // the trailing Schur complement is written to Dst (packed), or in place (Dst null), and
-// det^{-1/2} to *rs.  Two barriers; the caller's data must be visible on entry.
+// det^{-1/2} to *rs.  Two barriers; the caller's data must be visible on entry.  The last `lev` rows
+// belong to the levels.
 __device__ __forceinline__ void elim(const fl *Mx, fl *inplace, int D, int c0, fl *Dst, fl *U, int4 *Qs, fx *rs,
-                                     const uint32_t *inv20, int *flag) {
+                                     const uint32_t *inv20, int lev, int *flag) {
     const int t = threadIdx.x, Dt = D - c0 - 2;
     if (t < ((Dt + 31) & ~31)) {
         const fl p00 = Mx[pidx(D, c0, c0)], p01 = Mx[pidx(D, c0, c0 + 1)], p11 = Mx[pidx(D, c0 + 1, c0 + 1)];
@@ -157,7 +158,7 @@ __device__ __forceinline__ void elim(const fl *Mx, fl *inplace, int D, int c0, f
             if (t == 0) {
                 *rs = yo;
                 // a positive determinant of a negative block is outside this form's range only
-                const int bad = fl_pivot_bad(det) | (fl_positive(p00) ? 0 : 2);
+                const int bad = fl_pivot_bad(det) | (fl_positive(p00) ? 0 : kFlLost);
                 if (bad) atomicOr(flag, bad);
             }
         }
@@ -166,7 +167,10 @@ __device__ __forceinline__ void elim(const fl *Mx, fl *inplace, int D, int c0, f
             const int4 qa = Q[0], qb = Q[1], qc = Q[2], qt = Q[3];
             const fl5 a{{qa.x, qa.y, qa.z, qa.w, qt.x}}, b{{qb.x, qb.y, qb.z, qb.w, qt.y}},
                 c{{qc.x, qc.y, qc.z, qc.w, qt.z}};
-            fl_urow(a, b, c, Mx[pidx(D, c0, c0 + 2 + t)], Mx[pidx(D, c0 + 1, c0 + 2 + t)], U[t], U[Dt + t]);
+            // a negative diagonal entry: refused where the levels will pivot on it; elsewhere the sign of
+            // the block's determinant decides, which is then beyond this form
+            if (fl_urow(a, b, c, Mx[pidx(D, c0, c0 + 2 + t)], Mx[pidx(D, c0 + 1, c0 + 2 + t)], U[t], U[Dt + t]))
+                atomicOr(flag, t >= Dt - lev && t < Dt - 2 ? 1 : kFlLost);
         }
     }
     __syncthreads();
@@ -266,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                 if (a < n && b < n) {
                     const int si = modes[a] + (i & 1) * M, sj = modes[b] + (j & 1) * M;
                     const double o = O[(size_t)si * N2 + sj];
-                    if (!(fabs(o) <= 4.0)) atomicOr(&s_flag, 2);
+                    if (!(fabs(o) <= 4.0)) atomicOr(&s_flag, kFlLost);
                     v = fl_from_fx(fx_from_double(i == j ? 1.0 : 0.0) - fx_from_double(o));
                 }
                 X[pidx(D0, i, j)] = v;
@@ -275,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
         __syncthreads();
         // eliminate the included prefix modes (2x2 block pivots)
         for (int e = 0; e < k; ++e)
-            elim(X, X, D0, 2 * e, nullptr, Wb, Qs, s_rs + kSub + e, inv20, &s_flag);
+            elim(X, X, D0, 2 * e, nullptr, Wb, Qs, s_rs + kSub + e, inv20, 2 * r, &s_flag);
         // the unit's trailing block -> Ub, through registers: the prefix matrix may extend over Ub
         {
             const int d = 2 * rp, o = 2 * k, E = (d >> 1) * (d + 1);
@@ -325,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
             if (leaf) {
                 in_x = ds + 1 == ss;
                 fl *dst = in_x ? X : Sl + (ds == 1 ? slot_off(2) : 0);
-                elim(src, nullptr, D, 2 * (ds - j0), dst, Wb, Qs, s_rs + leaf, inv20, &s_flag);
+                elim(src, nullptr, D, 2 * (ds - j0), dst, Wb, Qs, s_rs + leaf, inv20, 2 * r, &s_flag);
 #pragma unroll
                 for (int e = 0; e <= kS; ++e)
                     if (e > ds) jv[e] = ds + 1;
@@ -422,7 +426,8 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                         const int4 qa = Q[0], qb = Q[1], qc = Q[2], qt = Q[3];
                         const fl5 a{{qa.x, qa.y, qa.z, qa.w, qt.x}}, b{{qb.x, qb.y, qb.z, qb.w, qt.y}},
                             c{{qc.x, qc.y, qc.z, qc.w, qt.z}};
-                        fl_urow(a, b, c, P[pidx(d, 0, i + 2)], P[pidx(d, 1, i + 2)], Wb[f], Wb[nr + f]);
+                        if (fl_urow(a, b, c, P[pidx(d, 0, i + 2)], P[pidx(d, 1, i + 2)], Wb[f], Wb[nr + f]))
+                            atomicOr(&s_flag, i < dc - 2 ? 1 : kFlLost);
                     }
                 }
                 __syncthreads();
@@ -634,7 +639,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                 out[0] = s.hi;
                 out[1] = s.lo;
                 out[2] = a * tp.hi;
-                if (s_flag) atomicOr(pl.pflags + sp, s_flag);
+                if (s_flag) atomicOr(pl.pflags + sp, fl_unit_flags(s_flag));
             }
         }
     }
