@@ -473,7 +473,7 @@ __device__ __forceinline__ void dfs(const Src &A, T tau, int depth, int nreal, A
         const fx det = fl_det2(p00, p01, p11);
         const fx rs = fl_rsqrt(det);
         if constexpr (m == 1) {
-            acc.bad |= fl_last_bad(p00, p11, det);
+            acc.bad |= fl_pivot_bad(det);
             leaf_pair<NEG>(acc, ONE ? rs : fx_mul_uu(tau, rs), tau, real, cnt);
         } else {
             // symmetric form C - U U^T, U = B R^{-T}, in limbs
@@ -482,8 +482,7 @@ __device__ __forceinline__ void dfs(const Src &A, T tau, int depth, int nreal, A
             const fl_piv v = fl_pivot_from(p00, p01, fl_rsqrt(fl_pack(p00)), rs);
             fl u0[d], u1[d];
 #pragma unroll
-            for (int i = 0; i < d; ++i)
-                if (fl_urow(v.a, v.b, v.c, A(o, o + 2 + i), A(o + 1, o + 2 + i), u0[i], u1[i])) acc.bad |= i < d - 2 ? 1 : kFlLost;
+            for (int i = 0; i < d; ++i) fl_urow(v.a, v.b, v.c, A(o, o + 2 + i), A(o + 1, o + 2 + i), u0[i], u1[i]);
             RegMat<fl, m - 1> C;
 #pragma unroll
             for (int i = 0; i < d; ++i)

@@ -27,6 +27,8 @@ constexpr int B = Prec<fx>::B;
 constexpr int R = kL + B;     // modes of a sub-unit's level-0 matrix
 constexpr int kW = kThreads / 32;
 constexpr int kSub = 1 << kS;
+constexpr int kLast = kThreads - 32;  // the last warp
+static_assert(2 * R <= 32, "a row of a level-0 matrix a lane");
 
 // a node's prefactor m 2^e: m in [1, 2) as limbs at scale 117
 struct node {
@@ -134,10 +136,9 @@ constexpr int kInv = sym(2 * (R - 1)) + 1;  // reciprocals 2^20 / w + 1 of w < k
 
 // One 2x2 block pivot eliminated by the whole CTA: rows c0, c0 + 1 of the packed D x D matrix Mx;
 // the trailing Schur complement is written to Dst (packed), or in place (Dst null), and
-// det^{-1/2} to *rs.  Two barriers; the caller's data must be visible on entry.  The last `lev` rows
-// belong to the levels.
+// det^{-1/2} to *rs.  Two barriers; the caller's data must be visible on entry.
 __device__ __forceinline__ void elim(const fl *Mx, fl *inplace, int D, int c0, fl *Dst, fl *U, int4 *Qs, fx *rs,
-                                     const uint32_t *inv20, int lev, int *flag) {
+                                     const uint32_t *inv20, int *flag, uint32_t &out) {
     const int t = threadIdx.x, Dt = D - c0 - 2;
     if (t < ((Dt + 31) & ~31)) {
         const fl p00 = Mx[pidx(D, c0, c0)], p01 = Mx[pidx(D, c0, c0 + 1)], p11 = Mx[pidx(D, c0 + 1, c0 + 1)];
@@ -167,10 +168,8 @@ __device__ __forceinline__ void elim(const fl *Mx, fl *inplace, int D, int c0, f
             const int4 qa = Q[0], qb = Q[1], qc = Q[2], qt = Q[3];
             const fl5 a{{qa.x, qa.y, qa.z, qa.w, qt.x}}, b{{qb.x, qb.y, qb.z, qb.w, qt.y}},
                 c{{qc.x, qc.y, qc.z, qc.w, qt.z}};
-            // a negative diagonal entry: refused where the levels will pivot on it; elsewhere the sign of
-            // the block's determinant decides, which is then beyond this form
-            if (fl_urow(a, b, c, Mx[pidx(D, c0, c0 + 2 + t)], Mx[pidx(D, c0 + 1, c0 + 2 + t)], U[t], U[Dt + t]))
-                atomicOr(flag, t >= Dt - lev && t < Dt - 2 ? 1 : kFlLost);
+            fl_urow(a, b, c, Mx[pidx(D, c0, c0 + 2 + t)], Mx[pidx(D, c0 + 1, c0 + 2 + t)], U[t], U[Dt + t], out);
+            out |= fl_negative(Mx[pidx(D, c0 + 2 + t, c0 + 2 + t)]);
         }
     }
     __syncthreads();
@@ -185,6 +184,31 @@ __device__ __forceinline__ void elim(const fl *Mx, fl *inplace, int D, int c0, f
         else inplace[at] = v;
     }
     __syncthreads();
+}
+
+// The range check of one step of the chain of all includes (fl.cuh), t < d: the matrix's diagonal and, of its
+// rows below the first pivot, U.  Out of line: the sweep passes here once a pattern, on the last warp
+// beside the others' work.
+static __device__ __noinline__ uint32_t chain_rows(const fl *P, int d, const int4 *Q, int t) {
+    uint32_t out = fl_negative(P[pidx(d, t, t)]);
+    if (t >= 2) {
+        const int4 qa = Q[0], qb = Q[1], qc = Q[2], qt = Q[3];
+        const fl5 a{{qa.x, qa.y, qa.z, qa.w, qt.x}}, b{{qb.x, qb.y, qb.z, qb.w, qt.y}}, c{{qc.x, qc.y, qc.z, qc.w, qt.z}};
+        fl u0, u1;
+        fl_urow(a, b, c, P[pidx(d, 0, t)], P[pidx(d, 1, t)], u0, u1, out);
+    }
+    return out;
+}
+// ... with the pivot's quantities anew (at the register bottom, which keeps them to itself)
+static __device__ __noinline__ uint32_t chain_node(const fl *P, int d, int t) {
+    uint32_t out = fl_negative(P[pidx(d, t, t)]);
+    if (t >= 2) {
+        const fl p00 = P[pidx(d, 0, 0)], p01 = P[pidx(d, 0, 1)], p11 = P[pidx(d, 1, 1)];
+        const fl_piv v = fl_pivot_from(p00, p01, fl_rsqrt(fl_pack(p00)), fl_rsqrt(fl_det2(p00, p01, p11)));
+        fl u0, u1;
+        fl_urow(v.a, v.b, v.c, P[pidx(d, 0, t)], P[pidx(d, 1, t)], u0, u1, out);
+    }
+    return out;
 }
 
 template <bool BIN>
@@ -259,6 +283,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
         }
         __syncthreads();
         const int D0 = 2 * (k + rp);
+        uint32_t out = 0;  // bits of rows and diagonal entries beyond the limb form's range (fl.cuh)
         // gather I - O on those rows into X, padding modes as identity
         {
             const uint32_t inv = inv20[D0 + 1];
@@ -279,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
         __syncthreads();
         // eliminate the included prefix modes (2x2 block pivots)
         for (int e = 0; e < k; ++e)
-            elim(X, X, D0, 2 * e, nullptr, Wb, Qs, s_rs + kSub + e, inv20, 2 * r, &s_flag);
+            elim(X, X, D0, 2 * e, nullptr, Wb, Qs, s_rs + kSub + e, inv20, &s_flag, out);
         // the unit's trailing block -> Ub, through registers: the prefix matrix may extend over Ub
         {
             const int d = 2 * rp, o = 2 * k, E = (d >> 1) * (d + 1);
@@ -316,6 +341,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
         for (int e = 0; e <= kS; ++e) jv[e] = 0;
         for (int leaf = 0; leaf < nsub; ++leaf) {
             const int kk = __popc(leaf);
+            const bool all = k == qs && kk == ss;  // its last node at every level has all modes included
             // the depth whose choice turns include (none at the first leaf); deeper choices
             // are excludes
             const int ds = leaf ? ss - 1 - (31 - __clz(leaf ^ (leaf - 1))) : ss;
@@ -329,7 +355,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
             if (leaf) {
                 in_x = ds + 1 == ss;
                 fl *dst = in_x ? X : Sl + (ds == 1 ? slot_off(2) : 0);
-                elim(src, nullptr, D, 2 * (ds - j0), dst, Wb, Qs, s_rs + leaf, inv20, 2 * r, &s_flag);
+                elim(src, nullptr, D, 2 * (ds - j0), dst, Wb, Qs, s_rs + leaf, inv20, &s_flag, out);
 #pragma unroll
                 for (int e = 0; e <= kS; ++e)
                     if (e > ds) jv[e] = ds + 1;
@@ -426,9 +452,10 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                         const int4 qa = Q[0], qb = Q[1], qc = Q[2], qt = Q[3];
                         const fl5 a{{qa.x, qa.y, qa.z, qa.w, qt.x}}, b{{qb.x, qb.y, qb.z, qb.w, qt.y}},
                             c{{qc.x, qc.y, qc.z, qc.w, qt.z}};
-                        if (fl_urow(a, b, c, P[pidx(d, 0, i + 2)], P[pidx(d, 1, i + 2)], Wb[f], Wb[nr + f]))
-                            atomicOr(&s_flag, i < dc - 2 ? 1 : kFlLost);
+                        fl_urow(a, b, c, P[pidx(d, 0, i + 2)], P[pidx(d, 1, i + 2)], Wb[f], Wb[nr + f]);
                     }
+                    if (all && t >= kLast && t < kLast + d)
+                        out |= chain_rows(src + (np - 1) * sstr, d, Qb + 4 * (np - 1), t - kLast);
                 }
                 __syncthreads();
                 // (c) both children of every parent: the exclude child is the parent's
@@ -476,6 +503,8 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
             // the register bottom: each thread's two-mode node, relative to its prefactor m 2^e
             const fl *nodes = (L_eff & 1) ? Y : X;
             const bool has = t < (1 << L_eff);
+            if (all && t >= kLast && t < kLast + 2 * B)
+                out |= chain_node(nodes + ((1 << L_eff) - 1) * nstride(2 * B), 2 * B, t - kLast);
             int e = -(1 << 20);
             node tn = node_unit();
             const int nreal = n - (n_eff - B);
@@ -546,6 +575,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                 // next sub-unit writes Y after a barrier only
             }
         }
+        if (out) atomicOr(&s_flag, 2);  // not positive definite: beside a pivot that says so, or alone
         __syncthreads();
         if (t < 32) {
             // the prefix factor (a tree of products over the lanes) and each sub-unit's (the
