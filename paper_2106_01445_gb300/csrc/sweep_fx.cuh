@@ -123,7 +123,8 @@ struct Lay {
     static_assert(sizeof(fl) * sym(2 * kMaxN) <= W, "prefix matrix must fit in X, Y, Ub and Sl");
 };
 // 228 KB an SM, 1 KB of it reserved a CTA
-static_assert(3 * (Lay::bytes(true) + 1024 + 1600) <= 228 * 1024, "three CTAs must fit on an SM");
+static_assert(3 * (Lay::bytes(true) + 1024 + 2500) <= 228 * 1024 && 3 * (Lay::bytes(false) + 1024 + 1600) <= 228 * 1024,
+              "three CTAs must fit on an SM");
 
 // f / w for the folded-triangle indices (f < 2^12, w <= 2 kMaxN + 1), by a reciprocal
 __device__ __forceinline__ void fold_fast(int f, int D, uint32_t inv, int &i, int &j) {
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
     __shared__ long long s_unit;
     __shared__ int s_flag;
     __shared__ float s_abs[kSub * kW];
-    __shared__ int s_exp[kSub * kW];
+    __shared__ int s_exp[kSub * kW * (BIN ? 8 : 1)];
     __shared__ fx s_rs[kSub + kMaxN];  // the tree's and the prefix's det^{-1/2}
     __shared__ uint32_t inv20[kInv];
 
@@ -512,12 +513,23 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                 tn = node_ld((L_eff & 1) ? tauY : tauX, t);
                 e = tn.e;
             }
-            const int em = __reduce_max_sync(0xffffffffu, e);
             const int at = leaf * kW + wp;
             if constexpr (BIN) {
-                // unsigned, by subset size: the thread's sizes 0..B, aligned to the warp's
-                // exponent; then lane (z, part) sums every fourth lane's share of the warp's
-                // size z = 0..7 (a lane's bin b belongs to size popc(lane) + b)
+                // unsigned, by subset size (a lane's bin b, 0..B, belongs to the warp's size
+                // popc(lane) + b): every size aligned to the largest exponent among the lanes that
+                // hold it, so that a size keeps its last bits beside one of larger terms (a
+                // mode included may scale them by 16); then lane (z, part) sums every fourth
+                // lane's share of the warp's size z = 0..7
+                const int pc = __popc(lane);
+                int by = -(1 << 20);  // lane c: the largest exponent of the lanes with c includes
+#pragma unroll
+                for (int c = 0; c <= 5; ++c) {
+                    const int v = __reduce_max_sync(0xffffffffu, pc == c ? e : -(1 << 20));
+                    if (lane == c) by = v;
+                }
+                int ez = by;          // lane z: of the lanes that hold size z
+#pragma unroll
+                for (int b = 1; b <= B; ++b) ez = max(ez, __shfl_sync(0xffffffffu, by, (lane - b) & 31));
                 fx *scratch = (fx *)((L_eff & 1) ? X : Y) + wp * 32 * (B + 1);
                 BinAcc<fx, B + 1> acc;
 #pragma unroll
@@ -529,10 +541,11 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                     if (acc.bad) atomicOr(&s_flag, acc.bad);
                     const fx mp = node_packed(tn);
 #pragma unroll
-                    for (int b = 0; b <= B; ++b) acc.v[b] = fx_shr(fx_mul_uu(acc.v[b], mp), em - e + 4);
+                    for (int b = 0; b <= B; ++b) acc.v[b] = fx_mul_uu(acc.v[b], mp);
                 }
 #pragma unroll
-                for (int b = 0; b <= B; ++b) scratch[lane * (B + 1) + b] = acc.v[b];
+                for (int b = 0; b <= B; ++b)
+                    scratch[lane * (B + 1) + b] = fx_shr(acc.v[b], __shfl_sync(0xffffffffu, ez, pc + b) - e + 4);
                 __syncwarp();
                 const int z = lane & 7, part = lane >> 3;
                 fx s = fx_zero();
@@ -543,10 +556,13 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
                 }
                 s = s + fx_shfl_xor(s, 8);
                 s = s + fx_shfl_xor(s, 16);
-                if (lane < 8) s_sum[at * 8 + lane] = s;
-                if (lane == 0) s_exp[at] = em;
+                if (lane < 8) {
+                    s_sum[at * 8 + lane] = s;
+                    s_exp[at * 8 + lane] = ez;
+                }
                 __syncthreads();  // the scratch lies in the next sub-unit's matrices
             } else {
+                const int em = __reduce_max_sync(0xffffffffu, e);
                 fx v = fx_zero();
                 float ab = 0.0f;
                 if (has) {
@@ -602,21 +618,25 @@ __global__ void __launch_bounds__(kThreads, 3) sweep_fx_kernel(int M, const doub
         else __syncwarp();
         if constexpr (BIN) {
             // sub-unit `leaf`, size z (0..9 within it): the four warps' sums (warp w holds the
-            // sizes popc(w) + 0..7) times the sub-unit's factor, then per size of the unit
+            // sizes popc(w) + 0..7), aligned to the size's largest exponent, times the sub-unit's
+            // factor, then per size of the unit
             dd *part = (dd *)X;
             if (t < 10 * nsub) {
                 const int leaf = t / 10, z = t - 10 * leaf;
-                int em = s_exp[leaf * kW];
+                int em = -(1 << 20);
 #pragma unroll
-                for (int w = 1; w < kW; ++w) em = max(em, s_exp[leaf * kW + w]);
+                for (int w = 0; w < kW; ++w) {
+                    const int b = z - __popc(w);
+                    if (b >= 0 && b < 8) em = max(em, s_exp[(leaf * kW + w) * 8 + b]);
+                }
                 fx S = fx_zero();
 #pragma unroll
                 for (int w = 0; w < kW; ++w) {
-                    const int b = z - __popc(w), d = em - s_exp[leaf * kW + w];
-                    if (b >= 0 && b < 8) S = S + fx_shr(s_sum[(leaf * kW + w) * 8 + b], d);
+                    const int b = z - __popc(w), at = (leaf * kW + w) * 8 + b;
+                    if (b >= 0 && b < 8) S = S + fx_shr(s_sum[at], em - s_exp[at]);
                 }
                 const dd sv = fx_to_dd(S);
-                const double sc = ldexp(1.0, em + 4);
+                const double sc = ldexp(1.0, em + 4);  // (a size without terms: 0)
                 part[t] = node_dd(node_ld(s_ts, leaf)) * dd(sv.hi * sc, sv.lo * sc);
             }
             __syncthreads();
