@@ -112,7 +112,7 @@ __device__ __noinline__ void tree_forward(qf *base, int np, int d, const uint16_
             Q[3 * cp + k] = f;
         } else {
             rs[cp] = r;
-            if (!qf_positive(det)) atomicOr(bad, 1);
+            if (!qf_positive(det) || qf_saturated(det)) atomicOr(bad, 1);
             if (nchild) {
                 nchild[2 * cp] = (uint16_t)(noff[cp] + 2 * d - 1);
                 nchild[2 * cp + 1] = (uint16_t)(dst - base + cp * stc);
@@ -283,7 +283,9 @@ __global__ void __launch_bounds__(kTreeThreads, 2) grad_tree_kernel(int M, int n
         fold_ij(f, Ds, i, j);
         const int ri = smrow[i], rj = smrow[j];
         const int gi = modes[ri >> 1] + (ri & 1) * M, gj = modes[rj >> 1] + (rj & 1) * M;
-        SM[gpidx(Ds, i, j)] = (i == j ? qf_one() : qf_zero()) - qf_from_double(O[(size_t)gi * N2 + gj]);
+        const double o = O[(size_t)gi * N2 + gj];
+        if (!(fabs(o) <= 0x1p100)) atomicOr(&s_bad, 1);  // not finite, or far beyond any state: left to double-double
+        SM[gpidx(Ds, i, j)] = (i == j ? qf_one() : qf_zero()) - qf_from_double(o);
     }
     for (int f = t; f < gsym(Dr); f += kTreeThreads) Gam[f] = qf_zero();
     // where the packed trailing block of the last d rows of a D-row matrix starts

@@ -300,6 +300,8 @@ QF_FN bool qf_positive(const qf &a) {
     const int32_t t = (int32_t)a.w[3] >> 10;
     return t > 0 || (t == 0 && (a.w[0] | a.w[1] | a.w[2]) != 0u);
 }
+// overflowed, or from a double that is not finite
+QF_FN bool qf_saturated(const qf &a) { return (a.w[3] & 0x3ffu) == 1023u; }
 // exact (53 bits fit)
 QF_FN qf qf_from_double(double d) {
     using namespace qfn;

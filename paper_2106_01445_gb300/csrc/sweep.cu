@@ -198,8 +198,7 @@ template <> __device__ __forceinline__ fx6 mul_pos<fx6>(fx6 a, fx6 b) { return f
 // pivot check: 0 fine, 1 not positive (or NaN), 2 outside the fixed-point range
 template <typename T> __device__ __forceinline__ int pivot_bad(T det) { return det > T(0) ? 0 : 1; }
 template <> __device__ __forceinline__ int pivot_bad<fx6>(fx6 det) { return fx_pivot_bad(det); }
-__device__ __forceinline__ bool saturated(const qf &x) { return (x.w[3] & 0x3ffu) == 1023u; }
-template <> __device__ __forceinline__ int pivot_bad<sq>(sq det) { return qf_positive(det) && !saturated(det) ? 0 : 1; }
+template <> __device__ __forceinline__ int pivot_bad<sq>(sq det) { return qf_positive(det) && !qf_saturated(det) ? 0 : 1; }
 // complex pivots: their determinants may have any argument in (-pi, pi); only zero or NaN is bad
 template <> __device__ __forceinline__ int pivot_bad<zc>(zc det) {
     return fabs(det.re) + fabs(det.im) > 0.0 ? 0 : 1;
@@ -261,7 +260,7 @@ __device__ __forceinline__ float abs_part(fx6 x) { return (float)(int32_t)x.w[5]
 __device__ __forceinline__ bool is_nan(float x) { return x != x; }
 __device__ __forceinline__ bool is_nan(double x) { return x != x; }
 __device__ __forceinline__ bool is_nan(dd x) { return x.hi != x.hi; }
-__device__ __forceinline__ bool is_nan(const sq &x) { return saturated(x); }
+__device__ __forceinline__ bool is_nan(const sq &x) { return qf_saturated(x); }
 __device__ __forceinline__ bool is_nan(zc x) { return zc_nan(x); }
 __device__ __forceinline__ bool is_nan(zf x) { return zf_nan(x); }
 // a thread's subtree sum as (hi, lo) doubles
