@@ -373,11 +373,11 @@ __global__ void __launch_bounds__(kScanThreads) approx_scan_kernel(int n_pat, lo
     const int p0 = t * per < n_pat ? t * per : n_pat, p1 = p0 + per < n_pat ? p0 + per : n_pat;
     if (t == 0) {
         s_n = 0;
-        s_small = 0;
+        s_small = -1;
         s_L = 1;
     }
     long long units = 0, secs = 0;
-    int nmax = 0, nsmall = 0, Lmax = 1;
+    int nmax = 0, nsmall = -1, Lmax = 1;
     for (int p = p0; p < p1; ++p) {
         const int L = pl.pat_L[p], n = pl.pat_n[p];
         units += L > 0 ? L / 2 + 1 : 0;
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(kScanThreads) approx_scan_kernel(int n_pat, lo
         pl.info[1] = s_n;
         pl.info[2] = s_L;
         pl.info[3] = sc[kScanThreads - 1];
-        pl.info[4] = s_small;  // largest n of the one-CTA minors kernel
+        pl.info[4] = s_small;  // largest n of the one-CTA minors kernel (0: empty patterns only, -1: none)
     }
 }
 
@@ -2857,7 +2857,7 @@ int run_approx(gbs_ctx *ctx, int M, const double *O, const double *logdet, const
         }
         if (st) return st;
     }
-    if (n_two > 0) {
+    if (n_two >= 0) {  // empty patterns too: their sector tables come from here
         st = launch_minors<R, kMinorThreads>(ctx, M, O, pats, n_pat, order, 0, n_two, 0, pl);
         if (st) return st;
     }
