@@ -228,7 +228,7 @@ struct ApproxPlan {
     double *pat_max;      // per pattern: largest tilted sector
     double *sec_D;        // (kMaxOrder + 1) per sector: D_w^(k), w = 0..order
     double *sec_part;     // per sector: fitted last point (negative: the fit fell back)
-    int *sec_slow;        // sectors left to the slow fits' kernel
+    uint32_t *sec_slow;   // sectors left to the slow fits' kernel (below 2^32: a sector is 92 bytes of workspace)
     unsigned long long *slow;  // their number, and the kernel's work counter
 };
 
@@ -2031,7 +2031,7 @@ __global__ void __launch_bounds__(kFitThreads, 3) approx_sector_fit_lanes_kernel
     const int ok = maxent_fit_lanes<J>(act, n, m, a, x, xn, lane);
     if (act && ok == 1) val = mu[0] * exp(-a[0]);
     if (in) pl.sec_part[gs] = val;
-    if (fit && !(act && ok == 1)) pl.sec_slow[atomicAdd(pl.slow, 1ull)] = (int)gs;
+    if (fit && !(act && ok == 1)) pl.sec_slow[atomicAdd(pl.slow, 1ull)] = (uint32_t)gs;
 }
 
 // the sectors that approx_sector_fit_lanes_kernel left: fits that take many trial points, fits that
@@ -2749,7 +2749,7 @@ ApproxPlan approx_plan_from(void *ws, int n_pat, long long units = 0, long long 
     pl.pat_max = (double *)(b + o.pat_max);
     pl.sec_D = (double *)(b + o.sec_D);
     pl.sec_part = (double *)(b + o.sec_part);
-    pl.sec_slow = (int *)(b + o.sec_slow);
+    pl.sec_slow = (uint32_t *)(b + o.sec_slow);
     pl.slow = (unsigned long long *)(b + o.counter3);
     return pl;
 }
