@@ -59,7 +59,7 @@ typedef enum {
     GBS_DD = 2,          /* double-double (~106-bit) class factorisations and sum: for patterns whose
                             signed sum cancels beyond FP64 (kappa u64 >~ 1e-10).  110-bit software
                             floating point on the integer pipes, double-double itself on the FP64
-                            pipes where kappa exceeds 1e22 */
+                            pipes where kappa exceeds 1e24 */
     GBS_FX = 3,          /* exact sum only: 128-bit fixed-point (Q16.112) factorisations on the
                             integer pipes, double-double prefactors and sum; accuracy as GBS_DD
                             (~2^-100 per term) at a fraction of its cost.  Needs every pivot

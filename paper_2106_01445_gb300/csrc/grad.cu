@@ -20,6 +20,7 @@
 
 #include "dd.cuh"
 #include "gbs_internal.cuh"
+#include "kappa.cuh"
 #include "qf.cuh"
 
 namespace {
@@ -221,7 +222,7 @@ __device__ __noinline__ void tree_backward(const qf *base, int np, int d, const 
 // four lanes, long jobs on the last warps beside the short ones on the first).  Measured on the
 // 32-mode Clements workload (512 patterns, n = 8..16): 69.5 ms in double-double (FP64 pipe 70% busy),
 // 49.9 with the same kernel in qf (barriers, divergence), 18.0 as it is here.
-__global__ void __launch_bounds__(kTreeThreads, 2) grad_tree_kernel(int M, int n_max, const double *__restrict__ O,
+__global__ void __launch_bounds__(kTreeThreads, 2) grad_tree_kernel(int M, const double *__restrict__ O,
                                                                const uint64_t *__restrict__ pats,
                                                                const int *__restrict__ chunk_p,
                                                                const long long *__restrict__ chunk_u, size_t pst,
@@ -242,6 +243,7 @@ __global__ void __launch_bounds__(kTreeThreads, 2) grad_tree_kernel(int M, int n
     __shared__ int s_bad;
     __shared__ qf s_T, s_V, s_S[2];
     __shared__ double nA[kNodes], dA[kGroupBits], s_A[2], s_Asum;
+    __shared__ float s_guess;
     const int t = threadIdx.x, ch = blockIdx.x, p = chunk_p[ch], N2 = 2 * M;
     const long long u_begin = chunk_u[2 * ch], u_end = chunk_u[2 * ch + 1];
     const uint64_t wlo = pats[2 * p], whi = pats[2 * p + 1];
@@ -277,6 +279,17 @@ __global__ void __launch_bounds__(kTreeThreads, 2) grad_tree_kernel(int M, int n
         smrow[2 * r + 1] = (uint8_t)(2 * t + 1);
     }
     __syncthreads();
+    if (n >= kGuessFrom) {  // alike in all chunks of the pattern
+        if (t < 32) {
+            const float k = kappa_guess(O, M, modes, n);
+            if (t == 0) s_guess = k;
+        }
+        __syncthreads();
+        if (s_guess > kGuessRedo) {
+            if (t == 0) atomicOr(flags + p, 1);
+            return;
+        }
+    }
     // the chunk's rows of A = I - O, its high pivots, and a zero Gam
     for (int f = t; f < gsym(Ds); f += kTreeThreads) {
         int i, j;
@@ -866,8 +879,8 @@ __global__ void __launch_bounds__(kTreeThreads) grad_tree_dd_kernel(int M, const
 
 }  // namespace ddk
 
-// the patterns that the double-double kernel takes again: kappa = sum |terms| / |T| above kRedo (or
-// no number), or a pivot that is not positive; their flags start afresh
+// the patterns that the double-double kernel takes: kappa = sum |terms| / |T| above kRedo (or no number), a
+// pivot that is not positive, or left out by the first kernel (kappa.cuh); their flags start afresh
 constexpr double kRedo = 1e24;
 __global__ void grad_redo_kernel(int n_pat, const long long *__restrict__ chunk_off, const qf *__restrict__ part_T,
                                  const double *__restrict__ part_A, int *__restrict__ redo, int *__restrict__ flags) {
@@ -1301,8 +1314,8 @@ int grad_sigmaQ(gbs_ctx *ctx, int M, const double *O, const double *logdet, cons
     GBS_CUDA(ctx, cudaFuncSetAttribute(grad_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     st = gbs_timing_begin(ctx);
     if (st) return st;
-    grad_tree_kernel<<<(unsigned)chunks, kTreeThreads, smem, ctx->stream>>>(M, n_max, O, pats, chunk_p, chunk_u, pst,
-                                                                           part, pT, pA, flags);
+    grad_tree_kernel<<<(unsigned)chunks, kTreeThreads, smem, ctx->stream>>>(M, O, pats, chunk_p, chunk_u, pst, part, pT,
+                                                                           pA, flags);
     GBS_CUDA(ctx, cudaGetLastError());
     grad_redo_kernel<<<(n_pat + 127) / 128, 128, 0, ctx->stream>>>(n_pat, chunk_off, pT, pA, redo, flags);
     const size_t dsmem = sizeof(dd) * (size_t)ddk::kTreeSmem;

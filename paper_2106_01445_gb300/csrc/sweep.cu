@@ -33,6 +33,7 @@
 #include "fx.cuh"
 #include "fx6.cuh"
 #include "gbs_internal.cuh"
+#include "kappa.cuh"
 #include "qf.cuh"
 #include "zc.cuh"
 
@@ -568,10 +569,12 @@ struct Plan {
     bool redo;          // a second pass: only the patterns with kRedoFlag in their status bits
 };
 constexpr int kRedoFlag = 256;
-// GBS_DD: patterns with kappa above this, and those without a result, are taken again in
-// double-double.  There the two arithmetics' last digits differ by more than 1e-9 of the result
-// (kappa 2^-106 times a few), and the sign of a sum that is all cancellation is the arithmetic's.
-constexpr double kRedoKappa = 1e22;
+// GBS_DD: patterns with kappa above this, and those without a result, are taken again in double-double, and
+// those whose kappa is sure to be (kappa.cuh) there alone: a batch of such patterns else took both
+// passes' time, one and a half times double-double's.  The line: against the 192-bit sum the
+// result's error is below 2^-117 kappa here and 2^-112 in double-double (450 patterns of 13 to 19
+// clicks), so up to 1e24 the two agree to 5e-11 of the sum; beyond, callers keep the digits they had.
+constexpr double kRedoKappa = 1e24;
 
 template <typename T>
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(int M, const uint64_t *__restrict__ pats,
@@ -800,6 +803,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same_v<T, sq> ? 3 : 0) sweep
     T *Sl = (T *)(smem + Lay::off_Sl);       // the sub-unit tree's stored matrices
     using Tau = typename Prec<T>::Tau;
     __shared__ Tau s_tpre;
+    __shared__ float s_guess;
 
     const int t = threadIdx.x;
     const int N2 = 2 * M;
@@ -850,6 +854,20 @@ __global__ void __launch_bounds__(kThreads, std::is_same_v<T, sq> ? 3 : 0) sweep
         }
         __syncthreads();
         const int n = s_n;
+        if constexpr (std::is_same_v<T, sq>) {
+            if (n >= kGuessFrom) {  // alike in all units of the pattern
+                if (t < 32) {
+                    const float k = kappa_guess(O, M, modes, n);
+                    if (t == 0) s_guess = k;
+                }
+                __syncthreads();
+                if (s_guess > kGuessRedo) {
+                    if (t == 0) atomicOr(pl.pflags + sp, kRedoFlag);
+                    __syncthreads();
+                    continue;
+                }
+            }
+        }
         int n_eff, L_eff, q, ss;
         unit_shape<T>(n, n_eff, L_eff, q, ss, pl.split + kSubMore<T>);
         const int r = L_eff + B;           // modes of a sub-unit's level-0 matrix
@@ -1332,6 +1350,10 @@ __global__ void finalize_kernel(int n_pat, const double *__restrict__ logdet, Pl
     const bool batch_over = *pl.overflow != 0;
     if (std::is_same_v<T, sq> && sp == 0 && lane == 0) *pl.counter = 0;  // for the second pass
     if (pl.redo && !(pl.pflags[sp] & kRedoFlag)) return;
+    if (std::is_same_v<T, sq> && (pl.pflags[sp] & kRedoFlag)) {  // not swept
+        if (lane == 0) atomicAdd(pl.n_redo, 1);
+        return;
+    }
     double h, l, a;
     warp_unit_sum(pl.partials, pl.unit_off[sp], batch_over ? pl.unit_off[sp] : pl.unit_off[sp + 1], lane, h, l, a);
     if (lane) return;
