@@ -1987,9 +1987,39 @@ __global__ void __launch_bounds__(kSecThreads) approx_sector_fit_kernel(int n_pa
     }
 }
 
-// The same values, P consecutive sectors a warp (P <= 32): order J for all of them at once in
-// maxent_fit_lanes; the others go to approx_fit_slow_kernel.  Both kernels together, GB300: 256
+// The fits of the warp's sectors whose own order (the batch's, or less where the support is small) is J or below,
+// one order after the other: 1 it stands (val), else to be done by approx_fit_slow_kernel
+template <int J>
+__device__ __forceinline__ int fit_lane_orders(bool fit, int Jmax, int n, const double *Dk, const double *x, int xn,
+                                              int lane, double &val) {
+    int done = 0;
+    const bool act = fit && Jmax == J;
+    if (__any_sync(0xffffffffu, act)) {
+        double m[J + 1], a[J + 1], mu[J + 1];
+        if (act) {
+            raw_moments(Dk, J, mu);
+            double np = 1.0;
+#pragma unroll
+            for (int i = 0; i <= J; ++i) {
+                m[i] = mu[i] / np / mu[0];
+                np *= n;
+            }
+        }
+        const int ok = maxent_fit_lanes<J>(act, n, m, a, x, xn, lane);
+        if (act && ok == 1) {
+            val = mu[0] * exp(-a[0]);
+            done = 1;
+        }
+    }
+    if constexpr (J > 0) done |= fit_lane_orders<J - 1>(fit, Jmax, n, Dk, x, xn, lane, val);
+    return done;
+}
+
+// The same values, P consecutive sectors a warp (P <= 32), all of an order at once in maxent_fit_lanes; the
+// fits that take many trial points or fail go to approx_fit_slow_kernel.  Both kernels together, GB300: 256
 // 50-mode patterns at order 2 11.4 -> 5.2 ms, 96 at order 4 66 -> 14.8 ms (one warp a sector before).
+// Patterns of no more clicks than the order have their lower order here too: on the clusters, 200
+// patterns of 2 and 3 clicks at order 2 took 8.9 ms for 3.8.
 template <int J>
 __global__ void __launch_bounds__(kFitThreads, 3) approx_sector_fit_lanes_kernel(int n_pat, int P, double sector_eps,
                                                                                 ApproxPlan pl) {
@@ -2015,27 +2045,14 @@ __global__ void __launch_bounds__(kFitThreads, 3) approx_sector_fit_lanes_kernel
     const double D0 = Dk[0];
     double val = 0.0;
     const bool fit = in && n > 0 && k >= n && D0 >= sector_eps * pl.pat_max[p] && D0 > 0.0;
-    const int Jmax = J < n - 1 ? J : n - 1;
-    const bool act = fit && Jmax == J;
     if (in && n == 0) val = k == 0 ? D0 : 0.0;
-    double m[J + 1], a[J + 1], mu[J + 1];
-    if (act) {
-        raw_moments(Dk, J, mu);
-        double np = 1.0;
-#pragma unroll
-        for (int i = 0; i <= J; ++i) {
-            m[i] = mu[i] / np / mu[0];
-            np *= n;
-        }
-    }
-    const int ok = maxent_fit_lanes<J>(act, n, m, a, x, xn, lane);
-    if (act && ok == 1) val = mu[0] * exp(-a[0]);
+    const int done = fit_lane_orders<J>(fit, J < n - 1 ? J : n - 1, n, Dk, x, xn, lane, val);
     if (in) pl.sec_part[gs] = val;
-    if (fit && !(act && ok == 1)) pl.sec_slow[atomicAdd(pl.slow, 1ull)] = (uint32_t)gs;
+    if (fit && !done) pl.sec_slow[atomicAdd(pl.slow, 1ull)] = (uint32_t)gs;
 }
 
-// the sectors that approx_sector_fit_lanes_kernel left: fits that take many trial points, fits that
-// fail at their order and go on at lower ones, and supports smaller than the order
+// the sectors that approx_sector_fit_lanes_kernel left: fits that take many trial points, and fits that
+// fail at their order and go on at lower ones
 __global__ void __cluster_dims__(kSlowCtas, 1, 1) __launch_bounds__(kSlowThreads)
     approx_fit_slow_kernel(int n_pat, int order, ApproxPlan pl) {
     __shared__ SlowShared sh;
