@@ -1780,11 +1780,13 @@ __device__ int maxent_fit_lanes(bool act, int n, const double *m, double *a, con
     return ok;
 }
 
-// The same fit by a cluster of kSlowCtas CTAs of four warps: sixteen steps of a line search at once,
-// 2^-16r .. 2^-(16r+15) in round r, of which the first accepted one counts.  A few fits in ten thousand
+// The same fit by a cluster of kSlowCtas CTAs of four warps: W = sixteen steps of a line search at once,
+// 2^-Wr .. 2^-(Wr+W-1) in round r, of which the first accepted one counts.  A few fits in ten thousand
 // (moments on the boundary of their cone) search 30 and more halvings in each of up to 200 iterations,
-// and one of them on one warp (7,157 trial points, 66 ms) took longer than all others together.  The step is solved by one warp of each CTA (a CTA's four warps sit
-// on the four quarters of its SM, each with an FP64 pipe of its own); every thread keeps the state.
+// and one of them on one warp (7,157 trial points, 66 ms) took longer than all others together.  The step is solved
+// by one warp of each CTA (a CTA's four warps sit on the four quarters of its SM, each with an FP64 pipe of
+// its own); every thread keeps the state.
+// `one`: a CTA by itself, W = 4: where there are thousands of such fits the steps tried for nothing fill the pipes.
 constexpr int kSlowCtas = 4, kSlowThreads = 128, kSlowWarps = kSlowCtas * kSlowThreads / 32;
 struct SlowShared {
     double x[kApproxMaxN];
@@ -1794,11 +1796,16 @@ struct SlowShared {
     int singular;
     long long job;
 };
+__device__ __forceinline__ void slow_sync(const cooperative_groups::cluster_group &cl, bool one) {
+    if (one) __syncthreads();
+    else cl.sync();
+}
 template <int J>
-__device__ bool maxent_fit_cluster(const cooperative_groups::cluster_group &cl, SlowShared &sh, int n, const double *m,
-                                   double *a) {
+__device__ bool maxent_fit_cluster(const cooperative_groups::cluster_group &cl, bool one, SlowShared &sh, int n,
+                                   const double *m, double *a) {
     constexpr int NV = 2 * J + 2;
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, rank = (int)cl.block_rank(), me = rank * 4 + wp;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, rank = (int)cl.block_rank();
+    const int W = one ? kSlowThreads / 32 : kSlowWarps, me = one ? wp : rank * 4 + wp;
     double st[J + 1], an[J + 1], sum[NV], v[NV], gn[J + 1], phi = 0.0, phin, gmax = 0.0, gnmax, gst = 0.0;
     int buf = 0;
 #pragma unroll
@@ -1845,12 +1852,12 @@ __device__ bool maxent_fit_cluster(const cooperative_groups::cluster_group &cl, 
 #pragma unroll
                 for (int i = 0; i < NV; ++i) sh.sum[buf][wp][i] = sum[i];
             }
-            cl.sync();  // this round's sums are in; the other buffer is free again after the next one
+            slow_sync(cl, one);  // this round's sums are in; the other buffer is free again after the next one
             int found = -1;
-            for (int c = kSlowWarps - 1; c >= 0; --c)
-                if (cl.map_shared_rank(&sh, c / 4)->take[buf][c & 3]) found = c;
+            for (int c = W - 1; c >= 0; --c)
+                if ((one ? &sh : cl.map_shared_rank(&sh, c / 4))->take[buf][c & 3]) found = c;
             if (found >= 0) {
-                const double *src = cl.map_shared_rank(&sh, found / 4)->sum[buf][found & 3];
+                const double *src = (one ? &sh : cl.map_shared_rank(&sh, found / 4))->sum[buf][found & 3];
 #pragma unroll
                 for (int i = 0; i < NV; ++i) sum[i] = src[i];
                 t = tround;
@@ -1860,7 +1867,7 @@ __device__ bool maxent_fit_cluster(const cooperative_groups::cluster_group &cl, 
             }
             buf ^= 1;
             if (found >= 0) break;
-            for (int c = 0; c < kSlowWarps; ++c) tround *= 0.5;
+            for (int c = 0; c < W; ++c) tround *= 0.5;
             if (tround < 1e-12) return gmax <= 1e-10;
         }
         trial<J>(a, sum, m, true, 0.0, 0.0, 0.0, 1.0, phi, gn, gmax);
@@ -2058,14 +2065,18 @@ __global__ void __cluster_dims__(kSlowCtas, 1, 1) __launch_bounds__(kSlowThreads
     __shared__ SlowShared sh;
     const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
     const int t = threadIdx.x;
-    const bool first = cl.block_rank() == 0 && t == 0;
     if (*pl.overflow) return;
     const long long jobs = (long long)pl.slow[0];
+    // more than six a cluster: each CTA by itself (200 patterns of 2 and 3 clicks at order 2, 2121 such fits, whole
+    // calls: 6.3 -> 3.7 ms; 200 of 5 and 6 clicks at order 4, 4569 of them: 50 -> 27 ms).  With fewer the longest
+    // fit counts: of seven batches with 640 to 850 three were up to a third slower that way.
+    const bool one = jobs > 6ll * (gridDim.x / kSlowCtas);
+    const bool first = (one || cl.block_rank() == 0) && t == 0;
     for (;;) {
         if (first) sh.job = (long long)atomicAdd(pl.slow + 1, 1ull);
-        cl.sync();
-        const long long job = cl.map_shared_rank(&sh, 0)->job;
-        cl.sync();  // read by all before the next one is drawn, and before a CTA exits
+        slow_sync(cl, one);
+        const long long job = (one ? &sh : cl.map_shared_rank(&sh, 0))->job;
+        slow_sync(cl, one);  // read by all before the next one is drawn, and before a CTA exits
         if (job >= jobs) break;
         const long long gs = pl.sec_slow[job];
         int lo = 0, hi = n_pat;
@@ -2084,16 +2095,16 @@ __global__ void __cluster_dims__(kSlowCtas, 1, 1) __launch_bounds__(kSlowThreads
         for (int j = top; j >= 0 && !done; --j) {
             double np = 1.0;
             for (int i = 0; i <= j; ++i) { m[i] = mu[i] / np / mu[0]; np *= n; }
-            done = j == 4   ? maxent_fit_cluster<4>(cl, sh, n, m, a)
-                   : j == 3 ? maxent_fit_cluster<3>(cl, sh, n, m, a)
-                   : j == 2 ? maxent_fit_cluster<2>(cl, sh, n, m, a)
-                   : j == 1 ? maxent_fit_cluster<1>(cl, sh, n, m, a)
-                            : maxent_fit_cluster<0>(cl, sh, n, m, a);
+            done = j == 4   ? maxent_fit_cluster<4>(cl, one, sh, n, m, a)
+                   : j == 3 ? maxent_fit_cluster<3>(cl, one, sh, n, m, a)
+                   : j == 2 ? maxent_fit_cluster<2>(cl, one, sh, n, m, a)
+                   : j == 1 ? maxent_fit_cluster<1>(cl, one, sh, n, m, a)
+                            : maxent_fit_cluster<0>(cl, one, sh, n, m, a);
             if (done) {
                 val = mu[0] * exp(-a[0]);
                 if (j != top) fell = true;
             }
-            cl.sync();  // the next fit writes its sums where a slower CTA may still read this one's
+            slow_sync(cl, one);  // the next fit writes its sums where a slower CTA may still read this one's
         }
         if (!done) fell = true;
         if (first) pl.sec_part[gs] = fell ? -val : val;   // the sign marks a fallback
