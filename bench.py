@@ -406,7 +406,8 @@ def run_gpu(args):
     kms = sweep_ms / max(launches, 1)
     achieved = flops / (kms * 1e-3)
     kname = {"fp32": "sweep_kernel<float>", "fp64": "sweep_kernel<double>",
-             "dd": "sweep_kernel<sq> (110-bit software floating point)", "fx": "sweep_fx_kernel"}[prec]
+             "dd": "sweep_kernel<sq> (110-bit software floating point), with the result kernels and the "
+                   "double-double pass", "fx": "sweep_fx_kernel"}[prec]
     roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": DRAM_TRAFFIC.get(prec),
                 "kernel": kname, "kernel_ms": kms, "flops_per_launch": flops,

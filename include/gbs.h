@@ -45,8 +45,9 @@ typedef enum {
                               fixed number of steps and report GBS_E_FIT), and no kernel waits
                               on another */
     GBS_E_FIT = 7,         /* approximation: a sector fit fell back to a lower order */
-    GBS_E_RANGE = 8,       /* GBS_FX: a pivot determinant below 2^-8 or an entry of O beyond
-                              4 left the fixed-point range (evaluate in GBS_DD instead) */
+    GBS_E_RANGE = 8,       /* GBS_FX: a pivot determinant below 2^-8, an entry of O beyond 4 or an
+                              I - O that is not positive definite left the fixed-point range
+                              (evaluate in GBS_DD instead) */
     GBS_E_FLOOR = 9        /* approximation with FP32 minors: sectors below the FP32 noise floor
                               (1e-6 of the largest tilted sector) could carry 1e-4 or more of the
                               estimate, which FP32 moments cannot resolve; logP is returned but
@@ -60,17 +61,20 @@ typedef enum {
                             signed sum cancels beyond FP64 (kappa u64 >~ 1e-10).  110-bit software
                             floating point on the integer pipes, double-double itself on the FP64
                             pipes where kappa exceeds 1e24 */
-    GBS_FX = 3,          /* exact sum only: 128-bit fixed-point (Q16.112) factorisations on the
-                            integer pipes, double-double prefactors and sum; accuracy as GBS_DD
-                            (~2^-100 per term) at a fraction of its cost.  Needs every pivot
+    GBS_FX = 3,          /* exact sum only: 128-bit fixed-point factorisations (30-bit limbs, 2^-114) on
+                            the integer pipes, prefactors m 2^e and sums of 512 terms as 128-bit
+                            integers times 2^e, those added in double-double; ~2^-100 per term, at a
+                            fraction of GBS_DD's cost.  Needs every pivot
                             determinant of the Schur recursion >= 2^-8 (true when the largest
                             eigenvalue of sigma_Q is below 16); else GBS_E_RANGE */
     GBS_FF = 4,          /* approximation only: float-float (~48-bit) complex minors on the FP32
                             pipes; FP64-class moments at a fraction of FP64's cost (n <= 79) */
     GBS_AUTO = 5,        /* exact sum: GBS_FX, then GBS_DD for the patterns it reports GBS_E_RANGE,
                             then GBS_FX192 for the valid results whose err_bound exceeds 1e-10 (on
-                            the device, no host synchronisation; gbs_reserve covers it; a batch
-                            that needs neither rerun costs two sweeps over no units);
+                            the device; the host waits where GBS_FX would, once, and not at
+                            all after a gbs_reserve that covers the call (a rerun whose units
+                            might not fit an unreserved workspace reads their number back); a
+                            batch that needs neither rerun costs two sweeps over no units);
                             approximation: GBS_FF */
     GBS_FX192 = 6        /* exact sum only: 192-bit fixed point (Q16.176), prefactors and sums as
                             192-bit mantissas with exponents, unit sums added exactly per pattern:

@@ -150,14 +150,12 @@ __device__ __forceinline__ int fl_chol_bad(const fl &p00, const fx &det) {
 __device__ __forceinline__ fx fl_rsqrt(const fx &x) { return fx_rsqrt_at(x, 13); }  // ulp 2^-114
 
 // the 2x2 block elimination's quantities (see fx.cuh): a = p00^{-1/2}, b = det^{-1/2} p00^{1/2},
-// c = p01 det^{-1/2}, rs = det^{-1/2} (packed Q16.112)
+// c = p01 det^{-1/2}, from a and rs = det^{-1/2} (packed Q16.112)
 struct fl_piv {
     fl5 a, b, c;
-    fx rs;
 };
 __device__ __forceinline__ fl_piv fl_pivot_from(const fl &p00, const fl &p01, const fx &ya, const fx &rs) {
     fl_piv v;
-    v.rs = rs;
     v.a = fl5_at123(ya);
     const fl5 r = fl5_at126(rs);
     int64_t pc[5] = {0, 0, 0, 0, 0}, pq[5] = {0, 0, 0, 0, 0}, pb[5] = {0, 0, 0, 0, 0};

@@ -46,7 +46,6 @@ __device__ __forceinline__ fx &operator+=(fx &a, const fx &b) { return a = a + b
 __device__ __forceinline__ bool fx_positive(const fx &a) {
     return (int32_t)a.w[3] > 0 || (a.w[3] == 0u && (a.w[2] | a.w[1] | a.w[0]) != 0u);
 }
-__device__ __forceinline__ bool operator>(const fx &a, const fx &b) { return fx_positive(a - b); }
 
 // Limbs 3..7 of the unsigned 256-bit product a*b, without the partial products of
 // columns 0 and 1 and the low halves of column 2.  Row i adds a_i * b; after row i
@@ -114,28 +113,19 @@ __device__ __forceinline__ void fx_sub_masked(uint32_t &p4, uint32_t &p5, uint32
 }
 __device__ __forceinline__ uint32_t fx_sign_mask(const fx &a) { return (uint32_t)((int32_t)a.w[3] >> 31); }
 
-// signed product: the unsigned product minus 2^128 (b [a < 0] + a [b < 0]), bits 112..239
-__device__ __forceinline__ fx operator*(const fx &a, const fx &b) {
-    uint32_t p3, p4, p5, p6, p7;
-    fx_mul_upper(a, b, p3, p4, p5, p6, p7);
-    fx_sub_masked(p4, p5, p6, p7, b, fx_sign_mask(a));
-    fx_sub_masked(p4, p5, p6, p7, a, fx_sign_mask(b));
-    return fx_shift_out(p3, p4, p5, p6, p7);
-}
 // a * b for a, b >= 0
 __device__ __forceinline__ fx fx_mul_uu(const fx &a, const fx &b) {
     uint32_t p3, p4, p5, p6, p7;
     fx_mul_upper(a, b, p3, p4, p5, p6, p7);
     return fx_shift_out(p3, p4, p5, p6, p7);
 }
-// a * b for b >= 0, a of either sign
+// a * b for b >= 0, a of either sign: the unsigned product minus 2^128 b [a < 0], bits 112..239
 __device__ __forceinline__ fx fx_mul_su(const fx &a, const fx &b) {
     uint32_t p3, p4, p5, p6, p7;
     fx_mul_upper(a, b, p3, p4, p5, p6, p7);
     fx_sub_masked(p4, p5, p6, p7, b, fx_sign_mask(a));
     return fx_shift_out(p3, p4, p5, p6, p7);
 }
-__device__ __forceinline__ fx &operator*=(fx &a, const fx &b) { return a = a * b; }
 
 __device__ __forceinline__ fx fx_from_i128(__int128 v) {
     fx r;
@@ -178,7 +168,7 @@ __device__ __forceinline__ dd fx_to_dd(const fx &a) {
 
 
 // x^{-1/2} in Q16.112 for a packed x with ulp 2^-(127 - h0) (h0 = 15: Q16.112; h0 = 13: ulp
-// 2^-114) in [2^-11, 2^11); pivots lie in [2^-9, 25].
+// 2^-114) in [2^-11, 2^11); pivots that pass the checks lie in [2^-10.4, 25].
 //  * x = m 4^h', m in [1/2, 2): an odd shift s of X (m = 1 for the powers of four, which stay exact);
 //  * an FP32 estimate r0 of r = m^{-1/2} (relative error below 2^-22), 24 bits, scale 30;
 //  * one step of third order on the top 64 bits W of m: with e = 1 - m r0^2, r = r0 (1 + e/2 +
@@ -187,8 +177,8 @@ __device__ __forceinline__ dd fx_to_dd(const fx &a) {
 //  * one Newton step against the whole of x: with |e| < 2^-59 known, only the bits of m R^2 below
 //    2^-59 are formed (columns 3, 4 and the low half of 5 of X R^2: nine products instead of two
 //    full 128 x 64 ones), E = e 2^121, and y += y e / 2.
-// The result is within 1.1 units of 2^-112 (a big-integer emulation over [2^-10, 2^5]); exact for
-// powers of four.  Inputs outside the range (checked by the callers) give a finite, meaningless
+// The result is within one unit of 2^-112 (a big-integer emulation over the whole range, the FP32 estimate off
+// by up to two units); exact for powers of four.  Inputs outside the range (checked by the callers) give a finite, meaningless
 // result.
 static __device__ __noinline__ fx fx_rsqrt_at(fx x, int h0) {
     int lz = __clz((int)x.w[3]);

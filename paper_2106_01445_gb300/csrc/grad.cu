@@ -610,7 +610,7 @@ __device__ void reverse_pivots(const dd *Mx, dd *G, int D, int np, const dd *Qs,
 // (the adjoint of a shared step is linear in what flows into it), and the chunk's partial
 // Gbar and T are written; the chunks of a pattern are summed in order afterwards.
 __global__ void __launch_bounds__(kTreeThreads) grad_tree_dd_kernel(int M, const double *__restrict__ O,
-                                                               const uint64_t *__restrict__ pats, int n_pat,
+                                                               const uint64_t *__restrict__ pats,
                                                                const int *__restrict__ chunk_p,
                                                                const long long *__restrict__ chunk_u, size_t pst,
                                                                const int *__restrict__ redo, dd *__restrict__ part,
@@ -1321,7 +1321,7 @@ int grad_sigmaQ(gbs_ctx *ctx, int M, const double *O, const double *logdet, cons
     const size_t dsmem = sizeof(dd) * (size_t)ddk::kTreeSmem;
     GBS_CUDA(ctx, cudaFuncSetAttribute(ddk::grad_tree_dd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsmem));
     ddk::grad_tree_dd_kernel<<<(unsigned)chunks, ddk::kTreeThreads, dsmem, ctx->stream>>>(
-        M, O, pats, n_pat, chunk_p, chunk_u, pst, redo, (dd *)part, (dd *)pT, flags);
+        M, O, pats, chunk_p, chunk_u, pst, redo, (dd *)part, (dd *)pT, flags);
     GBS_CUDA(ctx, cudaGetLastError());
     st = gbs_timing_end(ctx);
     if (st) return st;

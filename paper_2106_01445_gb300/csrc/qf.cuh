@@ -1,14 +1,18 @@
 // Software floating point with a 110-bit significand on the integer pipes, for the double-double
 // paths.  The FP64 pipe of this GPU issues two lanes a clock and SM (a double-double multiply-
 // subtract c - a0 b0 - a1 b1 is 27 of its instructions, 216 clocks of an SM a warp); the same
-// operation here is about 130 integer instructions, 33 to 40 clocks, with four more bits.
+// operation here is about 130 integer instructions, 33 to 40 clocks, on 110 bits.
 //
 // A number is M 2^-110 4^e: M a signed 112-bit integer in three 30-bit limbs and a signed 22-bit top
-// limb, normalised to 2^109 <= |M| < 2^111 (zero: M = 0), e in [-512, 511] (the range of a double), in
-// 16 bytes: w[0..2] the limbs, w[3] = top limb 2^10 + e + 512.  Results are truncated (relative
-// error below 2^-109; a sum: of the larger operand).  Limbs of 30 bits let every partial product of
-// a column accumulate in 64 bits without a carry (fl.cuh); the exponent's base 4 keeps the
-// normalising shift even, so that reciprocal square roots need no odd case of their own.
+// limb, normalised to 2^109 <= |M| <= 2^111 (zero: M = 0), e in [-512, 511] (the range of a double), in
+// 16 bytes: w[0..2] the limbs, w[3] = top limb 2^10 + e + 512.  Results are truncated: a product below 2^-109
+// of itself, a sum below 2^-108 of the larger operand.  The fused forms shift the factor of a smaller
+// product in the product's place, which loses up to 2^-107 of the largest term a factor shifted: below
+// 2^-106 of it for two terms (dot2, fma), 2^-105 for three (fms2), k 2^-107 for k (dot).  (Against a 192-bit sum
+// the sweep's results are off by less than 2^-117 kappa, double-double's by 2^-112: truncations average out.)
+// Limbs of 30 bits let every partial product of a column accumulate in 64 bits without a carry (fl.cuh);
+// the exponent's base 4 keeps the normalising shift even, so that reciprocal square roots need no odd
+// case of their own.
 // Overflow saturates the exponent (a saturated number converts to NaN), underflow gives zero.
 #pragma once
 #include <stdint.h>
@@ -168,7 +172,7 @@ template <bool NEG> QF_FN qf qf_sum(const qf &x, const qf &y) {
 QF_FN qf operator+(const qf &x, const qf &y) { return qf_sum<false>(x, y); }
 QF_FN qf operator-(const qf &x, const qf &y) { return qf_sum<true>(x, y); }
 QF_FN qf operator-(const qf &x) { return qf_zero() - x; }
-// x / 2 (a product would be truncated; the shift is exact)
+// x / 2 (truncated by at most one unit of M)
 QF_FN qf qf_half(const qf &x) {
     using namespace qfn;
     const reg a = unpack(x);

@@ -106,11 +106,11 @@ template <> struct Prec<sq> {
     static constexpr bool fixed = false;
     static constexpr int wrow = 2;
 };
-// 128-bit fixed point: the matrices of the breadth-first levels and of the register bottom
-// in limb form (fl.cuh), the prefix, the prefactors and the sums packed Q16.112 (fx.cuh).
-// Products truncated to 2^-112 or finer and the pivot rsqrt (within 1.1 units of 2^-112) give
-// each factor a relative error far below 2^-100 while its pivot determinant stays >= 2^-8;
-// unit sums in double-double.
+// 128-bit fixed point (its sweep: sweep_fx.cuh): every matrix, from the gather to the register bottom, in limb
+// form (fl.cuh), prefactors m 2^e with m in limbs, sub-unit sums packed Q16.112 (fx.cuh) times 2^e, each
+// term truncated to 2^-108 of the largest prefactor.  Products truncated to 2^-112 or finer and the
+// pivot rsqrt (within one unit of 2^-112) give each factor a relative error far below 2^-100 while its
+// pivot determinant stays >= 2^-8; unit sums in double-double.
 template <> struct Prec<fx> {
     static constexpr int B = 2, idx = GBS_FX;
     using Tau = dd;
@@ -1158,15 +1158,9 @@ __global__ void __launch_bounds__(kThreads, std::is_same_v<T, sq> ? 3 : 0) sweep
                         S = S + s_vred[w];
                         AB += s_ared[w];
                     }
-                    if constexpr (std::is_same<T, fx6>::value) {
-                        // the sub-unit's sum S 2^(em + 4) times its prefix factor, added to the
-                        // unit's sum, all as m 2^e with 192-bit mantissas
-                        uacc6 = fxe6_add(uacc6, fxe6_norm(S, em + 4) * tsub);
-                    } else {
-                        const dd sv = fx_to_dd(S);
-                        const double sc = ldexp(1.0, em + 4);
-                        unit_add(u_hi, u_lo, tsub, sv.hi * sc, sv.lo * sc);
-                    }
+                    // the sub-unit's sum S 2^(em + 4) times its prefix factor, added to the
+                    // unit's sum, all as m 2^e with 192-bit mantissas
+                    uacc6 = fxe6_add(uacc6, fxe6_norm(S, em + 4) * tsub);
                     u_abs += tau_abs(tsub) * ldexp((double)AB, em);
                 }
             } else if (t < (1 << L_eff)) {
