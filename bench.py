@@ -36,7 +36,7 @@ import gbs_inputs as g  # noqa: E402
 METRIC = "subset logdets/sec and click-pattern log P/sec at stated rel. error vs FP64 oracle"
 # dram__bytes_read.sum + dram__bytes_write.sum of one sweep launch on this workload
 # (ncu captures summarised under profiles/); None where no capture of the current kernel exists
-DRAM_TRAFFIC = {"fp32": 129536.0, "dd": None, "fp64": 130048.0, "fx": 129280.0}
+DRAM_TRAFFIC = {"fp32": 129536.0, "dd": 297216.0, "fp64": 130048.0, "fx": 146688.0}
 UNIT = "subset logdets/s"
 # 32-bit multiply-adds of one fixed-point update entry: two products of four 30-bit limbs
 # without their lowest columns, 10 wide multiply-adds each, which take two issue slots of the
