@@ -480,9 +480,9 @@ __global__ void __launch_bounds__(kTreeThreads, 2) grad_tree_kernel(int M, const
 // ---- the same adjoint in double-double --------------------------------------------------------
 // For patterns whose sum cancels by more than kRedo: there the result is limited by the arithmetic
 // (a relative error of about 3e-34 kappa in double-double, a tenth of that in qf, against a quadruple
-// precision sum over the subsets), so the two differ by 1e-9 and more, and callers keep the values
-// they had.  CTAs of other patterns leave at once.  A batch that has such patterns pays for one chunk's
-// time here (about 5 ms on the 32-mode workload).
+// precision sum over the subsets), the two come to differ by 1e-9, and callers keep the values
+// they had.  What the guess names beforehand (kappa.cuh) comes here alone.  CTAs of other patterns leave at
+// once.  A batch with a few such patterns pays for one chunk's time here (about 5 ms on the 32-mode workload).
 namespace ddk {
 constexpr int kTM = 7;                   // modes of a unit's subtree (2^7 leaves)
 constexpr int kTreeThreads = 128;

@@ -8,8 +8,10 @@
 // 30 of the 35 patterns with kappa above 1e26, 8 of 22 between 1e24 and 1e26, 7 of 39 between 1e22 and 1e24
 // and 1 of 384 below.  (Blocks of four modes, at 25 times the work, told no better.)
 //
-// Measured on a GB300: GBS_DD on 40 patterns of 16 to 18 clicks at 100 modes, kappa 1e25 to 5e29, 7.68 -> 6.43 ms
-// (double-double alone 5.17); batches without such patterns unchanged.
+// Measured on a GB300: GBS_DD on 40 patterns of 18 clicks at 100 modes 12.50 -> 8.54 ms (double-double alone
+// 8.51), of 16 to 18 clicks (kappa 1e25 to 5e29, some guesses below the line) 7.68 -> 6.43 (5.17); the gradient of 64
+// patterns of 15 to 17 clicks at 40 modes, 62 of them above 1e24, 63.7 -> 50.8 ms (double-double alone 50.0);
+// batches without such patterns unchanged.
 #pragma once
 #include <stdint.h>
 
