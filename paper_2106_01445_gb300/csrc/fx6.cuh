@@ -7,6 +7,7 @@
 #pragma once
 #include <stdint.h>
 
+#include "fl.cuh"
 #include "fx.cuh"
 
 struct fx6 {
@@ -204,13 +205,11 @@ __device__ __forceinline__ fx6 fx6_from_double(double d) {
 __device__ __forceinline__ fx fx6_top(const fx6 &a) { return fx{{a.w[2], a.w[3], a.w[4], a.w[5]}}; }
 __device__ __forceinline__ fx6 fx6_widen(const fx &a) { return fx6{{0u, 0u, a.w[0], a.w[1], a.w[2], a.w[3]}}; }
 __device__ __forceinline__ double fx_to_double(const fx6 &a) { return fx_to_double(fx6_top(a)); }
-__device__ __forceinline__ int fx_pivot_bad(const fx6 &det) {
-    if (!fx_positive(det)) return 1;
-    return (int32_t)det.w[5] < 256 ? 2 : 0;
-}
-__device__ __forceinline__ int fx_chol_bad(const fx6 &p00, const fx6 &det) {
-    if (!fx_positive(p00)) return 1;
-    return fx_pivot_bad(det);
+// pivot check of a block with its determinant (flags: fl.cuh): its products are unsigned, so both diagonal
+// entries have to be positive before the determinant says anything
+__device__ __forceinline__ int fx_block_bad(const fx6 &p00, const fx6 &p11, const fx6 &det) {
+    if (!fx_positive(p00) || !fx_positive(p11) || !fx_positive(det)) return 1;
+    return (int32_t)det.w[5] < 256 ? kFlLost : 0;
 }
 // x^{-1/2}: the 128-bit reciprocal square root of x's leading 128 bits (relative error
 // ~2^-104 for x >= 2^-8), then one Newton step in 192 bits, y <- y + y e / 2 with
@@ -234,6 +233,13 @@ __device__ __forceinline__ fx6 fx_det2(const fx6 &p00, const fx6 &p01, const fx6
 // stored offset, u' = u + 2 > 0 (|u| <= sqrt(2) for a physical state), so that each entry needs
 // two unsigned products:
 //   c_ij - u_i . u_j = c_ij - (u'_i0 u'_j0 + u'_i1 u'_j1) + t_i + t_j,  t = 2 (u'0 + u'1) - 4.
+// An O that is no state's may leave that range and, past 2^15, the format: rows outside [-2, 6), and, where a
+// prefix pivot goes by W = B P^{-1} (below 113 for positive definite A <= 5 I), entries of W of 256 and more, are
+// noted in a word and reported as kFlLost.  Within them no entry wraps, and the pivots' checks tell the rest.
+__device__ __forceinline__ uint32_t fx_row_out(const fx6 &u0, const fx6 &u1) { return (u0.w[5] | u1.w[5]) >> 19; }
+__device__ __forceinline__ uint32_t fx_w_out(const fx6 &w0, const fx6 &w1) {
+    return ((w0.w[5] + (256u << 16)) | (w1.w[5] + (256u << 16))) >> 25;
+}
 struct fx6_piv {
     fx6 a, c, b, rs, det;
 };

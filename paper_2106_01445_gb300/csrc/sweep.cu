@@ -198,8 +198,12 @@ template <typename T> __device__ __forceinline__ T mul_pos(T a, T b) { return a 
 template <> __device__ __forceinline__ fx6 mul_pos<fx6>(fx6 a, fx6 b) { return fx_mul_uu(a, b); }
 // pivot check: 0 fine, 1 not positive (or NaN), 2 outside the fixed-point range
 template <typename T> __device__ __forceinline__ int pivot_bad(T det) { return det > T(0) ? 0 : 1; }
-template <> __device__ __forceinline__ int pivot_bad<fx6>(fx6 det) { return fx_pivot_bad(det); }
 template <> __device__ __forceinline__ int pivot_bad<sq>(sq det) { return qf_positive(det) && !qf_saturated(det) ? 0 : 1; }
+// the same of a pivot block; double-double and the like go by the determinant alone
+template <typename T> __device__ __forceinline__ int block_bad(const T &, const T &, const T &det) { return pivot_bad(det); }
+template <> __device__ __forceinline__ int block_bad<fx6>(const fx6 &p00, const fx6 &p11, const fx6 &det) {
+    return fx_block_bad(p00, p11, det);
+}
 // complex pivots: their determinants may have any argument in (-pi, pi); only zero or NaN is bad
 template <> __device__ __forceinline__ int pivot_bad<zc>(zc det) {
     return fabs(det.re) + fabs(det.im) > 0.0 ? 0 : 1;
@@ -494,7 +498,7 @@ __device__ __forceinline__ void dfs(const Src &A, T tau, int depth, int nreal, A
         }
     } else if constexpr (m == 1) {
         const T det = det2(p00, p01, p11);
-        if constexpr (Prec<T>::fixed || std::is_same_v<T, sq>) acc.bad |= pivot_bad(det);
+        if constexpr (Prec<T>::fixed || std::is_same_v<T, sq>) acc.bad |= block_bad(p00, p11, det);
         const T rs = rsq<T>(det);
         if constexpr (std::is_same_v<T, sq>) leaf_pair_sq<NEG, ONE>(acc, rs, tau, real);
         else leaf_pair<NEG>(acc, ONE ? rs : mul_pos(tau, rs), tau, real, cnt);
@@ -502,10 +506,13 @@ __device__ __forceinline__ void dfs(const Src &A, T tau, int depth, int nreal, A
         // symmetric form C - U U^T, U = B R^{-T} (offset rows)
         constexpr int d = 2 * (m - 1);
         const typename Prec<T>::Piv v = fx_pivot(p00, p01, p11);
-        acc.bad |= fx_chol_bad(p00, v.det);
+        acc.bad |= fx_block_bad(p00, p11, v.det);
         T u0[d], u1[d], tt[d];
 #pragma unroll
-        for (int i = 0; i < d; ++i) fx_urow(v, A(o, o + 2 + i), A(o + 1, o + 2 + i), u0[i], u1[i], tt[i]);
+        for (int i = 0; i < d; ++i) {
+            fx_urow(v, A(o, o + 2 + i), A(o + 1, o + 2 + i), u0[i], u1[i], tt[i]);
+            acc.bad |= fx_row_out(u0[i], u1[i]) ? kFlLost : 0;
+        }
         RegMat<T, m - 1> C;
 #pragma unroll
         for (int i = 0; i < d; ++i)
@@ -695,7 +702,7 @@ __device__ __forceinline__ typename Prec<T>::Tau elim_pivot(T *Mx, int D, int c0
     const T p00 = Mx[pidx(D, c0, c0)], p01 = Mx[pidx(D, c0, c0 + 1)], p11 = Mx[pidx(D, c0 + 1, c0 + 1)];
     const T det = det2(p00, p01, p11);
     if (t == 0) {
-        const int bad = pivot_bad(det);
+        const int bad = block_bad(p00, p11, det);
         if (bad) atomicOr(flag, bad);
     }
     const int Dt = D - c0 - 2;
@@ -704,8 +711,11 @@ __device__ __forceinline__ typename Prec<T>::Tau elim_pivot(T *Mx, int D, int c0
         const T inv = rs * rs;
         const T q00 = p11 * inv, q01 = mul_neg(p01, inv), q11 = p00 * inv;
         const T b0 = Mx[pidx(D, c0, c0 + 2 + t)], b1 = Mx[pidx(D, c0 + 1, c0 + 2 + t)];
-        Wb[2 * t] = dot2(q00, b0, q01, b1);
-        Wb[2 * t + 1] = dot2(q01, b0, q11, b1);
+        const T w0 = dot2(q00, b0, q01, b1), w1 = dot2(q01, b0, q11, b1);
+        Wb[2 * t] = w0;
+        Wb[2 * t + 1] = w1;
+        if constexpr (Prec<T>::fixed)
+            if (fx_w_out(w0, w1)) atomicOr(flag, kFlLost);
     }
     const typename Prec<T>::Tau rt = tau_of(det, rs);
     __syncthreads();
@@ -729,7 +739,7 @@ __device__ __forceinline__ typename Prec<T>::Tau elim_into(const T *Mx, int D, i
     const T p00 = Mx[pidx(D, c0, c0)], p01 = Mx[pidx(D, c0, c0 + 1)], p11 = Mx[pidx(D, c0 + 1, c0 + 1)];
     const T det = det2(p00, p01, p11);
     if (t == 0) {
-        const int bad = pivot_bad(det);
+        const int bad = block_bad(p00, p11, det);
         if (bad) atomicOr(flag, bad);
     }
     const int Dt = D - c0 - 2;
@@ -738,8 +748,11 @@ __device__ __forceinline__ typename Prec<T>::Tau elim_into(const T *Mx, int D, i
         const T inv = rs * rs;
         const T q00 = p11 * inv, q01 = mul_neg(p01, inv), q11 = p00 * inv;
         const T b0 = Mx[pidx(D, c0, c0 + 2 + t)], b1 = Mx[pidx(D, c0 + 1, c0 + 2 + t)];
-        Wb[2 * t] = dot2(q00, b0, q01, b1);
-        Wb[2 * t + 1] = dot2(q01, b0, q11, b1);
+        const T w0 = dot2(q00, b0, q01, b1), w1 = dot2(q01, b0, q11, b1);
+        Wb[2 * t] = w0;
+        Wb[2 * t + 1] = w1;
+        if constexpr (Prec<T>::fixed)
+            if (fx_w_out(w0, w1)) atomicOr(flag, kFlLost);
     }
     const typename Prec<T>::Tau rt = tau_of(det, rs);
     __syncthreads();
@@ -896,7 +909,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same_v<T, sq> ? 3 : 0) sweep
             } else {
                 const int si = modes[a] + (i & 1) * M, sj = modes[b] + (j & 1) * M;
                 const double o = O[(size_t)si * N2 + sj];
-                if (Prec<T>::fixed && !(fabs(o) <= 4.0)) atomicOr(&s_flag, 2);
+                if (Prec<T>::fixed && !(fabs(o) <= 4.0)) atomicOr(&s_flag, kFlLost);
                 if (std::is_same_v<T, sq> && !(fabs(o) <= 0x1p100)) atomicOr(&s_flag, 1);
                 v = a_entry_t<T>(i == j ? 1.0 : 0.0, o, pl.t_re, pl.t_im);
             }
@@ -1009,7 +1022,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same_v<T, sq> ? 3 : 0) sweep
                             const Node tp = NIO::ld(tsrc, cp);
                             NIO::st(tdst, 2 * cp, tp);
                             NIO::st(tdst, 2 * cp + 1, node_times(tp, v.rs));
-                            const int bad = fx_chol_bad(p00, det);
+                            const int bad = fx_block_bad(p00, p11, det);
                             if (bad) atomicOr(&s_flag, bad);
                         }
                     }
@@ -1030,6 +1043,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same_v<T, sq> ? 3 : 0) sweep
                 }
                 __syncthreads();
                 // (b) the rows of W = B P^{-1} (fixed point: of U = B R^{-T}), dc per parent
+                uint32_t out = 0;
                 for (int f = t; f < np * dc; f += kThreads) {
                     const int cp = f / dc, i = f - cp * dc;
                     const T *P = src + cp * sstr;
@@ -1037,13 +1051,18 @@ __global__ void __launch_bounds__(kThreads, std::is_same_v<T, sq> ? 3 : 0) sweep
                     if constexpr (Prec<T>::fixed) {
                         const typename Prec<T>::Piv v{Qb[3 * cp], Qb[3 * cp + 1], Qb[3 * cp + 2], konst<T>(0.0),
                                                       konst<T>(0.0)};
-                        fx_urow(v, b0, b1, Wb[3 * f], Wb[3 * f + 1], Wb[3 * f + 2]);
+                        T u0, u1;
+                        fx_urow(v, b0, b1, u0, u1, Wb[3 * f + 2]);
+                        Wb[3 * f] = u0;
+                        Wb[3 * f + 1] = u1;
+                        out |= fx_row_out(u0, u1);
                     } else {
                         const T q00 = Qb[3 * cp], q01 = Qb[3 * cp + 1], q11 = Qb[3 * cp + 2];
                         Wb[2 * f] = dot2(q00, b0, q01, b1);
                         Wb[2 * f + 1] = dot2(q01, b0, q11, b1);
                     }
                 }
+                if (out) atomicOr(&s_flag, kFlLost);
                 __syncthreads();
                 // (c) both children of every parent: the exclude child is the parent's
                 // trailing block, the include child its Schur complement
@@ -1206,7 +1225,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same_v<T, sq> ? 3 : 0) sweep
                 for (int k = 0; k < 6; ++k) mw[k] = r.m.w[k];
                 out[3] = (double)r.e;
                 out[4] = u_abs * tau_abs(tpre);
-                if (s_flag) atomicOr(pl.pflags + sp, s_flag);
+                if (s_flag) atomicOr(pl.pflags + sp, fl_unit_flags(s_flag));
             }
             __syncthreads();
         } else {
